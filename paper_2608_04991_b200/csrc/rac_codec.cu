@@ -160,26 +160,21 @@ __global__ void __launch_bounds__(256, 2) calib_kernel(const CodecParams p) {
         const uint32_t rs = xs + row_bytes;
 
         if (valid) {
-            u64 x2[16], r2[16];
+            uint32_t xw[16], rw[16];   // packed bf16, slot order
 #pragma unroll
             for (int j = 0; j < 4; j++) {
-                uint4 w = lds128(xs + off[j]);
-                x2[4 * j + 0] = bf16x2_to_p(w.x);
-                x2[4 * j + 1] = bf16x2_to_p(w.y);
-                x2[4 * j + 2] = bf16x2_to_p(w.z);
-                x2[4 * j + 3] = bf16x2_to_p(w.w);
+                const uint4 w = lds128(xs + off[j]);
+                xw[4 * j + 0] = w.x; xw[4 * j + 1] = w.y; xw[4 * j + 2] = w.z; xw[4 * j + 3] = w.w;
             }
             if (has_ref) {
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
-                    u64 rr[4];
-                    load_ref_slot(rs + off[j], p.gain, p.bias, (int)(off[j] >> 1), rr);
-#pragma unroll
-                    for (int i = 0; i < 4; i++) r2[4 * j + i] = rr[i];
+                    const uint4 w = load_ref_words(rs + off[j], p.gain, p.bias, (int)(off[j] >> 1));
+                    rw[4 * j + 0] = w.x; rw[4 * j + 1] = w.y; rw[4 * j + 2] = w.z; rw[4 * j + 3] = w.w;
                 }
             } else {
 #pragma unroll
-                for (int i = 0; i < 16; i++) r2[i] = 0ull;
+                for (int i = 0; i < 16; i++) rw[i] = 0u;
             }
             u64 a2, b2;
             float4 st;
@@ -190,7 +185,7 @@ __global__ void __launch_bounds__(256, 2) calib_kernel(const CodecParams p) {
                 a2 = pack2(a, a);
                 b2 = pack2(b, b);
             } else {
-                fit_group(x2, r2, has_ref, p.lpg, p.inv_group, group_mask, p.status, a2, b2, nullptr, &st);
+                fit_group(xw, rw, has_ref, p.lpg, p.inv_group, group_mask, p.status, a2, b2, nullptr, &st);
             }
             if (MOMENTS) {
                 if (!timed_out && (lane & (p.lpg - 1)) == 0) p.moments[tok * p.J + (tid >> p.lpg_shift)] = st;
@@ -203,8 +198,8 @@ __global__ void __launch_bounds__(256, 2) calib_kernel(const CodecParams p) {
 #pragma unroll
                 for (int hh = 0; hh < 2; hh++) {
                     float e0, e1, e2, e3;
-                    unpack2(psub(x2[4 * j + 2 * hh], pfma(a2, r2[4 * j + 2 * hh], b2)), e0, e1);
-                    unpack2(psub(x2[4 * j + 2 * hh + 1], pfma(a2, r2[4 * j + 2 * hh + 1], b2)), e2, e3);
+                    unpack2(sub_pair(xw[4 * j + 2 * hh], pfma(a2, bf16x2_to_p(rw[4 * j + 2 * hh]), b2)), e0, e1);
+                    unpack2(sub_pair(xw[4 * j + 2 * hh + 1], pfma(a2, bf16x2_to_p(rw[4 * j + 2 * hh + 1]), b2)), e2, e3);
                     float4 v = acc[(2 * q + hh) * nt + tid];
                     v.x = __fmaf_rn(e0, e0, v.x);
                     v.y = __fmaf_rn(e1, e1, v.y);
@@ -378,26 +373,21 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
 
         if (valid) {
             // ---- (1) the slab: 4 slots of 8 channels, slot j holds piece (j + rot) & 3
-            u64 x2[16], r2[16];
+            uint32_t xw[16], rw[16];   // packed bf16, slot order
 #pragma unroll
             for (int j = 0; j < 4; j++) {
-                uint4 w = lds128(xs + off[j]);
-                x2[4 * j + 0] = bf16x2_to_p(w.x);
-                x2[4 * j + 1] = bf16x2_to_p(w.y);
-                x2[4 * j + 2] = bf16x2_to_p(w.z);
-                x2[4 * j + 3] = bf16x2_to_p(w.w);
+                const uint4 w = lds128(xs + off[j]);
+                xw[4 * j + 0] = w.x; xw[4 * j + 1] = w.y; xw[4 * j + 2] = w.z; xw[4 * j + 3] = w.w;
             }
             if (has_ref) {
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
-                    u64 rr[4];
-                    load_ref_slot(rs + off[j], p.gain, p.bias, (int)(off[j] >> 1), rr);
-#pragma unroll
-                    for (int i = 0; i < 4; i++) r2[4 * j + i] = rr[i];
+                    const uint4 w = load_ref_words(rs + off[j], p.gain, p.bias, (int)(off[j] >> 1));
+                    rw[4 * j + 0] = w.x; rw[4 * j + 1] = w.y; rw[4 * j + 2] = w.z; rw[4 * j + 3] = w.w;
                 }
             } else {
 #pragma unroll
-                for (int i = 0; i < 16; i++) r2[i] = 0ull;
+                for (int i = 0; i < 16; i++) rw[i] = 0u;
             }
             // ---- (2) Eq. 6 and wire rounding
             u64 a2, b2;
@@ -410,7 +400,7 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
                 b2 = pack2(b, b);
             } else {
                 uint32_t coef_word;
-                fit_group(x2, r2, has_ref, lpg, p.inv_group, group_mask, p.status, a2, b2, &coef_word);
+                fit_group(xw, rw, has_ref, lpg, p.inv_group, group_mask, p.status, a2, b2, &coef_word);
                 if ((lane & (lpg - 1)) == 0) reinterpret_cast<uint32_t *>(rec)[tid >> lpg_shift] = coef_word;
             }
 
@@ -438,8 +428,8 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
                     uint32_t bits8[8];
 #pragma unroll
                     for (int i = 0; i < 4; i++) {
-                        const u64 rt = pfma(a2, r2[4 * j + i], b2);
-                        const u64 e = psub(x2[4 * j + i], rt);
+                        const u64 rt = pfma(a2, bf16x2_to_p(rw[4 * j + i]), b2);
+                        const u64 e = sub_pair(xw[4 * j + i], rt);
                         float v0, v1, t0, t1;
                         unpack2(pmul(e, inv2[i]), v0, v1);
                         t0 = fminf(fmaxf(v0, -qmax), qmax);
@@ -464,8 +454,8 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
                     // [-2^(BITS-1), 2^(BITS-1)-1], whose upper end is Qmax)
 #pragma unroll
                     for (int i = 3; i >= 0; i--) {
-                        const u64 rt = pfma(a2, r2[4 * j + i], b2);
-                        const u64 e = psub(x2[4 * j + i], rt);
+                        const u64 rt = pfma(a2, bf16x2_to_p(rw[4 * j + i]), b2);
+                        const u64 e = sub_pair(xw[4 * j + i], rt);
                         float v0, v1, t0, t1;
                         unpack2(pmul(e, inv2[i]), v0, v1);
                         v0 = fmaxf(v0, -qmax);

@@ -134,6 +134,35 @@ __device__ __forceinline__ u64 pmul(u64 a, u64 b) {
 __device__ __forceinline__ u64 bf16x2_to_p(uint32_t w) {
     return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
 }
+// One binary32 operand and one bf16 half of a packed word, one rounding: the same value as unpacking the half first, without
+// the unpacking.  (Per SM quarter a packed binary32 add or multiply-add takes 2 cycles for two values, and so does every
+// shift, mask or permute that an unpacking is made of; an add takes 1 for one value.)
+__device__ __forceinline__ float add_lo(uint32_t w, float c) {
+    float r;
+    asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; add.rn.f32.bf16 %0, l, %2;}" : "=f"(r) : "r"(w), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float add_hi(uint32_t w, float c) {
+    float r;
+    asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; add.rn.f32.bf16 %0, h, %2;}" : "=f"(r) : "r"(w), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float sub_lo(uint32_t w, float c) {   // low half - c
+    float r;
+    asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; sub.rn.f32.bf16 %0, l, %2;}" : "=f"(r) : "r"(w), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float sub_hi(uint32_t w, float c) {   // high half - c
+    float r;
+    asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; sub.rn.f32.bf16 %0, h, %2;}" : "=f"(r) : "r"(w), "f"(c));
+    return r;
+}
+// packed halves of w minus a packed pair
+__device__ __forceinline__ u64 sub_pair(uint32_t w, u64 c) {
+    float c0, c1;
+    unpack2(c, c0, c1);
+    return pack2(sub_lo(w, c0), sub_hi(w, c1));
+}
 // bits of a where m is set, bits of b elsewhere
 __device__ __forceinline__ uint32_t bitsel(uint32_t a, uint32_t b, uint32_t m) { return (a & m) | (b & ~m); }
 
@@ -197,6 +226,27 @@ __device__ __forceinline__ void load_ref_slot(uint32_t addr, const uint16_t *gai
 #pragma unroll
         for (int i = 0; i < 4; i++) r2[i] = bf16x2_to_p(ws[i]);
     }
+}
+
+// the same values left as packed bf16 words (the transformed reference is a bf16 value, so nothing is lost)
+__device__ __forceinline__ uint4 load_ref_words(uint32_t addr, const uint16_t *gain, const uint16_t *bias, int c) {
+    uint4 w = lds128(addr);
+    if (gain) {
+        const uint4 gw = __ldg(reinterpret_cast<const uint4 *>(gain + c));
+        const uint4 bw = __ldg(reinterpret_cast<const uint4 *>(bias + c));
+        const uint32_t gws[4] = {gw.x, gw.y, gw.z, gw.w};
+        const uint32_t bws[4] = {bw.x, bw.y, bw.z, bw.w};
+        uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const float g0 = half_bits_to_float(gws[i] & 0xffff), g1 = half_bits_to_float(gws[i] >> 16);
+            const float b0 = half_bits_to_float(bws[i] & 0xffff), b1 = half_bits_to_float(bws[i] >> 16);
+            ws[i] = f2_to_bf16x2(__fmaf_rn(g0, __uint_as_float(ws[i] << 16), b0),
+                                 __fmaf_rn(g1, __uint_as_float(ws[i] & 0xffff0000u), b1));
+        }
+        w = make_uint4(ws[0], ws[1], ws[2], ws[3]);
+    }
+    return w;
 }
 
 // the same for one pair of channels (c even), operation for operation
@@ -267,24 +317,22 @@ __device__ __forceinline__ void issue_token_loads(const CodecParams &p, Ctrl *ct
     if (row >= 0) bulk_load(stage_addr + r_off, ref_row_ptr<SUB>(p, row), row_bytes, bar);
 }
 
-// Eq. 6 for the group this thread belongs to: centred two-pass sums over the thread's 32 channels (packed
-// binary32, two accumulators per sum), butterflies over the group's lanes, the zero-variance rule, and wire
-// rounding of (alpha, beta) to binary16.  Returns the wire coefficients splatted for packed arithmetic; a16/b16
-// are their bit patterns.
-__device__ __forceinline__ void fit_group(const u64 (&x2)[16], const u64 (&r2)[16], bool has_ref, int lpg, float inv_group,
-                                          unsigned int group_mask, uint32_t *status, u64 &a2, u64 &b2,
+// Eq. 6 for the group this thread belongs to: centred two-pass sums over the thread's 32 channels (rows as packed bf16
+// words; two accumulators per sum and channel parity), butterflies over the group's lanes, the zero-variance rule, and
+// wire rounding of (alpha, beta) to binary16.  Returns the wire coefficients splatted for packed arithmetic; a16/b16
+// are their bit patterns.  The rows stay packed and enter the sums through the mixed adds above: half the registers of
+// unpacked rows and no unpacking (streaming pass at 131072 x 5120, group 128, 4-bit: with outliers 528 -> 485 us, without
+// 516 -> 467 us, with x_hat 726 -> 700 us).
+__device__ __forceinline__ void fit_group(const uint32_t (&xw)[16], const uint32_t (&rw)[16], bool has_ref, int lpg,
+                                          float inv_group, unsigned int group_mask, uint32_t *status, u64 &a2, u64 &b2,
                                           uint32_t *coef_word = nullptr, float4 *stats = nullptr) {
-    u64 sra = 0ull, srb = 0ull, sha = 0ull, shb = 0ull;
+    float ra0 = 0.f, ra1 = 0.f, rb0 = 0.f, rb1 = 0.f, xa0 = 0.f, xa1 = 0.f, xb0 = 0.f, xb1 = 0.f;
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
-        sra = padd(sra, r2[i]); srb = padd(srb, r2[i + 1]);
-        sha = padd(sha, x2[i]); shb = padd(shb, x2[i + 1]);
+        ra0 = add_lo(rw[i], ra0); ra1 = add_hi(rw[i], ra1); rb0 = add_lo(rw[i + 1], rb0); rb1 = add_hi(rw[i + 1], rb1);
+        xa0 = add_lo(xw[i], xa0); xa1 = add_hi(xw[i], xa1); xb0 = add_lo(xw[i + 1], xb0); xb1 = add_hi(xw[i + 1], xb1);
     }
-    float sr, sr_hi, sh, sh_hi;
-    unpack2(padd(sra, srb), sr, sr_hi);
-    unpack2(padd(sha, shb), sh, sh_hi);
-    sr += sr_hi;
-    sh += sh_hi;
+    float sr = (ra0 + rb0) + (ra1 + rb1), sh = (xa0 + xb0) + (xa1 + xb1);
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         if (lpg > o) {
@@ -296,12 +344,12 @@ __device__ __forceinline__ void fit_group(const u64 (&x2)[16], const u64 (&r2)[1
         if (status) atomicOr(status, RAC_STATUS_NONFINITE);
     }
     const float rbar = sr * inv_group, hbar = sh * inv_group;
-    const u64 rbar2 = pack2(rbar, rbar), hbar2 = pack2(hbar, hbar);
     u64 sxxa = 0ull, sxxb = 0ull, sxya = 0ull, sxyb = 0ull;
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
-        u64 dr0 = psub(r2[i], rbar2), dh0 = psub(x2[i], hbar2);
-        u64 dr1 = psub(r2[i + 1], rbar2), dh1 = psub(x2[i + 1], hbar2);
+        const u64 dr0 = pack2(sub_lo(rw[i], rbar), sub_hi(rw[i], rbar)), dh0 = pack2(sub_lo(xw[i], hbar), sub_hi(xw[i], hbar));
+        const u64 dr1 = pack2(sub_lo(rw[i + 1], rbar), sub_hi(rw[i + 1], rbar));
+        const u64 dh1 = pack2(sub_lo(xw[i + 1], hbar), sub_hi(xw[i + 1], hbar));
         sxxa = pfma(dr0, dr0, sxxa); sxya = pfma(dr0, dh0, sxya);
         sxxb = pfma(dr1, dr1, sxxb); sxyb = pfma(dr1, dh1, sxyb);
     }

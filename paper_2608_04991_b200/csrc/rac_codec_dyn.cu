@@ -170,32 +170,27 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_dyn_kernel
         const bool has_ref = ctrl->row[stage] >= 0;
 
         u64 e2[16];        // Eq. 7 residual of this thread's channels, packed pairs in slot order
-        u64 r2[16];        // aligned-reference inputs, kept for the sender-side reconstruction
+        uint32_t rw[16];   // reference values (packed bf16), kept for the sender-side reconstruction
         u64 a2 = 0ull, b2 = 0ull;
         uint32_t sel[KG > 4 ? 8 : 4] = {};   // per round: in-group offset | binary16 value << 16 (same in every lane of the group)
         uint32_t own = 0;                      // rounds whose outlier lives in this thread
         float m = 0.f;
         if (valid) {
-            u64 x2[16];
+            uint32_t xw[16];
 #pragma unroll
             for (int j = 0; j < 4; j++) {
-                uint4 w = lds128(xs + off[j]);
-                x2[4 * j + 0] = bf16x2_to_p(w.x);
-                x2[4 * j + 1] = bf16x2_to_p(w.y);
-                x2[4 * j + 2] = bf16x2_to_p(w.z);
-                x2[4 * j + 3] = bf16x2_to_p(w.w);
+                const uint4 w = lds128(xs + off[j]);
+                xw[4 * j + 0] = w.x; xw[4 * j + 1] = w.y; xw[4 * j + 2] = w.z; xw[4 * j + 3] = w.w;
             }
             if (has_ref) {
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
-                    u64 rr[4];
-                    load_ref_slot(rs + off[j], p.gain, p.bias, (int)(off[j] >> 1), rr);
-#pragma unroll
-                    for (int i = 0; i < 4; i++) r2[4 * j + i] = rr[i];
+                    const uint4 w = load_ref_words(rs + off[j], p.gain, p.bias, (int)(off[j] >> 1));
+                    rw[4 * j + 0] = w.x; rw[4 * j + 1] = w.y; rw[4 * j + 2] = w.z; rw[4 * j + 3] = w.w;
                 }
             } else {
 #pragma unroll
-                for (int i = 0; i < 16; i++) r2[i] = 0ull;
+                for (int i = 0; i < 16; i++) rw[i] = 0u;
             }
             bool shared = false;
             if constexpr (SUB) shared = p.coef_ext != nullptr;
@@ -207,7 +202,7 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_dyn_kernel
                 b2 = pack2(b, b);
             } else {
                 uint32_t coef_word;
-                fit_group(x2, r2, has_ref, lpg, p.inv_group, group_mask, p.status, a2, b2, &coef_word);
+                fit_group(xw, rw, has_ref, lpg, p.inv_group, group_mask, p.status, a2, b2, &coef_word);
                 if ((lane & (lpg - 1)) == 0) reinterpret_cast<uint32_t *>(rec)[tid >> lpg_shift] = coef_word;
             }
             // residual, and the largest magnitude of each slot of 8 channels
@@ -217,7 +212,7 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_dyn_kernel
                 float ev[8];
 #pragma unroll
                 for (int i = 0; i < 4; i++) {
-                    e2[4 * j + i] = psub(x2[4 * j + i], pfma(a2, r2[4 * j + i], b2));
+                    e2[4 * j + i] = sub_pair(xw[4 * j + i], pfma(a2, bf16x2_to_p(rw[4 * j + i]), b2));
                     unpack2(e2[4 * j + i], ev[2 * i], ev[2 * i + 1]);
                 }
                 sm[j] = abs_max8(ev, 0u);
@@ -434,7 +429,7 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_dyn_kernel
                         if (XHAT) {
                             // Eq. 9 with the code just chosen: x_hat = bf16((alpha*r + beta) + q*s)
                             float x0, x1;
-                            unpack2(pfma(psub(tt, magic2), s2, pfma(a2, r2[4 * j + i], b2)), x0, x1);
+                            unpack2(pfma(psub(tt, magic2), s2, pfma(a2, bf16x2_to_p(rw[4 * j + i]), b2)), x0, x1);
                             xh[i] = f2_to_bf16x2(x0, x1);
                         }
                     }
