@@ -8,7 +8,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "librac.so")
-SOURCES = ["rac_codec.cu", "rac_codec_dyn.cu", "rac_match.cu"]
+SOURCES = ["rac_codec.cu", "rac_codec_dyn.cu", "rac_calib.cu", "rac_match.cu"]
 HEADERS = ["rac_common.cuh", "rac_codec_dev.cuh", os.path.join("..", "..", "include", "rac.h")]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

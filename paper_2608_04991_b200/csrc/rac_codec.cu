@@ -1,5 +1,4 @@
-// RAC codec kernels for sm_100a: encode (Sec. IV-C, Eq. 6-8 + packing, outlier split), reconstruct (Eq. 9),
-// and the residual-RMS pass behind the step tables.
+// RAC codec kernels for sm_100a: encode (Sec. IV-C, Eq. 6-8 + packing, outlier split) and reconstruct (Eq. 9).
 //
 // Shape of the streaming kernels: persistent CTAs, one token per CTA iteration, one thread per 32
 // consecutive channels.  Rows travel between HBM and shared memory only as 1-D bulk copies (TMA without a
@@ -15,11 +14,9 @@
 //
 // Kernels: encode_ws_kernel (streaming pass of encode, optionally also the sender-side x_hat),
 // outlier_kernel (second launch of encode: the k largest |e| per token), decode_kernel and decode_ws_kernel
-// (receiver and sender reconstruction, with and without per-token outliers), calib_kernel +
-// calib_finalize_kernel (step tables; in its second form the statistics pass of the segment fit),
-// segment_fit_kernel + seg_of_kernel (Eq. 6 over several fitting positions), split_waves_kernel (tokens that
-// reference the same prompt go second), recon_error_kernel (error of a sender-path run).  The kernels of the
-// per-group-scale quantiser (Eq. 8 as printed) live in rac_codec_dyn.cu; this file holds the C ABI of both.
+// (receiver and sender reconstruction, with and without per-token outliers), split_waves_kernel (tokens that
+// reference the same prompt go second).  The kernels of the per-group-scale quantiser (Eq. 8 as printed) live in
+// rac_codec_dyn.cu; this file holds the C ABI of both.  Step tables, segment fit and reconstruction error: rac_calib.cu.
 #include <cstring>
 
 #include "rac_codec_dev.cuh"
@@ -85,167 +82,6 @@ int make_geometry(const rac_codec_cfg *cfg, Geometry *g) {
     const int raw = g->gval_off + 2 * ng;
     g->rec = (raw + 15) / 16 * 16;
     return RAC_OK;
-}
-
-// ------------------------------------------------------------------------------------------------
-// calibration pass: per-channel sums of e^2 (the residual of Eq. 7 with wire coefficients)
-// ------------------------------------------------------------------------------------------------
-// Same front end as the encoder (slab loads, Eq. 6 statistics, wire coefficients); instead of codes, every
-// thread accumulates e^2 of its own 32 channels in shared memory, separately for tokens with a reference
-// (row 0) and tokens coded directly (row 1).  One CTA barrier per token; the grid is fixed.
-// MOMENTS: the first pass of the segment fit instead -- the centred statistics of Eq. 6 of every (token, group)
-// go to p.moments and nothing is accumulated.
-template <bool MOMENTS>
-__global__ void __launch_bounds__(256, 2) calib_kernel(const CodecParams p) {
-    constexpr bool SUB = false;  // always over all tokens
-    extern __shared__ __align__(128) unsigned char smem[];
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int lane = tid & 31;
-    const int rot = (lane >> 1) & 3;
-    const int d = p.d;
-    const bool valid = tid * 32 < d;
-    const EncSmem L = enc_smem_layout(d, p.stages, nt);
-    Ctrl *ctrl = reinterpret_cast<Ctrl *>(smem);
-    const uint32_t sbase = smem_u32(smem);
-    const int S = p.stages;
-    const uint32_t row_bytes = 2u * (uint32_t)d;
-
-    if (tid == 0) {
-        for (int s = 0; s < S; s++) mbar_init(smem_u32(&ctrl->bar[s]), 1);
-        mbar_init_fence();
-    }
-    for (int o = tid; o < 2 * nt * 32; o += nt) reinterpret_cast<float *>(smem + L.acc0)[o] = 0.f;
-    __syncthreads();
-
-    const int first = blockIdx.x, stride = gridDim.x;
-    const long long n_tok = tokens_to_do<SUB>(p);
-    const int n_my = (n_tok > first) ? (int)((n_tok - first + stride - 1) / stride) : 0;
-    int next_raw = 0;
-    auto raw_row_of = [&](int k) -> int {  // raw ref_row entry of this CTA's k-th token
-        long long t = token_at<SUB>(p, first + (long long)k * stride);
-        return p.ref_row ? p.ref_row[t] : (int)t;
-    };
-    if (tid == 0) {
-        for (int k = 0; k < S - 1 && k < n_my; k++) {
-            long long t = token_at<SUB>(p, first + (long long)k * stride);
-            ctrl->tok[k] = t;
-            issue_token_loads<SUB>(p, ctrl, sbase + L.stage0 + k * L.stage_bytes, row_bytes, k, resolve_row<SUB>(p, raw_row_of(k)),
-                              p.X + t * d, row_bytes);
-        }
-        if (S - 1 < n_my) next_raw = raw_row_of(S - 1);
-    }
-    int cnt_ref = 0, cnt_dir = 0;  // tokens per table row (thread 0 only)
-    uint32_t off[4];
-#pragma unroll
-    for (int j = 0; j < 4; j++) off[j] = (uint32_t)(tid * 64 + ((j + rot) & 3) * 16);
-    const unsigned int group_mask = __ballot_sync(0xffffffffu, valid);
-
-    int stage = 0, issue_stage = S - 1;
-    bool aborted = false;
-    uint32_t parity = 0;
-    for (int it = 0; it < n_my; it++) {
-        if (tid == 0 && it + S - 1 < n_my) {
-            const int k = it + S - 1;
-            const long long tk = token_at<SUB>(p, first + (long long)k * stride);
-            ctrl->tok[issue_stage] = tk;
-            issue_token_loads<SUB>(p, ctrl, sbase + L.stage0 + issue_stage * L.stage_bytes, row_bytes, issue_stage,
-                              resolve_row<SUB>(p, next_raw), p.X + tk * d, row_bytes);
-            if (k + 1 < n_my) next_raw = raw_row_of(k + 1);
-        }
-        const bool timed_out = !mbar_wait_bounded(smem_u32(&ctrl->bar[stage]), parity);
-        if (timed_out && p.status) atomicOr(p.status, RAC_STATUS_TIMEOUT);
-        const bool has_ref = ctrl->row[stage] >= 0;
-        const long long tok = ctrl->tok[stage];
-        const uint32_t xs = sbase + L.stage0 + stage * L.stage_bytes;
-        const uint32_t rs = xs + row_bytes;
-
-        if (valid) {
-            uint32_t xw[16], rw[16];   // packed bf16, slot order
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const uint4 w = lds128(xs + off[j]);
-                xw[4 * j + 0] = w.x; xw[4 * j + 1] = w.y; xw[4 * j + 2] = w.z; xw[4 * j + 3] = w.w;
-            }
-            if (has_ref) {
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    const uint4 w = load_ref_words(rs + off[j], p.gain, p.bias, (int)(off[j] >> 1));
-                    rw[4 * j + 0] = w.x; rw[4 * j + 1] = w.y; rw[4 * j + 2] = w.z; rw[4 * j + 3] = w.w;
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 16; i++) rw[i] = 0u;
-            }
-            u64 a2, b2;
-            float4 st;
-            if (!MOMENTS && p.coef_ext) {
-                // shared coefficients: the residual of Eq. 7 with the words of the token's segment
-                const uint32_t cw = p.coef_ext[(long long)p.seg_of[tok] * p.J + (tid >> p.lpg_shift)];
-                const float a = half_bits_to_float(cw & 0xffffu), b = half_bits_to_float(cw >> 16);
-                a2 = pack2(a, a);
-                b2 = pack2(b, b);
-            } else {
-                fit_group(xw, rw, has_ref, p.lpg, p.inv_group, group_mask, p.status, a2, b2, nullptr, &st);
-            }
-            if (MOMENTS) {
-                if (!timed_out && (lane & (p.lpg - 1)) == 0) p.moments[tok * p.J + (tid >> p.lpg_shift)] = st;
-            }
-            float4 *acc = reinterpret_cast<float4 *>(smem + L.acc0) + (has_ref ? 0 : 8 * nt);
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                if (MOMENTS) break;
-                const int q = (j + rot) & 3;
-#pragma unroll
-                for (int hh = 0; hh < 2; hh++) {
-                    float e0, e1, e2, e3;
-                    unpack2(sub_pair(xw[4 * j + 2 * hh], pfma(a2, bf16x2_to_p(rw[4 * j + 2 * hh]), b2)), e0, e1);
-                    unpack2(sub_pair(xw[4 * j + 2 * hh + 1], pfma(a2, bf16x2_to_p(rw[4 * j + 2 * hh + 1]), b2)), e2, e3);
-                    float4 v = acc[(2 * q + hh) * nt + tid];
-                    v.x = __fmaf_rn(e0, e0, v.x);
-                    v.y = __fmaf_rn(e1, e1, v.y);
-                    v.z = __fmaf_rn(e2, e2, v.z);
-                    v.w = __fmaf_rn(e3, e3, v.w);
-                    acc[(2 * q + hh) * nt + tid] = v;
-                }
-            }
-        }
-        if (tid == 0) { if (has_ref) cnt_ref++; else cnt_dir++; }
-        if (__syncthreads_or(timed_out)) { aborted = true; break; }  // one vote: every thread leaves together
-        if (++stage == S) { stage = 0; parity ^= 1u; }
-        if (++issue_stage == S) issue_stage = 0;
-    }
-
-    __syncthreads();
-    if (MOMENTS) {
-        if (tid == 0 && aborted) {
-            for (int s = 0; s < S; s++) {
-                mbar_wait_bounded(smem_u32(&ctrl->bar[s]), 0);
-                mbar_wait_bounded(smem_u32(&ctrl->bar[s]), 1);
-            }
-        }
-        return;
-    }
-    // partial sums of this CTA, channel order, then its token counts
-    float *out = p.calib_partial + (long long)blockIdx.x * 2 * d;
-    const float *acc = reinterpret_cast<const float *>(smem + L.acc0);
-    if (valid) {
-        for (int rrow = 0; rrow < 2; rrow++)
-            for (int f = 0; f < 8; f++)
-                for (int cc = 0; cc < 4; cc++)
-                    out[rrow * d + tid * 32 + f * 4 + cc] = acc[rrow * nt * 32 + ((f * nt) + tid) * 4 + cc];
-    }
-    if (tid == 0) {
-        int *cnt = reinterpret_cast<int *>(p.calib_partial + (long long)gridDim.x * 2 * d) + 2 * blockIdx.x;
-        cnt[0] = cnt_ref;
-        cnt[1] = cnt_dir;
-        if (aborted) {
-            // give copies that may still be in flight a bounded chance to land before the CTA retires
-            for (int s = 0; s < S; s++) {
-                mbar_wait_bounded(smem_u32(&ctrl->bar[s]), 0);
-                mbar_wait_bounded(smem_u32(&ctrl->bar[s]), 1);
-            }
-        }
-    }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -646,7 +482,7 @@ __global__ void __launch_bounds__(W * 32, W == 7 ? 4 : 3) outlier_kernel(const C
     if constexpr (SUB) shared = p.coef_ext != nullptr;
     const int coff = shared ? 0 : 4 * p.J;
     // everything this kernel reads was written by the streaming pass launched just before it
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    grid_dependency_wait();
     const long long n_tok = tokens_to_do<SUB>(p);
 
     for (long long ti0 = ((long long)blockIdx.x * W + warp) * U; ti0 < n_tok; ti0 += tstride) {
@@ -871,35 +707,6 @@ __global__ void __launch_bounds__(W * 32, W == 7 ? 4 : 3) outlier_kernel(const C
         }
         __syncwarp();
     }
-}
-
-// step tables from the per-CTA partial sums (fixed summation order -> deterministic)
-__global__ void calib_finalize_kernel(const float *partial, int nblocks, int d, int bits, float clip_sigmas, float *step,
-                                      float *inv_step) {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= 2 * d) return;
-    int row = c / d;
-    const int *cnt = reinterpret_cast<const int *>(partial + (long long)nblocks * 2 * d);
-    double sum = 0.0;
-    long long n = 0;
-    for (int b = 0; b < nblocks; b++) {
-        sum += (double)partial[(long long)b * 2 * d + c];
-        n += cnt[2 * b + row];
-    }
-    float s = 0.f, is = 0.f;
-    if (n > 0) {
-        double qmax = (double)((1 << (bits - 1)) - 1);
-        double want = (double)clip_sigmas * sqrt(sum / (double)n) / qmax;
-        if (want > 0.0) {
-            if (want > 65504.0) want = 65504.0;
-            __half h = __double2half(want);
-            if ((double)__half2float(h) < want) h = __ushort_as_half((unsigned short)(__half_as_ushort(h) + 1));  // round up
-            s = __half2float(h);
-            if (s != 0.f) is = __fdiv_rn(1.0f, s);
-        }
-    }
-    step[c] = s;
-    inv_step[c] = is;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1368,7 +1175,7 @@ __global__ void __launch_bounds__(256, 2) decode_ws_kernel(const CodecParams p) 
 // host side: launch plumbing
 // ------------------------------------------------------------------------------------------------
 
-static int fill_common(const Geometry &g, CodecParams *p, long long T, const void *ref_base, long long ref_rows,
+int fill_common(const Geometry &g, CodecParams *p, long long T, const void *ref_base, long long ref_rows,
                        const int32_t *ref_row, const void *gain, const void *bias, uint32_t *status) {
     if (T < 0 || ref_rows < 0) return RAC_EINVAL;
     if ((gain == nullptr) != (bias == nullptr)) return RAC_EINVAL;
@@ -1404,23 +1211,6 @@ static int fill_common(const Geometry &g, CodecParams *p, long long T, const voi
     p->gval_off = g.gval_off;
     p->test_extra_tx = 0;
     return RAC_OK;
-}
-
-// Launch of a kernel that runs after the one before it on the stream, allowed to be set up while that one drains
-// (programmatic dependent launch): the kernel itself waits for its predecessor's memory before it reads anything.
-template <typename K, typename... Args>
-static void launch_after(K kernel, unsigned grid, unsigned block, cudaStream_t stream, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 // Encode: the streaming kernel, then (with outliers) the selection kernel.  Variant 4 of the streaming kernel
@@ -1482,9 +1272,9 @@ static int launch_encode(const Geometry &g, CodecParams &p, long long max_ctas, 
     const int nth = g.d / 32;
     const unsigned nb = (unsigned)blocks, nt = wpc * 32;
 #define RAC_OUT(NV, KT)                                                                    \
-    (wide ? launch_after(outlier_kernel<NV, KT, false, 8>, nb, nt, stream, p, g.bits)     \
-          : launch_after(outlier_kernel<NV, KT, false, 7>, nb, nt, stream, p, g.bits))
-    if (sub) launch_after(outlier_kernel<8, 0, true, 8>, nb, nt, stream, p, g.bits);
+    (wide ? launch_after(outlier_kernel<NV, KT, false, 8>, nb, nt, 0, stream, p, g.bits)     \
+          : launch_after(outlier_kernel<NV, KT, false, 7>, nb, nt, 0, stream, p, g.bits))
+    if (sub) launch_after(outlier_kernel<8, 0, true, 8>, nb, nt, 0, stream, p, g.bits);
     else if (g.topk == 8) {
         if (nth <= 128) RAC_OUT(4, 8);
         else if (nth <= 160) RAC_OUT(5, 8);
@@ -1590,132 +1380,6 @@ __global__ void __launch_bounds__(1024) split_waves_kernel(const int32_t *ref_ro
         wave_count[0] = T - total2;
     }
 }
-
-// ------------------------------------------------------------------------------------------------
-// Eq. 6 over several fitting positions: one coefficient pair per (segment of tokens, group)
-// ------------------------------------------------------------------------------------------------
-// Pass 1 (calib_kernel<true>) leaves the centred statistics of every (token, group).  Pass 2: one warp per
-// (segment, group) merges them with the pairwise update of means and centred sums, in binary64 and in a fixed
-// order (lane l takes tokens l, l+32, ... of the segment in order, then a shuffle tree), applies the
-// zero-variance rule and rounds to the wire format.
-struct Mom {
-    double n, mr, mh, sxx, sxy;
-};
-__device__ __forceinline__ Mom mom_merge(const Mom &a, const Mom &b) {
-    if (b.n == 0.0) return a;
-    if (a.n == 0.0) return b;
-    Mom o;
-    o.n = a.n + b.n;
-    const double dr = b.mr - a.mr, dh = b.mh - a.mh, w = b.n / o.n, f = a.n * w;
-    o.mr = a.mr + dr * w;
-    o.mh = a.mh + dh * w;
-    o.sxx = a.sxx + b.sxx + dr * dr * f;
-    o.sxy = a.sxy + b.sxy + dr * dh * f;
-    return o;
-}
-__global__ void __launch_bounds__(256) segment_fit_kernel(const float4 *moments, const int32_t *seg_off, long long n_seg,
-                                                          int J, int group, long long T, uint32_t *coef_seg) {
-    const long long wid = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (wid >= n_seg * J) return;
-    const long long k = wid / J;
-    const int j = (int)(wid - k * J);
-    long long t0 = seg_off[k], t1 = seg_off[k + 1];
-    t0 = t0 < 0 ? 0 : (t0 > T ? T : t0);
-    t1 = t1 < t0 ? t0 : (t1 > T ? T : t1);
-    Mom m = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (long long t = t0 + lane; t < t1; t += 32) {
-        const float4 s = moments[t * J + j];
-        const Mom one = {(double)group, (double)s.x, (double)s.y, (double)s.z, (double)s.w};
-        m = mom_merge(m, one);
-    }
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {   // lane l absorbs lane l + o: earlier tokens stay on the left
-        Mom b;
-        b.n = __shfl_down_sync(0xffffffffu, m.n, o);
-        b.mr = __shfl_down_sync(0xffffffffu, m.mr, o);
-        b.mh = __shfl_down_sync(0xffffffffu, m.mh, o);
-        b.sxx = __shfl_down_sync(0xffffffffu, m.sxx, o);
-        b.sxy = __shfl_down_sync(0xffffffffu, m.sxy, o);
-        if (lane + o < 32) m = mom_merge(m, b);
-    }
-    if (lane == 0) {
-        double a = 0.0, b = m.mh;
-        if (m.sxx > 1e-12 && fabs(m.sxy) < 65504.0 * m.sxx) {
-            a = m.sxy / m.sxx;
-            b = m.mh - a * m.mr;
-        }
-        a = fmin(fmax(a, -65504.0), 65504.0);
-        b = fmin(fmax(b, -65504.0), 65504.0);
-        const uint32_t a16 = __half_as_ushort(__double2half(a)), b16 = __half_as_ushort(__double2half(b));
-        coef_seg[k * J + j] = a16 | (b16 << 16);
-    }
-}
-// segment of every token: the last k with seg_off[k] <= t (empty segments have equal offsets and are skipped)
-__global__ void seg_of_kernel(const int32_t *seg_off, long long n_seg, long long T, int32_t *seg_of) {
-    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    long long lo = 0, hi = n_seg;   // invariant: seg_off[lo] <= t (seg_off[0] = 0), answer in [lo, hi)
-    while (hi - lo > 1) {
-        const long long mid = (lo + hi) >> 1;
-        if (seg_off[mid] <= t) lo = mid; else hi = mid;
-    }
-    seg_of[t] = (int32_t)lo;
-}
-
-// ------------------------------------------------------------------------------------------------
-// reconstruction error of a sender-path run (input of the byte-cost side of calibration, Sec. IV-C)
-// ------------------------------------------------------------------------------------------------
-constexpr int kErrGrid = 592;     // fixed, so that the summation order does not depend on the device
-constexpr int kErrThreads = 256;
-
-// partial[b] = (sum (x - x_hat)^2, sum x^2, max |x - x_hat|) over the 8-element chunks b, b + grid, ...
-__global__ void __launch_bounds__(kErrThreads) recon_error_kernel(const uint4 *X, const uint4 *Xh, long long n8,
-                                                                  double *partial) {
-    double se = 0.0, sx = 0.0;
-    float mx = 0.f;
-    for (long long i = blockIdx.x * (long long)kErrThreads + threadIdx.x; i < n8; i += (long long)kErrGrid * kErrThreads) {
-        const uint4 a = X[i], b = Xh[i];
-        const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            const float x0 = __uint_as_float(aw[k] << 16), x1 = __uint_as_float(aw[k] & 0xffff0000u);
-            const float y0 = __uint_as_float(bw[k] << 16), y1 = __uint_as_float(bw[k] & 0xffff0000u);
-            const float d0 = __fsub_rn(x0, y0), d1 = __fsub_rn(x1, y1);   // exact or one rounding: both are bf16
-            se += (double)d0 * (double)d0 + (double)d1 * (double)d1;
-            sx += (double)x0 * (double)x0 + (double)x1 * (double)x1;
-            mx = fmaxf(mx, fmaxf(fabsf(d0), fabsf(d1)));
-        }
-    }
-    __shared__ double s_se[kErrThreads], s_sx[kErrThreads];
-    __shared__ float s_mx[kErrThreads];
-    s_se[threadIdx.x] = se; s_sx[threadIdx.x] = sx; s_mx[threadIdx.x] = mx;
-    __syncthreads();
-    for (int o = kErrThreads / 2; o > 0; o >>= 1) {   // fixed tree: the same order on every run
-        if (threadIdx.x < o) {
-            s_se[threadIdx.x] += s_se[threadIdx.x + o];
-            s_sx[threadIdx.x] += s_sx[threadIdx.x + o];
-            s_mx[threadIdx.x] = fmaxf(s_mx[threadIdx.x], s_mx[threadIdx.x + o]);
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        partial[3 * blockIdx.x + 0] = s_se[0];
-        partial[3 * blockIdx.x + 1] = s_sx[0];
-        partial[3 * blockIdx.x + 2] = (double)s_mx[0];
-    }
-}
-__global__ void recon_error_finalize_kernel(const double *partial, double *out) {
-    double se = 0.0, sx = 0.0, mx = 0.0;
-    for (int b = 0; b < kErrGrid; b++) {
-        se += partial[3 * b];
-        sx += partial[3 * b + 1];
-        mx = fmax(mx, partial[3 * b + 2]);
-    }
-    out[0] = se; out[1] = sx; out[2] = mx;
-}
-
-constexpr int kCalibGrid = 128;  // fixed, so that the summation order does not depend on the device
 
 // A subset of the tokens and a second reference buffer (the *_list entry points); all null/0 otherwise.
 struct Subset {
@@ -2002,122 +1666,6 @@ int rac_split_waves(const int32_t *ref_row, int64_t T, int64_t first_intra_row, 
     split_waves_kernel<<<1, 1024, 0, static_cast<cudaStream_t>(stream)>>>(ref_row, (int)T, first_intra_row, wave1, wave2,
                                                                          wave_count);
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
-}
-
-size_t rac_fit_segments_workspace_bytes(const rac_codec_cfg *cfg, int64_t T) {
-    Geometry g;
-    if (make_geometry(cfg, &g) != RAC_OK || T < 0) return 0;
-    return ((size_t)T * (size_t)g.J * sizeof(float4) + 15) / 16 * 16 + 16;
-}
-
-int rac_fit_segments(const rac_codec_cfg *cfg, const void *X, int64_t T, const void *ref_base, int64_t ref_rows,
-                     const int32_t *ref_row, const void *ref_gain, const void *ref_bias, const int32_t *seg_off,
-                     int64_t n_seg, uint32_t *coef_seg, int32_t *seg_of, void *workspace, size_t workspace_bytes,
-                     uint32_t *dev_status, void *stream) {
-    Geometry g;
-    int rc = make_geometry(cfg, &g);
-    if (rc != RAC_OK) return rc;
-    CodecParams p = {};
-    rc = fill_common(g, &p, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, dev_status);
-    if (rc != RAC_OK) return rc;
-    if (n_seg < 0 || n_seg >= (1ll << 30) || T >= (1ll << 31)) return RAC_EUNSUPPORTED;
-    if (n_seg == 0) return T == 0 ? RAC_OK : RAC_EINVAL;
-    if (!seg_off || !coef_seg || !workspace || (T > 0 && (!X || !seg_of))) return RAC_EINVAL;
-    if (!aligned16(X) || !aligned16(workspace)) return RAC_EALIGN;
-    if (workspace_bytes < rac_fit_segments_workspace_bytes(cfg, T)) return RAC_ESIZE;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    p.X = static_cast<const uint16_t *>(X);
-    p.moments = static_cast<float4 *>(workspace);
-    if (T > 0) {
-        p.stages = 2;
-        EncSmem L = enc_smem_layout(g.d, p.stages, g.nthreads);
-        rc = launch_persistent(calib_kernel<true>, p, g.nthreads, L.total, T, st);
-        if (rc != RAC_OK) return rc;
-        seg_of_kernel<<<(unsigned)((T + 255) / 256), 256, 0, st>>>(seg_off, n_seg, T, seg_of);
-    }
-    const long long warps = n_seg * g.J;
-    segment_fit_kernel<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>(p.moments, seg_off, n_seg, g.J, g.group, T,
-                                                                            coef_seg);
-    return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
-}
-
-size_t rac_recon_error_workspace_bytes(void) { return (size_t)kErrGrid * 3 * sizeof(double); }
-
-int rac_recon_error(const void *X, const void *X_hat, int64_t T, int32_t d, double *out, void *workspace,
-                    size_t workspace_bytes, void *stream) {
-    if (T < 0 || d <= 0 || !out || !workspace) return RAC_EINVAL;
-    if (d % 8) return RAC_EUNSUPPORTED;
-    if (T > 0 && (!X || !X_hat)) return RAC_EINVAL;
-    if (!aligned16(X) || !aligned16(X_hat) || !aligned16(workspace) || (reinterpret_cast<uintptr_t>(out) & 7u)) return RAC_EALIGN;
-    if (workspace_bytes < rac_recon_error_workspace_bytes()) return RAC_ESIZE;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    double *partial = static_cast<double *>(workspace);
-    recon_error_kernel<<<kErrGrid, kErrThreads, 0, st>>>(static_cast<const uint4 *>(X), static_cast<const uint4 *>(X_hat),
-                                                       (long long)T * d / 8, partial);
-    recon_error_finalize_kernel<<<1, 1, 0, st>>>(partial, out);
-    return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
-}
-
-size_t rac_calibrate_workspace_bytes(const rac_codec_cfg *cfg) {
-    Geometry g;
-    if (make_geometry(cfg, &g) != RAC_OK) return 0;
-    return (size_t)kCalibGrid * 2 * (size_t)g.d * sizeof(float) + (size_t)kCalibGrid * 2 * sizeof(int);
-}
-
-static int calibrate_impl(const rac_codec_cfg *cfg, const void *X, int64_t T, const void *ref_base, int64_t ref_rows,
-                          const int32_t *ref_row, const void *ref_gain, const void *ref_bias, const uint32_t *coef_seg,
-                          const int32_t *seg_of, float clip_sigmas, float *step, float *inv_step, void *workspace,
-                          size_t workspace_bytes, uint32_t *dev_status, void *stream) {
-    Geometry g;
-    int rc = make_geometry(cfg, &g);
-    if (rc != RAC_OK) return rc;
-    CodecParams p = {};
-    rc = fill_common(g, &p, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, dev_status);
-    if (rc != RAC_OK) return rc;
-    if (g.scale_mode != 0) return RAC_EUNSUPPORTED;   // the tables belong to the static quantiser only
-    if ((g.coef_fmt == 1) != (coef_seg != nullptr) || (coef_seg != nullptr) != (seg_of != nullptr)) return RAC_EINVAL;
-    p.coef_ext = coef_seg;
-    p.seg_of = seg_of;
-    if (!step || !inv_step || !workspace || !(clip_sigmas > 0.f)) return RAC_EINVAL;
-    if (T > 0 && !X) return RAC_EINVAL;
-    if (!aligned16(X) || !aligned16(workspace) || !aligned16(step) || !aligned16(inv_step)) return RAC_EALIGN;
-    if (workspace_bytes < rac_calibrate_workspace_bytes(cfg)) return RAC_ESIZE;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    p.X = static_cast<const uint16_t *>(X);
-    p.calib_partial = static_cast<float *>(workspace);
-    // every CTA of the fixed grid writes its partials, also when it has no token
-    {
-        p.stages = 2;
-        EncSmem L = enc_smem_layout(g.d, p.stages, g.nthreads);
-        DeviceInfo di;
-        rc = device_info(&di);
-        if (rc != RAC_OK) return rc;
-        if (L.total > di.max_smem_optin) return RAC_EUNSUPPORTED;
-        if (cudaFuncSetAttribute(calib_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total) != cudaSuccess) return RAC_ECUDA;
-        calib_kernel<false><<<kCalibGrid, g.nthreads, L.total, st>>>(p);
-        if (cudaGetLastError() != cudaSuccess) return RAC_ECUDA;
-    }
-    int n = 2 * g.d;
-    calib_finalize_kernel<<<(n + 255) / 256, 256, 0, st>>>(p.calib_partial, kCalibGrid, g.d, g.bits, clip_sigmas, step, inv_step);
-    return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
-}
-
-int rac_calibrate_steps(const rac_codec_cfg *cfg, const void *X, int64_t T, const void *ref_base, int64_t ref_rows,
-                        const int32_t *ref_row, const void *ref_gain, const void *ref_bias, float clip_sigmas,
-                        float *step, float *inv_step, void *workspace, size_t workspace_bytes, uint32_t *dev_status,
-                        void *stream) {
-    return calibrate_impl(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, nullptr, nullptr, clip_sigmas, step,
-                          inv_step, workspace, workspace_bytes, dev_status, stream);
-}
-
-int rac_calibrate_steps_shared(const rac_codec_cfg *cfg, const void *X, int64_t T, const void *ref_base, int64_t ref_rows,
-                               const int32_t *ref_row, const void *ref_gain, const void *ref_bias,
-                               const uint32_t *coef_seg, const int32_t *seg_of, float clip_sigmas, float *step,
-                               float *inv_step, void *workspace, size_t workspace_bytes, uint32_t *dev_status,
-                               void *stream) {
-    if (!coef_seg || !seg_of) return RAC_EINVAL;
-    return calibrate_impl(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, coef_seg, seg_of, clip_sigmas, step,
-                          inv_step, workspace, workspace_bytes, dev_status, stream);
 }
 
 }  // extern "C"

@@ -28,7 +28,7 @@ struct CodecParams {
     const float *inv_step;     // [2,d]
     uint8_t *payload;          // encode out / decode in
     uint16_t *X_hat;           // decode out
-    float *calib_partial;      // calibrate out: [grid][2][d] sums of e^2, then [grid][2] token counts
+    float *calib_partial;      // calibrate out: [parts][2][d] sums of e^2, then [parts][2] token counts
     float *tmax;               // encode with outliers: [T][d/32] largest |e| per thread slab (caller workspace)
     uint32_t *status;
     long long T;
@@ -53,6 +53,9 @@ struct CodecParams {
     uint32_t test_extra_tx;
 };
 
+// parameters every call has in common, with the checks of the arguments they come from (defined in rac_codec.cu)
+int fill_common(const Geometry &g, CodecParams *p, long long T, const void *ref_base, long long ref_rows,
+                const int32_t *ref_row, const void *gain, const void *bias, uint32_t *status);
 // scale_mode 1 (defined in rac_codec_dyn.cu)
 int launch_encode_dyn(const Geometry &g, CodecParams &p, long long max_ctas, cudaStream_t stream);
 int launch_decode_dyn(const Geometry &g, CodecParams &p, cudaStream_t stream);
@@ -66,22 +69,9 @@ struct Ctrl {
     unsigned long long bar[kMaxStages];
     int row[kMaxStages];        // reference row of the token in each stage, -1 = direct
     int seg[kMaxStages];        // segment of the token in each stage (shared coefficients only)
-    long long tok[kMaxStages];  // the token in each stage (segment fit only)
 };
 
 __host__ __device__ inline int align_up(int v, int a) { return (v + a - 1) / a * a; }
-
-struct EncSmem {  // calibration kernel
-    int stage0, stage_bytes, acc0, total;
-};
-__host__ __device__ inline EncSmem enc_smem_layout(int d, int stages, int nthreads) {
-    EncSmem s;
-    s.stage0 = align_up((int)sizeof(Ctrl), 128);
-    s.stage_bytes = 4 * d;  // X row + R row
-    s.acc0 = s.stage0 + stages * s.stage_bytes;   // e^2 accumulators: 2 table rows x 32 floats per thread
-    s.total = s.acc0 + 2 * nthreads * 32 * 4;
-    return s;
-}
 
 struct DecSmem {
     int ctrl, stage0, stage_bytes, rec_pad, out0, total;
@@ -436,6 +426,23 @@ static int resident_ctas(const void *kernel, int dev, int nthreads, int smem_byt
     }
     *occ_out = it->second;
     return RAC_OK;
+}
+
+// Launch of a kernel that may be set up while the one before it on the stream drains (programmatic dependent launch):
+// the kernel itself waits for its predecessor's memory (grid_dependency_wait) before it reads anything.
+template <typename K, typename... Args>
+static void launch_after(K kernel, unsigned grid, unsigned block, size_t smem, cudaStream_t stream, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 template <typename K>
