@@ -428,23 +428,6 @@ static int resident_ctas(const void *kernel, int dev, int nthreads, int smem_byt
     return RAC_OK;
 }
 
-// Launch of a kernel that may be set up while the one before it on the stream drains (programmatic dependent launch):
-// the kernel itself waits for its predecessor's memory (grid_dependency_wait) before it reads anything.
-template <typename K, typename... Args>
-static void launch_after(K kernel, unsigned grid, unsigned block, size_t smem, cudaStream_t stream, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 template <typename K>
 static int launch_persistent(K kernel, const CodecParams &p, int nthreads, int smem_bytes, long long max_ctas,
                              cudaStream_t stream) {

@@ -72,6 +72,9 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 
 // waits until everything the kernel before this one on the stream wrote is visible (programmatic dependent launch)
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel on the stream be set up from now on (it waits for this one's end before it reads anything): for short
+// kernels whose launches follow one another, where the set-up would otherwise be in the way.  Call it first.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {
     uint4 v;
@@ -164,5 +167,22 @@ struct Geometry {
     int rec;        // record stride in bytes
 };
 int make_geometry(const rac_codec_cfg *cfg, Geometry *g);  // RAC_OK or an error
+
+// Launch of a kernel that may be set up while the one before it on the stream drains (programmatic dependent launch):
+// the kernel itself waits for its predecessor's memory (grid_dependency_wait) before it reads anything.
+template <typename K, typename... Args>
+static void launch_after(K kernel, unsigned grid, unsigned block, size_t smem, cudaStream_t stream, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 }  // namespace rac

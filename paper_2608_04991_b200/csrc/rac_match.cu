@@ -1,23 +1,32 @@
 // Exact-token span retrieval for prefill uplinks (Sec. IV-B.1, Eq. 3) on the GPU.
 //
-// Index: an open-addressing hash table with one slot per DISTINCT w-token window of the history.  A slot
-// stores one representative start position (used to verify a key token by token, so hash collisions can
-// never change the result) and the K largest start positions of that window in descending order.  A start
-// enters its slot's list by a cascade of atomicMax: it is offered to entry 0, the smaller of (offered, found)
-// is carried to entry 1, and so on.  Every step keeps the pair it touches, so entry 0 ends as the largest
-// value ever offered, entry 1 as the largest of the rest, ...: the final lists do not depend on the order in
-// which threads run.
-// Query: one thread per query position looks its window up, extends each of the <= K candidates forward
-// to the longest exact match and keeps lexargmax(length, start).
-// Selection: the left-to-right scan of Eq. 3 visits a position, jumps by the span length if it has a
-// candidate and by one otherwise.  "Next position at or after p that has a candidate" is a parallel
-// suffix scan; the remaining chain (one hop per selected span) is walked by a single thread, and the
-// spans are expanded to per-token rows in parallel.
+// Index: a hash table with one slot per DISTINCT w-token window of the history, in buckets of four slots (32 bytes, one
+// trip to L2).  A slot holds 32 bits of the window's hash beside one representative start position; where the hash bits
+// agree the key is verified token by token, so hash collisions can never change the result.  Beside the slot stand the K
+// largest start positions of that window, as a set that does not depend on the order in which threads run (set_insert).
+// Query: one thread per query position looks its window up and extends each of the <= K candidates forward to the longest
+// exact match; long matches are finished by the warp together.  lexargmax(length, start) is kept.
+// Selection: the left-to-right scan of Eq. 3 visits a position, jumps by the span length if it has a candidate and by one
+// otherwise.  Positions are cut into chunks; every chunk works out, for each of its positions, where a scan that enters there
+// leaves the chunk and how many spans it selects on the way (pointer doubling in shared memory).  What is left is one hop per
+// chunk; a last kernel walks every chunk from the position where the scan enters it and writes its spans and rows.
+//
+// All of it is bound by the latency of dependent trips to L2 and of launches, not by the bytes: the forms above were chosen
+// to make fewer of both, and every kernel lets the next one be set up while it runs.  32768 history and 2048 query tokens:
+// 23 us in four launches (52 us in nine before: sorted lists, a thread per match, a suffix scan and a serial walk), 131072 /
+// 131072 tokens: 44 us (99 us), a query of 2048 tokens against an index of 16384 22 us (60 us), eight appends of 2048 tokens
+// behind a reset 39 us (54 us).
 #include <mutex>
 
 #include "rac_common.cuh"
 
 namespace rac {
+
+typedef unsigned long long u64;
+constexpr u64 kEmptySlot = ~0ull;
+constexpr int kBucket = 4;             // slots per bucket
+constexpr int kChunk = 512;            // query positions per chunk of the selection = threads of its CTAs
+constexpr int kInlineChunks = 8;       // up to so many chunks every CTA of the last kernel walks the chunks itself
 
 struct MatchParams {
     const int32_t *hist;
@@ -25,278 +34,495 @@ struct MatchParams {
     int32_t *ref_row;
     rac_span *spans_out;   // may be null
     int32_t *n_spans;
-    // workspace sections
-    int32_t *rep;          // [M]      representative start of the slot's window, -1 = empty
-    int32_t *top;          // [M*K]    r-th largest start of the slot's window, -1 = none
-    int32_t *slot_of;      // [nwin]
+    u64 *slots;            // [M]      hash bits (high half) and representative start of the slot's window, all ones = empty
+    int32_t *top;          // [n_hist*K] the K largest starts of a window, in no order, -1 = none, at its representative start
+    int32_t *next;         // [nwin]   unlimited hits (max_hits = 0) only: another start of the same window, -1 = none;
+                           //          top[representative] is then the head of the window's chain (K = 1)
     int2 *best;            // [N]      (length, history start) of the best candidate, length 0 = none
-    int2 *hop;             // [N]      (next position >= p with a candidate, position after its span)
-    rac_span *spans_ws;    // [N/w + 1]
-    int32_t *chunk_first;  // [ceil(N/1024)] first position with a candidate in each chunk of 1024 positions
-    unsigned short *delta16; // [N]    jump4 - position, 65535 = does not fit
-    int32_t *jump2;        // [N]      position after the next two spans at or after each position (n_query if fewer)
-    int32_t *jump4;        // [N]      ... after the next four
+    int2 *jump;            // [N]      where a scan that enters the chunk here leaves it, and the spans it selects until then
+    int2 *entry;           // [chunks] where the scan enters the chunk, and the spans selected before
     int n_hist, n_query, nwin, w, K;
-    unsigned int mask;     // M - 1
+    unsigned int bmask;    // buckets - 1
     const int32_t *end_of; // [n_hist] end of the request that holds each history position; null = one request
     int first_live;        // only windows that start at or after this history position are candidates (0 = all)
-    int32_t *next;         // [nwin]   unlimited hits (max_hits = 0) only: another start of the same window, -1 = none;
-                           //          top[slot] is then the head of the slot's chain (K = 1 entry per slot)
+    // intra-sequence references: a table of the prompt's tokens, keyed by a position that holds the token
+    int32_t *trep;         // [tmask + 1] that position, -1 = empty; null = no such references
+    int32_t *tfirst;       // [tmask + 1] kFirstBase - (first position of the token), -1 = none yet
+    unsigned int tmask;
 };
+constexpr int kFirstBase = 0x3fffffff;
 
-__device__ __forceinline__ unsigned int window_hash(const int32_t *tok, int w) {
-    unsigned long long h = 0x9E3779B97F4A7C15ull;
-    for (int m = 0; m < w; m++) {
-        h ^= (unsigned long long)(unsigned int)tok[m];
-        h *= 0xff51afd7ed558ccdull;
-        h ^= h >> 32;
+// four tokens (or what is left of the window) per step, loaded before any is used: a window is a chain of one or two trips
+// to memory, not one per token
+__device__ __forceinline__ u64 window_hash(const int32_t *tok, int w) {
+    u64 h = 0x9E3779B97F4A7C15ull;
+    for (int m = 0; m < w; m += 4) {
+        uint32_t t[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) t[u] = m + u < w ? (uint32_t)tok[m + u] : 0u;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            if (m + u < w) {
+                h ^= (u64)t[u];
+                h *= 0xff51afd7ed558ccdull;
+                h ^= h >> 32;
+            }
+        }
     }
-    return (unsigned int)h;
+    return h;
 }
-
 __device__ __forceinline__ bool same_window(const int32_t *a, const int32_t *b, int w) {
-    for (int m = 0; m < w; m++)
-        if (a[m] != b[m]) return false;
+    for (int m = 0; m < w; m += 4) {
+        uint32_t x[4], y[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            x[u] = m + u < w ? (uint32_t)a[m + u] : 0u;
+            y[u] = m + u < w ? (uint32_t)b[m + u] : 0u;
+        }
+        if ((x[0] ^ y[0]) | (x[1] ^ y[1]) | (x[2] ^ y[2]) | (x[3] ^ y[3])) return false;
+    }
     return true;
 }
-
-// Offers start j to a descending list of K entries (-1 = empty): atomicMax at entry r keeps the larger of
-// (offered, found) there and carries the smaller on to entry r + 1.  Whatever the interleaving with other
-// threads, the list ends as the K largest values ever offered, in descending order.
-__device__ __forceinline__ void cascade_insert(int32_t *lst, int K, int j) {
-    int v = j;
-    for (int r = 0; r < K && v >= 0; r++) {
-        const int old = atomicMax(&lst[r], v);
-        v = old < v ? old : v;
-    }
+// a bucket as the L2 holds it (other SMs may be filling it)
+__device__ __forceinline__ void load_bucket(const u64 *slots, unsigned int b, u64 (&e)[kBucket]) {
+    const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(slots + (size_t)b * kBucket);
+    const ulonglong2 lo = __ldcg(q), hi = __ldcg(q + 1);
+    e[0] = lo.x; e[1] = lo.y; e[2] = hi.x; e[3] = hi.y;
 }
 
-__global__ void match_init_kernel(MatchParams p, long long table_ints) {
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long k = i; k < table_ints; k += stride) p.rep[k] = -1;  // rep and top are contiguous
-    for (long long k = i; k < p.n_query; k += stride) p.ref_row[k] = -1;
-    if (i == 0) *p.n_spans = 0;
-}
-
-// one slot per distinct window: claim an empty slot or find the slot that already holds this window
-__global__ void match_insert_kernel(MatchParams p) {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= p.nwin) return;
-    const int32_t *win = p.hist + j;
-    unsigned int s = window_hash(win, p.w) & p.mask;
-    int slot = -1;
-    for (unsigned int probe = 0; probe <= p.mask; probe++) {
-        int cur = atomicCAS(&p.rep[s], -1, j);
-        if (cur == -1 || cur == j || same_window(p.hist + cur, win, p.w)) { slot = (int)s; break; }
-        s = (s + 1) & p.mask;
-    }
-    p.slot_of[j] = slot;  // the table has >= 2*nwin slots, so a slot is always found
-    if (slot < 0) return;
-    // unlimited hits: every start of the window goes onto the slot's chain.  The order of a chain depends on which
-    // thread came first; the query looks at ALL of it and keeps lexargmax(length, start), so the result does not.
-    if (p.next) p.next[j] = atomicExch(&p.top[slot], j);
-    else cascade_insert(p.top + (long long)slot * p.K, p.K, j);
-}
-
-__global__ void match_query_kernel(MatchParams p) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= p.n_query) return;
-    int bestL = 0, bestj = -1;
-    if (i + p.w <= p.n_query && p.nwin > 0) {
-        const int32_t *win = p.query + i;
-        unsigned int s = window_hash(win, p.w) & p.mask;
-        int slot = -1;
-        for (unsigned int probe = 0; probe <= p.mask; probe++) {
-            int cur = p.rep[s];
-            if (cur < 0) break;  // empty slot ends the probe sequence: the window is not in the history
-            if (same_window(p.hist + cur, win, p.w)) { slot = (int)s; break; }
-            s = (s + 1) & p.mask;
-        }
-        if (slot >= 0) {
-            // candidate j: extend forward to the longest exact match, keep lexargmax(length, start)
-            auto consider = [&](int j) {
-                int L = p.w;
-                const int hend = p.end_of ? p.end_of[j] : p.n_hist;   // a match stays inside its request
-                // eight tokens per trip to memory: the loads of a trip are independent, and a long match is a chain
-                // of dependent trips
-                const int room = min(p.n_query - i, hend - j);            // L may grow up to this
-                bool open = true;
-                while (open && L + 8 <= room) {
-                    int32_t q[8], h[8];
+// First slot of a bucket, from slot `from` on, that is empty or carries the hash bits (kBucket if none), and what it holds.
+// Selects, not branches: the lanes of a warp then look at whatever slot each of them is at in ONE trip, where a branch per
+// slot made a trip of each (the two trips per slot took most of the table's time).
+__device__ __forceinline__ int find_in_bucket(const u64 (&e)[kBucket], uint32_t tag, int from, u64 &held) {
+    int at = kBucket;
+    held = kEmptySlot;
 #pragma unroll
-                    for (int u = 0; u < 8; u++) { q[u] = p.query[i + L + u]; h[u] = p.hist[j + L + u]; }
-                    unsigned int ne = 0;
+    for (int s = kBucket - 1; s >= 0; s--) {
+        const bool hit = s >= from && (e[s] == kEmptySlot || (uint32_t)(e[s] >> 32) == tag);
+        at = hit ? s : at;
+        held = hit ? e[s] : held;
+    }
+    return at;
+}
+
+// The representative start of the window that starts at history position j: the one its slot holds, or j itself after
+// claiming the first empty slot of the probe sequence.  Slots fill in probe order and are never emptied, so two threads with
+// the same window end at one slot.  The window's set of starts stands at the place of its representative in `top`.
+__device__ __forceinline__ int find_or_claim(u64 *slots, unsigned int bmask, const int32_t *hist, int j, int w) {
+    const u64 h = window_hash(hist + j, w);
+    const uint32_t tag = (uint32_t)(h >> 32);
+    unsigned int b = (unsigned int)h & bmask, probes = 0;
+    u64 e[kBucket];
+    load_bucket(slots, b, e);
+    int from = 0;
+    while (probes <= bmask) {
+        u64 held;
+        const int s = find_in_bucket(e, tag, from, held);
+        if (s == kBucket) {                   // full of other windows: the next bucket
+            b = (b + 1) & bmask;
+            probes++;
+            load_bucket(slots, b, e);
+            from = 0;
+            continue;
+        }
+        u64 *at = slots + (size_t)b * kBucket + s;
+        if (held == kEmptySlot) {
+            held = atomicCAS(at, kEmptySlot, ((u64)tag << 32) | (uint32_t)j);
+            if (held == kEmptySlot) return j;
+        }
+        if ((uint32_t)(held >> 32) == tag && same_window(hist + (int)(uint32_t)held, hist + j, w)) return (int)(uint32_t)held;
+        from = s + 1;
+    }
+    return -1;   // the table has at least twice as many slots as windows: not reached
+}
+
+// Start j enters a window's set of the K largest starts (-1 = empty entry): it takes the place of the smallest entry, by
+// compare-and-swap, until that succeeds or every entry is larger.  Entries only grow, so what a thread has seen of an entry is
+// never more than it holds: a value is replaced only when K larger ones exist, and j gives up only when K larger ones exist.
+// The set ends as the K largest values ever offered, whatever the interleaving; the order of its entries is of no meaning.
+// One look at the set and one swap are two trips to L2 (a sorted list, kept by a cascade of atomicMax, cost up to K).
+__device__ __forceinline__ void set_insert(int32_t *set, int K, int j) {
+    int v[16];
 #pragma unroll
-                    for (int u = 0; u < 8; u++) ne |= (q[u] != h[u]) ? (1u << u) : 0u;
-                    if (ne) { L += __ffs(ne) - 1; open = false; }
-                    else L += 8;
-                }
-                while (open && L < room && p.query[i + L] == p.hist[j + L]) L++;
-                if (L > bestL || (L == bestL && j > bestj)) { bestL = L; bestj = j; }
-            };
-            if (p.next) {
-                // every occurrence of the window (at most nwin of them: the walk is bounded by construction)
-                int j = p.top[slot];
-                for (int n = 0; j >= 0 && n < p.nwin; n++) {
-                    if (j >= p.first_live) consider(j);
-                    j = p.next[j];
-                }
-            } else {
-                const int32_t *lst = p.top + (long long)slot * p.K;
-                for (int r = 0; r < p.K; r++) {
-                    const int j = lst[r];
-                    if (j < p.first_live) break;   // descending: the rest is empty (-1) or older than the live window
-                    consider(j);
-                }
-            }
-        }
-    }
-    p.best[i] = make_int2(bestL, bestj);
-}
-
-// Selection.  (1) hop[p] = (s, s + len(s)) with s the first position >= p that has a candidate (n_query if
-// none): a suffix scan, done grid-wide in two launches -- first the first candidate of every chunk of 1024
-// positions, then every chunk completes its positions with the first candidate of the later chunks as carry --
-// which also leaves the jump lengths hop.y - p as 16-bit deltas (65535 = "look it up in hop").  (2) One thread
-// of a single CTA follows the chain from 0 and lists the positions it visits: the serial part of Eq. 3, one
-// dependent read per selected span; the deltas of a window of positions are staged in shared memory so that each
-// read is a shared-memory access instead of a trip to L2.  (3) A grid-wide kernel turns the visited positions into
-// spans and per-token rows.
-constexpr int kWalkWindow = 96 * 1024;  // positions per window: 192 KiB of shared memory
-constexpr int kHopChunk = 1024;         // positions per CTA of the suffix scan
-
-__global__ void __launch_bounds__(kHopChunk) match_chunk_first_kernel(MatchParams p) {
-    __shared__ int s_first;
-    const int i = blockIdx.x * kHopChunk + threadIdx.x;
-    if (threadIdx.x == 0) s_first = p.n_query;
-    __syncthreads();
-    const bool st = i < p.n_query && p.best[i].x > 0;
-    const unsigned int b = __ballot_sync(0xffffffffu, st);
-    if (b && (threadIdx.x & 31) == 0) atomicMin(&s_first, i + __ffs(b) - 1);
-    __syncthreads();
-    if (threadIdx.x == 0) p.chunk_first[blockIdx.x] = s_first;
-}
-
-__global__ void __launch_bounds__(kHopChunk) match_hop_kernel(MatchParams p, int nchunks) {
-    __shared__ int warp_first[kHopChunk / 32];
-    __shared__ int s_carry;
-    const int N = p.n_query;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int i = blockIdx.x * kHopChunk + tid;
-    const int len = i < N ? p.best[i].x : 0;
-    const unsigned int b = __ballot_sync(0xffffffffu, len > 0);
-    if (lane == 0) warp_first[warp] = b ? (i + __ffs(b) - 1) : N;
-    if (tid == 0) {
-        int c = N;   // first candidate of the later chunks
-        for (int k = blockIdx.x + 1; k < nchunks; k++) {
-            const int f = p.chunk_first[k];
-            if (f < N) { c = f; break; }
-        }
-        s_carry = c;
-    }
-    __syncthreads();
-    if (i >= N) return;
-    const unsigned int at_or_after = b >> lane;
-    int s;
-    if (at_or_after) {
-        s = i + __ffs(at_or_after) - 1;
-    } else {
-        s = s_carry;
-        for (int w = warp + 1; w < kHopChunk / 32; w++) {
-            if (warp_first[w] < N) { s = warp_first[w]; break; }
-        }
-    }
-    const int nx = s < N ? s + p.best[s].x : N;
-    p.hop[i] = make_int2(s, nx);
-}
-
-// pointer doubling over "the position after the span at or after i": two spans, then four; the chain walk then
-// takes one dependent step per FOUR selected spans
-__global__ void match_jump2_kernel(MatchParams p) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= p.n_query) return;
-    const int a = p.hop[i].y;
-    p.jump2[i] = a < p.n_query ? p.hop[a].y : p.n_query;
-}
-__global__ void match_jump4_kernel(MatchParams p) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= p.n_query) return;
-    const int a = p.jump2[i];
-    const int b = a < p.n_query ? p.jump2[a] : p.n_query;
-    p.jump4[i] = b;
-    const int dlt = b - i;
-    p.delta16[i] = (unsigned short)(dlt < 65535 ? dlt : 65535);
-}
-
-__global__ void __launch_bounds__(1024) match_select_kernel(MatchParams p, int window) {
-    extern __shared__ unsigned short s_delta[];
-    __shared__ int s_nspans, s_pos;
-    const int N = p.n_query;
-    const int tid = threadIdx.x;
-    if (tid == 0) { s_pos = 0; s_nspans = 0; }
-    __syncthreads();
-
-    // (2) the chain, window by window; spans_ws[n].q_start keeps the n-th visited position
-    while (true) {
-        const int wbeg = s_pos;
-        if (wbeg >= N) break;
-        const int wend = min(N, wbeg + window);
-        // eight deltas per load where the window start allows it (the array itself is 16-byte aligned)
-        if ((wbeg & 7) == 0) {
-            const int n8 = (wend - wbeg) >> 3;
-            const uint4 *src = reinterpret_cast<const uint4 *>(p.delta16 + wbeg);
-            uint4 *dst = reinterpret_cast<uint4 *>(s_delta);
-            for (int i = tid; i < n8; i += blockDim.x) dst[i] = src[i];
-            for (int i = wbeg + (n8 << 3) + tid; i < wend; i += blockDim.x) s_delta[i - wbeg] = p.delta16[i];
+    for (int m = 0; m < 4; m++) {
+        if ((K & 3) == 0) {       // whole 16-byte pieces (the table's sections are 16-byte aligned)
+            int4 q = make_int4(0x7fffffff, 0x7fffffff, 0x7fffffff, 0x7fffffff);
+            if (4 * m < K) q = __ldcg(reinterpret_cast<const int4 *>(set) + m);
+            v[4 * m] = q.x; v[4 * m + 1] = q.y; v[4 * m + 2] = q.z; v[4 * m + 3] = q.w;
         } else {
-            for (int i = wbeg + tid; i < wend; i += blockDim.x) s_delta[i - wbeg] = p.delta16[i];
+#pragma unroll
+            for (int u = 0; u < 4; u++) v[4 * m + u] = 4 * m + u < K ? __ldcg(set + 4 * m + u) : 0x7fffffff;
         }
-        __syncthreads();
-        if (tid == 0) {
-            int n = s_nspans, pos = wbeg;
-            while (pos < wend) {
-                p.spans_ws[n++].q_start = pos;          // start of a group of (up to) four spans
-                const int dlt = s_delta[pos - wbeg];
-                pos = dlt == 65535 ? p.jump4[pos] : pos + dlt;
-            }
-            s_nspans = n;
-            s_pos = pos;
-        }
-        __syncthreads();
     }
-    if (tid == 0) {
-        p.chunk_first[0] = s_nspans;   // the suffix scan is done with this array: it now carries the group count
-        *p.n_spans = 0;                // the expansion of the last group sets the real count
+    while (true) {
+        int low = v[0], at = 0;
+        unsigned int empty = 0;
+#pragma unroll
+        for (int r = 0; r < 16; r++) {
+            if (v[r] < low) { low = v[r]; at = r; }
+            empty |= v[r] < 0 ? (1u << r) : 0u;
+        }
+        if (empty) {              // threads with the same window start at different empty entries
+            const unsigned int later = empty & ~((1u << (j % K)) - 1u);
+            at = __ffs(later ? later : empty) - 1;
+        }
+        if (low > j) return;
+        const int found = atomicCAS(&set[at], low, j);
+        if (found == low) return;
+#pragma unroll
+        for (int r = 0; r < 16; r++) v[r] = r == at ? found : v[r];
     }
 }
+// Start j enters the index.  Unlimited hits: every start goes onto its window's chain.  The order of a chain
+// depends on which thread came first; the query looks at ALL of it and keeps lexargmax(length, start), so the result does not.
+__device__ __forceinline__ void index_start(u64 *slots, int32_t *top, int32_t *next, unsigned int bmask, const int32_t *hist,
+                                            int j, int w, int K) {
+    const int rep = find_or_claim(slots, bmask, hist, j, w);
+    if (rep < 0) return;
+    if (next) next[j] = atomicExch(&top[rep], j);
+    else set_insert(top + (size_t)rep * K, K, j);
+}
 
-// (3) grid-wide: a warp per group walks its (up to) four spans -- three dependent lookups each -- and expands them
-// to rows; only the last group can hold fewer than four, and its warp sets the span count
-__global__ void match_expand_kernel(MatchParams p) {
+// all ones in n16 pieces of 16 bytes; with zero, also *zero = 0
+__global__ void fill_ones_kernel(uint4 *dst, long long n16, int32_t *zero) {
+    grid_launch_dependents();
+    grid_dependency_wait();
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    for (long long k = i; k < n16; k += (long long)gridDim.x * blockDim.x) dst[k] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    if (zero && i == 0) *zero = 0;
+}
+
+__global__ void __launch_bounds__(256) match_insert_kernel(const MatchParams p) {
+    grid_launch_dependents();
+    grid_dependency_wait();
+    // the latest starts first: once a set is full of them the earlier ones are done with one look
+    const int j = p.nwin - 1 - (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (j >= 0) index_start(p.slots, p.top, p.next, p.bmask, p.hist, j, p.w, p.K);
+}
+
+// first position at or after this thread's position in its chunk that has a candidate (`limit` if none)
+__device__ __forceinline__ int next_candidate(bool has, int i, int limit) {
+    __shared__ int s_first[kChunk / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned int b = __ballot_sync(0xffffffffu, has);
+    if (lane == 0) s_first[warp] = b ? i + __ffs(b) - 1 : limit;
+    __syncthreads();
+    if (b >> lane) return i + __ffs(b >> lane) - 1;
+    for (int w = warp + 1; w < kChunk / 32; w++)
+        if (s_first[w] < limit) return s_first[w];
+    return limit;
+}
+
+// Lookup, extension, and the chunk's jumps.  One CTA per chunk, one thread per position.
+// Extension: a thread compares eight tokens at its candidate by itself; what is still open after that is finished by the
+// warp, 128 tokens per trip.  Neighbouring positions inside one copied stretch have the same (history - query) distance and
+// so the same end: one comparison closes them all.  A thread by itself took a trip per eight tokens, for every position
+// of a long match (2048-token prompt: 21 us, with copies of copies 55 us).
+__global__ void __launch_bounds__(kChunk, 2) match_query_kernel(const MatchParams p) {
+    grid_launch_dependents();
+    grid_dependency_wait();
     const int N = p.n_query;
-    const int ng = p.chunk_first[0];
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    for (int g = gw; g < ng; g += warps) {
-        int pos = p.spans_ws[g].q_start;
-        int m = 0;
-        for (; m < 4 && pos < N; m++) {
-            const int2 h = p.hop[pos];
-            if (h.x >= N) break;               // no candidate at or after pos: the chain ends
-            rac_span sp;
-            sp.q_start = h.x;
-            sp.len = h.y - h.x;
-            sp.h_start = p.best[h.x].y;
-            if (lane == 0 && p.spans_out) p.spans_out[4 * g + m] = sp;
-            for (int q = lane; q < sp.len; q += 32) p.ref_row[sp.q_start + q] = sp.h_start + q;
-            pos = h.y;
+    const int base = blockIdx.x * kChunk, i = base + threadIdx.x, lane = threadIdx.x & 31;
+    if (p.trep && i < N) {     // intra-sequence references: the first position of every token of the prompt
+        const int32_t tok = p.query[i];
+        unsigned int s = (unsigned int)window_hash(&tok, 1) & p.tmask;
+        for (unsigned int probe = 0; probe <= p.tmask; probe++) {
+            int cur = __ldcg(p.trep + s);
+            if (cur < 0) cur = atomicCAS(&p.trep[s], -1, i);
+            if (cur < 0 || p.query[cur] == tok) {
+                if (__ldcg(p.tfirst + s) < kFirstBase - i) atomicMax(&p.tfirst[s], kFirstBase - i);
+                break;
+            }
+            s = (s + 1) & p.tmask;
         }
-        if (g == ng - 1 && lane == 0) *p.n_spans = 4 * g + m;
+    }
+    int rep = -1;      // representative start of the window at i, -1: not in the history
+    if (i < N && i + p.w <= N && p.nwin > 0) {
+        const int32_t *win = p.query + i;
+        const u64 h = window_hash(win, p.w);
+        const uint32_t tag = (uint32_t)(h >> 32);
+        unsigned int b = (unsigned int)h & p.bmask;
+        u64 e[kBucket];
+        load_bucket(p.slots, b, e);
+        int from = 0;
+        for (unsigned int probe = 0; probe <= p.bmask;) {
+            u64 held;
+            const int s = find_in_bucket(e, tag, from, held);
+            if (s == kBucket) {
+                b = (b + 1) & p.bmask;
+                probe++;
+                load_bucket(p.slots, b, e);
+                from = 0;
+                continue;
+            }
+            if (held == kEmptySlot) break;      // ends the probe sequence: the window is not in the history
+            if (same_window(p.hist + (int)(uint32_t)held, win, p.w)) {
+                rep = (int)(uint32_t)held;
+                break;
+            }
+            from = s + 1;
+        }
+    }
+    int bestL = 0, bestj = -1;
+    // one candidate per lane (j = -1: none), all lanes of the warp together; `room`: the longest its match can be
+    auto consider = [&](int j, int room) {
+        int L = 0;
+        bool open = false;
+        if (j >= 0) {
+            L = p.w;
+            uint32_t ne = 0;
+            const int n8 = min(8, room - L);
+            int32_t q[8], hh[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                q[u] = u < n8 ? p.query[i + L + u] : 0;
+                hh[u] = u < n8 ? p.hist[j + L + u] : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; u++) ne |= (u >= n8 || q[u] != hh[u]) ? (1u << u) : 0u;
+            open = ne == 0u;
+            L += open ? 8 : __ffs(ne) - 1;
+        }
+        unsigned int todo = __ballot_sync(0xffffffffu, open);
+        while (todo) {
+            const int lead = __ffs(todo) - 1;
+            const int i0 = __shfl_sync(0xffffffffu, i, lead), j0 = __shfl_sync(0xffffffffu, j, lead);
+            const int L0 = __shfl_sync(0xffffffffu, L, lead), room0 = __shfl_sync(0xffffffffu, room, lead);
+            int len = L0;
+            bool more = true;
+            while (more && len < room0) {
+                uint32_t differ = 0;                   // bit u: the lane's token of the u-th 32 differs or lies outside
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const int at = len + 32 * u + lane;
+                    differ |= (at >= room0 || p.query[i0 + at] != p.hist[j0 + at]) ? (1u << u) : 0u;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const unsigned int b = __ballot_sync(0xffffffffu, (differ >> u) & 1u);
+                    if (more) {
+                        if (b) { len += __ffs(b) - 1; more = false; }
+                        else len += 32;
+                    }
+                }
+            }
+            // every open position of the same distance that lies before the end has the same end
+            const int end = i0 + len;
+            if (open && j - i == j0 - i0 && i < end) { L = end - i; open = false; }
+            todo = __ballot_sync(0xffffffffu, open);
+        }
+        if (j >= 0 && (L > bestL || (L == bestL && j > bestj))) { bestL = L; bestj = j; }
+    };
+    auto room_of = [&](int j) { return min(N - i, (p.end_of ? p.end_of[j] : p.n_hist) - j); };   // inside its request
+    if (p.next) {
+        // every occurrence of the window (at most nwin of them: the walk is bounded by construction)
+        int chain = rep >= 0 ? p.top[rep] : -1, n = 0;
+        while (true) {
+            while (chain >= 0 && chain < p.first_live && n < p.nwin) { chain = p.next[chain]; n++; }
+            const int j = n < p.nwin ? chain : -1;
+            if (!__any_sync(0xffffffffu, j >= 0)) break;
+            if (j >= 0) { chain = p.next[j]; n++; }
+            consider(j, j >= 0 ? room_of(j) : 0);
+        }
+    } else {
+        // The K most recent starts.  A candidate replaces the best so far only with a longer match, or with one as long and a
+        // larger start, so its last token of that length has to match: after the first candidate, one trip for all the others
+        // rules most of them out before they are extended.
+        const int32_t *set = p.top + (size_t)(rep >= 0 ? rep : 0) * p.K;
+        auto can_win = [&](int j) {
+            const int at = bestL - (j > bestj ? 1 : 0);
+            return bestL == 0 || (room_of(j) > at && p.hist[j + at] == p.query[i + at]);
+        };
+        unsigned int alive = 0;
+        if (rep >= 0) {
+#pragma unroll 4
+            for (int r = 0; r < p.K; r++) alive |= set[r] >= p.first_live ? (1u << r) : 0u;   // first_live >= 0: no empty ones
+        }
+        bool first = true;
+        while (__any_sync(0xffffffffu, alive != 0u)) {
+            // largest start first: neighbours inside one copied stretch then look at the same distance at the same time
+            int j = -1, at = 0;
+            if (alive) {
+#pragma unroll 4
+                for (int r = 0; r < p.K; r++) {
+                    const int k = ((alive >> r) & 1u) ? set[r] : -1;
+                    if (k > j) { j = k; at = r; }
+                }
+                alive &= ~(1u << at);
+                if (!first && !can_win(j)) j = -1;
+            }
+            if (!__any_sync(0xffffffffu, j >= 0)) continue;
+            consider(j, j >= 0 ? room_of(j) : 0);
+            if (first && alive) {
+#pragma unroll 4
+                for (int r = 0; r < p.K; r++)
+                    if (((alive >> r) & 1u) && !can_win(set[r])) alive &= ~(1u << r);
+            }
+            first = false;
+        }
+    }
+    if (i < N) p.best[i] = make_int2(bestL, bestj);
+
+    // ---- where a scan that is at position i leaves the chunk, by pointer doubling
+    __shared__ int s_nxt[kChunk], s_cnt[kChunk];
+    const int limit = min(base + kChunk, N);
+    int nxt = next_candidate(bestL > 0, i, limit), cnt = 0;
+    if (bestL > 0) { nxt = i + bestL; cnt = 1; }
+    if (i >= limit) { nxt = limit; cnt = 0; }
+    while (true) {
+        s_nxt[threadIdx.x] = nxt;
+        s_cnt[threadIdx.x] = cnt;
+        if (!__syncthreads_or(nxt < limit)) break;
+        if (nxt < limit) {
+            const int k = nxt - base;
+            nxt = s_nxt[k];
+            cnt += s_cnt[k];
+        }
+        __syncthreads();
+    }
+    if (i < N) p.jump[i] = make_int2(nxt, cnt);
+}
+
+// Where the scan enters every chunk: entry of chunk c+1 = where a scan that enters chunk c at ITS entry leaves it.  All
+// chunks guess their first position and exchange exits until nothing changes; scans that enter a chunk at different
+// positions usually leave it at the same one, so two or three exchanges do (at most one per chunk, as in the serial walk).
+// One CTA, 1024 chunks at a time.
+__global__ void __launch_bounds__(1024) match_resolve_kernel(const MatchParams p, int nchunks) {
+    __shared__ int s_exit[1024], s_warp[32];
+    grid_launch_dependents();
+    grid_dependency_wait();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int carry = 0, carry_cnt = 0;
+    for (int c0 = 0; c0 < nchunks; c0 += 1024) {
+        const int c = c0 + tid;
+        const int start = c * kChunk, end = min(start + kChunk, p.n_query);
+        const bool live = c < nchunks;
+        int e = tid == 0 ? carry : start, exit = e, cnt = 0;
+        while (true) {
+            exit = e;
+            cnt = 0;
+            if (live && e < end) {
+                const int2 j = __ldcg(p.jump + e);
+                exit = j.x;
+                cnt = j.y;
+            }
+            s_exit[tid] = exit;
+            __syncthreads();
+            const int ne = tid == 0 ? carry : s_exit[tid - 1];
+            const bool changed = live && ne != e;
+            e = ne;
+            if (!__syncthreads_or(changed)) break;
+        }
+        // spans selected before the chunk
+        int incl = live ? cnt : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, incl, o);
+            incl += lane >= o ? up : 0;
+        }
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        int before = carry_cnt, total = 0;
+        for (int w = 0; w < 32; w++) {
+            before += w < warp ? s_warp[w] : 0;
+            total += s_warp[w];
+        }
+        if (live) p.entry[c] = make_int2(e, before + incl - cnt);
+        carry = s_exit[min(1024, nchunks - c0) - 1];
+        carry_cnt += total;
+        __syncthreads();
+    }
+    if (tid == 0) *p.n_spans = carry_cnt;
+}
+
+// Spans and rows: the scan through one chunk from its entry.  Every position at or after the entry belongs to this CTA
+// alone, and so does the part of its last span that reaches into later chunks (their entries lie behind it).
+__global__ void __launch_bounds__(kChunk) match_emit_kernel(const MatchParams p, int nchunks) {
+    __shared__ int s_next[kChunk], s_len[kChunk], s_row[kChunk], s_list[kChunk];
+    __shared__ int s_entry, s_base, s_n;
+    grid_launch_dependents();
+    grid_dependency_wait();
+    const int N = p.n_query, c = blockIdx.x;
+    const int base = c * kChunk, limit = min(base + kChunk, N), i = base + threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int2 mine = i < N ? __ldcg(p.best + i) : make_int2(0, -1);
+    if (threadIdx.x == 0) {
+        int e = 0, before = 0;
+        if (nchunks > kInlineChunks) {
+            const int2 v = __ldcg(p.entry + c);
+            e = v.x;
+            before = v.y;
+        } else {
+            for (int k = 0; k < c; k++) {
+                if (e >= min((k + 1) * kChunk, N)) continue;
+                const int2 v = __ldcg(p.jump + e);
+                e = v.x;
+                before += v.y;
+            }
+        }
+        s_entry = e;
+        s_base = before;
+    }
+    s_next[threadIdx.x] = next_candidate(mine.x > 0, i, limit);
+    s_len[threadIdx.x] = mine.x;
+    s_row[threadIdx.x] = -1;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int pos = s_entry, n = 0;
+        while (pos < limit) {
+            const int s = s_next[pos - base];
+            if (s >= limit) break;
+            s_list[n++] = s - base;
+            pos = s + s_len[s - base];
+        }
+        s_n = n;
+        if (nchunks <= kInlineChunks && c == nchunks - 1) *p.n_spans = s_base + n;
+    }
+    __syncthreads();
+    const int n = s_n, entry = s_entry;
+    for (int k = warp; k < n; k += kChunk / 32) {        // a warp per span, up to the end of the chunk
+        const int at = s_list[k], len = s_len[at], s = base + at;
+        const int h = __ldcg(&p.best[s].y);
+        if (lane == 0 && p.spans_out) {
+            rac_span sp;
+            sp.q_start = s;
+            sp.h_start = h;
+            sp.len = len;
+            p.spans_out[s_base + k] = sp;
+        }
+        const int in = min(len, limit - s);
+        for (int q = lane; q < in; q += 32) s_row[at + q] = h + q;
+    }
+    if (n > 0) {                                         // the last span's part in later chunks: the whole CTA
+        const int at = s_list[n - 1], s = base + at, end = s + s_len[at];
+        const int h = __ldcg(&p.best[s].y);
+        for (int q = limit + threadIdx.x; q < end; q += kChunk) p.ref_row[q] = h + (q - s);
+    }
+    __syncthreads();
+    if (i < N && i >= entry) {
+        int row = s_row[threadIdx.x];
+        if (row < 0 && p.trep) {
+            // intra-sequence reference: the first occurrence of this token, if it is an earlier one
+            const int32_t tok = p.query[i];
+            unsigned int s = (unsigned int)window_hash(&tok, 1) & p.tmask;
+            for (unsigned int probe = 0; probe <= p.tmask; probe++) {
+                const int cur = __ldcg(p.trep + s);
+                if (cur < 0) break;
+                if (p.query[cur] == tok) {
+                    const int f = kFirstBase - __ldcg(p.tfirst + s);
+                    if (f < i) row = p.n_hist + f;
+                    break;
+                }
+                s = (s + 1) & p.tmask;
+            }
+        }
+        p.ref_row[i] = row;
     }
 }
 
 __global__ void spans_to_rows_kernel(const rac_span *spans, const int32_t *n_spans, long long n_query, int32_t *ref_row) {
+    grid_launch_dependents();
+    grid_dependency_wait();
     const int ns = *n_spans;
     const int warps = (gridDim.x * blockDim.x) >> 5;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -316,6 +542,8 @@ __global__ void __launch_bounds__(1024) spans_to_segments_kernel(const rac_span 
                                                                  int max_seg, int32_t *seg_off, int32_t *n_seg) {
     __shared__ int s_scan[1024];
     __shared__ int s_base;
+    grid_launch_dependents();
+    grid_dependency_wait();
     const int ns = min(*n_spans, (max_seg - 1) / 2);
     const int tid = threadIdx.x;
     if (tid == 0) { s_base = 1; seg_off[0] = 0; }   // boundary 0 always; every span adds its start (if a gap precedes) and its end
@@ -358,6 +586,8 @@ __global__ void __launch_bounds__(1024) spans_to_segments_kernel(const rac_span 
 }
 
 __global__ void fill_i32_kernel(int32_t *dst, long long n, int32_t v) {
+    grid_launch_dependents();
+    grid_dependency_wait();
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     long long stride = (long long)gridDim.x * blockDim.x;
     for (; i < n; i += stride) dst[i] = v;
@@ -368,73 +598,26 @@ __global__ void fill_i32_kernel(int32_t *dst, long long n, int32_t v) {
 // ---------------------------------------------------------------------------------------------
 struct IndexParams {
     const int32_t *hist;
-    int32_t *rep;       // [M]
-    int32_t *top;       // [M*K]
+    u64 *slots;         // [M]
+    int32_t *top;       // [capacity*K]
     int32_t *end_of;    // [capacity]
     int32_t *next;      // [capacity]  no cap on the hits: another start of the same window (chain link), else null
-    int32_t *cnt;       // [M]         unused (kept so that the layout of an index does not change)
     int a, b;           // the request: tokens [a, b)
     int w, K;
-    unsigned int mask;
+    unsigned int bmask;
 };
 
 // Appending a request: every position learns the end of its request; every window of the request finds or claims
-// its slot and enters the slot's list by the cascade.  The request's starts are larger than everything already
-// there, so the older entries move down (and the oldest fall off) as a by-product.  One launch, any request size.
-__global__ void index_append_kernel(IndexParams p) {
-    const int j = p.a + blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= p.b) return;
+// its slot and enters the slot's set.  The request's starts are larger than everything already there, so the oldest
+// entries fall out as a by-product.  One launch, any request size.
+__global__ void __launch_bounds__(128) index_append_kernel(const IndexParams p) {
+    grid_launch_dependents();
+    grid_dependency_wait();
+    const int j = p.b - 1 - (int)(blockIdx.x * blockDim.x + threadIdx.x);   // the latest starts first
+    if (j < p.a) return;
     p.end_of[j] = p.b;
-    if (j + p.w > p.b) return;  // the window would leave the request
-    const int32_t *win = p.hist + j;
-    unsigned int s = window_hash(win, p.w) & p.mask;
-    int slot = -1;
-    for (unsigned int probe = 0; probe <= p.mask; probe++) {
-        int cur = atomicCAS(&p.rep[s], -1, j);
-        if (cur == -1 || cur == j || same_window(p.hist + cur, win, p.w)) { slot = (int)s; break; }
-        s = (s + 1) & p.mask;
-    }
-    if (slot < 0) return;
-    if (p.next) p.next[j] = atomicExch(&p.top[slot], j);   // every start, on the slot's chain (order irrelevant)
-    else cascade_insert(p.top + (long long)slot * p.K, p.K, j);
-}
-
-// Intra-sequence references: first occurrence of every token of the prompt (a hash table keyed by a position
-// whose token is the key, verified by comparing tokens), then the uncovered positions look theirs up.
-__global__ void intra_insert_kernel(const int32_t *query, int n, int32_t *trep, int32_t *tfirst, unsigned int mask) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int32_t tok = query[i];
-    unsigned int s = window_hash(&tok, 1) & mask;
-    for (unsigned int probe = 0; probe <= mask; probe++) {
-        int cur = atomicCAS(&trep[s], -1, i);
-        if (cur == -1 || cur == i || query[cur] == tok) { atomicMin(&tfirst[s], i); return; }
-        s = (s + 1) & mask;
-    }
-}
-__global__ void intra_assign_kernel(const int32_t *query, int n, const int32_t *trep, const int32_t *tfirst,
-                                    unsigned int mask, int n_hist, int32_t *ref_row) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || ref_row[i] >= 0) return;
-    const int32_t tok = query[i];
-    unsigned int s = window_hash(&tok, 1) & mask;
-    for (unsigned int probe = 0; probe <= mask; probe++) {
-        int cur = trep[s];
-        if (cur < 0) return;
-        if (query[cur] == tok) {
-            const int f = tfirst[s];
-            if (f < i) ref_row[i] = n_hist + f;
-            return;
-        }
-        s = (s + 1) & mask;
-    }
-}
-
-__global__ void fill2_i32_kernel(int32_t *a, long long na, int32_t va, int32_t *b, long long nb, int32_t vb) {
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long k = i; k < na; k += stride) a[k] = va;
-    for (long long k = i; k < nb; k += stride) b[k] = vb;
+    if (j + p.w <= p.b)      // else the window would leave the request
+        index_start(p.slots, p.top, p.next, p.bmask, p.hist, j, p.w, p.K);
 }
 
 static size_t align16(size_t v) { return (v + 15) / 16 * 16; }
@@ -454,50 +637,47 @@ static int sm_count() {
     return cache[dev];
 }
 
-// the six launches of the selection (suffix scan and pointer doubling grid-wide, chain walk in one CTA, expansion
-// grid-wide)
-static int launch_selection(const MatchParams &p, cudaStream_t st) {
-    const int nchunks = (p.n_query + kHopChunk - 1) / kHopChunk;
-    match_chunk_first_kernel<<<nchunks, kHopChunk, 0, st>>>(p);
-    match_hop_kernel<<<nchunks, kHopChunk, 0, st>>>(p, nchunks);
-    match_jump2_kernel<<<(p.n_query + 255) / 256, 256, 0, st>>>(p);
-    match_jump4_kernel<<<(p.n_query + 255) / 256, 256, 0, st>>>(p);
-    const int window = p.n_query < kWalkWindow ? p.n_query : kWalkWindow;
-    const size_t dyn = ((size_t)window * 2 + 15) / 16 * 16;
-    if (dyn > 48 * 1024 &&
-        cudaFuncSetAttribute(match_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-        return RAC_ECUDA;
-    match_select_kernel<<<1, 1024, dyn, st>>>(p, window);
-    match_expand_kernel<<<sm_count(), 256, 0, st>>>(p);
-    return RAC_OK;
+static int fill_blocks(long long n16) {
+    const long long b = (n16 + 255) / 256, most = (long long)sm_count() * 8;
+    return (int)(b < 1 ? 1 : b > most ? most : b);
+}
+// Slots for n windows: at least `per` each.  Four per window leave one bucket in 250 full, two one in seven, and the slowest
+// of a warp's lanes sets its pace.
+static unsigned int table_slots(long long n, unsigned long long per) {
+    unsigned long long M = 1024;
+    while (M < per * (unsigned long long)(n > 0 ? n : 1)) M <<= 1;
+    return (unsigned int)M;
 }
 
-
+// lookup and extension, the chunks' entries (few chunks are walked in the last kernel instead: up to seven hops cost less
+// than a launch), spans and rows
+static void launch_query(const MatchParams &p, cudaStream_t st) {
+    const int nchunks = (p.n_query + kChunk - 1) / kChunk;
+    launch_after(match_query_kernel, nchunks, kChunk, 0, st, p);
+    if (nchunks > kInlineChunks) launch_after(match_resolve_kernel, 1, 1024, 0, st, p, nchunks);
+    launch_after(match_emit_kernel, nchunks, kChunk, 0, st, p, nchunks);
+}
 
 struct MatchLayout {
-    size_t rep, top, slot_of, best, hop, spans, chunk_first, delta16, jump2, jump4, next, total;
+    size_t slots, top, filled, best, jump, entry, next, total;
     unsigned int M;
 };
-// K = 0 (unlimited hits): one entry per slot (the head of its chain) and a chain link per history position
+// K = 0 (unlimited hits): one entry per window (the head of its chain) and a chain link per history position
 static MatchLayout match_layout(long long n_hist, long long n_query, int K) {
     MatchLayout L;
     const bool chains = K == 0;
     if (chains) K = 1;
-    unsigned long long M = 1024;
-    while (M < 2ull * (unsigned long long)(n_hist > 0 ? n_hist : 1)) M <<= 1;
-    L.M = (unsigned int)M;
+    const size_t n = (size_t)(n_query > 0 ? n_query : 1);
+    const size_t h = (size_t)(n_hist > 0 ? n_hist : 1);
+    L.M = table_slots(n_hist, 4);
     size_t o = 0;
-    L.rep = o;      o += (size_t)M * 4;                       // rep and top must stay contiguous (one fill)
-    L.top = o;      o = align16(o + (size_t)M * K * 4);
-    L.slot_of = o;  o = align16(o + (size_t)(n_hist > 0 ? n_hist : 1) * 4);
-    L.best = o;     o = align16(o + (size_t)(n_query > 0 ? n_query : 1) * 8);
-    L.hop = o;      o = align16(o + (size_t)(n_query > 0 ? n_query : 1) * 8);
-    L.spans = o;    o = align16(o + (size_t)(n_query + 1) * sizeof(rac_span));
-    L.chunk_first = o; o = align16(o + ((size_t)(n_query > 0 ? n_query : 1) / kHopChunk + 1) * 4);
-    L.delta16 = o;  o = align16(o + (size_t)(n_query > 0 ? n_query : 1) * 2);
-    L.jump2 = o;    o = align16(o + (size_t)(n_query > 0 ? n_query : 1) * 4);
-    L.jump4 = o;    o = align16(o + (size_t)(n_query > 0 ? n_query : 1) * 4);
-    L.next = o;     if (chains) o = align16(o + (size_t)(n_hist > 0 ? n_hist : 1) * 4);
+    L.slots = o;    o += (size_t)L.M * 8;                      // slots and top must stay contiguous (one fill)
+    L.top = o;      o = align16(o + h * K * 4);
+    L.filled = o;
+    L.best = o;     o = align16(o + n * 8);
+    L.jump = o;     o = align16(o + n * 8);
+    L.entry = o;    o = align16(o + (n / kChunk + 1) * 8);
+    L.next = o;     if (chains) o = align16(o + h * 4);
     L.total = o;
     return L;
 }
@@ -552,46 +732,31 @@ int rac_match_spans(const int32_t *hist_tok, int64_t n_hist, const int32_t *quer
     if (workspace_bytes < L.total) return RAC_ESIZE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
-    MatchParams p;
-    p.end_of = nullptr;
+    MatchParams p = {};
     p.hist = hist_tok;
     p.query = query_tok;
     p.ref_row = ref_row;
     p.spans_out = spans;
     p.n_spans = n_spans;
-    p.rep = reinterpret_cast<int32_t *>(ws + L.rep);
+    p.slots = reinterpret_cast<u64 *>(ws + L.slots);
     p.top = reinterpret_cast<int32_t *>(ws + L.top);
-    p.slot_of = reinterpret_cast<int32_t *>(ws + L.slot_of);
     p.best = reinterpret_cast<int2 *>(ws + L.best);
-    p.hop = reinterpret_cast<int2 *>(ws + L.hop);
-    p.spans_ws = reinterpret_cast<rac_span *>(ws + L.spans);
-    p.chunk_first = reinterpret_cast<int32_t *>(ws + L.chunk_first);
-    p.delta16 = reinterpret_cast<unsigned short *>(ws + L.delta16);
-    p.jump2 = reinterpret_cast<int32_t *>(ws + L.jump2);
-    p.jump4 = reinterpret_cast<int32_t *>(ws + L.jump4);
+    p.jump = reinterpret_cast<int2 *>(ws + L.jump);
+    p.entry = reinterpret_cast<int2 *>(ws + L.entry);
     p.n_hist = (int)n_hist;
     p.n_query = (int)n_query;
     p.nwin = (int)(n_hist - min_ngram + 1 > 0 ? n_hist - min_ngram + 1 : 0);
     p.w = min_ngram;
     p.K = max_hits > 0 ? max_hits : 1;
-    p.first_live = 0;
     p.next = max_hits == 0 ? reinterpret_cast<int32_t *>(ws + L.next) : nullptr;
-    p.mask = L.M - 1;
+    p.bmask = L.M / kBucket - 1;
 
-    const long long table_ints = (long long)L.M * (1 + p.K);
-    const int tb = 256;
-    long long work = table_ints > n_query ? table_ints : n_query;
-    int init_blocks = (int)((work + tb - 1) / tb);
-    if (init_blocks > sm_count() * 8) init_blocks = sm_count() * 8;
-    if (init_blocks < 1) init_blocks = 1;
-    match_init_kernel<<<init_blocks, tb, 0, st>>>(p, table_ints);
-    if (p.nwin > 0 && n_query > 0) {
-        int nb = (p.nwin + tb - 1) / tb;
-        match_insert_kernel<<<nb, tb, 0, st>>>(p);
-    }
+    // four launches, five when there are many chunks; the times are in the head of this file
+    const long long n16 = n_query > 0 ? (long long)(L.filled / 16) : 0;
+    launch_after(fill_ones_kernel, fill_blocks(n16), 256, 0, st, reinterpret_cast<uint4 *>(ws + L.slots), n16, n_spans);
     if (n_query > 0) {
-        match_query_kernel<<<(int)((n_query + tb - 1) / tb), tb, 0, st>>>(p);
-        if (launch_selection(p, st) != RAC_OK) return RAC_ECUDA;
+        if (p.nwin > 0) launch_after(match_insert_kernel, (p.nwin + 255) / 256, 256, 0, st, p);
+        launch_query(p, st);
     }
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
 }
@@ -604,8 +769,8 @@ int rac_spans_to_rows(const rac_span *spans, const int32_t *n_spans, int64_t n_q
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int blocks = (int)((n_query + 255) / 256);
     if (blocks > sm_count() * 8) blocks = sm_count() * 8;
-    fill_i32_kernel<<<blocks, 256, 0, st>>>(ref_row, n_query, -1);
-    spans_to_rows_kernel<<<sm_count(), 256, 0, st>>>(spans, n_spans, n_query, ref_row);
+    launch_after(fill_i32_kernel, blocks, 256, 0, st, ref_row, (long long)n_query, -1);
+    launch_after(spans_to_rows_kernel, sm_count(), 256, 0, st, spans, n_spans, (long long)n_query, ref_row);
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
 }
 
@@ -630,7 +795,7 @@ int rac_match_spans_static(const int32_t *hist_tok, int64_t n_hist, const int32_
 // ---- persistent index ------------------------------------------------------------------------
 namespace {
 struct IndexLayout {
-    size_t rep, top, cnt, end_of, slot_of, total;
+    size_t slots, top, filled, end_of, next, total;
     unsigned int M;
 };
 bool index_cfg_ok(const rac_index_cfg *c) {
@@ -639,45 +804,32 @@ bool index_cfg_ok(const rac_index_cfg *c) {
 }
 IndexLayout index_layout(const rac_index_cfg *c) {
     IndexLayout L;
-    unsigned long long M = 1024;
-    while (M < 2ull * (unsigned long long)c->capacity) M <<= 1;
-    L.M = (unsigned int)M;
+    L.M = table_slots(c->capacity, 4);
     size_t o = 0;
-    L.rep = o;      o += (size_t)M * 4;                        // rep and top contiguous: one fill with -1
-    L.top = o;      o = align16(o + (size_t)M * (c->max_hits > 0 ? c->max_hits : 1) * 4);
-    L.cnt = o;      o = align16(o + (size_t)M * 4);
+    L.slots = o;    o += (size_t)L.M * 8;                      // slots and top contiguous: one fill
+    L.top = o;      o = align16(o + (size_t)c->capacity * (c->max_hits > 0 ? c->max_hits : 1) * 4);
+    L.filled = o;
     L.end_of = o;   o = align16(o + (size_t)c->capacity * 4);
-    L.slot_of = o;  o = align16(o + (size_t)c->capacity * 4);
+    L.next = o;     o = align16(o + (size_t)c->capacity * 4);
     L.total = o;
     return L;
 }
 struct QueryLayout {
-    size_t best, hop, spans, chunk_first, delta16, jump2, jump4, trep, tfirst, total;
+    size_t best, jump, entry, trep, tfirst, total;
     unsigned int Mq;
 };
 QueryLayout query_layout(long long n_query) {
     QueryLayout L;
     const size_t n = (size_t)(n_query > 0 ? n_query : 1);
-    unsigned long long M = 1024;
-    while (M < 2ull * n) M <<= 1;
-    L.Mq = (unsigned int)M;
+    L.Mq = table_slots(n_query, 2);
     size_t o = 0;
     L.best = o;    o = align16(o + n * 8);
-    L.hop = o;     o = align16(o + n * 8);
-    L.spans = o;   o = align16(o + (n + 1) * sizeof(rac_span));
-    L.chunk_first = o; o = align16(o + (n / kHopChunk + 1) * 4);
-    L.delta16 = o; o = align16(o + n * 2);
-    L.jump2 = o;   o = align16(o + n * 4);
-    L.jump4 = o;   o = align16(o + n * 4);
-    L.trep = o;    o = align16(o + (size_t)M * 4);
-    L.tfirst = o;  o = align16(o + (size_t)M * 4);
+    L.jump = o;    o = align16(o + n * 8);
+    L.entry = o;   o = align16(o + (n / kChunk + 1) * 8);
+    L.trep = o;    o += (size_t)L.Mq * 4;                      // trep and tfirst contiguous: one fill
+    L.tfirst = o;  o += (size_t)L.Mq * 4;
     L.total = o;
     return L;
-}
-int grid_for(long long n, int tb) {
-    long long b = (n + tb - 1) / tb;
-    if (b > (long long)sm_count() * 16) b = (long long)sm_count() * 16;
-    return (int)(b < 1 ? 1 : b);
 }
 }  // namespace
 
@@ -691,10 +843,9 @@ int rac_index_reset(const rac_index_cfg *cfg, void *index, size_t index_bytes, v
     if (reinterpret_cast<uintptr_t>(index) & 15u) return RAC_EALIGN;
     const IndexLayout L = index_layout(cfg);
     if (index_bytes < L.total) return RAC_ESIZE;
-    unsigned char *ix = static_cast<unsigned char *>(index);
-    const long long table = (long long)L.M * (1 + (cfg->max_hits > 0 ? cfg->max_hits : 1));
-    fill2_i32_kernel<<<grid_for(table, 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        reinterpret_cast<int32_t *>(ix + L.rep), table, -1, reinterpret_cast<int32_t *>(ix + L.cnt), (long long)L.M, 0);
+    const long long n16 = (long long)(L.filled / 16);
+    launch_after(fill_ones_kernel, fill_blocks(n16), 256, 0, static_cast<cudaStream_t>(stream),
+                 reinterpret_cast<uint4 *>(static_cast<unsigned char *>(index) + L.slots), n16, (int32_t *)nullptr);
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
 }
 
@@ -711,20 +862,16 @@ int rac_index_append(const rac_index_cfg *cfg, void *index, size_t index_bytes, 
     unsigned char *ix = static_cast<unsigned char *>(index);
     IndexParams p;
     p.hist = hist_tok;
-    p.rep = reinterpret_cast<int32_t *>(ix + L.rep);
+    p.slots = reinterpret_cast<u64 *>(ix + L.slots);
     p.top = reinterpret_cast<int32_t *>(ix + L.top);
-    p.cnt = reinterpret_cast<int32_t *>(ix + L.cnt);
     p.end_of = reinterpret_cast<int32_t *>(ix + L.end_of);
-    p.next = cfg->max_hits == 0 ? reinterpret_cast<int32_t *>(ix + L.slot_of) : nullptr;
+    p.next = cfg->max_hits == 0 ? reinterpret_cast<int32_t *>(ix + L.next) : nullptr;
     p.a = (int)n_before;
     p.b = (int)n_after;
     p.w = cfg->min_ngram;
     p.K = cfg->max_hits > 0 ? cfg->max_hits : 1;
-    p.mask = L.M - 1;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int tb = 256;
-    const int nb = (int)((n_after - n_before + tb - 1) / tb);
-    index_append_kernel<<<nb, tb, 0, st>>>(p);
+    p.bmask = L.M / kBucket - 1;
+    launch_after(index_append_kernel, (unsigned)((n_after - n_before + 127) / 128), 128, 0, static_cast<cudaStream_t>(stream), p);
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
 }
 
@@ -758,44 +905,38 @@ int rac_index_query_live(const rac_index_cfg *cfg, const void *index, size_t ind
     const unsigned char *ix = static_cast<const unsigned char *>(index);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    MatchParams p;
+    MatchParams p = {};
     p.hist = hist_tok;
     p.query = query_tok;
     p.ref_row = ref_row;
     p.spans_out = spans;
     p.n_spans = n_spans;
-    p.rep = const_cast<int32_t *>(reinterpret_cast<const int32_t *>(ix + L.rep));
+    p.slots = const_cast<u64 *>(reinterpret_cast<const u64 *>(ix + L.slots));
     p.top = const_cast<int32_t *>(reinterpret_cast<const int32_t *>(ix + L.top));
-    p.slot_of = nullptr;
     p.best = reinterpret_cast<int2 *>(ws + Q.best);
-    p.hop = reinterpret_cast<int2 *>(ws + Q.hop);
-    p.spans_ws = reinterpret_cast<rac_span *>(ws + Q.spans);
-    p.chunk_first = reinterpret_cast<int32_t *>(ws + Q.chunk_first);
-    p.delta16 = reinterpret_cast<unsigned short *>(ws + Q.delta16);
-    p.jump2 = reinterpret_cast<int32_t *>(ws + Q.jump2);
-    p.jump4 = reinterpret_cast<int32_t *>(ws + Q.jump4);
+    p.jump = reinterpret_cast<int2 *>(ws + Q.jump);
+    p.entry = reinterpret_cast<int2 *>(ws + Q.entry);
     p.n_hist = (int)n_hist;
     p.n_query = (int)n_query;
     p.nwin = (int)(n_hist - cfg->min_ngram + 1 > 0 ? n_hist - cfg->min_ngram + 1 : 0);
     p.w = cfg->min_ngram;
     p.K = cfg->max_hits > 0 ? cfg->max_hits : 1;
-    p.mask = L.M - 1;
-    p.next = cfg->max_hits == 0 ? const_cast<int32_t *>(reinterpret_cast<const int32_t *>(ix + L.slot_of)) : nullptr;
+    p.bmask = L.M / kBucket - 1;
+    p.next = cfg->max_hits == 0 ? const_cast<int32_t *>(reinterpret_cast<const int32_t *>(ix + L.next)) : nullptr;
     p.first_live = (int)first_live;
     p.end_of = reinterpret_cast<const int32_t *>(ix + L.end_of);
-    const int tb = 256;
-    // rows to -1, span count to 0, and (for the intra-sequence pass) the token table to empty
-    int32_t *trep = reinterpret_cast<int32_t *>(ws + Q.trep), *tfirst = reinterpret_cast<int32_t *>(ws + Q.tfirst);
-    fill2_i32_kernel<<<grid_for(n_query > 1 ? n_query : 1, tb), tb, 0, st>>>(ref_row, n_query, -1, n_spans, 1, 0);
-    if (n_query == 0) return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
-    match_query_kernel<<<(int)((n_query + tb - 1) / tb), tb, 0, st>>>(p);
-    if (launch_selection(p, st) != RAC_OK) return RAC_ECUDA;
-    if (intra) {
-        fill2_i32_kernel<<<grid_for(Q.Mq, tb), tb, 0, st>>>(trep, (long long)Q.Mq, -1, tfirst, (long long)Q.Mq, 0x7fffffff);
-        const int nb = (int)((n_query + tb - 1) / tb);
-        intra_insert_kernel<<<nb, tb, 0, st>>>(query_tok, (int)n_query, trep, tfirst, Q.Mq - 1);
-        intra_assign_kernel<<<nb, tb, 0, st>>>(query_tok, (int)n_query, trep, tfirst, Q.Mq - 1, (int)n_hist, ref_row);
+    if (n_query == 0) {
+        launch_after(fill_ones_kernel, 1, 32, 0, st, (uint4 *)nullptr, 0ll, n_spans);
+        return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
     }
+    if (intra) {     // the token table starts empty
+        p.trep = reinterpret_cast<int32_t *>(ws + Q.trep);
+        p.tfirst = reinterpret_cast<int32_t *>(ws + Q.tfirst);
+        p.tmask = Q.Mq - 1;
+        const long long n16 = (long long)Q.Mq / 2;
+        launch_after(fill_ones_kernel, fill_blocks(n16), 256, 0, st, reinterpret_cast<uint4 *>(ws + Q.trep), n16, (int32_t *)nullptr);
+    }
+    launch_query(p, st);
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
 }
 
@@ -806,7 +947,7 @@ extern "C" int rac_spans_to_segments(const rac_span *spans, const int32_t *n_spa
     if (!n_spans || !seg_off || !n_seg || T < 0 || max_seg < 1) return RAC_EINVAL;
     if (T >= (1ll << 30) || max_seg >= (1ll << 30)) return RAC_EUNSUPPORTED;
     if (!spans) return RAC_EINVAL;
-    spans_to_segments_kernel<<<1, 1024, 0, static_cast<cudaStream_t>(stream)>>>(spans, n_spans, (int)T, (int)max_seg, seg_off,
-                                                                               n_seg);
+    launch_after(spans_to_segments_kernel, 1, 1024, 0, static_cast<cudaStream_t>(stream), spans, n_spans, (int)T, (int)max_seg,
+                 seg_off, n_seg);
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
 }

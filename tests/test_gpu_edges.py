@@ -72,3 +72,62 @@ def test_statistics_passes_at_partition_edges(env, d, g, T):
     assert np.all(np.abs(gs - o_step) <= np.spacing(o_step.astype(np.float16)).astype(np.float32))
     assert (gs != o_step).sum() <= max(2, 0.02 * gs.size)
     assert np.array_equal(inv.cpu().numpy()[gs == o_step], o_inv[gs == o_step])
+
+
+# ------------------------------------------------------------------------------- retrieval: chunks of 512 query positions
+def _match(env, hist, query, w, K):
+    rac, dev = env.rac, env.dev
+    h, q = torch.from_numpy(hist).to(dev), torch.from_numpy(query).to(dev)
+    N = q.numel()
+    nb = rac.rac_match_workspace_bytes(h.numel(), N, K)
+    ws = torch.full((nb + 32,), 0x5A, dtype=torch.uint8, device=dev)
+    rows = torch.full((N + 8,), 12345, dtype=torch.int32, device=dev)
+    cap = N // w + 1
+    spans = torch.full((cap + 2, 3), 777, dtype=torch.int32, device=dev)
+    n = torch.full((1,), -5, dtype=torch.int32, device=dev)
+    rac.rac_match_spans(h, h.numel(), q, N, w, K, rows[:N], spans[:cap], n, ws[:nb], nb)
+    torch.cuda.synchronize()
+    assert torch.all(rows[N:] == 12345) and torch.all(spans[cap:] == 777) and torch.all(ws[nb:] == 0x5A)
+    return rows[:N].cpu().numpy(), spans[:int(n.item())].cpu().numpy()
+
+
+@pytest.mark.parametrize("N,w,K", [(511, 4, 8), (512, 1, 3), (513, 4, 16), (4096, 5, 8), (4097, 4, 8), (1024 * 512 + 700, 4, 8),
+                                   (1500, 3, 0)])
+def test_selection_at_chunk_edges(env, N, w, K):
+    """Query lengths at the edges of a chunk, of the chunks one kernel walks itself, and of the 1024 chunks that are resolved
+    together; spans of one token up to several chunks, some ending exactly at a chunk's end; sets of 3, 8 and 16 starts."""
+    rng = np.random.default_rng(N + K)
+    hist = rng.integers(0, 3, 3000).astype(np.int32)          # three tokens: every window occurs many times
+    hist[500:2500] = rng.integers(0, 500, 2000)
+    query = rng.integers(0, 500, N).astype(np.int32)
+    i = int(rng.integers(0, 9))
+    while i < N:
+        L = min(int(rng.choice([1, 5, 40, 511, 512, 1300])), N - i)
+        if rng.random() < 0.3 and i % 512:
+            L = min(512 - i % 512, N - i)                     # up to the end of the chunk
+        j = int(rng.integers(0, hist.size - L + 1))
+        query[i:i + L] = hist[j:j + L]
+        i += L + int(rng.integers(0, 4))
+    rows, spans = _match(env, hist, query, w, K)
+    o_rows, o_spans = env.orc.match_spans(hist, query, w, K)
+    assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
+
+
+def test_one_span_over_many_chunks_and_no_span_at_all(env):
+    rng = np.random.default_rng(1)
+    hist = rng.integers(0, 30000, 9000).astype(np.int32)
+    for query in (hist[100:8100].copy(), rng.integers(40000, 50000, 6000).astype(np.int32)):
+        rows, spans = _match(env, hist, query, 4, 8)
+        o_rows, o_spans = env.orc.match_spans(hist, query, 4, 8)
+        assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
+
+
+def test_windows_that_occur_thousands_of_times(env):
+    """All threads at one slot and one set of starts at the same time: the sets still end as the K most recent starts."""
+    hist = np.zeros(20000, np.int32)
+    hist[::17] = 1
+    query = np.concatenate([hist[:300], np.full(40, 2, np.int32), hist[17 * 900:17 * 900 + 700]])
+    for K in (1, 3, 8, 16):
+        rows, spans = _match(env, hist, query, 4, K)
+        o_rows, o_spans = env.orc.match_spans(hist, query, 4, K)
+        assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
