@@ -1,12 +1,14 @@
-"""ctypes binding of ``librac.so`` -- argument marshalling only.
+"""Binding of ``librac.so`` -- argument marshalling only.
 
 Every function has the name and the argument order of its C entry point in
 ``include/rac.h``.  Arguments are either raw addresses (int) or torch tensors
 living where the C function expects them (device pointers for the ``rac_*``
-calls); the binding checks dtype, contiguity and device, takes
-``tensor.data_ptr()`` and the current CUDA stream, calls the library and raises
-on a non-zero return code.  No arithmetic of the method happens here and there
-is no fallback: if the library cannot be loaded, importing callers get an error.
+calls); the binding checks dtype, contiguity and device, takes the tensor's
+address and the current CUDA stream, calls the library and raises on a non-zero
+return code.  The launching calls are marshalled by the extension module
+``_native`` (``csrc/rac_py.cpp``), the others and the plain library by ctypes.
+No arithmetic of the method happens here and there is no fallback: if the
+library cannot be loaded, importing callers get an error.
 """
 from __future__ import annotations
 
@@ -14,7 +16,7 @@ import ctypes as C
 import os
 from typing import Optional
 
-import torch
+import torch  # noqa: F401  (the extension module needs its libraries in the process)
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "librac.so")
@@ -74,24 +76,21 @@ _lib: Optional[C.CDLL] = None
 
 
 class _Recorder:
-    """Stands in for the library while `prepare` runs a wrapper once: launches are recorded instead of made."""
+    """Stands in for the extension module while `prepare` runs a wrapper once: calls are recorded instead of made."""
 
-    def __init__(self, lib):
-        self._lib = lib
+    def __init__(self, native):
+        self._native = native
         self.calls = []
 
     def __getattr__(self, name):
-        real = getattr(self._lib, name)
-        if real.restype is not C.c_int:      # size queries, strings: answer them
-            return real
+        entry = getattr(self._native, name)
 
         def record(*args):
-            self.calls.append((name, real, args))
-            return RAC_OK
+            self.calls.append((entry, args))
         return record
 
 
-_recorder = None
+_native = None        # the extension module, or the recorder while a call is prepared
 
 
 def prepare(wrapper, *args, **kwargs):
@@ -101,33 +100,26 @@ def prepare(wrapper, *args, **kwargs):
     ``rac_decode_reconstruct``, ...), ``args`` what it would be given.  Tensor addresses, sizes and the stream
     (``stream=`` or the current one at the time of this call) are fixed here; the tensors must stay alive and in
     place.  For loops that issue the same small call many times (a decode step per token), where looking at a dozen
-    tensors costs more than the launch.  Not thread safe while it prepares."""
-    global _recorder
-    lib = load()
-    rec = _Recorder(lib)
-    _recorder = rec
+    tensors takes a share of the call.  Not thread safe while it prepares."""
+    global _native
+    load()
+    native = _native
+    rec = _Recorder(native)
+    _native = rec
     try:
         wrapper(*args, **kwargs)
     finally:
-        _recorder = None
+        _native = native
     if len(rec.calls) != 1:
         raise ValueError("prepare() wants a wrapper that makes exactly one library call")
-    name, real, cargs = rec.calls[0]
-    keep = (args, kwargs)      # the tensors (and the configuration struct the pointers refer to) stay referenced
-
-    def call():
-        rc = real(*cargs)
-        if rc != RAC_OK:
-            _check(name, rc)
-    call.keepalive = keep
-    return call
+    entry, cargs = rec.calls[0]
+    # the tensors (and the configuration struct the pointers refer to) stay referenced
+    return native.prepare(entry, cargs, (args, kwargs))
 
 
 def load():
     """Load the C-ABI library.  Raises if it has not been built (``__graft_entry__.build()``)."""
-    global _lib
-    if _recorder is not None:
-        return _recorder
+    global _lib, _native
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -204,41 +196,23 @@ def load():
     l.rac_calibrate_steps.argtypes = [cfgp, vp, i64, vp, i64, vp, vp, vp, C.c_float, vp, vp, vp, sz, vp, vp]
     l.rac_calibrate_steps_shared.restype = C.c_int
     l.rac_calibrate_steps_shared.argtypes = [cfgp, vp, i64, vp, i64, vp, vp, vp, vp, vp, C.c_float, vp, vp, vp, sz, vp, vp]
+    from . import _native as native
+    native.set_check(_check)
+    _native = native
     _lib = l
     return l
+
+
+def _calls():
+    """Where launching calls go: the extension module (loaded on first use)."""
+    if _native is None:
+        load()
+    return _native
 
 
 def _check(fn: str, rc: int) -> None:
     if rc != RAC_OK:
         raise RacError(fn, rc, load().rac_strerror(rc).decode())
-
-
-def _ptr(t, dtype=None, name="tensor") -> Optional[int]:
-    """Address of a tensor (or pass an int / None through)."""
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return t
-    if not isinstance(t, torch.Tensor):
-        raise TypeError(f"{name}: expected a torch tensor, an address or None")
-    if not t.is_cuda:
-        raise ValueError(f"{name}: must be a CUDA tensor")
-    if not t.is_contiguous():
-        raise ValueError(f"{name}: must be contiguous")
-    if dtype is not None and t.dtype not in (dtype if isinstance(dtype, tuple) else (dtype,)):
-        raise TypeError(f"{name}: expected {dtype}, got {t.dtype}")
-    return t.data_ptr()
-
-
-def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
-
-
-_BF16 = torch.bfloat16
-_F16 = torch.float16
-_I32 = torch.int32
-_F32 = torch.float32
-_U8 = (torch.uint8, torch.int8)
 
 
 # ----------------------------------------------------------------------------- plain queries
@@ -287,44 +261,27 @@ def rac_encode_workspace_bytes(cfg: CodecCfg, T: int) -> int:
 
 
 def rac_split_waves(ref_row, T, first_intra_row, wave1, wave2, wave_count, stream=None) -> None:
-    rc = load().rac_split_waves(_ptr(ref_row, _I32, "ref_row"), int(T), int(first_intra_row), _ptr(wave1, _I32, "wave1"),
-                                _ptr(wave2, _I32, "wave2"), _ptr(wave_count, _I32, "wave_count"),
-                                _stream() if stream is None else stream)
-    _check("rac_split_waves", rc)
+    _calls().rac_split_waves(ref_row, T, first_intra_row, wave1, wave2, wave_count, stream)
 
 
 def rac_encode_reconstruct_list(cfg, X, T, tok_list, tok_count, ref_base, ref_rows, ref_row, intra_base, intra_rows,
                                 ref_gain, ref_bias, step, inv_step, payload, payload_cap, X_hat, workspace,
                                 workspace_bytes, dev_status, stream=None, coef_seg=None, seg_of=None) -> None:
-    rc = load().rac_encode_reconstruct_list(
-        C.byref(cfg), _ptr(X, _BF16, "X"), int(T), _ptr(tok_list, _I32, "tok_list"), _ptr(tok_count, _I32, "tok_count"),
-        _ptr(ref_base, _BF16, "ref_base"), int(ref_rows), _ptr(ref_row, _I32, "ref_row"),
-        _ptr(intra_base, _BF16, "intra_base"), int(intra_rows), _ptr(coef_seg, _I32, "coef_seg"),
-        _ptr(seg_of, _I32, "seg_of"), _ptr(ref_gain, _F16, "ref_gain"),
-        _ptr(ref_bias, _F16, "ref_bias"), _ptr(step, _F32, "step"), _ptr(inv_step, _F32, "inv_step"),
-        _ptr(payload, _U8, "payload"), int(payload_cap), _ptr(X_hat, _BF16, "X_hat"), _ptr(workspace, None, "workspace"),
-        int(workspace_bytes), _ptr(dev_status, _I32, "dev_status"), _stream() if stream is None else stream)
-    _check("rac_encode_reconstruct_list", rc)
+    _calls().rac_encode_reconstruct_list(cfg, X, T, tok_list, tok_count, ref_base, ref_rows, ref_row, intra_base,
+                                         intra_rows, coef_seg, seg_of, ref_gain, ref_bias, step, inv_step, payload,
+                                         payload_cap, X_hat, workspace, workspace_bytes, dev_status, stream)
 
 
 def rac_decode_reconstruct_list(cfg, payload, T, tok_list, tok_count, ref_base, ref_rows, ref_row, intra_base,
                                 intra_rows, ref_gain, ref_bias, step, X_hat, dev_status, stream=None, coef_seg=None,
                                 seg_of=None) -> None:
-    rc = load().rac_decode_reconstruct_list(
-        C.byref(cfg), _ptr(payload, _U8, "payload"), int(T), _ptr(tok_list, _I32, "tok_list"),
-        _ptr(tok_count, _I32, "tok_count"), _ptr(ref_base, _BF16, "ref_base"), int(ref_rows),
-        _ptr(ref_row, _I32, "ref_row"), _ptr(intra_base, _BF16, "intra_base"), int(intra_rows),
-        _ptr(coef_seg, _I32, "coef_seg"), _ptr(seg_of, _I32, "seg_of"),
-        _ptr(ref_gain, _F16, "ref_gain"), _ptr(ref_bias, _F16, "ref_bias"), _ptr(step, _F32, "step"),
-        _ptr(X_hat, _BF16, "X_hat"), _ptr(dev_status, _I32, "dev_status"), _stream() if stream is None else stream)
-    _check("rac_decode_reconstruct_list", rc)
+    _calls().rac_decode_reconstruct_list(cfg, payload, T, tok_list, tok_count, ref_base, ref_rows, ref_row, intra_base,
+                                         intra_rows, coef_seg, seg_of, ref_gain, ref_bias, step, X_hat, dev_status,
+                                         stream)
 
 
 def rac_spans_to_segments(spans, n_spans, T, max_seg, seg_off, n_seg, stream=None) -> None:
-    rc = load().rac_spans_to_segments(_ptr(spans, _I32, "spans"), _ptr(n_spans, _I32, "n_spans"), int(T), int(max_seg),
-                                      _ptr(seg_off, _I32, "seg_off"), _ptr(n_seg, _I32, "n_seg"),
-                                      _stream() if stream is None else stream)
-    _check("rac_spans_to_segments", rc)
+    _calls().rac_spans_to_segments(spans, n_spans, T, max_seg, seg_off, n_seg, stream)
 
 
 def rac_fit_segments_workspace_bytes(cfg: CodecCfg, T: int) -> int:
@@ -334,13 +291,8 @@ def rac_fit_segments_workspace_bytes(cfg: CodecCfg, T: int) -> int:
 def rac_fit_segments(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, seg_off, n_seg, coef_seg, seg_of,
                      workspace, workspace_bytes, dev_status, stream=None) -> None:
     """Eq. 6 over several fitting positions; ``coef_seg`` is an int32 tensor [n_seg, J] holding the u32 words."""
-    rc = load().rac_fit_segments(C.byref(cfg), _ptr(X, _BF16, "X"), int(T), _ptr(ref_base, _BF16, "ref_base"),
-                                 int(ref_rows), _ptr(ref_row, _I32, "ref_row"), _ptr(ref_gain, _F16, "ref_gain"),
-                                 _ptr(ref_bias, _F16, "ref_bias"), _ptr(seg_off, _I32, "seg_off"), int(n_seg),
-                                 _ptr(coef_seg, _I32, "coef_seg"), _ptr(seg_of, _I32, "seg_of"),
-                                 _ptr(workspace, None, "workspace"), int(workspace_bytes),
-                                 _ptr(dev_status, _I32, "dev_status"), _stream() if stream is None else stream)
-    _check("rac_fit_segments", rc)
+    _calls().rac_fit_segments(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, seg_off, n_seg, coef_seg,
+                              seg_of, workspace, workspace_bytes, dev_status, stream)
 
 
 def rac_recon_error_workspace_bytes() -> int:
@@ -348,10 +300,7 @@ def rac_recon_error_workspace_bytes() -> int:
 
 
 def rac_recon_error(X, X_hat, T, d, out, workspace, workspace_bytes, stream=None) -> None:
-    rc = load().rac_recon_error(_ptr(X, _BF16, "X"), _ptr(X_hat, _BF16, "X_hat"), int(T), int(d), _ptr(out, None, "out"),
-                                _ptr(workspace, None, "workspace"), int(workspace_bytes),
-                                _stream() if stream is None else stream)
-    _check("rac_recon_error", rc)
+    _calls().rac_recon_error(X, X_hat, T, d, out, workspace, workspace_bytes, stream)
 
 
 def rac_calibrate_workspace_bytes(cfg: CodecCfg) -> int:
@@ -359,14 +308,10 @@ def rac_calibrate_workspace_bytes(cfg: CodecCfg) -> int:
 
 
 # ----------------------------------------------------------------------------- device calls
-def rac_match_spans(hist_tok, n_hist, query_tok, n_query, min_ngram, max_hits, ref_row, spans, n_spans,
-                    workspace, workspace_bytes, stream=None) -> None:
-    rc = load().rac_match_spans(_ptr(hist_tok, _I32, "hist_tok"), int(n_hist), _ptr(query_tok, _I32, "query_tok"),
-                                int(n_query), int(min_ngram), int(max_hits), _ptr(ref_row, _I32, "ref_row"),
-                                _ptr(spans, _I32, "spans"), _ptr(n_spans, _I32, "n_spans"),
-                                _ptr(workspace, None, "workspace"), int(workspace_bytes),
-                                _stream() if stream is None else stream)
-    _check("rac_match_spans", rc)
+def rac_match_spans(hist_tok, n_hist, query_tok, n_query, min_ngram, max_hits, ref_row, spans, n_spans, workspace,
+                    workspace_bytes, stream=None) -> None:
+    _calls().rac_match_spans(hist_tok, n_hist, query_tok, n_query, min_ngram, max_hits, ref_row, spans, n_spans,
+                             workspace, workspace_bytes, stream)
 
 
 MATCH_STATIC_BYTES = 3 << 20  # RAC_MATCH_STATIC_BYTES in rac.h
@@ -376,11 +321,8 @@ def rac_match_spans_static(hist_tok, n_hist, query_tok, n_query, min_ngram, max_
                            stream=None) -> None:
     """Span retrieval on the library's built-in 3 MiB scratch: for callers that may not allocate device memory.
     Calls on one device must not overlap on the GPU (they share the scratch)."""
-    rc = load().rac_match_spans_static(_ptr(hist_tok, _I32, "hist_tok"), int(n_hist), _ptr(query_tok, _I32, "query_tok"),
-                                       int(n_query), int(min_ngram), int(max_hits), _ptr(ref_row, _I32, "ref_row"),
-                                       _ptr(spans, _I32, "spans"), _ptr(n_spans, _I32, "n_spans"),
-                                       _stream() if stream is None else stream)
-    _check("rac_match_spans_static", rc)
+    _calls().rac_match_spans_static(hist_tok, n_hist, query_tok, n_query, min_ngram, max_hits, ref_row, spans, n_spans,
+                                    stream)
 
 
 def rac_index_bytes(cfg: IndexCfg) -> int:
@@ -392,119 +334,67 @@ def rac_index_query_workspace_bytes(n_query: int) -> int:
 
 
 def rac_index_reset(cfg, index, index_bytes, stream=None) -> None:
-    rc = load().rac_index_reset(C.byref(cfg), _ptr(index, None, "index"), int(index_bytes),
-                                _stream() if stream is None else stream)
-    _check("rac_index_reset", rc)
+    _calls().rac_index_reset(cfg, index, index_bytes, stream)
 
 
 def rac_index_append(cfg, index, index_bytes, hist_tok, n_before, n_after, stream=None) -> None:
-    rc = load().rac_index_append(C.byref(cfg), _ptr(index, None, "index"), int(index_bytes),
-                                 _ptr(hist_tok, _I32, "hist_tok"), int(n_before), int(n_after),
-                                 _stream() if stream is None else stream)
-    _check("rac_index_append", rc)
+    _calls().rac_index_append(cfg, index, index_bytes, hist_tok, n_before, n_after, stream)
 
 
-def rac_index_query_live(cfg, index, index_bytes, hist_tok, n_hist, first_live, query_tok, n_query, intra, ref_row, spans,
-                         n_spans, workspace, workspace_bytes, stream=None) -> None:
-    rc = load().rac_index_query_live(C.byref(cfg), _ptr(index, None, "index"), int(index_bytes),
-                                     _ptr(hist_tok, _I32, "hist_tok"), int(n_hist), int(first_live),
-                                     _ptr(query_tok, _I32, "query_tok"), int(n_query), int(bool(intra)),
-                                     _ptr(ref_row, _I32, "ref_row"), _ptr(spans, _I32, "spans"), _ptr(n_spans, _I32, "n_spans"),
-                                     _ptr(workspace, None, "workspace"), int(workspace_bytes),
-                                     _stream() if stream is None else stream)
-    _check("rac_index_query_live", rc)
+def rac_index_query_live(cfg, index, index_bytes, hist_tok, n_hist, first_live, query_tok, n_query, intra, ref_row,
+                         spans, n_spans, workspace, workspace_bytes, stream=None) -> None:
+    _calls().rac_index_query_live(cfg, index, index_bytes, hist_tok, n_hist, first_live, query_tok, n_query, intra,
+                                  ref_row, spans, n_spans, workspace, workspace_bytes, stream)
 
 
 def rac_index_query(cfg, index, index_bytes, hist_tok, n_hist, query_tok, n_query, intra, ref_row, spans, n_spans,
                     workspace, workspace_bytes, stream=None) -> None:
-    rc = load().rac_index_query(C.byref(cfg), _ptr(index, None, "index"), int(index_bytes),
-                                _ptr(hist_tok, _I32, "hist_tok"), int(n_hist), _ptr(query_tok, _I32, "query_tok"),
-                                int(n_query), int(bool(intra)), _ptr(ref_row, _I32, "ref_row"),
-                                _ptr(spans, _I32, "spans"), _ptr(n_spans, _I32, "n_spans"),
-                                _ptr(workspace, None, "workspace"), int(workspace_bytes),
-                                _stream() if stream is None else stream)
-    _check("rac_index_query", rc)
+    _calls().rac_index_query(cfg, index, index_bytes, hist_tok, n_hist, query_tok, n_query, intra, ref_row, spans,
+                             n_spans, workspace, workspace_bytes, stream)
 
 
 def rac_spans_to_rows(spans, n_spans, n_query, ref_row, stream=None) -> None:
-    rc = load().rac_spans_to_rows(_ptr(spans, _I32, "spans"), _ptr(n_spans, _I32, "n_spans"), int(n_query),
-                                  _ptr(ref_row, _I32, "ref_row"), _stream() if stream is None else stream)
-    _check("rac_spans_to_rows", rc)
+    _calls().rac_spans_to_rows(spans, n_spans, n_query, ref_row, stream)
 
 
 def rac_encode(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step, inv_step, payload, payload_cap,
                workspace, workspace_bytes, dev_status, stream=None) -> None:
-    rc = load().rac_encode(C.byref(cfg), _ptr(X, _BF16, "X"), int(T), _ptr(ref_base, _BF16, "ref_base"), int(ref_rows),
-                           _ptr(ref_row, _I32, "ref_row"), _ptr(ref_gain, _F16, "ref_gain"),
-                           _ptr(ref_bias, _F16, "ref_bias"), _ptr(step, _F32, "step"), _ptr(inv_step, _F32, "inv_step"),
-                           _ptr(payload, _U8, "payload"), int(payload_cap), _ptr(workspace, None, "workspace"),
-                           int(workspace_bytes), _ptr(dev_status, _I32, "dev_status"),
-                           _stream() if stream is None else stream)
-    _check("rac_encode", rc)
+    _calls().rac_encode(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step, inv_step, payload,
+                        payload_cap, workspace, workspace_bytes, dev_status, stream)
 
 
 def rac_encode_reconstruct(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step, inv_step, payload,
                            payload_cap, X_hat, workspace, workspace_bytes, dev_status, stream=None) -> None:
-    rc = load().rac_encode_reconstruct(C.byref(cfg), _ptr(X, _BF16, "X"), int(T), _ptr(ref_base, _BF16, "ref_base"),
-                                       int(ref_rows), _ptr(ref_row, _I32, "ref_row"), _ptr(ref_gain, _F16, "ref_gain"),
-                                       _ptr(ref_bias, _F16, "ref_bias"), _ptr(step, _F32, "step"),
-                                       _ptr(inv_step, _F32, "inv_step"), _ptr(payload, _U8, "payload"), int(payload_cap),
-                                       _ptr(X_hat, _BF16, "X_hat"), _ptr(workspace, None, "workspace"),
-                                       int(workspace_bytes), _ptr(dev_status, _I32, "dev_status"),
-                                       _stream() if stream is None else stream)
-    _check("rac_encode_reconstruct", rc)
+    _calls().rac_encode_reconstruct(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step, inv_step,
+                                    payload, payload_cap, X_hat, workspace, workspace_bytes, dev_status, stream)
 
 
-def _reconstruct(fn, cfg, payload, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step, X_hat, dev_status, stream):
-    rc = getattr(load(), fn)(C.byref(cfg), _ptr(payload, _U8, "payload"), int(T), _ptr(ref_base, _BF16, "ref_base"),
-                             int(ref_rows), _ptr(ref_row, _I32, "ref_row"), _ptr(ref_gain, _F16, "ref_gain"),
-                             _ptr(ref_bias, _F16, "ref_bias"), _ptr(step, _F32, "step"), _ptr(X_hat, _BF16, "X_hat"),
-                             _ptr(dev_status, _I32, "dev_status"), _stream() if stream is None else stream)
-    _check(fn, rc)
+def rac_decode_reconstruct(cfg, payload, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step, X_hat, dev_status,
+                           stream=None) -> None:
+    _calls().rac_decode_reconstruct(cfg, payload, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step, X_hat,
+                                    dev_status, stream)
 
 
-def rac_decode_reconstruct(cfg, payload, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step, X_hat,
-                           dev_status, stream=None) -> None:
-    _reconstruct("rac_decode_reconstruct", cfg, payload, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step,
-                 X_hat, dev_status, stream)
-
-
-def rac_sender_reconstruct(cfg, payload, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step, X_hat,
-                           dev_status, stream=None) -> None:
-    _reconstruct("rac_sender_reconstruct", cfg, payload, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step,
-                 X_hat, dev_status, stream)
+def rac_sender_reconstruct(cfg, payload, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step, X_hat, dev_status,
+                           stream=None) -> None:
+    _calls().rac_sender_reconstruct(cfg, payload, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, step, X_hat,
+                                    dev_status, stream)
 
 
 def rac_selftest_bounded_wait(cfg, which, inp, T, ref_base, ref_rows, step, inv_step, out, out_cap, workspace,
                               workspace_bytes, dev_status, stream=None) -> None:
     """Runs the encode (which=0) or reconstruction (which=1) kernels with waits that cannot complete; see rac.h."""
-    rc = load().rac_selftest_bounded_wait(C.byref(cfg), int(which), _ptr(inp, None, "in"), int(T),
-                                          _ptr(ref_base, _BF16, "ref_base"), int(ref_rows), _ptr(step, _F32, "step"),
-                                          _ptr(inv_step, _F32, "inv_step"), _ptr(out, None, "out"), int(out_cap),
-                                          _ptr(workspace, None, "workspace"), int(workspace_bytes),
-                                          _ptr(dev_status, _I32, "dev_status"), _stream() if stream is None else stream)
-    _check("rac_selftest_bounded_wait", rc)
+    _calls().rac_selftest_bounded_wait(cfg, which, inp, T, ref_base, ref_rows, step, inv_step, out, out_cap, workspace,
+                                       workspace_bytes, dev_status, stream)
 
 
 def rac_calibrate_steps(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, clip_sigmas, step, inv_step,
                         workspace, workspace_bytes, dev_status, stream=None) -> None:
-    rc = load().rac_calibrate_steps(C.byref(cfg), _ptr(X, _BF16, "X"), int(T), _ptr(ref_base, _BF16, "ref_base"),
-                                    int(ref_rows), _ptr(ref_row, _I32, "ref_row"), _ptr(ref_gain, _F16, "ref_gain"),
-                                    _ptr(ref_bias, _F16, "ref_bias"), float(clip_sigmas), _ptr(step, _F32, "step"),
-                                    _ptr(inv_step, _F32, "inv_step"), _ptr(workspace, None, "workspace"),
-                                    int(workspace_bytes), _ptr(dev_status, _I32, "dev_status"),
-                                    _stream() if stream is None else stream)
-    _check("rac_calibrate_steps", rc)
+    _calls().rac_calibrate_steps(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, clip_sigmas, step,
+                                 inv_step, workspace, workspace_bytes, dev_status, stream)
 
 
-def rac_calibrate_steps_shared(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, coef_seg, seg_of, clip_sigmas,
-                               step, inv_step, workspace, workspace_bytes, dev_status, stream=None) -> None:
-    rc = load().rac_calibrate_steps_shared(C.byref(cfg), _ptr(X, _BF16, "X"), int(T), _ptr(ref_base, _BF16, "ref_base"),
-                                           int(ref_rows), _ptr(ref_row, _I32, "ref_row"),
-                                           _ptr(ref_gain, _F16, "ref_gain"), _ptr(ref_bias, _F16, "ref_bias"),
-                                           _ptr(coef_seg, _I32, "coef_seg"), _ptr(seg_of, _I32, "seg_of"),
-                                           float(clip_sigmas), _ptr(step, _F32, "step"),
-                                           _ptr(inv_step, _F32, "inv_step"), _ptr(workspace, None, "workspace"),
-                                           int(workspace_bytes), _ptr(dev_status, _I32, "dev_status"),
-                                           _stream() if stream is None else stream)
-    _check("rac_calibrate_steps_shared", rc)
+def rac_calibrate_steps_shared(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, coef_seg, seg_of,
+                               clip_sigmas, step, inv_step, workspace, workspace_bytes, dev_status, stream=None) -> None:
+    _calls().rac_calibrate_steps_shared(cfg, X, T, ref_base, ref_rows, ref_row, ref_gain, ref_bias, coef_seg, seg_of,
+                                        clip_sigmas, step, inv_step, workspace, workspace_bytes, dev_status, stream)

@@ -1,0 +1,63 @@
+"""What the binding accepts and refuses, without a GPU: nothing here gets as far as a launch."""
+import pytest
+import torch
+
+A = 1 << 20      # a made-up, 16-byte aligned device address: never dereferenced here
+
+
+@pytest.fixture(scope="module")
+def rac():
+    from paper_2608_04991_b200 import build, binding
+    build.build()
+    binding.load()
+    return binding
+
+
+def decode(rac, cfg, payload=A, T=16, ref_base=A, step=A, X_hat=A):
+    rac.rac_decode_reconstruct(cfg, payload, T, ref_base, 16, None, None, None, step, X_hat, A, stream=0)
+
+
+@pytest.mark.parametrize("kw,exc,text", [
+    (dict(payload="x"), TypeError, "payload: expected a torch tensor, an address or None"),
+    (dict(step=1.5), TypeError, "step: expected a torch tensor"),
+    (dict(X_hat=torch.zeros(4, dtype=torch.bfloat16)), ValueError, "X_hat: must be a CUDA tensor"),
+    (dict(T="many"), ValueError, "invalid literal"),
+    (dict(T=None), TypeError, "int"),
+])
+def test_arguments_that_are_refused(rac, kw, exc, text):
+    with pytest.raises(exc, match=text):
+        decode(rac, rac.CodecCfg(4096, 128, 4, 0), **kw)
+
+
+def test_configuration_types_are_told_apart(rac):
+    with pytest.raises(TypeError):
+        decode(rac, rac.IndexCfg(100))
+    with pytest.raises(TypeError):
+        decode(rac, None)
+    with pytest.raises(TypeError):
+        rac.rac_index_reset(rac.CodecCfg(4096, 128, 4, 0), A, 1 << 30, stream=0)
+
+
+def test_addresses_and_numbers_reach_the_library(rac):
+    cfg = rac.CodecCfg(4096, 128, 4, 0)
+    for kw, code in [(dict(payload=None), -1), (dict(payload=A + 2), -2), (dict(T=-1), -1), (dict(T=17), -1)]:
+        with pytest.raises(rac.RacError) as e:
+            decode(rac, cfg, **kw)
+        assert e.value.code == code
+    with pytest.raises(rac.RacError) as e:
+        decode(rac, rac.CodecCfg(4096, 100, 4, 0))
+    assert e.value.code == -1 and "rac_decode_reconstruct" in str(e.value)
+    decode(rac, cfg, T=0)                        # a no-op
+    decode(rac, cfg, T=True and 0)
+
+
+def test_prepared_call_checks_like_the_plain_one(rac):
+    cfg = rac.CodecCfg(4096, 128, 4, 0)
+    call = rac.prepare(rac.rac_decode_reconstruct, cfg, A + 2, 16, A, 16, None, None, None, A, A, A, stream=0)
+    with pytest.raises(rac.RacError) as e:
+        call()
+    assert e.value.code == -2
+    with pytest.raises(TypeError):
+        call(1)
+    none = rac.prepare(rac.rac_decode_reconstruct, cfg, A, 0, A, 16, None, None, None, A, A, A, stream=0)
+    assert none() is None
