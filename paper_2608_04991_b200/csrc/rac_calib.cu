@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(32 * kFinSlices) calib_finalize_kernel(const f
     const int row = c >= d;
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
+    grid_launch_dependents();
     grid_dependency_wait();
     const int *cnt = reinterpret_cast<const int *>(partial + (long long)parts * 2 * d);
     double sum = 0.0;
@@ -273,6 +274,8 @@ __device__ __forceinline__ Mom mom_merge(const Mom &a, const Mom &b) {
 }
 __global__ void __launch_bounds__(256) segment_fit_kernel(const float4 *moments, const int32_t *seg_off, long long n_seg,
                                                           int J, int group, long long T, uint32_t *coef_seg) {
+    grid_launch_dependents();
+    grid_dependency_wait();
     const long long wid = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (wid >= n_seg * J) return;
@@ -311,6 +314,8 @@ __global__ void __launch_bounds__(256) segment_fit_kernel(const float4 *moments,
 }
 // segment of every token: the last k with seg_off[k] <= t (empty segments have equal offsets and are skipped)
 __global__ void seg_of_kernel(const int32_t *seg_off, long long n_seg, long long T, int32_t *seg_of) {
+    grid_launch_dependents();
+    grid_dependency_wait();
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (t >= T) return;
     long long lo = 0, hi = n_seg;   // invariant: seg_off[lo] <= t (seg_off[0] = 0), answer in [lo, hi)
@@ -384,6 +389,7 @@ __global__ void __launch_bounds__(kErrThreads) recon_error_kernel(const uint4 *X
 }
 // one CTA adds the partial sums: each thread every 256th, then the same tree (one thread for all 592 took 63 us, this takes 4 us)
 __global__ void __launch_bounds__(kErrThreads) recon_error_finalize_kernel(const double *partial, double *out) {
+    grid_launch_dependents();
     grid_dependency_wait();
     double se = 0.0, sx = 0.0, mx = 0.0;
     for (int b = threadIdx.x; b < kErrGrid; b += kErrThreads) {
@@ -453,11 +459,11 @@ int rac_fit_segments(const rac_codec_cfg *cfg, const void *X, int64_t T, const v
     if (T > 0) {
         rc = launch_calib<true>(p, 0, st);
         if (rc != RAC_OK) return rc;
-        seg_of_kernel<<<(unsigned)((T + 255) / 256), 256, 0, st>>>(seg_off, n_seg, T, seg_of);
+        launch_after(seg_of_kernel, (unsigned)((T + 255) / 256), 256, 0, st, seg_off, (long long)n_seg, (long long)T, seg_of);
     }
     const long long warps = n_seg * g.J;
-    segment_fit_kernel<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>(p.moments, seg_off, n_seg, g.J, g.group, T,
-                                                                            coef_seg);
+    launch_after(segment_fit_kernel, (unsigned)((warps * 32 + 255) / 256), 256, 0, st, p.moments, seg_off, (long long)n_seg, g.J,
+                 g.group, (long long)T, coef_seg);
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
 }
 

@@ -145,26 +145,7 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
     constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
     const uint32_t row_bytes = 2u * (uint32_t)d;
 
-    const int first = blockIdx.x, stride = gridDim.x;
-    const long long n_tok = tokens_to_do<SUB>(p);
-    const int n_my = (n_tok > first) ? (int)((n_tok - first + stride - 1) / stride) : 0;
-    auto raw_row_of = [&](int k) -> int {  // raw ref_row entry of this CTA's k-th token
-        long long t = token_at<SUB>(p, first + (long long)k * stride);
-        return p.ref_row ? p.ref_row[t] : (int)t;
-    };
-    // one lane: start the copies of this CTA's k-th token into stage s
-    auto issue = [&](int k, int s, int raw_row) {
-        const long long t = token_at<SUB>(p, first + (long long)k * stride);
-        const int row = resolve_row<SUB>(p, raw_row);
-        ctrl->row[s] = row;
-        if constexpr (SUB) ctrl->seg[s] = p.seg_of ? p.seg_of[t] : 0;
-        const uint32_t bar = smem_u32(&ctrl->full[s]);
-        const uint32_t base = sbase + L.stage0 + s * L.stage_bytes;
-        mbar_arrive_expect_tx(bar, p.test_extra_tx + row_bytes + (row >= 0 ? row_bytes : 0u));
-        bulk_load(base, p.X + t * d, row_bytes, bar);
-        if (row >= 0) bulk_load(base + row_bytes, ref_row_ptr<SUB>(p, row), row_bytes, bar);
-    };
-
+    if (p.T <= gridDim.x) grid_launch_dependents();
     if (tid == 0) {
         for (int s = 0; s < S; s++) {
             mbar_init(smem_u32(&ctrl->full[s]), 1);
@@ -186,6 +167,26 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
                 *reinterpret_cast<uint32_t *>(smem + L.stage0 + (s >> 1) * L.stage_bytes + L.rec_off + (s & 1) * recb + o) = 0u;
     }
     __syncthreads();
+    grid_dependency_wait();
+    const int first = blockIdx.x, stride = gridDim.x;
+    const long long n_tok = tokens_to_do<SUB>(p);
+    const int n_my = (n_tok > first) ? (int)((n_tok - first + stride - 1) / stride) : 0;
+    auto raw_row_of = [&](int k) -> int {  // raw ref_row entry of this CTA's k-th token
+        long long t = token_at<SUB>(p, first + (long long)k * stride);
+        return p.ref_row ? p.ref_row[t] : (int)t;
+    };
+    // one lane: start the copies of this CTA's k-th token into stage s
+    auto issue = [&](int k, int s, int raw_row) {
+        const long long t = token_at<SUB>(p, first + (long long)k * stride);
+        const int row = resolve_row<SUB>(p, raw_row);
+        ctrl->row[s] = row;
+        if constexpr (SUB) ctrl->seg[s] = p.seg_of ? p.seg_of[t] : 0;
+        const uint32_t bar = smem_u32(&ctrl->full[s]);
+        const uint32_t base = sbase + L.stage0 + s * L.stage_bytes;
+        mbar_arrive_expect_tx(bar, p.test_extra_tx + row_bytes + (row >= 0 ? row_bytes : 0u));
+        bulk_load(base, p.X + t * d, row_bytes, bar);
+        if (row >= 0) bulk_load(base + row_bytes, ref_row_ptr<SUB>(p, row), row_bytes, bar);
+    };
     if (tid == 0)
         for (int k = 0; k < S && k < n_my; k++) issue(k, k, raw_row_of(k));
 
@@ -482,6 +483,7 @@ __global__ void __launch_bounds__(W * 32, W == 7 ? 4 : 3) outlier_kernel(const C
     if constexpr (SUB) shared = p.coef_ext != nullptr;
     const int coff = shared ? 0 : 4 * p.J;
     // everything this kernel reads was written by the streaming pass launched just before it
+    if (p.T <= gridDim.x * W * U) grid_launch_dependents();
     grid_dependency_wait();
     const long long n_tok = tokens_to_do<SUB>(p);
 
@@ -737,11 +739,13 @@ __global__ void __launch_bounds__(256) decode_kernel(const CodecParams p) {
     constexpr float kBase = 8388608.0f + (float)H;  // 2^23 + H
     const uint32_t row_bytes = 2u * (uint32_t)d;
 
+    if (p.T <= gridDim.x) grid_launch_dependents();
     if (tid == 0) {
         for (int s = 0; s < S; s++) mbar_init(smem_u32(&ctrl->bar[s]), 1);
         mbar_init_fence();
     }
     __syncthreads();
+    grid_dependency_wait();
 
     bool shared = false;   // coefficient words per segment, outside the records
     if constexpr (SUB) shared = p.coef_ext != nullptr;
@@ -959,6 +963,17 @@ __global__ void __launch_bounds__(256, 2) decode_ws_kernel(const CodecParams p) 
     constexpr float kBase = 8388608.0f + (float)H;  // 2^23 + H
     const uint32_t row_bytes = 2u * (uint32_t)d;
 
+    if (p.T <= gridDim.x) grid_launch_dependents();
+    if (tid == 0) {
+        for (int s = 0; s < S; s++) {
+            mbar_init(smem_u32(&ctrl->full[s]), 1);
+            mbar_init(smem_u32(&ctrl->done[s]), nwarps);
+        }
+        ctrl->abort = 0;
+        mbar_init_fence();
+    }
+    __syncthreads();
+    grid_dependency_wait();
     const int first = blockIdx.x, stride = gridDim.x;
     const long long n_tok = tokens_to_do<SUB>(p);
     const int n_my = (n_tok > first) ? (int)((n_tok - first + stride - 1) / stride) : 0;
@@ -976,16 +991,6 @@ __global__ void __launch_bounds__(256, 2) decode_ws_kernel(const CodecParams p) 
         bulk_load(base, p.payload + t * p.rec, (uint32_t)p.rec, bar);
         if (row >= 0) bulk_load(base + L.rec_pad, ref_row_ptr<SUB>(p, row), row_bytes, bar);
     };
-
-    if (tid == 0) {
-        for (int s = 0; s < S; s++) {
-            mbar_init(smem_u32(&ctrl->full[s]), 1);
-            mbar_init(smem_u32(&ctrl->done[s]), nwarps);
-        }
-        ctrl->abort = 0;
-        mbar_init_fence();
-    }
-    __syncthreads();
     if (tid == 0)
         for (int k = 0; k < S && k < n_my; k++) issue(k, k, raw_row_of(k));
 
@@ -1332,6 +1337,8 @@ static int launch_decode(const Geometry &g, CodecParams &p, cudaStream_t stream)
 __global__ void __launch_bounds__(1024) split_waves_kernel(const int32_t *ref_row, int T, long long first_intra_row,
                                                            int32_t *wave1, int32_t *wave2, int32_t *wave_count) {
     __shared__ int s_cnt[32];
+    grid_launch_dependents();
+    grid_dependency_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tiles = (T + 31) / 32;
     const int per = (tiles + 31) / 32;
@@ -1663,8 +1670,8 @@ int rac_split_waves(const int32_t *ref_row, int64_t T, int64_t first_intra_row, 
     if (T < 0 || first_intra_row < 0 || !wave_count) return RAC_EINVAL;
     if (T >= (1ll << 30)) return RAC_EUNSUPPORTED;
     if (T > 0 && (!ref_row || !wave1 || !wave2)) return RAC_EINVAL;
-    split_waves_kernel<<<1, 1024, 0, static_cast<cudaStream_t>(stream)>>>(ref_row, (int)T, first_intra_row, wave1, wave2,
-                                                                         wave_count);
+    launch_after(split_waves_kernel, 1, 1024, 0, static_cast<cudaStream_t>(stream), ref_row, (int)T, (long long)first_intra_row,
+                 wave1, wave2, wave_count);
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
 }
 

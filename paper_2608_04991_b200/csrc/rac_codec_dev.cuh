@@ -442,7 +442,7 @@ static int launch_persistent(K kernel, const CodecParams &p, int nthreads, int s
     long long grid = (long long)di.sms * occ;
     if (grid > max_ctas) grid = max_ctas;
     if (grid < 1) grid = 1;
-    kernel<<<(unsigned)grid, nthreads, smem_bytes, stream>>>(p);
+    launch_after(kernel, (unsigned)grid, (unsigned)nthreads, (size_t)smem_bytes, stream, p);
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
 }
 

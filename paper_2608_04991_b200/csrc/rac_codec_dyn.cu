@@ -111,6 +111,22 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_dyn_kernel
     constexpr int WPT = BITS;  // code words per thread (32 channels)
     const uint32_t row_bytes = 2u * (uint32_t)d;
 
+    if (p.T <= gridDim.x) grid_launch_dependents();
+    if (tid == 0) {
+        for (int s = 0; s < S; s++) {
+            mbar_init(smem_u32(&ctrl->full[s]), 1);
+            mbar_init(smem_u32(&ctrl->done[s]), nwarps);
+            mbar_init(smem_u32(&ctrl->tokmax[s]), nwarps);
+        }
+        ctrl->abort = 0;
+        mbar_init_fence();
+    }
+    // padding bytes of the record slots are zero from here on: every field is rewritten per token, the gaps never
+    for (int s = 0; s < S; s++)
+        for (int o = 4 * tid; o < 2 * recb; o += 4 * nt)
+            *reinterpret_cast<uint32_t *>(smem + L.stage0 + s * L.stage_bytes + L.rec_off + o) = 0u;
+    __syncthreads();
+    grid_dependency_wait();
     const int first = blockIdx.x, stride = gridDim.x;
     const long long n_tok = tokens_to_do<SUB>(p);
     const int n_my = (n_tok > first) ? (int)((n_tok - first + stride - 1) / stride) : 0;
@@ -129,21 +145,6 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_dyn_kernel
         bulk_load(base, p.X + t * d, row_bytes, bar);
         if (row >= 0) bulk_load(base + row_bytes, ref_row_ptr<SUB>(p, row), row_bytes, bar);
     };
-
-    if (tid == 0) {
-        for (int s = 0; s < S; s++) {
-            mbar_init(smem_u32(&ctrl->full[s]), 1);
-            mbar_init(smem_u32(&ctrl->done[s]), nwarps);
-            mbar_init(smem_u32(&ctrl->tokmax[s]), nwarps);
-        }
-        ctrl->abort = 0;
-        mbar_init_fence();
-    }
-    // padding bytes of the record slots are zero from here on: every field is rewritten per token, the gaps never
-    for (int s = 0; s < S; s++)
-        for (int o = 4 * tid; o < 2 * recb; o += 4 * nt)
-            *reinterpret_cast<uint32_t *>(smem + L.stage0 + s * L.stage_bytes + L.rec_off + o) = 0u;
-    __syncthreads();
     if (tid == 0)
         for (int k = 0; k < S && k < n_my; k++) issue(k, k, raw_row_of(k));
 
@@ -569,11 +570,13 @@ __global__ void __launch_bounds__(256) decode_dyn_kernel(const CodecParams p) {
     const uint32_t row_bytes = 2u * (uint32_t)d;
     const int jq = lpq == 0 ? (p.qgen ? tid / p.qgen : 0) : (tid >> lpq_shift);
 
+    if (p.T <= gridDim.x) grid_launch_dependents();
     if (tid == 0) {
         for (int s = 0; s < S; s++) mbar_init(smem_u32(&ctrl->bar[s]), 1);
         mbar_init_fence();
     }
     __syncthreads();
+    grid_dependency_wait();
 
     const int first = blockIdx.x, stride = gridDim.x;
     const long long n_tok = tokens_to_do<SUB>(p);

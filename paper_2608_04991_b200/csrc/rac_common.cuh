@@ -73,7 +73,9 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 // waits until everything the kernel before this one on the stream wrote is visible (programmatic dependent launch)
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel on the stream be set up from now on (it waits for this one's end before it reads anything): for short
-// kernels whose launches follow one another, where the set-up would otherwise be in the way.  Call it first.
+// kernels whose launches follow one another, where the set-up would otherwise be in the way.  Call it first.  Kernels that
+// work through several rounds do not: CTAs that wait beside them for their end take their place in the SMs apart
+// (encode of 16384 x 4096 with outliers 79 -> 85 us, 20001 x 5120 both ends 202 -> 233 us with it).
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {
