@@ -87,7 +87,8 @@ int make_geometry(const rac_codec_cfg *cfg, Geometry *g) {
 // ------------------------------------------------------------------------------------------------
 // encode
 // ------------------------------------------------------------------------------------------------
-// Two launches.  (1) The streaming pass (this kernel): statistics, coefficients, residual, codes; every
+// Without outliers one launch of the streaming pass, with outliers and no x_hat one launch of encode_top_kernel (below), with
+// both two launches.  (1) The streaming pass (this kernel): statistics, coefficients, residual, codes; every
 // warp of the CTA works on its 1024 channels of the token and ends with ONE arrival on the stage's `done`
 // mbarrier -- there is no CTA barrier in the loop.  Handing the finished record to the copy engine and
 // refilling the stage is the duty of warp (i mod warps) for token i; the other warps are already in the
@@ -117,6 +118,139 @@ __host__ __device__ inline WsSmem ws_smem_layout(int d, int rec, int stages, boo
     return s;
 }
 
+// One thread's 32 channels of one token, rows and record in shared memory: Eq. 6, Eq. 7, Eq. 8 with the static table, packing,
+// the sender-side reconstruction (over the X row), and the largest |e| of the slab.
+template <int BITS, bool TOPK, bool XHAT, int LPG>
+__device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int lane, int rot, int d, int Jc, bool shared, int coff,
+                                            const uint32_t (&off)[4], unsigned int group_mask, uint32_t xs, uint32_t rs,
+                                            bool has_ref, int seg, unsigned char *rec, float *tm) {
+    constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
+    const u64 magic2 = pack2(kMagic, kMagic);
+    // ---- (1) the slab: 4 slots of 8 channels, slot j holds piece (j + rot) & 3
+    uint32_t xw[16], rw[16];   // packed bf16, slot order
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const uint4 w = lds128(xs + off[j]);
+        xw[4 * j + 0] = w.x; xw[4 * j + 1] = w.y; xw[4 * j + 2] = w.z; xw[4 * j + 3] = w.w;
+    }
+    if (has_ref) {
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const uint4 w = load_ref_words(rs + off[j], p.gain, p.bias, (int)(off[j] >> 1));
+            rw[4 * j + 0] = w.x; rw[4 * j + 1] = w.y; rw[4 * j + 2] = w.z; rw[4 * j + 3] = w.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 16; i++) rw[i] = 0u;
+    }
+    // ---- (2) Eq. 6 and wire rounding
+    u64 a2, b2;
+    constexpr int kShift = LPG == 4 ? 2 : 1;
+    const int lpg = LPG ? LPG : p.lpg, lpg_shift = LPG ? kShift : p.lpg_shift;
+    if (shared) {
+        const uint32_t cw = p.coef_ext[(long long)seg * Jc + (tid >> lpg_shift)];
+        const float a = half_bits_to_float(cw & 0xffffu), b = half_bits_to_float(cw >> 16);
+        a2 = pack2(a, a);
+        b2 = pack2(b, b);
+    } else {
+        uint32_t coef_word;
+        fit_group(xw, rw, has_ref, lpg, p.inv_group, group_mask, p.status, a2, b2, &coef_word);
+        if ((lane & (lpg - 1)) == 0) reinterpret_cast<uint32_t *>(rec)[tid >> lpg_shift] = coef_word;
+    }
+
+    // ---- (3) Eq. 7 residual, Eq. 8 quantisation with the static table, packing
+    const float *inv_tab = p.inv_step + (has_ref ? 0 : d);
+    const float *step_tab = p.step + (has_ref ? 0 : d);
+    uint32_t words[4];
+    float tmax = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const int c = (int)(off[j] >> 1);
+        const float4 iv0 = __ldg(reinterpret_cast<const float4 *>(inv_tab + c));
+        const float4 iv1 = __ldg(reinterpret_cast<const float4 *>(inv_tab + c + 4));
+        const u64 inv2[4] = {pack2(iv0.x, iv0.y), pack2(iv0.z, iv0.w), pack2(iv1.x, iv1.y), pack2(iv1.z, iv1.w)};
+        u64 st2[4] = {0ull, 0ull, 0ull, 0ull};
+        if (XHAT) {
+            const float4 s0 = __ldg(reinterpret_cast<const float4 *>(step_tab + c));
+            const float4 s1 = __ldg(reinterpret_cast<const float4 *>(step_tab + c + 4));
+            st2[0] = pack2(s0.x, s0.y); st2[1] = pack2(s0.z, s0.w); st2[2] = pack2(s1.x, s1.y); st2[3] = pack2(s1.z, s1.w);
+        }
+        float ev[8];
+        uint32_t xh[4];
+        uint32_t w = 0;
+        if (BITS == 3) {
+            uint32_t bits8[8];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const u64 rt = pfma(a2, bf16x2_to_p(rw[4 * j + i]), b2);
+                const u64 e = sub_pair(xw[4 * j + i], rt);
+                float v0, v1, t0, t1;
+                unpack2(pmul(e, inv2[i]), v0, v1);
+                t0 = fminf(fmaxf(v0, -qmax), qmax);
+                t1 = fminf(fmaxf(v1, -qmax), qmax);
+                const u64 tt = padd(pack2(t0, t1), magic2);
+                unpack2(tt, t0, t1);
+                bits8[2 * i] = __float_as_uint(t0);
+                bits8[2 * i + 1] = __float_as_uint(t1);
+                unpack2(e, ev[2 * i], ev[2 * i + 1]);
+                if (XHAT) {
+                    // Eq. 9 with the code just chosen: x_hat = bf16(fma(q, step, alpha*r + beta)); a binary16-valued
+                    // step makes q*step exact, so the fused form and (alpha*r + beta) + q*step are the same bits
+                    float x0, x1;
+                    unpack2(pfma(psub(tt, magic2), st2[i], rt), x0, x1);
+                    xh[i] = f2_to_bf16x2(x0, x1);
+                }
+            }
+            w = pack8<BITS>(bits8);
+        } else {
+            // 4- and 2-bit codes: clamp from below in binary32, round by the magic add, take the integer
+            // out of the mantissa and let the saturating pack clamp from above (its range is
+            // [-2^(BITS-1), 2^(BITS-1)-1], whose upper end is Qmax)
+#pragma unroll
+            for (int i = 3; i >= 0; i--) {
+                const u64 rt = pfma(a2, bf16x2_to_p(rw[4 * j + i]), b2);
+                const u64 e = sub_pair(xw[4 * j + i], rt);
+                float v0, v1, t0, t1;
+                unpack2(pmul(e, inv2[i]), v0, v1);
+                v0 = fmaxf(v0, -qmax);
+                v1 = fmaxf(v1, -qmax);
+                if (XHAT) { v0 = fminf(v0, qmax); v1 = fminf(v1, qmax); }  // the float is used again below
+                const u64 tt = padd(pack2(v0, v1), magic2);
+                unpack2(tt, t0, t1);
+                w = sat_pack2<BITS>((int)__float_as_uint(t1) - 0x4b400000, (int)__float_as_uint(t0) - 0x4b400000, w);
+                unpack2(e, ev[2 * i], ev[2 * i + 1]);
+                if (XHAT) {
+                    float x0, x1;
+                    unpack2(pfma(psub(tt, magic2), st2[i], rt), x0, x1);
+                    xh[i] = f2_to_bf16x2(x0, x1);
+                }
+            }
+        }
+        words[j] = w;
+        // sender-side reconstruction: the thread's own slab of the X row now carries x_hat
+        if (XHAT) sts128(xs + off[j], make_uint4(xh[0], xh[1], xh[2], xh[3]));
+        if (TOPK) {
+            const float m0 = fmaxf(fmaxf(fabsf(ev[0]), fabsf(ev[1])), fmaxf(fabsf(ev[2]), fabsf(ev[3])));
+            const float m1 = fmaxf(fmaxf(fabsf(ev[4]), fabsf(ev[5])), fmaxf(fabsf(ev[6]), fabsf(ev[7])));
+            tmax = fmaxf(tmax, fmaxf(m0, m1));
+        }
+    }
+    rot_right4(words, rot);  // words[q] is now the code word of piece q
+    uint32_t *cw = reinterpret_cast<uint32_t *>(rec + coff) + tid * BITS;
+    if (BITS == 4) {
+        cw[0] = words[0]; cw[1] = words[1]; cw[2] = words[2]; cw[3] = words[3];
+    } else if (BITS == 3) {
+        cw[0] = words[0] | (words[1] << 24);
+        cw[1] = (words[1] >> 8) | (words[2] << 16);
+        cw[2] = (words[2] >> 16) | (words[3] << 8);
+    } else {
+        cw[0] = words[0] | (words[1] << 16);
+        cw[1] = words[2] | (words[3] << 16);
+    }
+    // (4) the largest |e| of this thread's 32 channels, for the outlier pass
+    if (TOPK) tm[tid] = tmax;
+}
+
 // SUB: the token-list / second-reference-buffer form (see rac_codec_dev.cuh).
 // LPG: lanes per alignment group as a compile-time constant (4 = groups of 128 channels, 2 = groups of 64), or 0 to
 // read it from the parameters; the constant removes the uniform branches of the shuffle reductions.
@@ -142,7 +276,6 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
     const WsSmem L = ws_smem_layout(d, recb, S, TOPK);
     WsCtrl *ctrl = reinterpret_cast<WsCtrl *>(smem);
     const uint32_t sbase = smem_u32(smem);
-    constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
     const uint32_t row_bytes = 2u * (uint32_t)d;
 
     if (p.T <= gridDim.x) grid_launch_dependents();
@@ -194,7 +327,6 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
 #pragma unroll
     for (int j = 0; j < 4; j++) off[j] = (uint32_t)(tid * 64 + ((j + rot) & 3) * 16);
     const unsigned int group_mask = __ballot_sync(0xffffffffu, valid);
-    const u64 magic2 = pack2(kMagic, kMagic);
 
     int stage = 0, duty = 0;  // duty: the warp whose turn the tail of this token is
     uint32_t parity = 0;
@@ -208,131 +340,10 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
         if (!__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&ctrl->full[stage]), parity))) { timed_out = true; break; }
         const bool has_ref = REF ? true : ctrl->row[stage] >= 0;
 
-        if (valid) {
-            // ---- (1) the slab: 4 slots of 8 channels, slot j holds piece (j + rot) & 3
-            uint32_t xw[16], rw[16];   // packed bf16, slot order
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const uint4 w = lds128(xs + off[j]);
-                xw[4 * j + 0] = w.x; xw[4 * j + 1] = w.y; xw[4 * j + 2] = w.z; xw[4 * j + 3] = w.w;
-            }
-            if (has_ref) {
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    const uint4 w = load_ref_words(rs + off[j], p.gain, p.bias, (int)(off[j] >> 1));
-                    rw[4 * j + 0] = w.x; rw[4 * j + 1] = w.y; rw[4 * j + 2] = w.z; rw[4 * j + 3] = w.w;
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 16; i++) rw[i] = 0u;
-            }
-            // ---- (2) Eq. 6 and wire rounding
-            u64 a2, b2;
-            constexpr int kShift = LPG == 4 ? 2 : 1;
-            const int lpg = LPG ? LPG : p.lpg, lpg_shift = LPG ? kShift : p.lpg_shift;
-            if (shared) {
-                const uint32_t cw = p.coef_ext[(long long)ctrl->seg[stage] * Jc + (tid >> lpg_shift)];
-                const float a = half_bits_to_float(cw & 0xffffu), b = half_bits_to_float(cw >> 16);
-                a2 = pack2(a, a);
-                b2 = pack2(b, b);
-            } else {
-                uint32_t coef_word;
-                fit_group(xw, rw, has_ref, lpg, p.inv_group, group_mask, p.status, a2, b2, &coef_word);
-                if ((lane & (lpg - 1)) == 0) reinterpret_cast<uint32_t *>(rec)[tid >> lpg_shift] = coef_word;
-            }
-
-            // ---- (3) Eq. 7 residual, Eq. 8 quantisation with the static table, packing
-            const float *inv_tab = p.inv_step + (has_ref ? 0 : d);
-            const float *step_tab = p.step + (has_ref ? 0 : d);
-            uint32_t words[4];
-            float tmax = 0.f;
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const int c = (int)(off[j] >> 1);
-                const float4 iv0 = __ldg(reinterpret_cast<const float4 *>(inv_tab + c));
-                const float4 iv1 = __ldg(reinterpret_cast<const float4 *>(inv_tab + c + 4));
-                const u64 inv2[4] = {pack2(iv0.x, iv0.y), pack2(iv0.z, iv0.w), pack2(iv1.x, iv1.y), pack2(iv1.z, iv1.w)};
-                u64 st2[4] = {0ull, 0ull, 0ull, 0ull};
-                if (XHAT) {
-                    const float4 s0 = __ldg(reinterpret_cast<const float4 *>(step_tab + c));
-                    const float4 s1 = __ldg(reinterpret_cast<const float4 *>(step_tab + c + 4));
-                    st2[0] = pack2(s0.x, s0.y); st2[1] = pack2(s0.z, s0.w); st2[2] = pack2(s1.x, s1.y); st2[3] = pack2(s1.z, s1.w);
-                }
-                float ev[8];
-                uint32_t xh[4];
-                uint32_t w = 0;
-                if (BITS == 3) {
-                    uint32_t bits8[8];
-#pragma unroll
-                    for (int i = 0; i < 4; i++) {
-                        const u64 rt = pfma(a2, bf16x2_to_p(rw[4 * j + i]), b2);
-                        const u64 e = sub_pair(xw[4 * j + i], rt);
-                        float v0, v1, t0, t1;
-                        unpack2(pmul(e, inv2[i]), v0, v1);
-                        t0 = fminf(fmaxf(v0, -qmax), qmax);
-                        t1 = fminf(fmaxf(v1, -qmax), qmax);
-                        const u64 tt = padd(pack2(t0, t1), magic2);
-                        unpack2(tt, t0, t1);
-                        bits8[2 * i] = __float_as_uint(t0);
-                        bits8[2 * i + 1] = __float_as_uint(t1);
-                        unpack2(e, ev[2 * i], ev[2 * i + 1]);
-                        if (XHAT) {
-                            // Eq. 9 with the code just chosen: x_hat = bf16(fma(q, step, alpha*r + beta)); a binary16-valued
-                            // step makes q*step exact, so the fused form and (alpha*r + beta) + q*step are the same bits
-                            float x0, x1;
-                            unpack2(pfma(psub(tt, magic2), st2[i], rt), x0, x1);
-                            xh[i] = f2_to_bf16x2(x0, x1);
-                        }
-                    }
-                    w = pack8<BITS>(bits8);
-                } else {
-                    // 4- and 2-bit codes: clamp from below in binary32, round by the magic add, take the integer
-                    // out of the mantissa and let the saturating pack clamp from above (its range is
-                    // [-2^(BITS-1), 2^(BITS-1)-1], whose upper end is Qmax)
-#pragma unroll
-                    for (int i = 3; i >= 0; i--) {
-                        const u64 rt = pfma(a2, bf16x2_to_p(rw[4 * j + i]), b2);
-                        const u64 e = sub_pair(xw[4 * j + i], rt);
-                        float v0, v1, t0, t1;
-                        unpack2(pmul(e, inv2[i]), v0, v1);
-                        v0 = fmaxf(v0, -qmax);
-                        v1 = fmaxf(v1, -qmax);
-                        if (XHAT) { v0 = fminf(v0, qmax); v1 = fminf(v1, qmax); }  // the float is used again below
-                        const u64 tt = padd(pack2(v0, v1), magic2);
-                        unpack2(tt, t0, t1);
-                        w = sat_pack2<BITS>((int)__float_as_uint(t1) - 0x4b400000, (int)__float_as_uint(t0) - 0x4b400000, w);
-                        unpack2(e, ev[2 * i], ev[2 * i + 1]);
-                        if (XHAT) {
-                            float x0, x1;
-                            unpack2(pfma(psub(tt, magic2), st2[i], rt), x0, x1);
-                            xh[i] = f2_to_bf16x2(x0, x1);
-                        }
-                    }
-                }
-                words[j] = w;
-                // sender-side reconstruction: the thread's own slab of the X row now carries x_hat
-                if (XHAT) sts128(xs + off[j], make_uint4(xh[0], xh[1], xh[2], xh[3]));
-                if (TOPK) {
-                    const float m0 = fmaxf(fmaxf(fabsf(ev[0]), fabsf(ev[1])), fmaxf(fabsf(ev[2]), fabsf(ev[3])));
-                    const float m1 = fmaxf(fmaxf(fabsf(ev[4]), fabsf(ev[5])), fmaxf(fabsf(ev[6]), fabsf(ev[7])));
-                    tmax = fmaxf(tmax, fmaxf(m0, m1));
-                }
-            }
-            rot_right4(words, rot);  // words[q] is now the code word of piece q
-            uint32_t *cw = reinterpret_cast<uint32_t *>(rec + coff) + tid * BITS;
-            if (BITS == 4) {
-                cw[0] = words[0]; cw[1] = words[1]; cw[2] = words[2]; cw[3] = words[3];
-            } else if (BITS == 3) {
-                cw[0] = words[0] | (words[1] << 24);
-                cw[1] = (words[1] >> 8) | (words[2] << 16);
-                cw[2] = (words[2] >> 16) | (words[3] << 8);
-            } else {
-                cw[0] = words[0] | (words[1] << 16);
-                cw[1] = words[2] | (words[3] << 16);
-            }
-            // (4) the largest |e| of this thread's 32 channels, for the outlier pass
-            if (TOPK) reinterpret_cast<float *>(stg + L.tm_off + parity * L.tm_bytes)[tid] = tmax;
-        }
+        if (valid)
+            encode_slab<BITS, TOPK, XHAT, LPG>(p, tid, lane, rot, d, Jc, shared, coff, off, group_mask, xs, rs, has_ref,
+                                               SUB ? ctrl->seg[stage] : 0, rec,
+                                               reinterpret_cast<float *>(stg + L.tm_off + parity * L.tm_bytes));
         // this warp's share of the token is in shared memory: one arrival per warp
         fence_async_smem();  // the record (and x_hat) bytes written above will be read by the copy engine
         __syncwarp();
@@ -708,6 +719,322 @@ __global__ void __launch_bounds__(W * 32, W == 7 ? 4 : 3) outlier_kernel(const C
             }
         }
         __syncwarp();
+    }
+}
+
+// ------------------------------------------------------------------------------------------------
+// encode with outliers in one launch (calls without x_hat)
+// ------------------------------------------------------------------------------------------------
+// The streaming pass with NSEL further warps per CTA, the selectors.  A selector takes every NSEL-th token: when the streaming
+// warps have finished it, it refills the stage at once (two stages), finds the k largest |e| from the slab maxima by the steps
+// of outlier_kernel -- the rows of the few slabs that hold them are read again, from L2, where they passed microseconds ago --,
+// patches the record in shared memory and sends it off.  Nothing goes through DRAM twice, and there is
+// no second launch.  A token's selection is a chain of ~3000 cycles; NSEL of them
+// run beside the streaming warps of NSEL later tokens, so records live in four slots (token mod 4), with a barrier each for
+// "all streaming warps are done" and "the record has left".
+// The row reads bypass L1, which holds the step table.  Shapes by width (streaming warps + selectors, CTAs per SM): measured at
+// 131072 x 5120 3 CTAs of 5 + 3 warps 0.537 ms, 3 of 5 + 2 0.570, 4 of 5 + 2 0.589 to 0.649, 4 of 5 + 3 0.611 (two launches
+// 0.601); at 16384 x 4096 4 CTAs of 4 + 2 66 us, 4 of 4 + 3 68, 5 of 4 + 2 72 (two launches 81).  Reading the slabs from the
+// stage and refilling it afterwards was slower in every shape.  With x_hat the outliers would have to replace elements of a row
+// that has left by a bulk store, and waiting for its completion in the loop costs 0.2 ms: those calls keep the two launches.
+struct TopCtrl {
+    unsigned long long full[2];     // data of the stage has landed
+    unsigned long long done[4];     // every streaming warp has finished token (mod 4)
+    unsigned long long left[4];     // the record in slot (token mod 4) has been read by the copy engine
+    int row[2];
+    int abort;
+};
+template <int NSEL>
+struct TopSel {
+    float e[NSEL][kOutCap];
+    unsigned short c[NSEL][kOutCap];
+    unsigned char hot[NSEL][256];
+};
+struct TopSmem {
+    int stage0, stage_bytes, rec_off, tm_off, sel0, total;
+};
+__host__ __device__ inline TopSmem top_smem_layout(int d, int rec, int sel_bytes) {
+    TopSmem s;
+    s.stage0 = align_up((int)sizeof(TopCtrl), 128);
+    s.rec_off = 4 * d;                        // behind X row and R row: two record slots
+    s.tm_off = s.rec_off + 2 * rec;           // slab maxima (read before the stage is refilled)
+    s.stage_bytes = align_up(s.tm_off + d / 8, 128);
+    s.sel0 = s.stage0 + 2 * s.stage_bytes;
+    s.total = s.sel0 + sel_bytes;
+    return s;
+}
+
+// NV: slab maxima per lane (d <= 1024 * NV).  KT: the number of outliers when it is 8, else 0 = p.topk.  LPG, D, REF: as for
+// encode_ws_kernel.
+template <int BITS, int KT, int NV, int NSEL, int MAXT, int MINB, int LPG, int D = 0, bool REF = false>
+__global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParams p) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int lane = tid & 31, warp = tid >> 5, nstream = D ? (D / 32 + 31) / 32 : (nt >> 5) - NSEL;
+    const int rot = (lane >> 1) & 3;
+    const int d = D ? D : p.d;
+    constexpr bool kGeo = D != 0 && LPG != 0 && KT == 8;
+    const int Jc = kGeo ? D / (32 * (LPG ? LPG : 1)) : p.J;
+    const int codeb = kGeo ? D * BITS / 8 : p.code_bytes;
+    const int recb = kGeo ? (4 * (D / (32 * (LPG ? LPG : 1))) + D * BITS / 8 + 32 + 15) / 16 * 16 : p.rec;
+    const int coff = 4 * Jc;
+    const TopSmem L = top_smem_layout(d, recb, (int)sizeof(TopSel<NSEL>));
+    TopCtrl *ctrl = reinterpret_cast<TopCtrl *>(smem);
+    const uint32_t sbase = smem_u32(smem);
+    const uint32_t row_bytes = 2u * (uint32_t)d;
+
+    if (p.T <= gridDim.x) grid_launch_dependents();
+    if (tid == 0) {
+        for (int s = 0; s < 2; s++) mbar_init(smem_u32(&ctrl->full[s]), 1);
+        for (int s = 0; s < 4; s++) {
+            mbar_init(smem_u32(&ctrl->done[s]), nstream);
+            mbar_init(smem_u32(&ctrl->left[s]), 1);
+        }
+        ctrl->abort = 0;
+        mbar_init_fence();
+    }
+    {
+        // padding words of the records are written once and never touched again
+        const int raw = coff + codeb + 4 * p.topk;
+        for (int s = 0; s < 4; s++)
+            for (int o = raw + 4 * tid; o < recb; o += 4 * nt)
+                *reinterpret_cast<uint32_t *>(smem + L.stage0 + (s >> 1) * L.stage_bytes + L.rec_off + (s & 1) * recb + o) = 0u;
+    }
+    __syncthreads();
+    grid_dependency_wait();
+    const int first = blockIdx.x, stride = gridDim.x;
+    const int n_my = (p.T > first) ? (int)((p.T - first + stride - 1) / stride) : 0;
+    auto token = [&](int k) -> long long { return first + (long long)k * stride; };   // this CTA's k-th token
+    auto raw_row_of = [&](int k) -> int { return p.ref_row ? p.ref_row[token(k)] : (int)token(k); };
+    // one lane: start the copies of this CTA's k-th token
+    auto issue = [&](int k, int raw_row) {
+        const int s = k & 1, row = resolve_row<false>(p, raw_row);
+        ctrl->row[s] = row;
+        const uint32_t bar = smem_u32(&ctrl->full[s]);
+        const uint32_t base = sbase + L.stage0 + s * L.stage_bytes;
+        mbar_arrive_expect_tx(bar, p.test_extra_tx + row_bytes + (row >= 0 ? row_bytes : 0u));
+        bulk_load(base, p.X + token(k) * d, row_bytes, bar);
+        if (row >= 0) bulk_load(base + row_bytes, p.ref_base + (long long)row * d, row_bytes, bar);
+    };
+
+    bool timed_out = false;
+    if (warp < nstream) {
+        // ---- streaming warps
+        const bool valid = tid * 32 < d;
+        uint32_t off[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) off[j] = (uint32_t)(tid * 64 + ((j + rot) & 3) * 16);
+        const unsigned int group_mask = __ballot_sync(0xffffffffu, valid);
+        for (int it = 0; it < n_my; it++) {
+            if (*reinterpret_cast<volatile int *>(&ctrl->abort)) break;
+            const int stage = it & 1;
+            const uint32_t parity = (it >> 1) & 1;
+            unsigned char *stg = smem + L.stage0 + stage * L.stage_bytes;
+            const uint32_t xs = sbase + L.stage0 + stage * L.stage_bytes;
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&ctrl->full[stage]), parity))) { timed_out = true; break; }
+            const bool has_ref = REF ? true : ctrl->row[stage] >= 0;
+            if (valid)
+                encode_slab<BITS, true, false, LPG>(p, tid, lane, rot, d, Jc, false, coff, off, group_mask, xs, xs + row_bytes,
+                                                    has_ref, 0, stg + L.rec_off + parity * recb,
+                                                    reinterpret_cast<float *>(stg + L.tm_off));
+            fence_async_smem();     // the record bytes written above will be read by the copy engine
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&ctrl->done[it & 3])) : "memory");
+        }
+    } else {
+        // ---- selectors
+        const int sel = warp - nstream;
+        TopSel<NSEL> *sc = reinterpret_cast<TopSel<NSEL> *>(smem + L.sel0);
+        float *s_e = sc->e[sel];
+        unsigned short *s_c = sc->c[sel];
+        unsigned char *s_hot = sc->hot[sel];
+        const int nth = d >> 5, k = KT ? KT : p.topk;
+        const unsigned int lt_mask = (1u << lane) - 1u;
+        constexpr uint32_t cmask = (1u << BITS) - 1u;
+        const int coef_shift = 5 + (LPG ? (LPG == 4 ? 2 : 1) : p.lpg_shift);
+        if (sel == 0 && lane == 0)
+            for (int q = 0; q < 2 && q < n_my; q++) issue(q, raw_row_of(q));
+        for (int it = sel; it < n_my; it += NSEL) {
+            if (*reinterpret_cast<volatile int *>(&ctrl->abort)) break;
+            const int s = it & 1, next = it + 2;
+            unsigned char *stg = smem + L.stage0 + s * L.stage_bytes;
+            unsigned char *rec = stg + L.rec_off + ((it >> 1) & 1) * recb;
+            const long long t = token(it);
+            int raw_next = 0;
+            if (lane == 0 && next < n_my) raw_next = raw_row_of(next);
+            if (lane == 0 && it >= NSEL) {      // this selector's last record
+                bulk_wait_read<0>();
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&ctrl->left[(it - NSEL) & 3])) : "memory");
+            }
+            // (a parity tells neighbouring phases apart only: this barrier's last token, it - 4, is done, since the streaming
+            // warps go through the tokens in order and this selector's last one was it - NSEL >= it - 4)
+            static_assert(NSEL <= 4, "one phase at a time");
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&ctrl->done[it & 3]), (it >> 2) & 1))) { timed_out = true; break; }
+            const int row = ctrl->row[s];
+            unsigned int tv[NV];                // maxima of slabs 32 * i + lane: bit patterns of non-negative floats order like integers
+#pragma unroll
+            for (int i = 0; i < NV; i++)
+                tv[i] = 32 * i + lane < nth ? *reinterpret_cast<volatile unsigned int *>(stg + L.tm_off + (32 * i + lane) * 4) : 0u;
+            __syncwarp();
+            if (next < n_my) {
+                // the next token of this stage writes the record slot of token it - 2
+                if (it >= 2 && !__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&ctrl->left[next & 3]), ((next >> 2) - 1) & 1))) {
+                    timed_out = true;
+                    break;
+                }
+                if (lane == 0) issue(next, raw_next);
+            }
+            // ---- threshold and the slabs that reach it, in slab order (see outlier_kernel)
+            unsigned int m1 = tv[0], m2 = 0u;
+#pragma unroll
+            for (int i = 1; i < NV; i++) {
+                m2 = max(m2, min(m1, tv[i]));
+                m1 = max(m1, tv[i]);
+            }
+#pragma unroll
+            for (int r = 1; r < k; r++) {
+                const unsigned int top = __reduce_max_sync(0xffffffffu, m1);
+                const unsigned int bal = __ballot_sync(0xffffffffu, m1 == top);
+                const bool pop = m1 == top && (bal & lt_mask) == 0u;
+                m1 = pop ? m2 : m1;
+                m2 = pop ? 0u : m2;
+            }
+            const unsigned int tau = __reduce_max_sync(0xffffffffu, m1);
+            const float tauf = __uint_as_float(tau);
+            // tau == 0: fewer than k slabs hold anything but zeros, every element is a candidate: whole-token path
+            int nh = 0, n = kOutCap + 1;
+            if (tau != 0u) {
+#pragma unroll
+                for (int i = 0; i < NV; i++) {
+                    const bool hit = tv[i] >= tau;
+                    const unsigned int bal = __ballot_sync(0xffffffffu, hit);
+                    if (hit) s_hot[nh + __popc(bal & lt_mask)] = (unsigned char)(32 * i + lane);
+                    nh += __popc(bal);
+                }
+                n = 0;
+            }
+            __syncwarp();
+            // ---- candidates: eight slabs per round, four lanes per slab, eight channels per lane
+            const uint16_t *xrow = p.X + t * d, *rrow = row >= 0 ? p.ref_base + (long long)row * d : nullptr;
+            const uint32_t *coefp = reinterpret_cast<const uint32_t *>(rec);
+            for (int base = 0; base < nh && n <= kOutCap; base += 8) {
+                const int hi = base + (lane >> 2);
+                const bool act = hi < nh;
+                const int c0 = act ? (int)s_hot[hi] * 32 + (lane & 3) * 8 : 0;
+                uint4 xv = make_uint4(0u, 0u, 0u, 0u), rv = xv;
+                uint32_t cf = 0u;
+                if (act) {
+                    xv = __ldcg(reinterpret_cast<const uint4 *>(xrow + c0));
+                    if (rrow) rv = __ldcg(reinterpret_cast<const uint4 *>(rrow + c0));
+                    cf = coefp[c0 >> coef_shift];
+                }
+                const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w};
+                uint32_t rw[4] = {rv.x, rv.y, rv.z, rv.w};      // zero without a reference, as in the streaming warps
+                if (rrow && p.gain) {
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        const int c = c0 + 2 * i;
+                        rw[i] = f2_to_bf16x2(__fmaf_rn(half_bits_to_float(p.gain[c]), __uint_as_float(rw[i] << 16), half_bits_to_float(p.bias[c])),
+                                             __fmaf_rn(half_bits_to_float(p.gain[c + 1]), __uint_as_float(rw[i] & 0xffff0000u),
+                                                       half_bits_to_float(p.bias[c + 1])));
+                    }
+                }
+                const float ca = half_bits_to_float(cf & 0xffff), cb = half_bits_to_float(cf >> 16);
+                const u64 a2 = pack2(ca, ca), b2 = pack2(cb, cb);
+                float e[8];
+                uint32_t m = 0u;
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    unpack2(sub_pair(xw[i], pfma(a2, bf16x2_to_p(rw[i]), b2)), e[2 * i], e[2 * i + 1]);
+                    m |= (fabsf(e[2 * i]) >= tauf ? 1u : 0u) << (2 * i) | (fabsf(e[2 * i + 1]) >= tauf ? 2u : 0u) << (2 * i);
+                }
+                if (!act) m = 0u;
+                const int cnt = __popc(m);
+                // position of the lane's first candidate (candidates come out in channel order).  Almost always no lane has two.
+                int pos, total;
+                if (!__any_sync(0xffffffffu, cnt > 1)) {
+                    const unsigned int bal = __ballot_sync(0xffffffffu, cnt != 0);
+                    pos = n + __popc(bal & lt_mask);
+                    total = __popc(bal);
+                } else {
+                    int incl = cnt;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int up = __shfl_up_sync(0xffffffffu, incl, o);
+                        incl += lane >= o ? up : 0;
+                    }
+                    pos = n + incl - cnt;
+                    total = __shfl_sync(0xffffffffu, incl, 31);
+                }
+                while (m) {
+                    const int i = __ffs(m) - 1;
+                    m &= m - 1u;
+                    if (pos < kOutCap) {
+                        s_e[pos] = pick8(e, i);
+                        s_c[pos] = (unsigned short)(c0 + i);
+                    }
+                    pos++;
+                }
+                n += total;
+            }
+            __syncwarp();
+            // ---- one candidate per lane, in channel order; while there are too many the smallest goes
+            bool won;
+            int wc = 0, pos;
+            float we = 0.f;
+            if (n <= kOutCap) {
+                won = lane < n;
+                if (won) {
+                    wc = s_c[lane];
+                    we = s_e[lane];
+                }
+                unsigned int mag = won ? (__float_as_uint(we) & 0x7fffffffu) : 0xffffffffu;
+                for (int extra = n - k; extra > 0; extra--) {
+                    const unsigned int low = __reduce_min_sync(0xffffffffu, mag);
+                    const unsigned int bal = __ballot_sync(0xffffffffu, mag == low);
+                    if (lane == 31 - __clz(bal)) { mag = 0xffffffffu; won = false; }   // among equals the highest channel
+                }
+                pos = __popc(__ballot_sync(0xffffffffu, won) & lt_mask);
+            } else {
+                float unused;
+                select_whole_token(d, k, coef_shift, xrow, rrow, p.gain, p.bias, coefp, lane, &wc, &we, &unused);
+                won = lane < k;
+                pos = 0;                         // the whole-token path returns its winners by rank, not by channel
+                for (int y = 0; y < k; y++) {
+                    const int cy = __shfl_sync(0xffffffffu, wc, y);
+                    pos += cy < wc ? 1 : 0;
+                }
+            }
+            // ---- outlier fields in channel order, dense codes at those channels cleared
+            if (won) {
+                unsigned short *oidx = reinterpret_cast<unsigned short *>(rec + coff + codeb);
+                oidx[pos] = (unsigned short)wc;
+                oidx[k + pos] = (unsigned short)float_to_half_bits_sat(we);
+                uint32_t *codes32 = reinterpret_cast<uint32_t *>(rec + coff);
+                const int bit = wc * BITS, wd = bit >> 5, sh = bit & 31;
+                atomicAnd(&codes32[wd], ~(cmask << sh));
+                if (BITS == 3 && sh + BITS > 32) atomicAnd(&codes32[wd + 1], ~(cmask >> (32 - sh)));
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                bulk_store(p.payload + t * recb, smem_u32(rec), (uint32_t)recb);
+                bulk_commit();
+            }
+        }
+    }
+    if (timed_out) {
+        ctrl->abort = 1;
+        if (p.status) atomicOr(p.status, RAC_STATUS_TIMEOUT);
+    }
+    __syncthreads();
+    if (lane == 0) bulk_wait_all();  // every lane that stored records waits for its own copies
+    if (tid == 0 && *reinterpret_cast<volatile int *>(&ctrl->abort)) {
+        // give copies that may still be in flight a bounded chance to land before the CTA retires
+        for (int s = 0; s < 2; s++) {
+            mbar_wait_bounded(smem_u32(&ctrl->full[s]), 0);
+            mbar_wait_bounded(smem_u32(&ctrl->full[s]), 1);
+        }
     }
 }
 
@@ -1218,24 +1545,65 @@ int fill_common(const Geometry &g, CodecParams *p, long long T, const void *ref_
     return RAC_OK;
 }
 
-// Encode: the streaming kernel, then (with outliers) the selection kernel.  Variant 4 of the streaming kernel
-// caps registers at 96 so that four 160-thread CTAs fit on an SM.
+// Encode with outliers, no x_hat, all tokens: the one-launch form.  The shape follows from the number of streaming warps; the
+// widths 4096 and 5120 with groups of 128 or 64 channels have variants with these compiled in, and of those one for calls in
+// which every token has its reference row.
+template <int BITS, int KT, int NV, int NSEL, int MAXT, int MINB, int D>
+static int launch_top_shape(const Geometry &g, CodecParams &p, bool allref, cudaStream_t stream) {
+    const int nt = g.nthreads + 32 * NSEL, smem = top_smem_layout(g.d, g.rec, (int)sizeof(TopSel<NSEL>)).total;
+#define RAC_TOP(G, R) launch_persistent(encode_top_kernel<BITS, KT, NV, NSEL, MAXT, MINB, G, D, R>, p, nt, smem, p.T, stream)
+    if constexpr (D != 0) {
+        if (g.lpg == 4) return allref ? RAC_TOP(4, true) : RAC_TOP(4, false);
+        return allref ? RAC_TOP(2, true) : RAC_TOP(2, false);
+    } else {
+        return g.lpg == 4 ? RAC_TOP(4, false) : RAC_TOP(0, false);
+    }
+#undef RAC_TOP
+}
+template <int BITS, int KT>
+static int launch_top_bits(const Geometry &g, CodecParams &p, cudaStream_t stream) {
+    const bool allref = p.ref_row == nullptr && p.ref_base != nullptr;   // identity rows
+    if constexpr (KT == 8) {
+        if (g.lpg == 4 || g.lpg == 2) {
+            if (g.d == 5120) return launch_top_shape<BITS, KT, 5, 3, 256, 3, 5120>(g, p, allref, stream);
+            if (g.d == 4096) return launch_top_shape<BITS, KT, 4, 2, 192, 4, 4096>(g, p, allref, stream);
+        }
+    }
+    if (g.nthreads <= 64) return launch_top_shape<BITS, KT, 2, 3, 160, 6, 0>(g, p, false, stream);
+    if (g.nthreads <= 128) return launch_top_shape<BITS, KT, 4, 2, 192, 4, 0>(g, p, false, stream);
+    if (g.nthreads <= 160) return launch_top_shape<BITS, KT, 5, 3, 256, 3, 0>(g, p, false, stream);
+    return launch_top_shape<BITS, KT, 8, 3, 352, 2, 0>(g, p, false, stream);
+}
+static int launch_top(const Geometry &g, CodecParams &p, cudaStream_t stream) {
+#define RAC_TOPB(B) (g.topk == 8 ? launch_top_bits<B, 8>(g, p, stream) : launch_top_bits<B, 0>(g, p, stream))
+    switch (g.bits) {
+        case 4: return RAC_TOPB(4);
+        case 3: return RAC_TOPB(3);
+        case 2: return RAC_TOPB(2);
+    }
+#undef RAC_TOPB
+    return RAC_EUNSUPPORTED;
+}
+
+// Encode: the streaming kernel, then (with outliers and x_hat, or over a token list) the selection kernel.  Variant 4 of the
+// streaming kernel caps registers at 96 so that four 160-thread CTAs fit on an SM.
 static int launch_encode(const Geometry &g, CodecParams &p, long long max_ctas, cudaStream_t stream) {
     if (g.scale_mode == 1) return launch_encode_dyn(g, p, max_ctas, stream);
     const bool topk = g.topk > 0;
+    const bool sub = p.tok_list || p.intra_base || p.coef_ext;   // the subset form has one variant per width: it is not the hot path
+    if (topk && !sub && !p.X_hat) return launch_top(g, p, stream);
     p.stages = 2;
     WsSmem L = ws_smem_layout(g.d, g.rec, p.stages, topk);
     // With x_hat the kernel reads both step tables every token; at four CTAs per SM the shared-memory carve-out
     // leaves too little L1 for them, so that variant runs three CTAs per SM at 128 registers.
     const bool tight = g.nthreads > 96 && g.nthreads <= 160 && !p.X_hat;
     int rc = RAC_EUNSUPPORTED;
-    const bool sub = p.tok_list || p.intra_base || p.coef_ext;   // the subset form has one variant per width: it is not the hot path
     // widths 4096 and 5120 with no or eight outliers per token run variants with the whole record geometry compiled in
     const bool geo = (g.d == 5120 || g.d == 4096) && (g.topk == 0 || g.topk == 8);
     const bool allref = p.ref_row == nullptr && p.ref_base != nullptr;   // identity rows: every token has its reference
 #define RAC_ENC4(B, K, X, G, W)                                                                                        \
-    (tight ? launch_persistent(encode_ws_kernel<B, K, X, 4, false, G, W>, p, g.nthreads, L.total, max_ctas, stream) \
-           : launch_persistent(encode_ws_kernel<B, K, X, 2, false, G, W>, p, g.nthreads, L.total, max_ctas, stream))
+    (!X && tight ? launch_persistent(encode_ws_kernel<B, K, X, X ? 2 : 4, false, G, W>, p, g.nthreads, L.total, max_ctas, stream) \
+                 : launch_persistent(encode_ws_kernel<B, K, X, 2, false, G, W>, p, g.nthreads, L.total, max_ctas, stream))
     // (at those widths the register variant follows from x_hat alone: 96 registers without it, 128 with it)
 #define RAC_ENC5(B, K, X, G, W, R) \
     launch_persistent(encode_ws_kernel<B, K, X, (X ? 2 : 4), false, G, W, R>, p, g.nthreads, L.total, max_ctas, stream)
@@ -1243,19 +1611,22 @@ static int launch_encode(const Geometry &g, CodecParams &p, long long max_ctas, 
     (!geo ? RAC_ENC4(B, K, X, G, 0)                                                                       \
      : g.d == 5120 ? (allref ? RAC_ENC5(B, K, X, G, 5120, true) : RAC_ENC5(B, K, X, G, 5120, false))     \
                    : (allref ? RAC_ENC5(B, K, X, G, 4096, true) : RAC_ENC5(B, K, X, G, 4096, false)))
-#define RAC_ENC2(B, K, X)                                                                                           \
-    (sub ? launch_persistent(encode_ws_kernel<B, K, X, 2, true, 0>, p, g.nthreads, L.total, max_ctas, stream)      \
-     : g.lpg == 4 ? RAC_ENC3(B, K, X, 4) : g.lpg == 2 ? RAC_ENC3(B, K, X, 2) : RAC_ENC4(B, K, X, 0, 0))
-#define RAC_ENC(B, K) (p.X_hat ? RAC_ENC2(B, K, true) : RAC_ENC2(B, K, false))
+#define RAC_ENC2(B, K, X) (g.lpg == 4 ? RAC_ENC3(B, K, X, 4) : g.lpg == 2 ? RAC_ENC3(B, K, X, 2) : RAC_ENC4(B, K, X, 0, 0))
+#define RAC_ENCS(B, K, X) launch_persistent(encode_ws_kernel<B, K, X, 2, true, 0>, p, g.nthreads, L.total, max_ctas, stream)
+#define RAC_ENC(B)                                                                                                  \
+    (sub ? (p.X_hat ? (topk ? RAC_ENCS(B, true, true) : RAC_ENCS(B, false, true))                                   \
+                    : (topk ? RAC_ENCS(B, true, false) : RAC_ENCS(B, false, false)))                                \
+     : topk ? RAC_ENC2(B, true, true) : (p.X_hat ? RAC_ENC2(B, false, true) : RAC_ENC2(B, false, false)))
     switch (g.bits) {
-        case 4: rc = topk ? RAC_ENC(4, true) : RAC_ENC(4, false); break;
-        case 3: rc = topk ? RAC_ENC(3, true) : RAC_ENC(3, false); break;
-        case 2: rc = topk ? RAC_ENC(2, true) : RAC_ENC(2, false); break;
+        case 4: rc = RAC_ENC(4); break;
+        case 3: rc = RAC_ENC(3); break;
+        case 2: rc = RAC_ENC(2); break;
     }
 #undef RAC_ENC5
 #undef RAC_ENC4
 #undef RAC_ENC3
 #undef RAC_ENC2
+#undef RAC_ENCS
 #undef RAC_ENC
     if (rc != RAC_OK || !topk) return rc;
     DeviceInfo di;

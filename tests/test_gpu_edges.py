@@ -131,3 +131,35 @@ def test_windows_that_occur_thousands_of_times(env):
         rows, spans = _match(env, hist, query, 4, K)
         o_rows, o_spans = env.orc.match_spans(hist, query, 4, K)
         assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
+
+
+# ------------------------------------------------------------------------------- encode with outliers in one launch
+@pytest.mark.parametrize("d,g,bits,k,T", [
+    (64, 32, 4, 2, 9000), (2048, 128, 3, 8, 8000), (2080, 32, 4, 16, 5000), (4096, 64, 2, 8, 5400), (4128, 32, 3, 5, 4100),
+    (5120, 128, 4, 8, 4100), (5152, 32, 4, 8, 2700), (8192, 1024, 4, 1, 2400), (8192, 64, 3, 8, 3)])
+def test_one_launch_outliers_at_shape_edges(env, d, g, bits, k, T):
+    """Widths on both sides of every CTA shape, more tokens than four rounds of the record slots (or fewer than CTAs), gathered
+    rows with direct tokens, some tokens with many equal residuals (the whole-token path): records equal the oracle's given the
+    device's coefficient words."""
+    s, rac, orc, dev, P = env.synth, env.rac, env.orc, env.dev, env.P
+    gen = s.generator(d + T, dev)
+    scale = s.channel_scale(d, 5, dev)
+    X = s.activations(T, d, scale, gen)
+    R = s.affine_noisy_reference(X, g, gen)
+    rng = np.random.default_rng(d)
+    rows = np.arange(T, dtype=np.int32)
+    rows[rng.random(T) < 0.2] = -1
+    equal = rng.random(T) < 0.02                       # reference equal to the token: an all-zero residual
+    R[torch.from_numpy(np.flatnonzero(equal)).to(dev)] = X[torch.from_numpy(np.flatnonzero(equal)).to(dev)]
+    flat = np.flatnonzero(rng.random(T) < 0.02)        # a few levels only: many equal magnitudes
+    X[torch.from_numpy(flat).to(dev)] = torch.sign(X[torch.from_numpy(flat).to(dev)].float()).to(torch.bfloat16)
+    cal = min(T, 512)
+    step, inv = orc.calibrate(d, g, bits, s.bf16_bits(X[:cal]), ref_base=s.bf16_bits(R[:cal]), ref_row=rows[:cal])
+    step_d, inv_d = P.to_dev(step, dev), P.to_dev(inv, dev)
+    cfg = rac.CodecCfg(d, g, bits, k)
+    pay, st = P.gpu_encode(cfg, X, R, torch.from_numpy(rows).to(dev), None, None, step_d, inv_d)
+    assert st == 0
+    P.compare_encode(cfg, pay, s.bf16_bits(X), s.bf16_bits(R), rows, None, None, step, inv)
+    # the same records as the two-launch form of the call with x_hat
+    pay2, xs, st = P.gpu_encode_reconstruct(cfg, X, R, torch.from_numpy(rows).to(dev), None, None, step_d, inv_d)
+    assert st == 0 and np.array_equal(pay, pay2)
