@@ -120,10 +120,11 @@ __host__ __device__ inline WsSmem ws_smem_layout(int d, int rec, int stages, boo
 
 // One thread's 32 channels of one token, rows and record in shared memory: Eq. 6, Eq. 7, Eq. 8 with the static table, packing,
 // the sender-side reconstruction (over the X row), and the largest |e| of the slab.
-template <int BITS, bool TOPK, bool XHAT, int LPG>
+// STEPREG: every token has a reference, and the thread holds its steps (row 0 of the table, slot order) in st0.
+template <int BITS, bool TOPK, bool XHAT, int LPG, bool STEPREG>
 __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int lane, int rot, int d, int Jc, bool shared, int coff,
                                             const uint32_t (&off)[4], unsigned int group_mask, uint32_t xs, uint32_t rs,
-                                            bool has_ref, int seg, unsigned char *rec, float *tm) {
+                                            bool has_ref, int seg, unsigned char *rec, float *tm, const u64 (&st0)[STEPREG ? 16 : 1]) {
     constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
     const u64 magic2 = pack2(kMagic, kMagic);
     // ---- (1) the slab: 4 slots of 8 channels, slot j holds piece (j + rot) & 3
@@ -171,9 +172,14 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
         const u64 inv2[4] = {pack2(iv0.x, iv0.y), pack2(iv0.z, iv0.w), pack2(iv1.x, iv1.y), pack2(iv1.z, iv1.w)};
         u64 st2[4] = {0ull, 0ull, 0ull, 0ull};
         if (XHAT) {
-            const float4 s0 = __ldg(reinterpret_cast<const float4 *>(step_tab + c));
-            const float4 s1 = __ldg(reinterpret_cast<const float4 *>(step_tab + c + 4));
-            st2[0] = pack2(s0.x, s0.y); st2[1] = pack2(s0.z, s0.w); st2[2] = pack2(s1.x, s1.y); st2[3] = pack2(s1.z, s1.w);
+            if (STEPREG) {
+#pragma unroll
+                for (int i = 0; i < 4; i++) st2[i] = st0[STEPREG ? 4 * j + i : 0];
+            } else {
+                const float4 s0 = __ldg(reinterpret_cast<const float4 *>(step_tab + c));
+                const float4 s1 = __ldg(reinterpret_cast<const float4 *>(step_tab + c + 4));
+                st2[0] = pack2(s0.x, s0.y); st2[1] = pack2(s0.z, s0.w); st2[2] = pack2(s1.x, s1.y); st2[3] = pack2(s1.z, s1.w);
+            }
         }
         float ev[8];
         uint32_t xh[4];
@@ -328,6 +334,26 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
     for (int j = 0; j < 4; j++) off[j] = (uint32_t)(tid * 64 + ((j + rot) & 3) * 16);
     const unsigned int group_mask = __ballot_sync(0xffffffffu, valid);
 
+    // x_hat where every token has a reference: the thread's steps stay in registers (it always owns the same channels), which
+    // leaves L1 to the other table (65536 x 5120 without outliers 346 -> 330 us, 9000 x 8192 130 -> 103 us).  Where a call can
+    // contain direct tokens the same with a branch per token was slower (long uplink 905 -> 980 us).
+    constexpr bool kStepReg = XHAT && REF;
+    u64 st0[kStepReg ? 16 : 1] = {};
+    if (kStepReg) {
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0;
+            if (valid) {
+                s0 = __ldg(reinterpret_cast<const float4 *>(p.step + (off[j] >> 1)));
+                s1 = __ldg(reinterpret_cast<const float4 *>(p.step + (off[j] >> 1) + 4));
+            }
+            st0[kStepReg ? 4 * j + 0 : 0] = pack2(s0.x, s0.y);
+            st0[kStepReg ? 4 * j + 1 : 0] = pack2(s0.z, s0.w);
+            st0[kStepReg ? 4 * j + 2 : 0] = pack2(s1.x, s1.y);
+            st0[kStepReg ? 4 * j + 3 : 0] = pack2(s1.z, s1.w);
+        }
+    }
+
     int stage = 0, duty = 0;  // duty: the warp whose turn the tail of this token is
     uint32_t parity = 0;
     bool timed_out = false;
@@ -341,9 +367,9 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
         const bool has_ref = REF ? true : ctrl->row[stage] >= 0;
 
         if (valid)
-            encode_slab<BITS, TOPK, XHAT, LPG>(p, tid, lane, rot, d, Jc, shared, coff, off, group_mask, xs, rs, has_ref,
+            encode_slab<BITS, TOPK, XHAT, LPG, kStepReg>(p, tid, lane, rot, d, Jc, shared, coff, off, group_mask, xs, rs, has_ref,
                                                SUB ? ctrl->seg[stage] : 0, rec,
-                                               reinterpret_cast<float *>(stg + L.tm_off + parity * L.tm_bytes));
+                                               reinterpret_cast<float *>(stg + L.tm_off + parity * L.tm_bytes), st0);
         // this warp's share of the token is in shared memory: one arrival per warp
         fence_async_smem();  // the record (and x_hat) bytes written above will be read by the copy engine
         __syncwarp();
@@ -825,6 +851,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
 #pragma unroll
         for (int j = 0; j < 4; j++) off[j] = (uint32_t)(tid * 64 + ((j + rot) & 3) * 16);
         const unsigned int group_mask = __ballot_sync(0xffffffffu, valid);
+        const u64 no_steps[1] = {0ull};
         for (int it = 0; it < n_my; it++) {
             if (*reinterpret_cast<volatile int *>(&ctrl->abort)) break;
             const int stage = it & 1;
@@ -834,9 +861,9 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
             if (!__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&ctrl->full[stage]), parity))) { timed_out = true; break; }
             const bool has_ref = REF ? true : ctrl->row[stage] >= 0;
             if (valid)
-                encode_slab<BITS, true, false, LPG>(p, tid, lane, rot, d, Jc, false, coff, off, group_mask, xs, xs + row_bytes,
+                encode_slab<BITS, true, false, LPG, false>(p, tid, lane, rot, d, Jc, false, coff, off, group_mask, xs, xs + row_bytes,
                                                     has_ref, 0, stg + L.rec_off + parity * recb,
-                                                    reinterpret_cast<float *>(stg + L.tm_off));
+                                                    reinterpret_cast<float *>(stg + L.tm_off), no_steps);
             fence_async_smem();     // the record bytes written above will be read by the copy engine
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&ctrl->done[it & 3])) : "memory");
@@ -1603,7 +1630,8 @@ static int launch_encode(const Geometry &g, CodecParams &p, long long max_ctas, 
     const bool allref = p.ref_row == nullptr && p.ref_base != nullptr;   // identity rows: every token has its reference
 #define RAC_ENC4(B, K, X, G, W)                                                                                        \
     (!X && tight ? launch_persistent(encode_ws_kernel<B, K, X, X ? 2 : 4, false, G, W>, p, g.nthreads, L.total, max_ctas, stream) \
-                 : launch_persistent(encode_ws_kernel<B, K, X, 2, false, G, W>, p, g.nthreads, L.total, max_ctas, stream))
+     : X && allref ? launch_persistent(encode_ws_kernel<B, K, X, 2, false, G, W, X>, p, g.nthreads, L.total, max_ctas, stream)    \
+                   : launch_persistent(encode_ws_kernel<B, K, X, 2, false, G, W>, p, g.nthreads, L.total, max_ctas, stream))
     // (at those widths the register variant follows from x_hat alone: 96 registers without it, 128 with it)
 #define RAC_ENC5(B, K, X, G, W, R) \
     launch_persistent(encode_ws_kernel<B, K, X, (X ? 2 : 4), false, G, W, R>, p, g.nthreads, L.total, max_ctas, stream)
