@@ -87,8 +87,8 @@ int make_geometry(const rac_codec_cfg *cfg, Geometry *g) {
 // ------------------------------------------------------------------------------------------------
 // encode
 // ------------------------------------------------------------------------------------------------
-// Without outliers one launch of the streaming pass, with outliers and no x_hat one launch of encode_top_kernel (below), with
-// both two launches.  (1) The streaming pass (this kernel): statistics, coefficients, residual, codes; every
+// Without outliers one launch of the streaming pass; with outliers one launch of encode_top_kernel (below) or two launches (the
+// rule is one_launch's).  (1) The streaming pass (this kernel): statistics, coefficients, residual, codes; every
 // warp of the CTA works on its 1024 channels of the token and ends with ONE arrival on the stage's `done`
 // mbarrier -- there is no CTA barrier in the loop.  Handing the finished record to the copy engine and
 // refilling the stage is the duty of warp (i mod warps) for token i; the other warps are already in the
@@ -749,7 +749,7 @@ __global__ void __launch_bounds__(W * 32, W == 7 ? 4 : 3) outlier_kernel(const C
 }
 
 // ------------------------------------------------------------------------------------------------
-// encode with outliers in one launch (calls without x_hat)
+// encode with outliers in one launch
 // ------------------------------------------------------------------------------------------------
 // The streaming pass with NSEL further warps per CTA, the selectors.  A selector takes every NSEL-th token: when the streaming
 // warps have finished it, it refills the stage at once (two stages), finds the k largest |e| from the slab maxima by the steps
@@ -761,8 +761,8 @@ __global__ void __launch_bounds__(W * 32, W == 7 ? 4 : 3) outlier_kernel(const C
 // The row reads bypass L1, which holds the step table.  Shapes by width (streaming warps + selectors, CTAs per SM): measured at
 // 131072 x 5120 3 CTAs of 5 + 3 warps 0.537 ms, 3 of 5 + 2 0.570, 4 of 5 + 2 0.589 to 0.649, 4 of 5 + 3 0.611 (two launches
 // 0.601); at 16384 x 4096 4 CTAs of 4 + 2 66 us, 4 of 4 + 3 68, 5 of 4 + 2 72 (two launches 81).  Reading the slabs from the
-// stage and refilling it afterwards was slower in every shape.  With x_hat the outliers would have to replace elements of a row
-// that has left by a bulk store, and waiting for its completion in the loop costs 0.2 ms: those calls keep the two launches.
+// stage and refilling it afterwards was slower in every shape.  With x_hat the CTAs keep two selectors and the registers that
+// three of them per SM leave; see one_launch for where that form is the better one.
 struct TopCtrl {
     unsigned long long full[2];     // data of the stage has landed
     unsigned long long done[4];     // every streaming warp has finished token (mod 4)
@@ -770,11 +770,15 @@ struct TopCtrl {
     int row[2];
     int abort;
 };
-template <int NSEL>
+constexpr int kHotCap = 64;        // slabs looked at; more (many maxima tie): the whole token
+constexpr int kPatchWords = 64;    // outliers of x_hat rows that have left, per selector
+template <int NSEL, bool XHAT>
 struct TopSel {
     float e[NSEL][kOutCap];
     unsigned short c[NSEL][kOutCap];
-    unsigned char hot[NSEL][256];
+    unsigned char hot[NSEL][kHotCap];
+    float rt[XHAT ? NSEL : 1][XHAT ? kOutCap : 1];
+    uint32_t patch[XHAT ? NSEL : 1][XHAT ? kPatchWords : 1];
 };
 struct TopSmem {
     int stage0, stage_bytes, rec_off, tm_off, sel0, total;
@@ -792,7 +796,7 @@ __host__ __device__ inline TopSmem top_smem_layout(int d, int rec, int sel_bytes
 
 // NV: slab maxima per lane (d <= 1024 * NV).  KT: the number of outliers when it is 8, else 0 = p.topk.  LPG, D, REF: as for
 // encode_ws_kernel.
-template <int BITS, int KT, int NV, int NSEL, int MAXT, int MINB, int LPG, int D = 0, bool REF = false>
+template <int BITS, int KT, bool XHAT, int NV, int NSEL, int MAXT, int MINB, int LPG, int D = 0, bool REF = false>
 __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -804,7 +808,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
     const int codeb = kGeo ? D * BITS / 8 : p.code_bytes;
     const int recb = kGeo ? (4 * (D / (32 * (LPG ? LPG : 1))) + D * BITS / 8 + 32 + 15) / 16 * 16 : p.rec;
     const int coff = 4 * Jc;
-    const TopSmem L = top_smem_layout(d, recb, (int)sizeof(TopSel<NSEL>));
+    const TopSmem L = top_smem_layout(d, recb, (int)sizeof(TopSel<NSEL, XHAT>));
     TopCtrl *ctrl = reinterpret_cast<TopCtrl *>(smem);
     const uint32_t sbase = smem_u32(smem);
     const uint32_t row_bytes = 2u * (uint32_t)d;
@@ -861,7 +865,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
             if (!__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&ctrl->full[stage]), parity))) { timed_out = true; break; }
             const bool has_ref = REF ? true : ctrl->row[stage] >= 0;
             if (valid)
-                encode_slab<BITS, true, false, LPG, false>(p, tid, lane, rot, d, Jc, false, coff, off, group_mask, xs, xs + row_bytes,
+                encode_slab<BITS, true, XHAT, LPG, false>(p, tid, lane, rot, d, Jc, false, coff, off, group_mask, xs, xs + row_bytes,
                                                     has_ref, 0, stg + L.rec_off + parity * recb,
                                                     reinterpret_cast<float *>(stg + L.tm_off), no_steps);
             fence_async_smem();     // the record bytes written above will be read by the copy engine
@@ -871,11 +875,27 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
     } else {
         // ---- selectors
         const int sel = warp - nstream;
-        TopSel<NSEL> *sc = reinterpret_cast<TopSel<NSEL> *>(smem + L.sel0);
+        const int nth = d >> 5, k = KT ? KT : p.topk;
+        TopSel<NSEL, XHAT> *sc = reinterpret_cast<TopSel<NSEL, XHAT> *>(smem + L.sel0);
         float *s_e = sc->e[sel];
         unsigned short *s_c = sc->c[sel];
         unsigned char *s_hot = sc->hot[sel];
-        const int nth = d >> 5, k = KT ? KT : p.topk;
+        // x_hat rows leave as bulk stores before their outliers are known.  The outliers wait here until the rows are in place:
+        // one wait for the stores of several tokens (a wait per token cost 0.2 ms at 131072 x 5120)
+        float *s_rt = sc->rt[XHAT ? sel : 0];
+        uint32_t *s_patch = sc->patch[XHAT ? sel : 0];
+        int n_patch = 0, it_patch = sel;        // tokens that wait, and the first of them
+        auto flush_patches = [&]() {
+            if (lane == 0) bulk_wait_all();
+            __syncwarp();
+            for (int q = lane; q < n_patch * k; q += 32) {
+                const uint32_t w = s_patch[q];
+                p.X_hat[token(it_patch + (q / k) * NSEL) * d + (w & 0xffffu)] = (uint16_t)(w >> 16);
+            }
+            __syncwarp();
+            it_patch += n_patch * NSEL;
+            n_patch = 0;
+        };
         const unsigned int lt_mask = (1u << lane) - 1u;
         constexpr uint32_t cmask = (1u << BITS) - 1u;
         const int coef_shift = 5 + (LPG ? (LPG == 4 ? 2 : 1) : p.lpg_shift);
@@ -889,6 +909,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
             const long long t = token(it);
             int raw_next = 0;
             if (lane == 0 && next < n_my) raw_next = raw_row_of(next);
+            if (XHAT && (n_patch + 1) * k > kPatchWords) flush_patches();
             if (lane == 0 && it >= NSEL) {      // this selector's last record
                 bulk_wait_read<0>();
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&ctrl->left[(it - NSEL) & 3])) : "memory");
@@ -903,6 +924,11 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
             for (int i = 0; i < NV; i++)
                 tv[i] = 32 * i + lane < nth ? *reinterpret_cast<volatile unsigned int *>(stg + L.tm_off + (32 * i + lane) * 4) : 0u;
             __syncwarp();
+            if (XHAT && lane == 0) {            // the X row carries x_hat now and must have been read before the refill
+                bulk_store(p.X_hat + t * d, sbase + L.stage0 + s * L.stage_bytes, row_bytes);
+                bulk_commit();
+                bulk_wait_read<0>();
+            }
             if (next < n_my) {
                 // the next token of this stage writes the record slot of token it - 2
                 if (it >= 2 && !__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&ctrl->left[next & 3]), ((next >> 2) - 1) & 1))) {
@@ -935,10 +961,11 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
                 for (int i = 0; i < NV; i++) {
                     const bool hit = tv[i] >= tau;
                     const unsigned int bal = __ballot_sync(0xffffffffu, hit);
-                    if (hit) s_hot[nh + __popc(bal & lt_mask)] = (unsigned char)(32 * i + lane);
+                    const int at = nh + __popc(bal & lt_mask);
+                    if (hit && at < kHotCap) s_hot[at] = (unsigned char)(32 * i + lane);
                     nh += __popc(bal);
                 }
-                n = 0;
+                n = nh <= kHotCap ? 0 : kOutCap + 1;
             }
             __syncwarp();
             // ---- candidates: eight slabs per round, four lanes per slab, eight channels per lane
@@ -968,11 +995,13 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
                 }
                 const float ca = half_bits_to_float(cf & 0xffff), cb = half_bits_to_float(cf >> 16);
                 const u64 a2 = pack2(ca, ca), b2 = pack2(cb, cb);
-                float e[8];
+                float e[8], rt[8];
                 uint32_t m = 0u;
 #pragma unroll
                 for (int i = 0; i < 4; i++) {
-                    unpack2(sub_pair(xw[i], pfma(a2, bf16x2_to_p(rw[i]), b2)), e[2 * i], e[2 * i + 1]);
+                    const u64 rt2 = pfma(a2, bf16x2_to_p(rw[i]), b2);
+                    unpack2(rt2, rt[2 * i], rt[2 * i + 1]);
+                    unpack2(sub_pair(xw[i], rt2), e[2 * i], e[2 * i + 1]);
                     m |= (fabsf(e[2 * i]) >= tauf ? 1u : 0u) << (2 * i) | (fabsf(e[2 * i + 1]) >= tauf ? 2u : 0u) << (2 * i);
                 }
                 if (!act) m = 0u;
@@ -999,6 +1028,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
                     if (pos < kOutCap) {
                         s_e[pos] = pick8(e, i);
                         s_c[pos] = (unsigned short)(c0 + i);
+                        if (XHAT) s_rt[pos] = pick8(rt, i);
                     }
                     pos++;
                 }
@@ -1008,12 +1038,13 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
             // ---- one candidate per lane, in channel order; while there are too many the smallest goes
             bool won;
             int wc = 0, pos;
-            float we = 0.f;
+            float we = 0.f, wrt = 0.f;
             if (n <= kOutCap) {
                 won = lane < n;
                 if (won) {
                     wc = s_c[lane];
                     we = s_e[lane];
+                    if (XHAT) wrt = s_rt[lane];
                 }
                 unsigned int mag = won ? (__float_as_uint(we) & 0x7fffffffu) : 0xffffffffu;
                 for (int extra = n - k; extra > 0; extra--) {
@@ -1023,8 +1054,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
                 }
                 pos = __popc(__ballot_sync(0xffffffffu, won) & lt_mask);
             } else {
-                float unused;
-                select_whole_token(d, k, coef_shift, xrow, rrow, p.gain, p.bias, coefp, lane, &wc, &we, &unused);
+                select_whole_token(d, k, coef_shift, xrow, rrow, p.gain, p.bias, coefp, lane, &wc, &we, &wrt);
                 won = lane < k;
                 pos = 0;                         // the whole-token path returns its winners by rank, not by channel
                 for (int y = 0; y < k; y++) {
@@ -1036,7 +1066,13 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
             if (won) {
                 unsigned short *oidx = reinterpret_cast<unsigned short *>(rec + coff + codeb);
                 oidx[pos] = (unsigned short)wc;
-                oidx[k + pos] = (unsigned short)float_to_half_bits_sat(we);
+                const uint32_t hv = float_to_half_bits_sat(we);
+                oidx[k + pos] = (unsigned short)hv;
+                // the sender-side reconstruction of an outlier channel: (alpha*r + beta) + the binary16 value
+                if (XHAT) {
+                    const uint16_t xh = __bfloat16_as_ushort(__float2bfloat16_rn(__fadd_rn(wrt, half_bits_to_float(hv))));
+                    s_patch[n_patch * k + pos] = (uint32_t)wc | (uint32_t)xh << 16;
+                }
                 uint32_t *codes32 = reinterpret_cast<uint32_t *>(rec + coff);
                 const int bit = wc * BITS, wd = bit >> 5, sh = bit & 31;
                 atomicAnd(&codes32[wd], ~(cmask << sh));
@@ -1048,7 +1084,9 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
                 bulk_store(p.payload + t * recb, smem_u32(rec), (uint32_t)recb);
                 bulk_commit();
             }
+            n_patch++;
         }
+        if (XHAT) flush_patches();
     }
     if (timed_out) {
         ctrl->abort = 1;
@@ -1572,16 +1610,18 @@ int fill_common(const Geometry &g, CodecParams *p, long long T, const void *ref_
     return RAC_OK;
 }
 
-// Encode with outliers, no x_hat, all tokens: the one-launch form.  The shape follows from the number of streaming warps; the
-// widths 4096 and 5120 with groups of 128 or 64 channels have variants with these compiled in, and of those one for calls in
-// which every token has its reference row.
-template <int BITS, int KT, int NV, int NSEL, int MAXT, int MINB, int D>
+// Encode with outliers, all tokens: the one-launch form.  The shape follows from the number of streaming warps; without x_hat
+// the widths 4096 and 5120 with groups of 128 or 64 channels have variants with these compiled in, and of those one for calls
+// in which every token has its reference row; with x_hat the width is compiled in for groups of 128.
+template <int BITS, int KT, bool XHAT, int NV, int NSEL, int MAXT, int MINB, int D>
 static int launch_top_shape(const Geometry &g, CodecParams &p, bool allref, cudaStream_t stream) {
-    const int nt = g.nthreads + 32 * NSEL, smem = top_smem_layout(g.d, g.rec, (int)sizeof(TopSel<NSEL>)).total;
-#define RAC_TOP(G, R) launch_persistent(encode_top_kernel<BITS, KT, NV, NSEL, MAXT, MINB, G, D, R>, p, nt, smem, p.T, stream)
-    if constexpr (D != 0) {
+    const int nt = g.nthreads + 32 * NSEL, smem = top_smem_layout(g.d, g.rec, (int)sizeof(TopSel<NSEL, XHAT>)).total;
+#define RAC_TOP(G, R) launch_persistent(encode_top_kernel<BITS, KT, XHAT, NV, NSEL, MAXT, MINB, G, D, R>, p, nt, smem, p.T, stream)
+    if constexpr (D != 0 && !XHAT) {
         if (g.lpg == 4) return allref ? RAC_TOP(4, true) : RAC_TOP(4, false);
         return allref ? RAC_TOP(2, true) : RAC_TOP(2, false);
+    } else if constexpr (D != 0) {
+        return RAC_TOP(4, false);
     } else {
         return g.lpg == 4 ? RAC_TOP(4, false) : RAC_TOP(0, false);
     }
@@ -1590,16 +1630,37 @@ static int launch_top_shape(const Geometry &g, CodecParams &p, bool allref, cuda
 template <int BITS, int KT>
 static int launch_top_bits(const Geometry &g, CodecParams &p, cudaStream_t stream) {
     const bool allref = p.ref_row == nullptr && p.ref_base != nullptr;   // identity rows
+    if (p.X_hat) {
+        if constexpr (KT == 8) {
+            if (g.lpg == 4 && g.d == 5120) return launch_top_shape<BITS, KT, true, 5, 2, 224, 3, 5120>(g, p, false, stream);
+            if (g.lpg == 4 && g.d == 4096) return launch_top_shape<BITS, KT, true, 4, 2, 192, 3, 4096>(g, p, false, stream);
+        }
+        if (g.nthreads <= 64) return launch_top_shape<BITS, KT, true, 2, 2, 128, 5, 0>(g, p, false, stream);
+        if (g.nthreads <= 96) return launch_top_shape<BITS, KT, true, 4, 2, 160, 4, 0>(g, p, false, stream);
+        if (g.nthreads <= 128) return launch_top_shape<BITS, KT, true, 4, 2, 192, 3, 0>(g, p, false, stream);
+        if (g.nthreads <= 160) return launch_top_shape<BITS, KT, true, 5, 2, 224, 3, 0>(g, p, false, stream);
+        return launch_top_shape<BITS, KT, true, 8, 2, 320, 2, 0>(g, p, false, stream);
+    }
     if constexpr (KT == 8) {
         if (g.lpg == 4 || g.lpg == 2) {
-            if (g.d == 5120) return launch_top_shape<BITS, KT, 5, 3, 256, 3, 5120>(g, p, allref, stream);
-            if (g.d == 4096) return launch_top_shape<BITS, KT, 4, 2, 192, 4, 4096>(g, p, allref, stream);
+            if (g.d == 5120) return launch_top_shape<BITS, KT, false, 5, 3, 256, 3, 5120>(g, p, allref, stream);
+            if (g.d == 4096) return launch_top_shape<BITS, KT, false, 4, 2, 192, 4, 4096>(g, p, allref, stream);
         }
     }
-    if (g.nthreads <= 64) return launch_top_shape<BITS, KT, 2, 3, 160, 6, 0>(g, p, false, stream);
-    if (g.nthreads <= 128) return launch_top_shape<BITS, KT, 4, 2, 192, 4, 0>(g, p, false, stream);
-    if (g.nthreads <= 160) return launch_top_shape<BITS, KT, 5, 3, 256, 3, 0>(g, p, false, stream);
-    return launch_top_shape<BITS, KT, 8, 3, 352, 2, 0>(g, p, false, stream);
+    if (g.nthreads <= 64) return launch_top_shape<BITS, KT, false, 2, 3, 160, 6, 0>(g, p, false, stream);
+    if (g.nthreads <= 128) return launch_top_shape<BITS, KT, false, 4, 2, 192, 4, 0>(g, p, false, stream);
+    if (g.nthreads <= 160) return launch_top_shape<BITS, KT, false, 5, 3, 256, 3, 0>(g, p, false, stream);
+    return launch_top_shape<BITS, KT, false, 8, 3, 352, 2, 0>(g, p, false, stream);
+}
+// Which calls with outliers take the one-launch form (two launches / one launch, 4-bit, eight outliers).  Without x_hat all of
+// them.  With x_hat everything up to 4096 channels: 512 x 4096 11.7 / 7.8 us, 2048 x 4096 22.3 / 17.4, gathered 100000 x 4096
+// 590 / 487, 40000 x 1536 128 / 114.  At 5120 channels the selectors' registers and the step tables in L1 are short: 2048 x 5120
+// 24.7 / 21.0, identity rows 100000 x 5120 627 / 619, but with direct tokens, which bring a second row of both tables, 8192
+// tokens 62.5 / 62.5 and 100000 tokens 647 / 662.  Beyond, 512 x 8192 19.5 / 17.4 but 4096 x 8192 54 / 62.
+static bool one_launch(const Geometry &g, const CodecParams &p) {
+    if (!p.X_hat || g.nthreads <= 128) return true;
+    if (g.nthreads <= 160) return p.ref_row == nullptr || p.T <= 8192;
+    return p.T <= 1024;
 }
 static int launch_top(const Geometry &g, CodecParams &p, cudaStream_t stream) {
 #define RAC_TOPB(B) (g.topk == 8 ? launch_top_bits<B, 8>(g, p, stream) : launch_top_bits<B, 0>(g, p, stream))
@@ -1618,7 +1679,7 @@ static int launch_encode(const Geometry &g, CodecParams &p, long long max_ctas, 
     if (g.scale_mode == 1) return launch_encode_dyn(g, p, max_ctas, stream);
     const bool topk = g.topk > 0;
     const bool sub = p.tok_list || p.intra_base || p.coef_ext;   // the subset form has one variant per width: it is not the hot path
-    if (topk && !sub && !p.X_hat) return launch_top(g, p, stream);
+    if (topk && !sub && one_launch(g, p)) return launch_top(g, p, stream);
     p.stages = 2;
     WsSmem L = ws_smem_layout(g.d, g.rec, p.stages, topk);
     // With x_hat the kernel reads both step tables every token; at four CTAs per SM the shared-memory carve-out
@@ -1660,11 +1721,11 @@ static int launch_encode(const Geometry &g, CodecParams &p, long long max_ctas, 
     DeviceInfo di;
     rc = device_info(&di);
     if (rc != RAC_OK) return rc;
-    // a warp per pair of tokens.  Without x_hat: four CTAs of seven warps per SM (72 registers); with x_hat (more state per
-    // token): three CTAs of eight warps (80 registers).  With more work than one round of them, every warp gets the same
-    // number of rounds (a grid of whole rounds, not a full grid with a ragged last round).
+    // A warp per pair of tokens.  Many rounds of them, or a token list: three CTAs of eight warps (80 registers, 48 tokens per
+    // SM); few rounds: four CTAs of seven warps (72 registers, 56 tokens).  With more work than one round, every warp gets the
+    // same number of rounds (a grid of whole rounds, not a full grid with a ragged last round).
     // (measured at 131072 x 5120: 0.901 against 0.910 ms; with few rounds the smaller CTAs win: 16384 x 4096 0.105 -> 0.102 ms)
-    const bool wide = sub || (p.X_hat != nullptr && p.T > (long long)di.sms * 3 * 8 * kOutPair * 6);
+    const bool wide = sub || p.T > (long long)di.sms * 3 * 8 * kOutPair * 6;
     const int wpc = wide ? 8 : 7;
     const long long per_cta = wpc * kOutPair;
     long long blocks = (p.T + per_cta - 1) / per_cta;

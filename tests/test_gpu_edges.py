@@ -136,7 +136,8 @@ def test_windows_that_occur_thousands_of_times(env):
 # ------------------------------------------------------------------------------- encode with outliers in one launch
 @pytest.mark.parametrize("d,g,bits,k,T", [
     (64, 32, 4, 2, 9000), (2048, 128, 3, 8, 8000), (2080, 32, 4, 16, 5000), (4096, 64, 2, 8, 5400), (4128, 32, 3, 5, 4100),
-    (5120, 128, 4, 8, 4100), (5152, 32, 4, 8, 2700), (8192, 1024, 4, 1, 2400), (8192, 64, 3, 8, 3)])
+    (3072, 64, 4, 8, 6000), (5120, 128, 4, 8, 4100), (5120, 64, 2, 12, 8193), (5152, 32, 4, 8, 2700), (8192, 1024, 4, 1, 2400),
+    (8192, 64, 3, 8, 3), (8192, 128, 4, 8, 1024)])
 def test_one_launch_outliers_at_shape_edges(env, d, g, bits, k, T):
     """Widths on both sides of every CTA shape, more tokens than four rounds of the record slots (or fewer than CTAs), gathered
     rows with direct tokens, some tokens with many equal residuals (the whole-token path): records equal the oracle's given the
@@ -160,6 +161,8 @@ def test_one_launch_outliers_at_shape_edges(env, d, g, bits, k, T):
     pay, st = P.gpu_encode(cfg, X, R, torch.from_numpy(rows).to(dev), None, None, step_d, inv_d)
     assert st == 0
     P.compare_encode(cfg, pay, s.bf16_bits(X), s.bf16_bits(R), rows, None, None, step, inv)
-    # the same records as the two-launch form of the call with x_hat
+    # with x_hat: the same records, and x_hat equal to the oracle's reconstruction of them
     pay2, xs, st = P.gpu_encode_reconstruct(cfg, X, R, torch.from_numpy(rows).to(dev), None, None, step_d, inv_d)
     assert st == 0 and np.array_equal(pay, pay2)
+    o_x = orc.reconstruct(d, g, bits, k, pay, T, ref_base=s.bf16_bits(R), ref_row=rows, step=step, nthreads=orc.max_threads())
+    assert np.array_equal(o_x.reshape(-1), s.bf16_bits(xs).reshape(-1))
