@@ -1673,50 +1673,73 @@ static int launch_top(const Geometry &g, CodecParams &p, cudaStream_t stream) {
     return RAC_EUNSUPPORTED;
 }
 
-// Encode: the streaming kernel, then (with outliers and x_hat, or over a token list) the selection kernel.  Variant 4 of the
-// streaming kernel caps registers at 96 so that four 160-thread CTAs fit on an SM.
+// The streaming kernel of one call.  REF (every token has a reference row: identity rows) drops the test per token; with x_hat it
+// also keeps the thread's steps in registers.  Register variants: 64 Ki registers hold two CTAs of 160 threads at 128 registers a
+// thread beside a third, or four at 96.  Without x_hat four CTAs are the better ones; with x_hat the kernel reads both step
+// tables every token, and at four CTAs per SM the shared-memory carve-out leaves too little L1 for them.
+template <int BITS, bool TOPK, bool XHAT, int LPG, int D>
+static int launch_stream_lpg(const Geometry &g, CodecParams &p, size_t smem, long long max_ctas, cudaStream_t stream) {
+    const bool allref = p.ref_row == nullptr && p.ref_base != nullptr;
+#define RAC_STREAM(M, R) \
+    launch_persistent(encode_ws_kernel<BITS, TOPK, XHAT, M, false, LPG, D, R>, p, g.nthreads, smem, max_ctas, stream)
+    if constexpr (XHAT) {
+        if constexpr (!(TOPK && D != 0)) {   // (at that width, identity rows with outliers are always one launch)
+            if (allref) return RAC_STREAM(2, true);
+        }
+        return RAC_STREAM(2, false);
+    } else if constexpr (D != 0) {
+        return allref ? RAC_STREAM(4, true) : RAC_STREAM(4, false);
+    } else {
+        return g.nthreads > 96 && g.nthreads <= 160 ? RAC_STREAM(4, false) : RAC_STREAM(2, false);
+    }
+#undef RAC_STREAM
+}
+
+// Widths 4096 and 5120 have variants with the record geometry compiled in; 4096 with outliers is always one launch (one_launch),
+// and so is every call with outliers and without x_hat: what those would need is not instantiated.
+template <int BITS, bool TOPK, bool XHAT>
+static int launch_stream(const Geometry &g, CodecParams &p, size_t smem, long long max_ctas, cudaStream_t stream) {
+    if (p.tok_list || p.intra_base || p.coef_ext)   // the subset form has one variant: it is not the hot path
+        return launch_persistent(encode_ws_kernel<BITS, TOPK, XHAT, 2, true, 0>, p, g.nthreads, smem, max_ctas, stream);
+    if constexpr (!TOPK || XHAT) {
+        if (g.d == 5120 && (!TOPK || g.topk == 8)) {
+            if (g.lpg == 4) return launch_stream_lpg<BITS, TOPK, XHAT, 4, 5120>(g, p, smem, max_ctas, stream);
+            if (g.lpg == 2) return launch_stream_lpg<BITS, TOPK, XHAT, 2, 5120>(g, p, smem, max_ctas, stream);
+        }
+        if constexpr (!TOPK) {
+            if (g.d == 4096 && g.lpg == 4) return launch_stream_lpg<BITS, TOPK, XHAT, 4, 4096>(g, p, smem, max_ctas, stream);
+            if (g.d == 4096 && g.lpg == 2) return launch_stream_lpg<BITS, TOPK, XHAT, 2, 4096>(g, p, smem, max_ctas, stream);
+        }
+        if (g.lpg == 4) return launch_stream_lpg<BITS, TOPK, XHAT, 4, 0>(g, p, smem, max_ctas, stream);
+        if (g.lpg == 2) return launch_stream_lpg<BITS, TOPK, XHAT, 2, 0>(g, p, smem, max_ctas, stream);
+        return launch_stream_lpg<BITS, TOPK, XHAT, 0, 0>(g, p, smem, max_ctas, stream);
+    }
+    return RAC_EUNSUPPORTED;
+}
+
+template <int BITS>
+static int launch_stream_bits(const Geometry &g, CodecParams &p, size_t smem, long long max_ctas, cudaStream_t stream) {
+    if (g.topk > 0)
+        return p.X_hat ? launch_stream<BITS, true, true>(g, p, smem, max_ctas, stream)
+                       : launch_stream<BITS, true, false>(g, p, smem, max_ctas, stream);
+    return p.X_hat ? launch_stream<BITS, false, true>(g, p, smem, max_ctas, stream)
+                   : launch_stream<BITS, false, false>(g, p, smem, max_ctas, stream);
+}
+
+// Encode: one launch (one_launch), or the streaming kernel and then, with outliers, the selection kernel.
 static int launch_encode(const Geometry &g, CodecParams &p, long long max_ctas, cudaStream_t stream) {
     if (g.scale_mode == 1) return launch_encode_dyn(g, p, max_ctas, stream);
     const bool topk = g.topk > 0;
-    const bool sub = p.tok_list || p.intra_base || p.coef_ext;   // the subset form has one variant per width: it is not the hot path
+    const bool sub = p.tok_list || p.intra_base || p.coef_ext;
     if (topk && !sub && one_launch(g, p)) return launch_top(g, p, stream);
     p.stages = 2;
-    WsSmem L = ws_smem_layout(g.d, g.rec, p.stages, topk);
-    // With x_hat the kernel reads both step tables every token; at four CTAs per SM the shared-memory carve-out
-    // leaves too little L1 for them, so that variant runs three CTAs per SM at 128 registers.
-    const bool tight = g.nthreads > 96 && g.nthreads <= 160 && !p.X_hat;
+    const size_t smem = ws_smem_layout(g.d, g.rec, p.stages, topk).total;
     int rc = RAC_EUNSUPPORTED;
-    // widths 4096 and 5120 with no or eight outliers per token run variants with the whole record geometry compiled in
-    const bool geo = (g.d == 5120 || g.d == 4096) && (g.topk == 0 || g.topk == 8);
-    const bool allref = p.ref_row == nullptr && p.ref_base != nullptr;   // identity rows: every token has its reference
-#define RAC_ENC4(B, K, X, G, W)                                                                                        \
-    (!X && tight ? launch_persistent(encode_ws_kernel<B, K, X, X ? 2 : 4, false, G, W>, p, g.nthreads, L.total, max_ctas, stream) \
-     : X && allref ? launch_persistent(encode_ws_kernel<B, K, X, 2, false, G, W, X>, p, g.nthreads, L.total, max_ctas, stream)    \
-                   : launch_persistent(encode_ws_kernel<B, K, X, 2, false, G, W>, p, g.nthreads, L.total, max_ctas, stream))
-    // (at those widths the register variant follows from x_hat alone: 96 registers without it, 128 with it)
-#define RAC_ENC5(B, K, X, G, W, R) \
-    launch_persistent(encode_ws_kernel<B, K, X, (X ? 2 : 4), false, G, W, R>, p, g.nthreads, L.total, max_ctas, stream)
-#define RAC_ENC3(B, K, X, G)                                                                              \
-    (!geo ? RAC_ENC4(B, K, X, G, 0)                                                                       \
-     : g.d == 5120 ? (allref ? RAC_ENC5(B, K, X, G, 5120, true) : RAC_ENC5(B, K, X, G, 5120, false))     \
-                   : (allref ? RAC_ENC5(B, K, X, G, 4096, true) : RAC_ENC5(B, K, X, G, 4096, false)))
-#define RAC_ENC2(B, K, X) (g.lpg == 4 ? RAC_ENC3(B, K, X, 4) : g.lpg == 2 ? RAC_ENC3(B, K, X, 2) : RAC_ENC4(B, K, X, 0, 0))
-#define RAC_ENCS(B, K, X) launch_persistent(encode_ws_kernel<B, K, X, 2, true, 0>, p, g.nthreads, L.total, max_ctas, stream)
-#define RAC_ENC(B)                                                                                                  \
-    (sub ? (p.X_hat ? (topk ? RAC_ENCS(B, true, true) : RAC_ENCS(B, false, true))                                   \
-                    : (topk ? RAC_ENCS(B, true, false) : RAC_ENCS(B, false, false)))                                \
-     : topk ? RAC_ENC2(B, true, true) : (p.X_hat ? RAC_ENC2(B, false, true) : RAC_ENC2(B, false, false)))
     switch (g.bits) {
-        case 4: rc = RAC_ENC(4); break;
-        case 3: rc = RAC_ENC(3); break;
-        case 2: rc = RAC_ENC(2); break;
+        case 4: rc = launch_stream_bits<4>(g, p, smem, max_ctas, stream); break;
+        case 3: rc = launch_stream_bits<3>(g, p, smem, max_ctas, stream); break;
+        case 2: rc = launch_stream_bits<2>(g, p, smem, max_ctas, stream); break;
     }
-#undef RAC_ENC5
-#undef RAC_ENC4
-#undef RAC_ENC3
-#undef RAC_ENC2
-#undef RAC_ENCS
-#undef RAC_ENC
     if (rc != RAC_OK || !topk) return rc;
     DeviceInfo di;
     rc = device_info(&di);
@@ -1734,19 +1757,17 @@ static int launch_encode(const Geometry &g, CodecParams &p, long long max_ctas, 
         const long long rounds = (blocks + resident - 1) / resident;
         blocks = (blocks + rounds - 1) / rounds;
     }
-    const int nth = g.d / 32;
+    const int nth = g.d / 32;      // up to 128 threads the call is always one launch (one_launch)
     const unsigned nb = (unsigned)blocks, nt = wpc * 32;
 #define RAC_OUT(NV, KT)                                                                    \
     (wide ? launch_after(outlier_kernel<NV, KT, false, 8>, nb, nt, 0, stream, p, g.bits)     \
           : launch_after(outlier_kernel<NV, KT, false, 7>, nb, nt, 0, stream, p, g.bits))
     if (sub) launch_after(outlier_kernel<8, 0, true, 8>, nb, nt, 0, stream, p, g.bits);
     else if (g.topk == 8) {
-        if (nth <= 128) RAC_OUT(4, 8);
-        else if (nth <= 160) RAC_OUT(5, 8);
+        if (nth <= 160) RAC_OUT(5, 8);
         else RAC_OUT(8, 8);
     } else {
-        if (nth <= 128) RAC_OUT(4, 0);
-        else if (nth <= 160) RAC_OUT(5, 0);
+        if (nth <= 160) RAC_OUT(5, 0);
         else RAC_OUT(8, 0);
     }
 #undef RAC_OUT
