@@ -171,7 +171,8 @@ struct Geometry {
 int make_geometry(const rac_codec_cfg *cfg, Geometry *g);  // RAC_OK or an error
 
 // Launch of a kernel that may be set up while the one before it on the stream drains (programmatic dependent launch):
-// the kernel itself waits for its predecessor's memory (grid_dependency_wait) before it reads anything.
+// the kernel itself waits for its predecessor's memory (grid_dependency_wait) before it reads anything (what was there before
+// the predecessor began may be read earlier, where the predecessor is known to let its successor begin only after its own wait).
 template <typename K, typename... Args>
 static void launch_after(K kernel, unsigned grid, unsigned block, size_t smem, cudaStream_t stream, Args... args) {
     cudaLaunchConfig_t cfg = {};
@@ -184,6 +185,26 @@ static void launch_after(K kernel, unsigned grid, unsigned block, size_t smem, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+// the same with clusters of `cluster` CTAs
+template <typename K, typename... Args>
+static void launch_cluster_after(K kernel, unsigned grid, unsigned cluster, unsigned block, size_t smem, cudaStream_t stream,
+                                 Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
     cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 

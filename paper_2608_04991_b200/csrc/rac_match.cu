@@ -9,24 +9,31 @@
 // Selection: the left-to-right scan of Eq. 3 visits a position, jumps by the span length if it has a candidate and by one
 // otherwise.  Positions are cut into chunks; every chunk works out, for each of its positions, where a scan that enters there
 // leaves the chunk and how many spans it selects on the way (pointer doubling in shared memory).  What is left is one hop per
-// chunk; a last kernel walks every chunk from the position where the scan enters it and writes its spans and rows.
+// chunk; then every chunk is walked from the position where the scan enters it, and writes its spans and rows.  Up to eight
+// chunks are the CTAs of one cluster, and all of the query is one launch; more take three.
 //
 // All of it is bound by the latency of dependent trips to L2 and of launches, not by the bytes: the forms above were chosen
 // to make fewer of both, and every kernel lets the next one be set up while it runs.  32768 history and 2048 query tokens:
-// 23 us in four launches (52 us in nine before: sorted lists, a thread per match, a suffix scan and a serial walk), 131072 /
-// 131072 tokens: 44 us (99 us), a query of 2048 tokens against an index of 16384 22 us (60 us), eight appends of 2048 tokens
-// behind a reset 39 us (54 us).
+// 20.5 us in three launches (52 us in nine before: sorted lists, a thread per match, a suffix scan and a serial walk; 23.5 us
+// with selection and emission in two launches and a test before every load of the extension), 131072 / 131072 tokens 40 us
+// (99 us, 43.6 us), a query of 2048 tokens against an index of 16384 16 us (60 us, 22 us), with intra-sequence references 18.5 us
+// (28 us), eight appends of 2048 tokens behind a reset 39 us (54 us).  Of the query's 16 us, 9 are the slowest warp's
+// candidates: up to eight of them, one after another, two trips each.
+#include <cooperative_groups.h>
+
 #include <mutex>
 
 #include "rac_common.cuh"
 
 namespace rac {
 
+namespace cg = cooperative_groups;
+
 typedef unsigned long long u64;
 constexpr u64 kEmptySlot = ~0ull;
 constexpr int kBucket = 4;             // slots per bucket
 constexpr int kChunk = 512;            // query positions per chunk of the selection = threads of its CTAs
-constexpr int kInlineChunks = 8;       // up to so many chunks every CTA of the last kernel walks the chunks itself
+constexpr int kClusterChunks = 8;      // up to so many chunks are one cluster of CTAs (the portable limit), and the query one launch
 
 struct MatchParams {
     const int32_t *hist;
@@ -45,41 +52,47 @@ struct MatchParams {
     unsigned int bmask;    // buckets - 1
     const int32_t *end_of; // [n_hist] end of the request that holds each history position; null = one request
     int first_live;        // only windows that start at or after this history position are candidates (0 = all)
-    // intra-sequence references: a table of the prompt's tokens, keyed by a position that holds the token
-    int32_t *trep;         // [tmask + 1] that position, -1 = empty; null = no such references
-    int32_t *tfirst;       // [tmask + 1] kFirstBase - (first position of the token), -1 = none yet
+    // intra-sequence references: a table of the prompt's tokens (TokenTable).  One cluster keeps it in shared memory.
+    unsigned int *tok;     // [tmask + 1] else null
     unsigned int tmask;
+    int intra;
+    int ahead;             // the launch before this one is of the same call and began after everything before the call had ended
 };
-constexpr int kFirstBase = 0x3fffffff;
 
-// four tokens (or what is left of the window) per step, loaded before any is used: a window is a chain of one or two trips
-// to memory, not one per token
-__device__ __forceinline__ u64 window_hash(const int32_t *tok, int w) {
-    u64 h = 0x9E3779B97F4A7C15ull;
+// Four tokens of a window (or what is left of it) per step, loaded before any is used: a chain of one or two trips to memory, not
+// one per token.  Kernels that may read the call's tokens ahead of their turn stage them in shared memory.
+__device__ __forceinline__ u64 hash_step(u64 h, int32_t t) {
+    h ^= (u64)(uint32_t)t;
+    h *= 0xff51afd7ed558ccdull;
+    return h ^ (h >> 32);
+}
+constexpr u64 kHashStart = 0x9E3779B97F4A7C15ull;
+__device__ __forceinline__ u64 window_hash(const int32_t *win, int w) {
+    u64 h = kHashStart;
     for (int m = 0; m < w; m += 4) {
-        uint32_t t[4];
+        int32_t t[4];
 #pragma unroll
-        for (int u = 0; u < 4; u++) t[u] = m + u < w ? (uint32_t)tok[m + u] : 0u;
+        for (int u = 0; u < 4; u++) t[u] = m + u < w ? win[m + u] : 0;
 #pragma unroll
-        for (int u = 0; u < 4; u++) {
-            if (m + u < w) {
-                h ^= (u64)t[u];
-                h *= 0xff51afd7ed558ccdull;
-                h ^= h >> 32;
-            }
-        }
+        for (int u = 0; u < 4; u++)
+            if (m + u < w) h = hash_step(h, t[u]);
     }
     return h;
 }
-__device__ __forceinline__ bool same_window(const int32_t *a, const int32_t *b, int w) {
-    for (int m = 0; m < w; m += 4) {
-        uint32_t x[4], y[4];
+// tokens [lo, lo + n) of src, as far as they lie before `end`, into shared memory; the caller synchronises
+__device__ __forceinline__ void stage_tokens(int32_t *dst, const int32_t *src, int lo, int n, int end) {
+    for (int t = threadIdx.x; t < n; t += blockDim.x) dst[t] = lo + t < end ? __ldcg(src + lo + t) : 0;
+}
+// the window at `win` (staged) is the one at `a` (history): eight tokens of it per trip
+__device__ __forceinline__ bool same_window(const int32_t *a, const int32_t *win, int w) {
+    for (int m = 0; m < w; m += 8) {
+        int32_t x[8];
 #pragma unroll
-        for (int u = 0; u < 4; u++) {
-            x[u] = m + u < w ? (uint32_t)a[m + u] : 0u;
-            y[u] = m + u < w ? (uint32_t)b[m + u] : 0u;
-        }
-        if ((x[0] ^ y[0]) | (x[1] ^ y[1]) | (x[2] ^ y[2]) | (x[3] ^ y[3])) return false;
+        for (int u = 0; u < 8; u++) x[u] = m + u < w ? a[m + u] : 0;
+        int32_t ne = 0;
+#pragma unroll
+        for (int u = 0; u < 8; u++) ne |= m + u < w ? x[u] ^ win[m + u] : 0;
+        if (ne) return false;
     }
     return true;
 }
@@ -108,8 +121,8 @@ __device__ __forceinline__ int find_in_bucket(const u64 (&e)[kBucket], uint32_t 
 // The representative start of the window that starts at history position j: the one its slot holds, or j itself after
 // claiming the first empty slot of the probe sequence.  Slots fill in probe order and are never emptied, so two threads with
 // the same window end at one slot.  The window's set of starts stands at the place of its representative in `top`.
-__device__ __forceinline__ int find_or_claim(u64 *slots, unsigned int bmask, const int32_t *hist, int j, int w) {
-    const u64 h = window_hash(hist + j, w);
+__device__ __forceinline__ int find_or_claim(u64 *slots, unsigned int bmask, const int32_t *hist, int j, const int32_t *win, int w,
+                                             u64 h) {
     const uint32_t tag = (uint32_t)(h >> 32);
     unsigned int b = (unsigned int)h & bmask, probes = 0;
     u64 e[kBucket];
@@ -130,10 +143,25 @@ __device__ __forceinline__ int find_or_claim(u64 *slots, unsigned int bmask, con
             held = atomicCAS(at, kEmptySlot, ((u64)tag << 32) | (uint32_t)j);
             if (held == kEmptySlot) return j;
         }
-        if ((uint32_t)(held >> 32) == tag && same_window(hist + (int)(uint32_t)held, hist + j, w)) return (int)(uint32_t)held;
+        if ((uint32_t)(held >> 32) == tag && same_window(hist + (int)(uint32_t)held, win, w)) return (int)(uint32_t)held;
         from = s + 1;
     }
-    return -1;   // the table has at least twice as many slots as windows: not reached
+    return -1;   // the table has four times as many slots as windows: not reached
+}
+
+// a set as the L2 holds it, `none` beyond its K entries
+__device__ __forceinline__ void load_set(const int32_t *set, int K, int none, int (&v)[16]) {
+#pragma unroll
+    for (int m = 0; m < 4; m++) {
+        if ((K & 3) == 0) {       // whole 16-byte pieces (the table's sections are 16-byte aligned)
+            int4 q = make_int4(none, none, none, none);
+            if (4 * m < K) q = __ldcg(reinterpret_cast<const int4 *>(set) + m);
+            v[4 * m] = q.x; v[4 * m + 1] = q.y; v[4 * m + 2] = q.z; v[4 * m + 3] = q.w;
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; u++) v[4 * m + u] = 4 * m + u < K ? __ldcg(set + 4 * m + u) : none;
+        }
+    }
 }
 
 // Start j enters a window's set of the K largest starts (-1 = empty entry): it takes the place of the smallest entry, by
@@ -143,17 +171,7 @@ __device__ __forceinline__ int find_or_claim(u64 *slots, unsigned int bmask, con
 // One look at the set and one swap are two trips to L2 (a sorted list, kept by a cascade of atomicMax, cost up to K).
 __device__ __forceinline__ void set_insert(int32_t *set, int K, int j) {
     int v[16];
-#pragma unroll
-    for (int m = 0; m < 4; m++) {
-        if ((K & 3) == 0) {       // whole 16-byte pieces (the table's sections are 16-byte aligned)
-            int4 q = make_int4(0x7fffffff, 0x7fffffff, 0x7fffffff, 0x7fffffff);
-            if (4 * m < K) q = __ldcg(reinterpret_cast<const int4 *>(set) + m);
-            v[4 * m] = q.x; v[4 * m + 1] = q.y; v[4 * m + 2] = q.z; v[4 * m + 3] = q.w;
-        } else {
-#pragma unroll
-            for (int u = 0; u < 4; u++) v[4 * m + u] = 4 * m + u < K ? __ldcg(set + 4 * m + u) : 0x7fffffff;
-        }
-    }
+    load_set(set, K, 0x7fffffff, v);
     while (true) {
         int low = v[0], at = 0;
         unsigned int empty = 0;
@@ -176,28 +194,36 @@ __device__ __forceinline__ void set_insert(int32_t *set, int K, int j) {
 // Start j enters the index.  Unlimited hits: every start goes onto its window's chain.  The order of a chain
 // depends on which thread came first; the query looks at ALL of it and keeps lexargmax(length, start), so the result does not.
 __device__ __forceinline__ void index_start(u64 *slots, int32_t *top, int32_t *next, unsigned int bmask, const int32_t *hist,
-                                            int j, int w, int K) {
-    const int rep = find_or_claim(slots, bmask, hist, j, w);
+                                            int j, const int32_t *win, int w, int K, u64 h) {
+    const int rep = find_or_claim(slots, bmask, hist, j, win, w, h);
     if (rep < 0) return;
     if (next) next[j] = atomicExch(&top[rep], j);
     else set_insert(top + (size_t)rep * K, K, j);
 }
 
-// all ones in n16 pieces of 16 bytes; with zero, also *zero = 0
+// All ones in n16 pieces of 16 bytes; with zero, also *zero = 0.  The kernel after it may begin once the work before this call
+// has ended (not at once): it then reads the call's tokens while the fill is under way.
 __global__ void fill_ones_kernel(uint4 *dst, long long n16, int32_t *zero) {
-    grid_launch_dependents();
     grid_dependency_wait();
+    grid_launch_dependents();
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     for (long long k = i; k < n16; k += (long long)gridDim.x * blockDim.x) dst[k] = make_uint4(~0u, ~0u, ~0u, ~0u);
     if (zero && i == 0) *zero = 0;
 }
 
+// Tokens and hashes before the wait for the fill: the tokens are of before the call, and the fill let this kernel begin only
+// once that had ended.  (The query kernel does the same behind this one.)
 __global__ void __launch_bounds__(256) match_insert_kernel(const MatchParams p) {
-    grid_launch_dependents();
-    grid_dependency_wait();
+    __shared__ int32_t s_tok[256 + 32];
     // the latest starts first: once a set is full of them the earlier ones are done with one look
-    const int j = p.nwin - 1 - (int)(blockIdx.x * blockDim.x + threadIdx.x);
-    if (j >= 0) index_start(p.slots, p.top, p.next, p.bmask, p.hist, j, p.w, p.K);
+    const int j = p.nwin - 1 - (int)(blockIdx.x * 256 + threadIdx.x), lo = p.nwin - 256 - (int)(blockIdx.x * 256);
+    for (int t = threadIdx.x; t < 256 + p.w - 1; t += 256) s_tok[t] = lo + t >= 0 ? __ldcg(p.hist + lo + t) : 0;
+    __syncthreads();
+    const int32_t *win = s_tok + (255 - threadIdx.x);
+    const u64 h = window_hash(win, p.w);
+    grid_dependency_wait();
+    grid_launch_dependents();
+    if (j >= 0) index_start(p.slots, p.top, p.next, p.bmask, p.hist, j, win, p.w, p.K, h);
 }
 
 // first position at or after this thread's position in its chunk that has a candidate (`limit` if none)
@@ -213,33 +239,135 @@ __device__ __forceinline__ int next_candidate(bool has, int i, int limit) {
     return limit;
 }
 
-// Lookup, extension, and the chunk's jumps.  One CTA per chunk, one thread per position.
-// Extension: a thread compares eight tokens at its candidate by itself; what is still open after that is finished by the
-// warp, 128 tokens per trip.  Neighbouring positions inside one copied stretch have the same (history - query) distance and
-// so the same end: one comparison closes them all.  A thread by itself took a trip per eight tokens, for every position
-// of a long match (2048-token prompt: 21 us, with copies of copies 55 us).
-__global__ void __launch_bounds__(kChunk, 2) match_query_kernel(const MatchParams p) {
-    grid_launch_dependents();
-    grid_dependency_wait();
-    const int N = p.n_query;
-    const int base = blockIdx.x * kChunk, i = base + threadIdx.x, lane = threadIdx.x & 31;
-    if (p.trep && i < N) {     // intra-sequence references: the first position of every token of the prompt
-        const int32_t tok = p.query[i];
-        unsigned int s = (unsigned int)window_hash(&tok, 1) & p.tmask;
-        for (unsigned int probe = 0; probe <= p.tmask; probe++) {
-            int cur = __ldcg(p.trep + s);
-            if (cur < 0) cur = atomicCAS(&p.trep[s], -1, i);
-            if (cur < 0 || p.query[cur] == tok) {
-                if (__ldcg(p.tfirst + s) < kFirstBase - i) atomicMax(&p.tfirst[s], kFirstBase - i);
-                break;
+// The tokens of a prompt: open addressing, a slot holds the smallest position so far of the token that claimed it (positions of
+// one token only ever replace each other), all ones = empty.  In global memory, or spread over the shared memories of a cluster.
+constexpr int kTokSlots = 2 * kChunk;     // per CTA of a cluster
+struct TokenTable {
+    const int32_t *query;
+    unsigned int *base;
+    unsigned int mask;
+    bool spread;
+    __device__ __forceinline__ unsigned int *at(unsigned int s) const {
+        return spread ? cg::this_cluster().map_shared_rank(base, s / kTokSlots) + s % kTokSlots : base + s;
+    }
+    // slots: a power of two in global memory, any multiple of kTokSlots in a cluster
+    __device__ __forceinline__ unsigned int start(int32_t tok) const {
+        const unsigned int h = (unsigned int)hash_step(kHashStart, tok);
+        return spread ? __umulhi(h, mask + 1u) : h & mask;
+    }
+    __device__ __forceinline__ unsigned int after(unsigned int s) const { return s == mask ? 0u : s + 1u; }
+    __device__ __forceinline__ void insert(int32_t tok, unsigned int i) const {
+        unsigned int s = start(tok);
+        for (unsigned int probe = 0; probe <= mask; probe++, s = after(s)) {
+            unsigned int *slot = at(s);
+            unsigned int cur = *(volatile unsigned int *)slot;
+            if (cur == ~0u) cur = atomicCAS(slot, ~0u, i);
+            if (cur == ~0u) return;
+            if (query[cur] == tok) {
+                if (i < cur) atomicMin(slot, i);
+                return;
             }
-            s = (s + 1) & p.tmask;
         }
     }
+    // first position of the token (it is in the table)
+    __device__ __forceinline__ unsigned int first(int32_t tok) const {
+        unsigned int s = start(tok);
+        for (unsigned int probe = 0; probe <= mask; probe++, s = after(s)) {
+            const unsigned int cur = *(volatile unsigned int *)at(s);
+            if (cur == ~0u || query[cur] == tok) return cur;
+        }
+        return ~0u;
+    }
+};
+
+// What a chunk hands out: the scan through it from its entry.  Every position at or after the entry belongs to this CTA alone,
+// and so does the part of its last span that reaches into later chunks (their entries lie behind it).
+struct EmitSmem {
+    int next[kChunk], len[kChunk], start[kChunk], row[kChunk], list[kChunk];
+    int entry, before, n;
+};
+__device__ __forceinline__ void emit_chunk(const MatchParams &p, EmitSmem &m, int base, const int32_t *tokens, const TokenTable &tt) {
+    const int N = p.n_query, limit = min(base + kChunk, N), i = base + threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        int pos = m.entry, n = 0;
+        while (pos < limit) {
+            const int s = m.next[pos - base];
+            if (s >= limit) break;
+            m.list[n++] = s - base;
+            pos = s + m.len[s - base];
+        }
+        m.n = n;
+        if (limit == N) *p.n_spans = m.before + n;
+    }
+    m.row[threadIdx.x] = -1;
+    __syncthreads();
+    const int n = m.n;
+    for (int k = warp; k < n; k += kChunk / 32) {        // a warp per span, up to the end of the chunk
+        const int at = m.list[k], len = m.len[at], s = base + at, h = m.start[at];
+        if (lane == 0 && p.spans_out) {
+            rac_span sp;
+            sp.q_start = s;
+            sp.h_start = h;
+            sp.len = len;
+            p.spans_out[m.before + k] = sp;
+        }
+        const int in = min(len, limit - s);
+        for (int q = lane; q < in; q += 32) m.row[at + q] = h + q;
+    }
+    if (n > 0) {                                         // the last span's part in later chunks: the whole CTA
+        const int at = m.list[n - 1], s = base + at, end = s + m.len[at], h = m.start[at];
+        for (int q = limit + threadIdx.x; q < end; q += kChunk) p.ref_row[q] = h + (q - s);
+    }
+    __syncthreads();
+    if (i < N && i >= m.entry) {
+        int row = m.row[threadIdx.x];
+        if (row < 0 && p.intra) {
+            // intra-sequence reference: the first occurrence of this token, if it is an earlier one
+            const unsigned int f = tt.first(tokens[threadIdx.x]);
+            if (f < (unsigned int)i) row = p.n_hist + (int)f;
+        }
+        p.ref_row[i] = row;
+    }
+}
+
+// Lookup, extension, and the chunk's jumps.  One CTA per chunk, one thread per position.
+// Extension: a thread compares eight tokens at its candidate by itself; what is still open after that is finished by the
+// warp, 256 tokens per trip.  Neighbouring positions inside one copied stretch have the same (history - query) distance and
+// so the same end: one comparison closes them all.  A thread by itself took a trip per eight tokens, for every position
+// of a long match (2048-token prompt: 21 us, with copies of copies 55 us).
+// ONE: the chunks are the CTAs of one cluster, which hands out spans and rows as well: a cluster barrier and jumps read from the
+// neighbours' shared memory in place of a launch, a table of tokens in shared memory in place of one that a launch has to fill.
+template <bool ONE>
+__global__ void __launch_bounds__(kChunk, ONE ? 1 : 2) match_query_kernel(const MatchParams p) {
+    __shared__ int32_t s_tok[kChunk + 40];
+    __shared__ unsigned int s_slots[ONE ? kTokSlots : 1];
+    grid_launch_dependents();
+    const int N = p.n_query;
+    const int base = blockIdx.x * kChunk, i = base + threadIdx.x, lane = threadIdx.x & 31;
+    TokenTable tt{p.query, p.tok, p.tmask, false};
+    if constexpr (ONE) {
+        if (p.intra) {
+            tt = TokenTable{p.query, s_slots, gridDim.x * kTokSlots - 1u, true};
+            for (int t = threadIdx.x; t < kTokSlots; t += kChunk) s_slots[t] = ~0u;
+            cg::this_cluster().barrier_arrive();
+        }
+    }
+    if (!p.ahead) grid_dependency_wait();
+    stage_tokens(s_tok, p.query, base, kChunk + p.w + 8, N);
+    __syncthreads();
+    const int32_t *win = s_tok + threadIdx.x;
+    const u64 h = window_hash(win, p.w);
+    if (p.ahead) grid_dependency_wait();
+    if (p.intra) {
+        if constexpr (ONE) cg::this_cluster().barrier_wait();
+        if (i < N) tt.insert(win[0], i);
+    }
     int rep = -1;      // representative start of the window at i, -1: not in the history
+    int v[16];         // its set
+#pragma unroll
+    for (int r = 0; r < 16; r++) v[r] = -1;
     if (i < N && i + p.w <= N && p.nwin > 0) {
-        const int32_t *win = p.query + i;
-        const u64 h = window_hash(win, p.w);
         const uint32_t tag = (uint32_t)(h >> 32);
         unsigned int b = (unsigned int)h & p.bmask;
         u64 e[kBucket];
@@ -264,25 +392,24 @@ __global__ void __launch_bounds__(kChunk, 2) match_query_kernel(const MatchParam
         }
     }
     int bestL = 0, bestj = -1;
-    // one candidate per lane (j = -1: none), all lanes of the warp together; `room`: the longest its match can be
-    auto consider = [&](int j, int room) {
-        int L = 0;
-        bool open = false;
-        if (j >= 0) {
-            L = p.w;
-            uint32_t ne = 0;
-            const int n8 = min(8, room - L);
-            int32_t q[8], hh[8];
+    // One candidate per lane (j = -1: none), all lanes of the warp together.  It replaces the best so far only with a longer match,
+    // or with one as long and a larger start, so its token at has_to_match has to be equal.  That token, the first eight behind
+    // the window and the end of the request come in one trip (no test stands before a load: it would make a trip of each).
+    auto has_to_match = [&](int j) { return max(bestL - (j > bestj ? 1 : 0), 0); };
+    auto consider = [&](int j) {
+        const int jj = max(j, 0), at = has_to_match(j);
+        int32_t hh[8];
 #pragma unroll
-            for (int u = 0; u < 8; u++) {
-                q[u] = u < n8 ? p.query[i + L + u] : 0;
-                hh[u] = u < n8 ? p.hist[j + L + u] : 0;
-            }
+        for (int u = 0; u < 8; u++) hh[u] = p.hist[min(jj + p.w + u, p.n_hist - 1)];
+        const int32_t h_at = p.hist[min(jj + at, p.n_hist - 1)], q_at = p.query[min(i + at, N - 1)];
+        const int end_j = p.end_of ? p.end_of[jj] : p.n_hist;
+        const int room = min(N - i, end_j - jj);          // the longest the match can be, inside its request
+        uint32_t ne = 0;
 #pragma unroll
-            for (int u = 0; u < 8; u++) ne |= (u >= n8 || q[u] != hh[u]) ? (1u << u) : 0u;
-            open = ne == 0u;
-            L += open ? 8 : __ffs(ne) - 1;
-        }
+        for (int u = 0; u < 8; u++) ne |= win[p.w + u] != hh[u] ? (1u << u) : 0u;
+        const bool can_win = j >= 0 && (bestL == 0 || (at < room && h_at == q_at));
+        int L = min(p.w + (ne ? __ffs(ne) - 1 : 8), room);
+        bool open = can_win && ne == 0u && p.w + 8 < room;
         unsigned int todo = __ballot_sync(0xffffffffu, open);
         while (todo) {
             const int lead = __ffs(todo) - 1;
@@ -291,14 +418,19 @@ __global__ void __launch_bounds__(kChunk, 2) match_query_kernel(const MatchParam
             int len = L0;
             bool more = true;
             while (more && len < room0) {
+                // (every load is made, at the last token inside where the lane is beyond: a test before each makes a trip of each)
+                int32_t q[8], hh[8];
                 uint32_t differ = 0;                   // bit u: the lane's token of the u-th 32 differs or lies outside
 #pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    const int at = len + 32 * u + lane;
-                    differ |= (at >= room0 || p.query[i0 + at] != p.hist[j0 + at]) ? (1u << u) : 0u;
+                for (int u = 0; u < 8; u++) {
+                    const int at = min(len + 32 * u + lane, room0 - 1);
+                    q[u] = p.query[i0 + at];
+                    hh[u] = p.hist[j0 + at];
                 }
 #pragma unroll
-                for (int u = 0; u < 4; u++) {
+                for (int u = 0; u < 8; u++) differ |= (len + 32 * u + lane >= room0 || q[u] != hh[u]) ? (1u << u) : 0u;
+#pragma unroll
+                for (int u = 0; u < 8; u++) {
                     const unsigned int b = __ballot_sync(0xffffffffu, (differ >> u) & 1u);
                     if (more) {
                         if (b) { len += __ffs(b) - 1; more = false; }
@@ -307,13 +439,12 @@ __global__ void __launch_bounds__(kChunk, 2) match_query_kernel(const MatchParam
                 }
             }
             // every open position of the same distance that lies before the end has the same end
-            const int end = i0 + len;
-            if (open && j - i == j0 - i0 && i < end) { L = end - i; open = false; }
+            const int stop = i0 + len;
+            if (open && j - i == j0 - i0 && i < stop) { L = stop - i; open = false; }
             todo = __ballot_sync(0xffffffffu, open);
         }
-        if (j >= 0 && (L > bestL || (L == bestL && j > bestj))) { bestL = L; bestj = j; }
+        if (can_win && (L > bestL || (L == bestL && j > bestj))) { bestL = L; bestj = j; }
     };
-    auto room_of = [&](int j) { return min(N - i, (p.end_of ? p.end_of[j] : p.n_hist) - j); };   // inside its request
     if (p.next) {
         // every occurrence of the window (at most nwin of them: the walk is bounded by construction)
         int chain = rep >= 0 ? p.top[rep] : -1, n = 0;
@@ -322,51 +453,48 @@ __global__ void __launch_bounds__(kChunk, 2) match_query_kernel(const MatchParam
             const int j = n < p.nwin ? chain : -1;
             if (!__any_sync(0xffffffffu, j >= 0)) break;
             if (j >= 0) { chain = p.next[j]; n++; }
-            consider(j, j >= 0 ? room_of(j) : 0);
+            consider(j);
         }
     } else {
-        // The K most recent starts.  A candidate replaces the best so far only with a longer match, or with one as long and a
-        // larger start, so its last token of that length has to match: after the first candidate, one trip for all the others
-        // rules most of them out before they are extended.
-        const int32_t *set = p.top + (size_t)(rep >= 0 ? rep : 0) * p.K;
-        auto can_win = [&](int j) {
-            const int at = bestL - (j > bestj ? 1 : 0);
-            return bestL == 0 || (room_of(j) > at && p.hist[j + at] == p.query[i + at]);
-        };
-        unsigned int alive = 0;
-        if (rep >= 0) {
-#pragma unroll 4
-            for (int r = 0; r < p.K; r++) alive |= set[r] >= p.first_live ? (1u << r) : 0u;   // first_live >= 0: no empty ones
-        }
+        // The K most recent starts.  After the first candidate, one trip for all the others rules most of them out (the end of
+        // a request is left to consider()).
+        if (rep >= 0) load_set(p.top + (size_t)rep * p.K, p.K, -1, v);
+#pragma unroll
+        for (int r = 0; r < 16; r++) v[r] = v[r] >= p.first_live ? v[r] : -1;     // first_live >= 0: no empty ones
         bool first = true;
-        while (__any_sync(0xffffffffu, alive != 0u)) {
+        while (true) {
             // largest start first: neighbours inside one copied stretch then look at the same distance at the same time
-            int j = -1, at = 0;
-            if (alive) {
-#pragma unroll 4
-                for (int r = 0; r < p.K; r++) {
-                    const int k = ((alive >> r) & 1u) ? set[r] : -1;
-                    if (k > j) { j = k; at = r; }
+            int j = v[0];
+#pragma unroll
+            for (int r = 1; r < 16; r++) j = max(j, v[r]);
+            if (!__any_sync(0xffffffffu, j >= 0)) break;
+#pragma unroll
+            for (int r = 0; r < 16; r++) v[r] = v[r] == j ? -1 : v[r];
+            consider(j);
+            if (first && bestL > 0) {
+                const int32_t q_last = p.query[i + bestL - 1], q_beyond = p.query[min(i + bestL, N - 1)];
+#pragma unroll
+                for (int r0 = 0; r0 < 16; r0 += 8) {
+                    if (r0 < p.K) {
+                        int32_t tok[8];
+#pragma unroll
+                        for (int r = 0; r < 8; r++)
+                            tok[r] = p.hist[min(max(v[r0 + r], 0) + has_to_match(v[r0 + r]), p.n_hist - 1)];
+#pragma unroll
+                        for (int r = 0; r < 8; r++)
+                            if (tok[r] != (v[r0 + r] > bestj ? q_last : q_beyond)) v[r0 + r] = -1;
+                    }
                 }
-                alive &= ~(1u << at);
-                if (!first && !can_win(j)) j = -1;
-            }
-            if (!__any_sync(0xffffffffu, j >= 0)) continue;
-            consider(j, j >= 0 ? room_of(j) : 0);
-            if (first && alive) {
-#pragma unroll 4
-                for (int r = 0; r < p.K; r++)
-                    if (((alive >> r) & 1u) && !can_win(set[r])) alive &= ~(1u << r);
             }
             first = false;
         }
     }
-    if (i < N) p.best[i] = make_int2(bestL, bestj);
 
     // ---- where a scan that is at position i leaves the chunk, by pointer doubling
     __shared__ int s_nxt[kChunk], s_cnt[kChunk];
     const int limit = min(base + kChunk, N);
-    int nxt = next_candidate(bestL > 0, i, limit), cnt = 0;
+    const int cand = next_candidate(bestL > 0, i, limit);
+    int nxt = cand, cnt = 0;
     if (bestL > 0) { nxt = i + bestL; cnt = 1; }
     if (i >= limit) { nxt = limit; cnt = 0; }
     while (true) {
@@ -380,7 +508,30 @@ __global__ void __launch_bounds__(kChunk, 2) match_query_kernel(const MatchParam
         }
         __syncthreads();
     }
-    if (i < N) p.jump[i] = make_int2(nxt, cnt);
+    if constexpr (ONE) {
+        __shared__ EmitSmem s_emit;
+        s_emit.next[threadIdx.x] = cand;
+        s_emit.len[threadIdx.x] = bestL;
+        s_emit.start[threadIdx.x] = bestj;
+        cg::cluster_group cluster = cg::this_cluster();
+        cluster.sync();
+        if (threadIdx.x == 0) {          // a hop per chunk before this one
+            int e = 0, before = 0;
+            for (unsigned int k = 0; k < blockIdx.x; k++) {
+                if (e >= (int)(k + 1) * kChunk) continue;
+                const int at = e - (int)k * kChunk;
+                e = cluster.map_shared_rank(s_nxt, k)[at];
+                before += cluster.map_shared_rank(s_cnt, k)[at];
+            }
+            s_emit.entry = e;
+            s_emit.before = before;
+        }
+        emit_chunk(p, s_emit, base, s_tok, tt);
+        cluster.sync();                  // nobody leaves while its shared memory may be read
+    } else if (i < N) {
+        p.best[i] = make_int2(bestL, bestj);
+        p.jump[i] = make_int2(nxt, cnt);
+    }
 }
 
 // Where the scan enters every chunk: entry of chunk c+1 = where a scan that enters chunk c at ITS entry leaves it.  All
@@ -432,92 +583,27 @@ __global__ void __launch_bounds__(1024) match_resolve_kernel(const MatchParams p
         carry_cnt += total;
         __syncthreads();
     }
-    if (tid == 0) *p.n_spans = carry_cnt;
 }
 
-// Spans and rows: the scan through one chunk from its entry.  Every position at or after the entry belongs to this CTA
-// alone, and so does the part of its last span that reaches into later chunks (their entries lie behind it).
-__global__ void __launch_bounds__(kChunk) match_emit_kernel(const MatchParams p, int nchunks) {
-    __shared__ int s_next[kChunk], s_len[kChunk], s_row[kChunk], s_list[kChunk];
-    __shared__ int s_entry, s_base, s_n;
+// Spans and rows (emit_chunk) of more chunks than a cluster holds.
+__global__ void __launch_bounds__(kChunk) match_emit_kernel(const MatchParams p) {
+    __shared__ EmitSmem s_emit;
+    __shared__ int32_t s_tok[kChunk];
     grid_launch_dependents();
     grid_dependency_wait();
-    const int N = p.n_query, c = blockIdx.x;
-    const int base = c * kChunk, limit = min(base + kChunk, N), i = base + threadIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int2 mine = i < N ? __ldcg(p.best + i) : make_int2(0, -1);
+    const int base = blockIdx.x * kChunk, i = base + threadIdx.x;
+    const int2 mine = i < p.n_query ? __ldcg(p.best + i) : make_int2(0, -1);
+    if (p.intra && i < p.n_query) s_tok[threadIdx.x] = p.query[i];
     if (threadIdx.x == 0) {
-        int e = 0, before = 0;
-        if (nchunks > kInlineChunks) {
-            const int2 v = __ldcg(p.entry + c);
-            e = v.x;
-            before = v.y;
-        } else {
-            for (int k = 0; k < c; k++) {
-                if (e >= min((k + 1) * kChunk, N)) continue;
-                const int2 v = __ldcg(p.jump + e);
-                e = v.x;
-                before += v.y;
-            }
-        }
-        s_entry = e;
-        s_base = before;
+        const int2 e = __ldcg(p.entry + blockIdx.x);
+        s_emit.entry = e.x;
+        s_emit.before = e.y;
     }
-    s_next[threadIdx.x] = next_candidate(mine.x > 0, i, limit);
-    s_len[threadIdx.x] = mine.x;
-    s_row[threadIdx.x] = -1;
+    s_emit.next[threadIdx.x] = next_candidate(mine.x > 0, i, min(base + kChunk, p.n_query));
+    s_emit.len[threadIdx.x] = mine.x;
+    s_emit.start[threadIdx.x] = mine.y;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int pos = s_entry, n = 0;
-        while (pos < limit) {
-            const int s = s_next[pos - base];
-            if (s >= limit) break;
-            s_list[n++] = s - base;
-            pos = s + s_len[s - base];
-        }
-        s_n = n;
-        if (nchunks <= kInlineChunks && c == nchunks - 1) *p.n_spans = s_base + n;
-    }
-    __syncthreads();
-    const int n = s_n, entry = s_entry;
-    for (int k = warp; k < n; k += kChunk / 32) {        // a warp per span, up to the end of the chunk
-        const int at = s_list[k], len = s_len[at], s = base + at;
-        const int h = __ldcg(&p.best[s].y);
-        if (lane == 0 && p.spans_out) {
-            rac_span sp;
-            sp.q_start = s;
-            sp.h_start = h;
-            sp.len = len;
-            p.spans_out[s_base + k] = sp;
-        }
-        const int in = min(len, limit - s);
-        for (int q = lane; q < in; q += 32) s_row[at + q] = h + q;
-    }
-    if (n > 0) {                                         // the last span's part in later chunks: the whole CTA
-        const int at = s_list[n - 1], s = base + at, end = s + s_len[at];
-        const int h = __ldcg(&p.best[s].y);
-        for (int q = limit + threadIdx.x; q < end; q += kChunk) p.ref_row[q] = h + (q - s);
-    }
-    __syncthreads();
-    if (i < N && i >= entry) {
-        int row = s_row[threadIdx.x];
-        if (row < 0 && p.trep) {
-            // intra-sequence reference: the first occurrence of this token, if it is an earlier one
-            const int32_t tok = p.query[i];
-            unsigned int s = (unsigned int)window_hash(&tok, 1) & p.tmask;
-            for (unsigned int probe = 0; probe <= p.tmask; probe++) {
-                const int cur = __ldcg(p.trep + s);
-                if (cur < 0) break;
-                if (p.query[cur] == tok) {
-                    const int f = kFirstBase - __ldcg(p.tfirst + s);
-                    if (f < i) row = p.n_hist + f;
-                    break;
-                }
-                s = (s + 1) & p.tmask;
-            }
-        }
-        p.ref_row[i] = row;
-    }
+    emit_chunk(p, s_emit, base, s_tok, TokenTable{p.query, p.tok, p.tmask, false});
 }
 
 __global__ void spans_to_rows_kernel(const rac_span *spans, const int32_t *n_spans, long long n_query, int32_t *ref_row) {
@@ -617,7 +703,7 @@ __global__ void __launch_bounds__(128) index_append_kernel(const IndexParams p) 
     if (j < p.a) return;
     p.end_of[j] = p.b;
     if (j + p.w <= p.b)      // else the window would leave the request
-        index_start(p.slots, p.top, p.next, p.bmask, p.hist, j, p.w, p.K);
+        index_start(p.slots, p.top, p.next, p.bmask, p.hist, j, p.hist + j, p.w, p.K, window_hash(p.hist + j, p.w));
 }
 
 static size_t align16(size_t v) { return (v + 15) / 16 * 16; }
@@ -649,13 +735,17 @@ static unsigned int table_slots(long long n, unsigned long long per) {
     return (unsigned int)M;
 }
 
-// lookup and extension, the chunks' entries (few chunks are walked in the last kernel instead: up to seven hops cost less
-// than a launch), spans and rows
+// lookup and extension, the chunks' entries, spans and rows: one cluster does all of it for up to kClusterChunks chunks
+static bool query_in_one(long long n_query) { return n_query <= (long long)kClusterChunks * kChunk; }
 static void launch_query(const MatchParams &p, cudaStream_t st) {
     const int nchunks = (p.n_query + kChunk - 1) / kChunk;
-    launch_after(match_query_kernel, nchunks, kChunk, 0, st, p);
-    if (nchunks > kInlineChunks) launch_after(match_resolve_kernel, 1, 1024, 0, st, p, nchunks);
-    launch_after(match_emit_kernel, nchunks, kChunk, 0, st, p, nchunks);
+    if (query_in_one(p.n_query)) {
+        launch_cluster_after(match_query_kernel<true>, nchunks, nchunks, kChunk, 0, st, p);
+        return;
+    }
+    launch_after(match_query_kernel<false>, nchunks, kChunk, 0, st, p);
+    launch_after(match_resolve_kernel, 1, 1024, 0, st, p, nchunks);
+    launch_after(match_emit_kernel, nchunks, kChunk, 0, st, p);
 }
 
 struct MatchLayout {
@@ -751,7 +841,8 @@ int rac_match_spans(const int32_t *hist_tok, int64_t n_hist, const int32_t *quer
     p.next = max_hits == 0 ? reinterpret_cast<int32_t *>(ws + L.next) : nullptr;
     p.bmask = L.M / kBucket - 1;
 
-    // four launches, five when there are many chunks; the times are in the head of this file
+    // three launches, five when there are many chunks; the times are in the head of this file
+    p.ahead = 1;
     const long long n16 = n_query > 0 ? (long long)(L.filled / 16) : 0;
     launch_after(fill_ones_kernel, fill_blocks(n16), 256, 0, st, reinterpret_cast<uint4 *>(ws + L.slots), n16, n_spans);
     if (n_query > 0) {
@@ -815,7 +906,7 @@ IndexLayout index_layout(const rac_index_cfg *c) {
     return L;
 }
 struct QueryLayout {
-    size_t best, jump, entry, trep, tfirst, total;
+    size_t best, jump, entry, tok, total;
     unsigned int Mq;
 };
 QueryLayout query_layout(long long n_query) {
@@ -826,8 +917,7 @@ QueryLayout query_layout(long long n_query) {
     L.best = o;    o = align16(o + n * 8);
     L.jump = o;    o = align16(o + n * 8);
     L.entry = o;   o = align16(o + (n / kChunk + 1) * 8);
-    L.trep = o;    o += (size_t)L.Mq * 4;                      // trep and tfirst contiguous: one fill
-    L.tfirst = o;  o += (size_t)L.Mq * 4;
+    L.tok = o;     o += (size_t)L.Mq * 4;
     L.total = o;
     return L;
 }
@@ -929,12 +1019,13 @@ int rac_index_query_live(const rac_index_cfg *cfg, const void *index, size_t ind
         launch_after(fill_ones_kernel, 1, 32, 0, st, (uint4 *)nullptr, 0ll, n_spans);
         return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
     }
-    if (intra) {     // the token table starts empty
-        p.trep = reinterpret_cast<int32_t *>(ws + Q.trep);
-        p.tfirst = reinterpret_cast<int32_t *>(ws + Q.tfirst);
+    p.intra = intra != 0;
+    if (intra && !query_in_one(n_query)) {     // the token table starts empty
+        p.tok = reinterpret_cast<unsigned int *>(ws + Q.tok);
         p.tmask = Q.Mq - 1;
-        const long long n16 = (long long)Q.Mq / 2;
-        launch_after(fill_ones_kernel, fill_blocks(n16), 256, 0, st, reinterpret_cast<uint4 *>(ws + Q.trep), n16, (int32_t *)nullptr);
+        const long long n16 = (long long)Q.Mq / 4;
+        launch_after(fill_ones_kernel, fill_blocks(n16), 256, 0, st, reinterpret_cast<uint4 *>(ws + Q.tok), n16, (int32_t *)nullptr);
+        p.ahead = 1;
     }
     launch_query(p, st);
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;

@@ -94,7 +94,7 @@ def _match(env, hist, query, w, K):
 @pytest.mark.parametrize("N,w,K", [(511, 4, 8), (512, 1, 3), (513, 4, 16), (4096, 5, 8), (4097, 4, 8), (1024 * 512 + 700, 4, 8),
                                    (1500, 3, 0)])
 def test_selection_at_chunk_edges(env, N, w, K):
-    """Query lengths at the edges of a chunk, of the chunks one kernel walks itself, and of the 1024 chunks that are resolved
+    """Query lengths at the edges of a chunk, of the chunks of one cluster, and of the 1024 chunks that are resolved
     together; spans of one token up to several chunks, some ending exactly at a chunk's end; sets of 3, 8 and 16 starts."""
     rng = np.random.default_rng(N + K)
     hist = rng.integers(0, 3, 3000).astype(np.int32)          # three tokens: every window occurs many times
@@ -131,6 +131,43 @@ def test_windows_that_occur_thousands_of_times(env):
         rows, spans = _match(env, hist, query, 4, K)
         o_rows, o_spans = env.orc.match_spans(hist, query, 4, K)
         assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
+
+
+@pytest.mark.parametrize("N,w,K,live", [(1, 1, 8, 0), (31, 32, 1, 0), (513, 3, 16, 0), (1537, 32, 3, 2000), (4096, 4, 8, 0),
+                                        (4097, 4, 8, 3300), (3000, 2, 0, 1000)])
+def test_index_and_token_table_at_cluster_edges(env, N, w, K, live):
+    """Prompts of one chunk up to the chunks of one cluster and one token more, with intra-sequence references (the table of
+    tokens in the cluster's shared memory or in global memory; tokens of every sign, among them -1), requests of all lengths,
+    whose ends cut matches off, and windows of one token up to 32.  Every result is exact."""
+    rac, dev = env.rac, env.dev
+    rng = np.random.default_rng(1000 + N)
+    hist = rng.integers(-40, 400, 6000).astype(np.int32)
+    cuts = np.unique(np.concatenate([[0, 6000], rng.integers(0, 6000, 12), [700, 701]])).astype(np.int32)
+    query = rng.integers(-300, 4000, N).astype(np.int32)
+    i = int(rng.integers(0, 9))
+    while i < N:
+        L = min(int(rng.choice([1, 9, 33, 300, 1300])), N - i)
+        j = int(rng.choice(cuts[:-1])) if rng.random() < 0.3 else int(rng.integers(0, 6000 - L + 1))
+        L = min(L, 6000 - j)
+        query[i:i + L] = hist[j:j + L]
+        i += L + int(rng.integers(0, 30))
+    cfg = rac.IndexCfg(6000, w, K)
+    nb, nws = rac.rac_index_bytes(cfg), rac.rac_index_query_workspace_bytes(N)
+    mem = torch.full((nb,), 0x5A, dtype=torch.uint8, device=dev)
+    ws = torch.full((nws + 16,), 0x5A, dtype=torch.uint8, device=dev)
+    h, q = torch.from_numpy(hist).to(dev), torch.from_numpy(query).to(dev)
+    rows = torch.full((N + 4,), 12345, dtype=torch.int32, device=dev)
+    spans = torch.full((N // w + 1, 3), 777, dtype=torch.int32, device=dev)
+    n = torch.full((1,), -5, dtype=torch.int32, device=dev)
+    rac.rac_index_reset(cfg, mem, nb)
+    for a, b in zip(cuts, cuts[1:]):
+        rac.rac_index_append(cfg, mem, nb, h, int(a), int(b))
+    for intra in (True, False):
+        rac.rac_index_query_live(cfg, mem, nb, h, 6000, live, q, N, intra, rows[:N], spans, n, ws[:nws], nws)
+        o_rows, o_spans = env.orc.match_spans_req(hist, cuts, query, w=w, max_hits=K, intra=intra, first_live=live)
+        assert np.array_equal(rows[:N].cpu().numpy(), o_rows)
+        assert np.array_equal(spans[:int(n.item())].cpu().numpy(), o_spans)
+    assert torch.all(rows[N:] == 12345) and torch.all(ws[nws:] == 0x5A)
 
 
 # ------------------------------------------------------------------------------- encode with outliers in one launch
