@@ -14,11 +14,12 @@
 //
 // All of it is bound by the latency of dependent trips to L2 and of launches, not by the bytes: the forms above were chosen
 // to make fewer of both, and every kernel lets the next one be set up while it runs.  32768 history and 2048 query tokens:
-// 20.5 us in three launches (52 us in nine before: sorted lists, a thread per match, a suffix scan and a serial walk; 23.5 us
-// with selection and emission in two launches and a test before every load of the extension), 131072 / 131072 tokens 40 us
+// 18 us in three launches (52 us in nine before: sorted lists, a thread per match, a suffix scan and a serial walk; 23.5 us
+// with selection and emission in two launches and a test before every load of the extension), 131072 / 131072 tokens 36 us
 // (99 us, 43.6 us), a query of 2048 tokens against an index of 16384 16 us (60 us, 22 us), with intra-sequence references 18.5 us
-// (28 us), eight appends of 2048 tokens behind a reset 39 us (54 us).  Of the query's 16 us, 9 are the slowest warp's
-// candidates: up to eight of them, one after another, two trips each.
+// (28 us), eight appends of 2048 tokens behind a reset 36 us (54 us;
+// 38 us in CTAs of 128 threads).  Of the query's 16 us, 9 are the slowest warp's candidates: up to eight of them, one after
+// another, two trips each.
 #include <cooperative_groups.h>
 
 #include <mutex>
@@ -118,37 +119,6 @@ __device__ __forceinline__ int find_in_bucket(const u64 (&e)[kBucket], uint32_t 
     return at;
 }
 
-// The representative start of the window that starts at history position j: the one its slot holds, or j itself after
-// claiming the first empty slot of the probe sequence.  Slots fill in probe order and are never emptied, so two threads with
-// the same window end at one slot.  The window's set of starts stands at the place of its representative in `top`.
-__device__ __forceinline__ int find_or_claim(u64 *slots, unsigned int bmask, const int32_t *hist, int j, const int32_t *win, int w,
-                                             u64 h) {
-    const uint32_t tag = (uint32_t)(h >> 32);
-    unsigned int b = (unsigned int)h & bmask, probes = 0;
-    u64 e[kBucket];
-    load_bucket(slots, b, e);
-    int from = 0;
-    while (probes <= bmask) {
-        u64 held;
-        const int s = find_in_bucket(e, tag, from, held);
-        if (s == kBucket) {                   // full of other windows: the next bucket
-            b = (b + 1) & bmask;
-            probes++;
-            load_bucket(slots, b, e);
-            from = 0;
-            continue;
-        }
-        u64 *at = slots + (size_t)b * kBucket + s;
-        if (held == kEmptySlot) {
-            held = atomicCAS(at, kEmptySlot, ((u64)tag << 32) | (uint32_t)j);
-            if (held == kEmptySlot) return j;
-        }
-        if ((uint32_t)(held >> 32) == tag && same_window(hist + (int)(uint32_t)held, win, w)) return (int)(uint32_t)held;
-        from = s + 1;
-    }
-    return -1;   // the table has four times as many slots as windows: not reached
-}
-
 // a set as the L2 holds it, `none` beyond its K entries
 __device__ __forceinline__ void load_set(const int32_t *set, int K, int none, int (&v)[16]) {
 #pragma unroll
@@ -164,41 +134,92 @@ __device__ __forceinline__ void load_set(const int32_t *set, int K, int none, in
     }
 }
 
-// Start j enters a window's set of the K largest starts (-1 = empty entry): it takes the place of the smallest entry, by
-// compare-and-swap, until that succeeds or every entry is larger.  Entries only grow, so what a thread has seen of an entry is
-// never more than it holds: a value is replaced only when K larger ones exist, and j gives up only when K larger ones exist.
-// The set ends as the K largest values ever offered, whatever the interleaving; the order of its entries is of no meaning.
-// One look at the set and one swap are two trips to L2 (a sorted list, kept by a cascade of atomicMax, cost up to K).
-__device__ __forceinline__ void set_insert(int32_t *set, int K, int j) {
-    int v[16];
-    load_set(set, K, 0x7fffffff, v);
-    while (true) {
-        int low = v[0], at = 0;
-        unsigned int empty = 0;
+// Start c enters a window's set of the K largest starts (-1 = empty entry).  An atomicMax puts it into one entry, and the smaller
+// of it and what stood there is carried on, until that is -1 or every entry is larger.  Entries only grow, so what a thread has
+// seen of an entry is never more than it holds, and a value is dropped only when K larger ones exist: the set ends as the K
+// largest values ever offered, whatever the interleaving; the order of its entries is of no meaning.  Every swap either puts a
+// value in or shows an entry that the value need not try again.
+// The first swap goes to an entry picked by position, together with the look at the set: one trip for a window that occurs once,
+// as most do, and threads with the same window at different entries.  (Look, then compare-and-swap of the smallest entry: two
+// trips, and one winner per trip among such threads.  131072 tokens hold one window 65
+// times: 40.7 us for the match, 35.7 so; 32768 tokens 20.5 and 17.9.)
+__device__ __forceinline__ void set_insert(int32_t *set, int K, int c) {
+    const unsigned int first = (unsigned int)c % (unsigned int)K, behind = ~((1u << first) - 1u);
+    int at = (int)first;
+    for (bool spread = false;; spread = true) {
+        const int old = atomicMax(&set[at], c);
+        int v[16];
+        load_set(set, K, 0x7fffffff, v);
+        if (old < 0) return;
+        const int held = max(old, c);
+        c = min(old, c);
+        int low = 0x7fffffff, low_at = 0;
+        unsigned int empty = 0, less = 0;
 #pragma unroll
         for (int r = 0; r < 16; r++) {
-            if (v[r] < low) { low = v[r]; at = r; }
-            empty |= v[r] < 0 ? (1u << r) : 0u;
+            const int x = r == at ? held : v[r];
+            if (x < low) { low = x; low_at = r; }
+            empty |= x < 0 ? (1u << r) : 0u;
+            less |= x < c ? (1u << r) : 0u;
         }
-        if (empty) {              // threads with the same window start at different empty entries
-            const unsigned int later = empty & ~((1u << (j % K)) - 1u);
-            at = __ffs(later ? later : empty) - 1;
+        if (!less) return;
+        at = low_at;
+        if (empty | (spread ? less : 0u)) {      // several threads are at this set: each at an entry of its own
+            const unsigned int m = empty ? empty : less;
+            at = __ffs(m & behind ? m & behind : m) - 1;
         }
-        if (low > j) return;
-        const int found = atomicCAS(&set[at], low, j);
-        if (found == low) return;
-#pragma unroll
-        for (int r = 0; r < 16; r++) v[r] = r == at ? found : v[r];
     }
 }
-// Start j enters the index.  Unlimited hits: every start goes onto its window's chain.  The order of a chain
-// depends on which thread came first; the query looks at ALL of it and keeps lexargmax(length, start), so the result does not.
+// Start j enters the index, h = the hash of its window `win`.  Its window's slot holds a representative start; the first empty slot
+// of the probe sequence is claimed where there is none.  Slots fill in probe order and are never emptied, so two threads with the
+// same window end at one slot.  The window's set of starts stands at the place of its representative in `top`.
+// A claim goes out together with j's place in the set that j heads if the claim succeeds (else nobody reads that set), and beside
+// the verification of the lanes that found a slot taken: a window that occurs once, as most do, is the trip for its bucket and
+// one more.  (One after another 18.4 us for a match of 32768 tokens, so 17.9.)
+// Unlimited hits: every start goes onto its window's chain.  The order of a chain depends on which thread came first; the query
+// looks at ALL of it and keeps lexargmax(length, start), so the result does not.
 __device__ __forceinline__ void index_start(u64 *slots, int32_t *top, int32_t *next, unsigned int bmask, const int32_t *hist,
                                             int j, const int32_t *win, int w, int K, u64 h) {
-    const int rep = find_or_claim(slots, bmask, hist, j, win, w, h);
-    if (rep < 0) return;
+    const uint32_t tag = (uint32_t)(h >> 32);
+    unsigned int b = (unsigned int)h & bmask, probes = 0;
+    u64 e[kBucket];
+    load_bucket(slots, b, e);
+    int from = 0, rep = -1, carry = j, old = -1;
+    bool placed = next != nullptr;
+    while (probes <= bmask) {     // (the table has four times as many slots as windows: ends before)
+        u64 held;
+        const int s = find_in_bucket(e, tag, from, held);
+        if (s == kBucket) {                   // full of other windows: the next bucket
+            b = (b + 1) & bmask;
+            probes++;
+            load_bucket(slots, b, e);
+            from = 0;
+            continue;
+        }
+        const bool claim = held == kEmptySlot;
+        u64 found = kEmptySlot;
+        if (claim) {
+            found = atomicCAS(slots + (size_t)b * kBucket + s, kEmptySlot, ((u64)tag << 32) | (uint32_t)j);
+            if (!placed) {      // once: from then on the value is in the set, wherever others may have moved it
+                old = atomicMax(&top[(size_t)j * K + (unsigned int)j % (unsigned int)K], j);
+                placed = true;
+            }
+        }
+        const int r = claim ? j : (int)(uint32_t)held;
+        const bool same = same_window(hist + r, win, w);
+        if (claim && found != kEmptySlot) {   // another thread was faster: look at what it put there
+#pragma unroll
+            for (int u = 0; u < kBucket; u++) e[u] = u == s ? found : e[u];
+            from = s;
+        } else if (same) {
+            rep = r;
+            if (claim && !next) carry = min(old, j);
+            break;
+        } else from = s + 1;
+    }
+    if (rep < 0 || carry < 0) return;
     if (next) next[j] = atomicExch(&top[rep], j);
-    else set_insert(top + (size_t)rep * K, K, j);
+    else set_insert(top + (size_t)rep * K, K, carry);
 }
 
 // All ones in n16 pieces of 16 bytes; with zero, also *zero = 0.  The kernel after it may begin once the work before this call
@@ -696,7 +717,7 @@ struct IndexParams {
 // Appending a request: every position learns the end of its request; every window of the request finds or claims
 // its slot and enters the slot's set.  The request's starts are larger than everything already there, so the oldest
 // entries fall out as a by-product.  One launch, any request size.
-__global__ void __launch_bounds__(128) index_append_kernel(const IndexParams p) {
+__global__ void __launch_bounds__(64) index_append_kernel(const IndexParams p) {
     grid_launch_dependents();
     grid_dependency_wait();
     const int j = p.b - 1 - (int)(blockIdx.x * blockDim.x + threadIdx.x);   // the latest starts first
@@ -961,7 +982,7 @@ int rac_index_append(const rac_index_cfg *cfg, void *index, size_t index_bytes, 
     p.w = cfg->min_ngram;
     p.K = cfg->max_hits > 0 ? cfg->max_hits : 1;
     p.bmask = L.M / kBucket - 1;
-    launch_after(index_append_kernel, (unsigned)((n_after - n_before + 127) / 128), 128, 0, static_cast<cudaStream_t>(stream), p);
+    launch_after(index_append_kernel, (unsigned)((n_after - n_before + 63) / 64), 64, 0, static_cast<cudaStream_t>(stream), p);
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
 }
 
