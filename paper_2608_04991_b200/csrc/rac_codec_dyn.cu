@@ -747,8 +747,22 @@ __global__ void __launch_bounds__(256) decode_dyn_kernel(const CodecParams p) {
 // outliers only below 8-bit codes.
 template <int B, bool X, int K>
 static int launch_encode_variant(bool tight, const Geometry &g, CodecParams &p, int smem, long long max_ctas, cudaStream_t stream) {
-    if (p.tok_list || p.intra_base || p.coef_ext)   // the subset form: one variant, not the hot path
+    if (p.tok_list || p.intra_base || p.coef_ext) {
+        // The subset form: groups of 128 channels compiled in, with the width where few outliers are usual.  (The two waves of
+        // 2048 x 4096, one or two outliers per group, encode with x_hat and decode: 36.8 and 40.9 us with nothing compiled in,
+        // 34.4 and 37.5 with the groups, 33.0 and 36.0 with the width.)
+        if constexpr (B == 4 || B == 8) {
+            if constexpr (K <= 2) {
+                if (g.d == 5120 && g.lpg == 4 && g.lpq == 4)
+                    return launch_persistent(encode_dyn_kernel<B, X, K, 2, true, 4, 5120>, p, g.nthreads, smem, max_ctas, stream);
+                if (g.d == 4096 && g.lpg == 4 && g.lpq == 4)
+                    return launch_persistent(encode_dyn_kernel<B, X, K, 2, true, 4, 4096>, p, g.nthreads, smem, max_ctas, stream);
+            }
+            if (g.lpg == 4 && g.lpq == 4)
+                return launch_persistent(encode_dyn_kernel<B, X, K, 2, true, 4>, p, g.nthreads, smem, max_ctas, stream);
+        }
         return launch_persistent(encode_dyn_kernel<B, X, K, 2, true>, p, g.nthreads, smem, max_ctas, stream);
+    }
     // the paper's code widths (4 and 8 bits) at widths 5120 and 4096 with groups of 128 channels (alignment and
     // quantisation alike) run variants with those compiled in
     if constexpr (B == 4 || B == 8) {
@@ -814,14 +828,17 @@ int launch_decode_dyn(const Geometry &g, CodecParams &p, cudaStream_t stream) {
     const DecSmem L = dec_smem_layout(g.d, g.rec, p.stages);
     const bool kg = g.topk_group > 0;
     const bool sub = p.tok_list || p.intra_base || p.coef_ext;
-    const bool spec = g.d == 5120 && g.lpg == 4 && g.lpq == 4;   // width and groups of 128 compiled in
+    // groups of 128 channels compiled in, with the widths 4096 and 5120 (16384 x 4096, 4-bit, one outlier per group: 53.7 us with
+    // nothing compiled in, 49.5 so)
+    const bool g128 = g.lpg == 4 && g.lpq == 4;
+#define RAC_DYN_DECK(B, K, S) \
+    (!g128 ? launch_persistent(decode_dyn_kernel<B, K, S>, p, g.nthreads, L.total, p.T, stream) \
+     : g.d == 5120 ? launch_persistent(decode_dyn_kernel<B, K, S, 4, 5120>, p, g.nthreads, L.total, p.T, stream) \
+     : g.d == 4096 ? launch_persistent(decode_dyn_kernel<B, K, S, 4, 4096>, p, g.nthreads, L.total, p.T, stream) \
+                   : launch_persistent(decode_dyn_kernel<B, K, S, 4>, p, g.nthreads, L.total, p.T, stream))
 #define RAC_DYN_DEC(B) \
-    (sub ? (kg ? launch_persistent(decode_dyn_kernel<B, true, true>, p, g.nthreads, L.total, p.T, stream) \
-               : launch_persistent(decode_dyn_kernel<B, false, true>, p, g.nthreads, L.total, p.T, stream)) \
-     : spec ? (kg ? launch_persistent(decode_dyn_kernel<B, true, false, 4, 5120>, p, g.nthreads, L.total, p.T, stream) \
-                  : launch_persistent(decode_dyn_kernel<B, false, false, 4, 5120>, p, g.nthreads, L.total, p.T, stream)) \
-         : (kg ? launch_persistent(decode_dyn_kernel<B, true, false>, p, g.nthreads, L.total, p.T, stream) \
-               : launch_persistent(decode_dyn_kernel<B, false, false>, p, g.nthreads, L.total, p.T, stream)))
+    (sub ? (kg ? RAC_DYN_DECK(B, true, true) : RAC_DYN_DECK(B, false, true)) \
+         : (kg ? RAC_DYN_DECK(B, true, false) : RAC_DYN_DECK(B, false, false)))
     switch (g.bits) {
         case 8: return RAC_DYN_DEC(8);
         case 4: return RAC_DYN_DEC(4);
@@ -829,6 +846,7 @@ int launch_decode_dyn(const Geometry &g, CodecParams &p, cudaStream_t stream) {
         case 2: return RAC_DYN_DEC(2);
     }
 #undef RAC_DYN_DEC
+#undef RAC_DYN_DECK
     return RAC_EUNSUPPORTED;
 }
 

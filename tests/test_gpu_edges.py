@@ -203,3 +203,43 @@ def test_one_launch_outliers_at_shape_edges(env, d, g, bits, k, T):
     assert st == 0 and np.array_equal(pay, pay2)
     o_x = orc.reconstruct(d, g, bits, k, pay, T, ref_base=s.bf16_bits(R), ref_row=rows, step=step, nthreads=orc.max_threads())
     assert np.array_equal(o_x.reshape(-1), s.bf16_bits(xs).reshape(-1))
+
+
+# ------------------------------------------------------------------------------- token lists, one scale per group
+@pytest.mark.parametrize("d,bits,kg,T", [(4096, 4, 1, 700), (4096, 8, 2, 40), (5120, 4, 0, 700), (5120, 8, 1, 33), (3072, 4, 4, 50),
+                                         (4096, 4, 3, 5)])
+def test_listed_tokens_at_compiled_in_widths(env, d, bits, kg, T):
+    """Two lists in random order, together all tokens: the widths and outlier counts that are compiled in, one beyond each, one
+    token per CTA and several.  The records meet the oracle's, x_hat of both sides is the oracle's reconstruction of them."""
+    s, rac, orc, dev, P = env.synth, env.rac, env.orc, env.dev, env.P
+    gen = s.generator(T, dev)
+    X = s.activations(T, d, s.channel_scale(d, 3, dev), gen)
+    R = s.affine_noisy_reference(X, 128, gen)
+    rng = np.random.default_rng(T)
+    rows = np.arange(T, dtype=np.int32)
+    rows[rng.random(T) < 0.2] = -1
+    order = rng.permutation(T).astype(np.int32)
+    cut = T // 3
+    cfg = rac.CodecCfg(d, 128, bits, 0, scale_mode=1, topk_group=kg)
+    rec = rac.rac_record_bytes(cfg)
+    rows_d, st = torch.from_numpy(rows).to(dev), torch.zeros(1, dtype=torch.int32, device=dev)
+    pay = torch.full((T * rec,), 0xA5, dtype=torch.uint8, device=dev)
+    xs, xr = (torch.full((T, d), -7.0, dtype=torch.bfloat16, device=dev) for _ in range(2))
+    lists = []
+    for part in (order[:cut], order[cut:]):
+        lst = torch.from_numpy(part).to(dev) if part.size else torch.zeros(1, dtype=torch.int32, device=dev)
+        lists.append((lst, torch.tensor([part.size], dtype=torch.int32, device=dev)))
+    nws = rac.rac_encode_workspace_bytes(cfg, T)
+    ws = torch.empty(max(nws, 16), dtype=torch.uint8, device=dev)
+    for lst, cnt in lists:
+        rac.rac_encode_reconstruct_list(cfg, X, T, lst, cnt, R, T, rows_d, None, 0, None, None, None, None, pay, T * rec, xs,
+                                        ws if nws else None, nws, st)
+    for lst, cnt in lists:
+        rac.rac_decode_reconstruct_list(cfg, pay, T, lst, cnt, R, T, rows_d, None, 0, None, None, None, xr, st)
+    assert int(st.item()) == 0
+    p = pay.cpu().numpy()
+    P.compare_encode(cfg, p, s.bf16_bits(X), s.bf16_bits(R), rows)
+    o_x = orc.reconstruct(d, 128, bits, 0, p, T, ref_base=s.bf16_bits(R), ref_row=rows, nthreads=orc.max_threads(), scale_mode=1,
+                          topk_group=kg)
+    for x in (xs, xr):
+        assert np.array_equal(o_x.reshape(-1), s.bf16_bits(x).reshape(-1))
