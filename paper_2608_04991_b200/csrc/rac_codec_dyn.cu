@@ -414,6 +414,14 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_dyn_kernel
 #pragma unroll
                 for (int j = 0; j < 4; j++) {
                     uint32_t t8[8], xh[4];
+                    if constexpr (XHAT && MINB == 4) {     // the reference once more: 16 registers less over the outlier rounds
+                        if (has_ref) {
+                            const uint4 w = load_ref_words(rs + off[j], p.gain, p.bias, (int)(off[j] >> 1));
+                            rw[4 * j + 0] = w.x; rw[4 * j + 1] = w.y; rw[4 * j + 2] = w.z; rw[4 * j + 3] = w.w;
+                        } else {
+                            rw[4 * j + 0] = rw[4 * j + 1] = rw[4 * j + 2] = rw[4 * j + 3] = 0u;
+                        }
+                    }
 #pragma unroll
                     for (int i = 0; i < 4; i++) {
                         u64 vv = pmul(e2[4 * j + i], inv2);
@@ -743,8 +751,12 @@ __global__ void __launch_bounds__(256) decode_dyn_kernel(const CodecParams p) {
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
-// The 96-register variant (four 160-thread CTAs per SM) exists where it does not spill: without x_hat, and with
-// outliers only below 8-bit codes.
+// The 96-register variant (four 160-thread CTAs per SM, five of 128 threads) exists where it does not spill and more warps pay:
+// without x_hat (with outliers only below 8-bit codes) and, reading the reference a second time, with x_hat in calls of many
+// tokens whose chains are long.  128 against 96 registers: 20001 x 5120, 4-bit, one, two and four outliers per group 128 / 122,
+// 158 / 150 and 228 / 219 us, but none 87 / 88, and up to two rounds of three CTAs per SM 300 tokens 5.4 / 6.3, 800 tokens
+// 7.5 / 7.9, 1000 tokens 11.4 / 10.7; 4096 channels, 8-bit, no outliers, 16384 tokens 82 / 74, 9000 43.5 / 42.8, 7000 33.9 / 34.7,
+// but 8-bit with one outlier 82 / 88 and 4-bit with none or one 69 / 71 and 81 / 83.
 template <int B, bool X, int K>
 static int launch_encode_variant(bool tight, const Geometry &g, CodecParams &p, int smem, long long max_ctas, cudaStream_t stream) {
     if (p.tok_list || p.intra_base || p.coef_ext) {
@@ -763,17 +775,27 @@ static int launch_encode_variant(bool tight, const Geometry &g, CodecParams &p, 
         }
         return launch_persistent(encode_dyn_kernel<B, X, K, 2, true>, p, g.nthreads, smem, max_ctas, stream);
     }
+    DeviceInfo di;
+    if (int rc = device_info(&di)) return rc;
+    const int sms = di.sms;
     // the paper's code widths (4 and 8 bits) at widths 5120 and 4096 with groups of 128 channels (alignment and
     // quantisation alike) run variants with those compiled in
     if constexpr (B == 4 || B == 8) {
         if (g.d == 5120 && g.lpg == 4 && g.lpq == 4) {
-            if constexpr (!X && (K == 0 || B != 8))
-                return launch_persistent(encode_dyn_kernel<B, X, K, 4, false, 4, 5120>, p, g.nthreads, smem, max_ctas, stream);
-            else
+            if constexpr (X ? K >= 1 && B != 8 : K == 0 || B != 8) {
+                if (!X || p.T > 6ll * sms)
+                    return launch_persistent(encode_dyn_kernel<B, X, K, 4, false, 4, 5120>, p, g.nthreads, smem, max_ctas, stream);
+            }
+            if constexpr (X || (K != 0 && B == 8))
                 return launch_persistent(encode_dyn_kernel<B, X, K, 2, false, 4, 5120>, p, g.nthreads, smem, max_ctas, stream);
         }
-        if (g.d == 4096 && g.lpg == 4 && g.lpq == 4)
+        if (g.d == 4096 && g.lpg == 4 && g.lpq == 4) {
+            if constexpr (X && K == 0 && B == 8) {
+                if (p.T > 54ll * sms)
+                    return launch_persistent(encode_dyn_kernel<B, X, K, 4, false, 4, 4096>, p, g.nthreads, smem, max_ctas, stream);
+            }
             return launch_persistent(encode_dyn_kernel<B, X, K, 2, false, 4, 4096>, p, g.nthreads, smem, max_ctas, stream);
+        }
         if constexpr (K == 0) {   // the paper's decode mode: one scale per token
             if (g.lpg == 4 && g.lpq == 0 && g.qgen == 0) {
                 if (g.d == 5120) {

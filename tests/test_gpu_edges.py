@@ -243,3 +243,18 @@ def test_listed_tokens_at_compiled_in_widths(env, d, bits, kg, T):
                           topk_group=kg)
     for x in (xs, xr):
         assert np.array_equal(o_x.reshape(-1), s.bf16_bits(x).reshape(-1))
+
+
+@pytest.mark.parametrize("d,bits,kg,T,predictor", [(5120, 4, 1, 900, True), (5120, 4, 2, 889, False), (5120, 4, 8, 888, False),
+                                                   (4096, 8, 0, 8000, False)])
+def test_group_scales_in_calls_of_many_tokens(env, d, bits, kg, T, predictor):
+    """Encode with x_hat past the token counts where it reads the reference a second time (and at the last one where it does
+    not): direct tokens, a predictor's gain and bias on the reference, several tokens per CTA."""
+    s, rac, P = env.synth, env.rac, env.P
+    gen = s.generator(d + kg, env.dev)
+    X = s.activations(T, d, s.channel_scale(d, 4, env.dev), gen)
+    R = s.affine_noisy_reference(X, 128, gen)
+    rows = torch.arange(T, dtype=torch.int32, device=env.dev)
+    rows[::7] = -1
+    gain, bias = s.predictor_gain_bias(d, 4, env.dev) if predictor else (None, None)
+    P.round_trip_case(rac.CodecCfg(d, 128, bits, 0, scale_mode=1, topk_group=kg), X, R, rows, gain, bias)
