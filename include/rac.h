@@ -199,7 +199,7 @@ int rac_match_spans_static(const int32_t *hist_tok, int64_t n_hist, const int32_
  *                      workspace >= rac_index_query_workspace_bytes(n_query) bytes, scratch.
  * The index only grows.  Old requests are dropped from the RESULTS at no cost with rac_index_query_live (below);
  * to reclaim their memory, reset the index and append the requests that are kept (appending 131072 tokens as 64
- * requests takes about 0.7 ms on a B200), or alternate between two indices.
+ * requests takes about 0.3 ms on a B200), or alternate between two indices.
  * All three are asynchronous on `stream`; calls on one index must be ordered. */
 typedef struct {
     int64_t capacity;      /* history tokens the index can hold, 1 .. 2^30 - 1 */
