@@ -15,11 +15,10 @@
 // All of it is bound by the latency of dependent trips to L2 and of launches, not by the bytes: the forms above were chosen
 // to make fewer of both, and every kernel lets the next one be set up while it runs.  32768 history and 2048 query tokens:
 // 18 us in three launches (52 us in nine before: sorted lists, a thread per match, a suffix scan and a serial walk; 23.5 us
-// with selection and emission in two launches and a test before every load of the extension), 131072 / 131072 tokens 36 us
-// (99 us, 43.6 us), a query of 2048 tokens against an index of 16384 16 us (60 us, 22 us), with intra-sequence references 18.5 us
-// (28 us), eight appends of 2048 tokens behind a reset 36 us (54 us;
-// 38 us in CTAs of 128 threads).  Of the query's 16 us, 9 are the slowest warp's candidates: up to eight of them, one after
-// another, two trips each.
+// with selection and emission in two launches and a test before every load of the extension), 131072 / 131072 tokens 35.5 us
+// (99 us, 43.6 us), a query of 2048 tokens against an index of 16384 12 us (60 us, 22 us), with intra-sequence references 14.3 us
+// (28 us), eight appends of 2048 tokens behind a reset 36 us (54 us; 38 us in CTAs of 128 threads).  Of the query's 12 us, 5 are
+// the slowest warp's candidates: up to eight of them, two at a time, two trips each (one at a time 9 of 16 us).
 #include <cooperative_groups.h>
 
 #include <mutex>
@@ -354,7 +353,7 @@ __device__ __forceinline__ void emit_chunk(const MatchParams &p, EmitSmem &m, in
 
 // Lookup, extension, and the chunk's jumps.  One CTA per chunk, one thread per position.
 // Extension: a thread compares eight tokens at its candidate by itself; what is still open after that is finished by the
-// warp, 256 tokens per trip.  Neighbouring positions inside one copied stretch have the same (history - query) distance and
+// warp, 256 tokens per trip, or 128 each at two distances.  Neighbouring positions inside one copied stretch have the same (history - query) distance and
 // so the same end: one comparison closes them all.  A thread by itself took a trip per eight tokens, for every position
 // of a long match (2048-token prompt: 21 us, with copies of copies 55 us).
 // ONE: the chunks are the CTAs of one cluster, which hands out spans and rows as well: a cluster barrier and jumps read from the
@@ -413,58 +412,98 @@ __global__ void __launch_bounds__(kChunk, ONE ? 1 : 2) match_query_kernel(const 
         }
     }
     int bestL = 0, bestj = -1;
-    // One candidate per lane (j = -1: none), all lanes of the warp together.  It replaces the best so far only with a longer match,
-    // or with one as long and a larger start, so its token at has_to_match has to be equal.  That token, the first eight behind
-    // the window and the end of the request come in one trip (no test stands before a load: it would make a trip of each).
+    // Up to two candidates per lane (-1: none), all lanes of the warp together.  One replaces the best so far only with a longer
+    // match, or with one as long and a larger start, so its token at has_to_match has to be equal.  That token, the first eight
+    // behind the window and the end of the request come in one trip (no test stands before a load: it would make a trip of each).
+    // What is still open goes on to the extension, two distances at a time, one per half of the warp.
     auto has_to_match = [&](int j) { return max(bestL - (j > bestj ? 1 : 0), 0); };
-    auto consider = [&](int j) {
+    struct Candidate {
+        int j, L, room;
+        bool can_win, open;
+    };
+    auto begin = [&](int j) {
         const int jj = max(j, 0), at = has_to_match(j);
         int32_t hh[8];
 #pragma unroll
         for (int u = 0; u < 8; u++) hh[u] = p.hist[min(jj + p.w + u, p.n_hist - 1)];
         const int32_t h_at = p.hist[min(jj + at, p.n_hist - 1)], q_at = p.query[min(i + at, N - 1)];
         const int end_j = p.end_of ? p.end_of[jj] : p.n_hist;
-        const int room = min(N - i, end_j - jj);          // the longest the match can be, inside its request
+        Candidate c;
+        c.j = j;
+        c.room = min(N - i, end_j - jj);          // the longest the match can be, inside its request
         uint32_t ne = 0;
 #pragma unroll
         for (int u = 0; u < 8; u++) ne |= win[p.w + u] != hh[u] ? (1u << u) : 0u;
-        const bool can_win = j >= 0 && (bestL == 0 || (at < room && h_at == q_at));
-        int L = min(p.w + (ne ? __ffs(ne) - 1 : 8), room);
-        bool open = can_win && ne == 0u && p.w + 8 < room;
-        unsigned int todo = __ballot_sync(0xffffffffu, open);
-        while (todo) {
-            const int lead = __ffs(todo) - 1;
-            const int i0 = __shfl_sync(0xffffffffu, i, lead), j0 = __shfl_sync(0xffffffffu, j, lead);
-            const int L0 = __shfl_sync(0xffffffffu, L, lead), room0 = __shfl_sync(0xffffffffu, room, lead);
-            int len = L0;
+        c.can_win = j >= 0 && (bestL == 0 || (at < c.room && h_at == q_at));
+        c.L = min(p.w + (ne ? __ffs(ne) - 1 : 8), c.room);
+        c.open = c.can_win && ne == 0u && p.w + 8 < c.room;
+        return c;
+    };
+    auto consider = [&](int j1, int j2) {
+        Candidate c = begin(j1), e = begin(ONE ? j2 : -1);
+        while (true) {
+            const unsigned int mc = __ballot_sync(0xffffffffu, c.open), me = ONE ? __ballot_sync(0xffffffffu, e.open) : 0u;
+            if (!(mc | me)) break;
+            const int la = __ffs(mc ? mc : me) - 1;
+            const int da = __shfl_sync(0xffffffffu, (mc ? c.j : e.j) - i, la);
+            const unsigned int oc = __ballot_sync(0xffffffffu, c.open && c.j - i != da);
+            const unsigned int oe = ONE ? __ballot_sync(0xffffffffu, e.open && e.j - i != da) : 0u;
+            const int lb = oc | oe ? __ffs(oc ? oc : oe) - 1 : la;
+            const bool a_is_c = mc != 0u, b_is_c = oc | oe ? oc != 0u : a_is_c;
+            const bool mine_c = lane < 16 ? a_is_c : b_is_c;      // which of its lead's candidates this half extends
+            const int lead = lane < 16 ? la : lb;
+            const int jc = __shfl_sync(0xffffffffu, c.j, lead), je = ONE ? __shfl_sync(0xffffffffu, e.j, lead) : 0;
+            const int rc = __shfl_sync(0xffffffffu, c.room, lead), re = ONE ? __shfl_sync(0xffffffffu, e.room, lead) : 0;
+            const int i0 = __shfl_sync(0xffffffffu, i, lead), j0 = mine_c ? jc : je, room0 = mine_c ? rc : re;
+            // one distance only: the second half takes the tokens behind the first half's (131072 query tokens 37.5 -> 35.7 us; in
+            // the cluster's form it cost the query 4 of 16 us)
+            const bool one = !ONE && !(oc | oe);
+            const int mine = (lane & 15) + (one && lane >= 16 ? 128 : 0), step = one ? 256 : 128;
+            int len = p.w + 8;
             bool more = true;
-            while (more && len < room0) {
-                // (every load is made, at the last token inside where the lane is beyond: a test before each makes a trip of each)
+            while (__any_sync(0xffffffffu, more)) {
                 int32_t q[8], hh[8];
-                uint32_t differ = 0;                   // bit u: the lane's token of the u-th 32 differs or lies outside
 #pragma unroll
                 for (int u = 0; u < 8; u++) {
-                    const int at = min(len + 32 * u + lane, room0 - 1);
+                    const int at = min(len + 16 * u + mine, room0 - 1);
                     q[u] = p.query[i0 + at];
                     hh[u] = p.hist[j0 + at];
                 }
+                int first = 0x7fffffff;              // this lane's first position that differs or lies outside
 #pragma unroll
-                for (int u = 0; u < 8; u++) differ |= (len + 32 * u + lane >= room0 || q[u] != hh[u]) ? (1u << u) : 0u;
-#pragma unroll
-                for (int u = 0; u < 8; u++) {
-                    const unsigned int b = __ballot_sync(0xffffffffu, (differ >> u) & 1u);
-                    if (more) {
-                        if (b) { len += __ffs(b) - 1; more = false; }
-                        else len += 32;
-                    }
+                for (int u = 7; u >= 0; u--) {
+                    const int at = len + 16 * u + mine;
+                    first = at >= room0 || q[u] != hh[u] ? at : first;
+                }
+                const int fa = __reduce_min_sync(0xffffffffu, lane < 16 ? first : 0x7fffffff);
+                const int fb = __reduce_min_sync(0xffffffffu, lane < 16 ? 0x7fffffff : first);
+                const int f = one ? min(fa, fb) : lane < 16 ? fa : fb;
+                if (more) {
+                    more = f == 0x7fffffff;
+                    len = more ? len + step : f;
                 }
             }
             // every open position of the same distance that lies before the end has the same end
-            const int stop = i0 + len;
-            if (open && j - i == j0 - i0 && i < stop) { L = stop - i; open = false; }
-            todo = __ballot_sync(0xffffffffu, open);
+            const int sa = __shfl_sync(0xffffffffu, i0 + len, 0), sb = __shfl_sync(0xffffffffu, i0 + len, 16);
+            const int db = __shfl_sync(0xffffffffu, j0 - i0, 16);
+            auto close = [&](Candidate &x) {
+                const int d = x.j - i, stop = d == da ? sa : sb;
+                if (x.open && (d == da || d == db) && i < stop) {
+                    x.L = stop - i;
+                    x.open = false;
+                }
+            };
+            close(c);
+            if (ONE) close(e);
         }
-        if (can_win && (L > bestL || (L == bestL && j > bestj))) { bestL = L; bestj = j; }
+        auto keep = [&](const Candidate &x) {
+            if (x.can_win && (x.L > bestL || (x.L == bestL && x.j > bestj))) {
+                bestL = x.L;
+                bestj = x.j;
+            }
+        };
+        keep(c);
+        if (ONE) keep(e);
     };
     if (p.next) {
         // every occurrence of the window (at most nwin of them: the walk is bounded by construction)
@@ -474,7 +513,7 @@ __global__ void __launch_bounds__(kChunk, ONE ? 1 : 2) match_query_kernel(const 
             const int j = n < p.nwin ? chain : -1;
             if (!__any_sync(0xffffffffu, j >= 0)) break;
             if (j >= 0) { chain = p.next[j]; n++; }
-            consider(j);
+            consider(j, -1);
         }
     } else {
         // The K most recent starts.  After the first candidate, one trip for all the others rules most of them out (the end of
@@ -484,14 +523,18 @@ __global__ void __launch_bounds__(kChunk, ONE ? 1 : 2) match_query_kernel(const 
         for (int r = 0; r < 16; r++) v[r] = v[r] >= p.first_live ? v[r] : -1;     // first_live >= 0: no empty ones
         bool first = true;
         while (true) {
-            // largest start first: neighbours inside one copied stretch then look at the same distance at the same time
-            int j = v[0];
+            // largest starts first: neighbours inside one copied stretch then look at the same distances at the same time
+            auto take = [&]() {
+                int j = v[0];
 #pragma unroll
-            for (int r = 1; r < 16; r++) j = max(j, v[r]);
+                for (int r = 1; r < 16; r++) j = max(j, v[r]);
+#pragma unroll
+                for (int r = 0; r < 16; r++) v[r] = v[r] == j ? -1 : v[r];
+                return j;
+            };
+            const int j = take();
             if (!__any_sync(0xffffffffu, j >= 0)) break;
-#pragma unroll
-            for (int r = 0; r < 16; r++) v[r] = v[r] == j ? -1 : v[r];
-            consider(j);
+            consider(j, ONE ? take() : -1);
             if (first && bestL > 0) {
                 const int32_t q_last = p.query[i + bestL - 1], q_beyond = p.query[min(i + bestL, N - 1)];
 #pragma unroll
