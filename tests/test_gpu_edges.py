@@ -205,6 +205,24 @@ def test_one_launch_outliers_at_shape_edges(env, d, g, bits, k, T):
     assert np.array_equal(o_x.reshape(-1), s.bf16_bits(xs).reshape(-1))
 
 
+@pytest.mark.parametrize("T", [0, 1, 31, 128, 4095, 4096, 4097, 12289, 131072, 128 * 4096 + 1])
+def test_split_waves_at_range_edges(env, T):
+    """One token up to more ranges than CTAs; mixed rows, all of one wave, and a first row that only the last token reaches."""
+    rac, dev = env.rac, env.dev
+    rng = np.random.default_rng(T)
+    rows = rng.integers(-1, 2000, max(T, 1)).astype(np.int32)
+    rows[-1] = 2 ** 31 - 1
+    rows_d = torch.from_numpy(rows).to(dev)
+    for first in (1000, 0, 2 ** 31 - 1):
+        w1, w2 = (torch.full((T + 1,), -9, dtype=torch.int32, device=dev) for _ in range(2))
+        n = torch.full((2,), -5, dtype=torch.int32, device=dev)
+        rac.rac_split_waves(rows_d, T, first, w1, w2, n)
+        o1, o2 = np.flatnonzero(rows[:T] < first), np.flatnonzero(rows[:T] >= first)
+        assert n.tolist() == [o1.size, o2.size]
+        assert np.array_equal(w1[:o1.size].cpu().numpy(), o1) and np.array_equal(w2[:o2.size].cpu().numpy(), o2)
+        assert torch.all(w1[o1.size:] == -9) and torch.all(w2[o2.size:] == -9)
+
+
 # ------------------------------------------------------------------------------- token lists, one scale per group
 @pytest.mark.parametrize("d,bits,kg,T", [(4096, 4, 1, 700), (4096, 8, 2, 40), (5120, 4, 0, 700), (5120, 8, 1, 33), (3072, 4, 4, 50),
                                          (4096, 4, 3, 5)])
