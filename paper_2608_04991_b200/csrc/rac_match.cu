@@ -442,14 +442,17 @@ __global__ void __launch_bounds__(kChunk, ONE ? 1 : 2) match_query_kernel(const 
     auto consider = [&](int j1, int j2) {
         Candidate c = begin(j1), e = begin(ONE ? j2 : -1);
         while (true) {
+            // The leads: the lowest lane with an open candidate, and the lowest with one at another distance.  A lane's second
+            // candidate counts as its first does: nobody below a lead may be open at the lead's distance (see close()).
             const unsigned int mc = __ballot_sync(0xffffffffu, c.open), me = ONE ? __ballot_sync(0xffffffffu, e.open) : 0u;
             if (!(mc | me)) break;
-            const int la = __ffs(mc ? mc : me) - 1;
-            const int da = __shfl_sync(0xffffffffu, (mc ? c.j : e.j) - i, la);
+            const int la = __ffs(mc | me) - 1;
+            const bool a_is_c = (mc >> la) & 1u;
+            const int da = __shfl_sync(0xffffffffu, (a_is_c ? c.j : e.j) - i, la);
             const unsigned int oc = __ballot_sync(0xffffffffu, c.open && c.j - i != da);
             const unsigned int oe = ONE ? __ballot_sync(0xffffffffu, e.open && e.j - i != da) : 0u;
-            const int lb = oc | oe ? __ffs(oc ? oc : oe) - 1 : la;
-            const bool a_is_c = mc != 0u, b_is_c = oc | oe ? oc != 0u : a_is_c;
+            const int lb = oc | oe ? __ffs(oc | oe) - 1 : la;
+            const bool b_is_c = oc | oe ? ((oc >> lb) & 1u) != 0u : a_is_c;
             const bool mine_c = lane < 16 ? a_is_c : b_is_c;      // which of its lead's candidates this half extends
             const int lead = lane < 16 ? la : lb;
             const int jc = __shfl_sync(0xffffffffu, c.j, lead), je = ONE ? __shfl_sync(0xffffffffu, e.j, lead) : 0;
@@ -483,7 +486,9 @@ __global__ void __launch_bounds__(kChunk, ONE ? 1 : 2) match_query_kernel(const 
                     len = more ? len + step : f;
                 }
             }
-            // every open position of the same distance that lies before the end has the same end
+            // Every open position of the same distance that lies before the end has the same end: it lies at or behind the lead, and
+            // what the lead compared reaches from there to the end.  (Not so before the lead: between a lower lane's own first
+            // eight tokens and the lead there may be tokens that nobody has compared.)
             const int sa = __shfl_sync(0xffffffffu, i0 + len, 0), sb = __shfl_sync(0xffffffffu, i0 + len, 16);
             const int db = __shfl_sync(0xffffffffu, j0 - i0, 16);
             auto close = [&](Candidate &x) {

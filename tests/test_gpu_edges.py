@@ -170,6 +170,79 @@ def test_index_and_token_table_at_cluster_edges(env, N, w, K, live):
     assert torch.all(rows[N:] == 12345) and torch.all(ws[nws:] == 0x5A)
 
 
+def _index_query(env, hist, cuts, query, w, K, intra):
+    rac, dev = env.rac, env.dev
+    N, H = query.size, hist.size
+    cfg = rac.IndexCfg(H, w, K)
+    nb, nws = rac.rac_index_bytes(cfg), rac.rac_index_query_workspace_bytes(N)
+    mem, ws = (torch.full((n,), 0x5A, dtype=torch.uint8, device=dev) for n in (nb, nws))
+    h, q = torch.from_numpy(hist).to(dev), torch.from_numpy(query).to(dev)
+    rows = torch.full((N,), 12345, dtype=torch.int32, device=dev)
+    spans = torch.full((N // w + 1, 3), 777, dtype=torch.int32, device=dev)
+    n = torch.full((1,), -5, dtype=torch.int32, device=dev)
+    rac.rac_index_reset(cfg, mem, nb)
+    for a, b in zip(cuts, cuts[1:]):
+        rac.rac_index_append(cfg, mem, nb, h, int(a), int(b))
+    rac.rac_index_query(cfg, mem, nb, h, H, q, N, intra, rows, spans, n, ws, nws)
+    return rows.cpu().numpy(), spans[:int(n.item())].cpu().numpy()
+
+
+def _edited_copies(N, edit, seed):
+    """History: a text, and prefixes of 3 to 9 tokens of its stretches repeated behind it.  Query: stretches of the text with
+    single tokens replaced at `edit` and every 12 to 20 from there, so that a match resumes at the same distance."""
+    rng = np.random.default_rng(seed)
+    text = rng.integers(0, 3000, 2500).astype(np.int32)
+    starts = rng.integers(0, 2300, 40)
+    tail = np.concatenate([np.concatenate([rng.integers(5000, 9000, 5), text[s:s + int(rng.integers(3, 10))]])
+                           for s in np.concatenate([starts, starts, rng.integers(0, 2300, 40)])]).astype(np.int32)
+    query = np.empty(0, np.int32)
+    while query.size < N:
+        s = int(rng.choice(starts))
+        part = text[s:s + int(rng.integers(40, 200))].copy()
+        part[edit::int(rng.integers(12, 21))] = 20000
+        query = np.concatenate([query, rng.integers(10000, 12000, int(rng.integers(0, 32))).astype(np.int32), part])
+    return np.concatenate([text, tail]), np.ascontiguousarray(query[:N])
+
+
+def test_copy_that_resumes_after_a_changed_token(env):
+    """The later of two starts matches its window only, the earlier one up to the changed token; behind it the copy goes on at the
+    earlier one's distance.  Nothing may reach over the changed token."""
+    rng = np.random.default_rng(0)
+    A = rng.permutation(2000)[:96].astype(np.int32)
+    first = A.copy()
+    first[12] = 5000
+    cases = [(np.concatenate([first, np.arange(6000, 6005), A[:8], np.arange(7000, 7020)]).astype(np.int32), A)]
+    hist = rng.permutation(20000)[:400].astype(np.int32)
+    hist[300:304] = hist[100:104]
+    query = hist[100:164].copy()
+    query[12] = 30000
+    cases.append((hist, query))
+    for hist, query in cases:
+        o_rows, o_spans = env.orc.match_spans(hist, query, 4, 8)
+        assert o_spans[0, 2] == 12
+        rows, spans = _match(env, hist, query, 4, 8)
+        assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
+        rows, spans = _index_query(env, hist, [0, hist.size], query, 4, 8, False)
+        assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
+
+
+@pytest.mark.parametrize("N", [64, 512, 2048, 4096, 4097])
+@pytest.mark.parametrize("w,K", [(1, 8), (3, 2), (4, 3), (4, 8), (4, 16), (8, 8)])
+def test_edited_copies(env, N, w, K):
+    """Copies with single tokens changed, over windows that occur several times: the first change at 8 to 31 tokens, the copies at
+    every alignment to a warp; one history and an index of several requests, with and without intra-sequence references."""
+    for edit in (8, 11, 12, 13, 17, 20, 25, 31):
+        hist, query = _edited_copies(N, edit, 100 * edit + N + K)
+        rows, spans = _match(env, hist, query, w, K)
+        o_rows, o_spans = env.orc.match_spans(hist, query, w, K)
+        assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
+        cuts = [0, 700, 2500, 2600, hist.size]
+        for intra in (False, True):
+            rows, spans = _index_query(env, hist, cuts, query, w, K, intra)
+            o_rows, o_spans = env.orc.match_spans_req(hist, cuts, query, w=w, max_hits=K, intra=intra)
+            assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
+
+
 # ------------------------------------------------------------------------------- encode with outliers in one launch
 @pytest.mark.parametrize("d,g,bits,k,T", [
     (64, 32, 4, 2, 9000), (2048, 128, 3, 8, 8000), (2080, 32, 4, 16, 5000), (4096, 64, 2, 8, 5400), (4128, 32, 3, 5, 4100),
