@@ -185,7 +185,7 @@ __device__ __forceinline__ void index_start(u64 *slots, int32_t *top, int32_t *n
     load_bucket(slots, b, e);
     int from = 0, rep = -1, carry = j, old = -1;
     bool placed = next != nullptr;
-    while (probes <= bmask) {     // (the table has four times as many slots as windows: ends before)
+    while (probes <= bmask) {     // (the table has at least twice as many slots as windows: ends before)
         u64 held;
         const int s = find_in_bucket(e, tag, from, held);
         if (s == kBucket) {                   // full of other windows: the next bucket
@@ -796,11 +796,11 @@ static int fill_blocks(long long n16) {
     const long long b = (n16 + 255) / 256, most = (long long)sm_count() * 8;
     return (int)(b < 1 ? 1 : b > most ? most : b);
 }
-// Slots for n windows: at least `per` each.  Four per window leave one bucket in 250 full, two one in seven, and the slowest
-// of a warp's lanes sets its pace.
+// Slots for n windows: at least `per` each, but no more than 2^31 in all, which leaves two for each of up to 2^30 windows.  Four
+// per window leave one bucket in 250 full, two one in seven, and the slowest of a warp's lanes sets its pace.
 static unsigned int table_slots(long long n, unsigned long long per) {
     unsigned long long M = 1024;
-    while (M < per * (unsigned long long)(n > 0 ? n : 1)) M <<= 1;
+    while (M < per * (unsigned long long)(n > 0 ? n : 1) && M < (1ull << 31)) M <<= 1;
     return (unsigned int)M;
 }
 

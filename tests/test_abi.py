@@ -159,3 +159,18 @@ def test_prepare_marshals_once_and_launches_nothing(rac):
     with pytest.raises(TypeError):
         rac.prepare(rac.rac_decode_reconstruct, cfg, "not a tensor", 16, A, 16, None, None, None, A, A, A, stream=0)
     assert not isinstance(rac.load(), rac._Recorder)                                 # also after a failed prepare
+
+
+def test_retrieval_memory_grows_with_the_sizes(rac):
+    """Workspaces and indices up to the largest sizes that are taken: never less memory for more tokens, and at least two table
+    slots of eight bytes and the set of starts (at least one word) for every window."""
+    sizes = [0, 1, 255, 257, 1 << 20, (1 << 28) - 1, 1 << 28, (1 << 28) + 1, 1 << 29, (1 << 29) + 1, 3 << 28, (1 << 30) - 1]
+    for K in (0, 1, 8, 16):
+        ws = [rac.rac_match_workspace_bytes(n, 1, K) for n in sizes]
+        ix = [rac.rac_index_bytes(rac.IndexCfg(n, 4, K)) for n in sizes[1:]]
+        for got, of in ((ws, sizes), (ix, sizes[1:])):
+            assert all(a <= b for a, b in zip(got, got[1:])), (K, got)
+            assert all(b >= n * (16 + 4 * max(K, 1)) for b, n in zip(got, of)), (K, got)
+    q = [rac.rac_index_query_workspace_bytes(n) for n in sizes]
+    assert all(a <= b for a, b in zip(q, q[1:]))
+    assert rac.rac_match_workspace_bytes(1 << 30, 1, 8) == 0 and rac.rac_index_bytes(rac.IndexCfg(1 << 30)) == 0
