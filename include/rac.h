@@ -155,9 +155,10 @@ int rac_match_spans(const int32_t *hist_tok, int64_t n_hist, const int32_t *quer
  *
  * Same operation, arguments and results as rac_match_spans, minus the workspace: the scratch is a fixed array
  * of RAC_MATCH_STATIC_BYTES = 3 MiB inside the library image (every GPU that loads the library holds
- * it until the process ends).  That is enough for, e.g., a 32768-token history with 8192 query tokens and 8
- * hits; a problem whose rac_match_workspace_bytes() exceeds the capacity is refused with RAC_ESIZE and nothing is
- * launched.  The call allocates nothing and frees nothing, on the host side of CUDA or through any library.
+ * it until the process ends).  That is enough for every problem whose rac_match_workspace_bytes() is no more
+ * than that, e.g. a 32768-token history with 8192 query tokens and 8 hits, and, with a hash table of half the
+ * size, for some beyond: 65536 history and 2048 query tokens with 4 hits, 131072 and 2048 with one.  What does not
+ * fit either way is refused with RAC_ESIZE and nothing is launched.  The call allocates nothing and frees nothing, on the host side of CUDA or through any library.
  *
  * First call on a device: looks up the device address of the built-in array (one cudaGetSymbolAddress with
  * that device current).  Make that first call outside any stream capture.  The address is kept for the life of the

@@ -817,18 +817,20 @@ static void launch_query(const MatchParams &p, cudaStream_t st) {
     launch_after(match_emit_kernel, nchunks, kChunk, 0, st, p);
 }
 
+constexpr int kSlotsPerWindow = 4;
 struct MatchLayout {
     size_t slots, top, filled, best, jump, entry, next, total;
     unsigned int M;
 };
-// K = 0 (unlimited hits): one entry per window (the head of its chain) and a chain link per history position
-static MatchLayout match_layout(long long n_hist, long long n_query, int K) {
+// K = 0 (unlimited hits): one entry per window (the head of its chain) and a chain link per history position.  per: table slots
+// per window.
+static MatchLayout match_layout(long long n_hist, long long n_query, int K, int per) {
     MatchLayout L;
     const bool chains = K == 0;
     if (chains) K = 1;
     const size_t n = (size_t)(n_query > 0 ? n_query : 1);
     const size_t h = (size_t)(n_hist > 0 ? n_hist : 1);
-    L.M = table_slots(n_hist, 4);
+    L.M = table_slots(n_hist, per);
     size_t o = 0;
     L.slots = o;    o += (size_t)L.M * 8;                      // slots and top must stay contiguous (one fill)
     L.top = o;      o = align16(o + h * K * 4);
@@ -874,12 +876,12 @@ extern "C" {
 size_t rac_match_workspace_bytes(int64_t n_hist, int64_t n_query, int32_t max_hits) {
     if (n_hist < 0 || n_query < 0 || max_hits < 0 || max_hits > 16) return 0;
     if (n_hist >= (1ll << 30) || n_query >= (1ll << 30)) return 0;
-    return match_layout(n_hist, n_query, max_hits).total;
+    return match_layout(n_hist, n_query, max_hits, kSlotsPerWindow).total;
 }
 
-int rac_match_spans(const int32_t *hist_tok, int64_t n_hist, const int32_t *query_tok, int64_t n_query,
-                    int32_t min_ngram, int32_t max_hits, int32_t *ref_row, rac_span *spans, int32_t *n_spans,
-                    void *workspace, size_t workspace_bytes, void *stream) {
+static int match_spans(const int32_t *hist_tok, int64_t n_hist, const int32_t *query_tok, int64_t n_query,
+                       int32_t min_ngram, int32_t max_hits, int32_t *ref_row, rac_span *spans, int32_t *n_spans,
+                       void *workspace, size_t workspace_bytes, int per, void *stream) {
     if (n_hist < 0 || n_query < 0 || !n_spans) return RAC_EINVAL;
     if (n_hist >= (1ll << 30) || n_query >= (1ll << 30)) return RAC_EUNSUPPORTED;
     if (min_ngram < 1 || min_ngram > 32) return RAC_EUNSUPPORTED;
@@ -887,7 +889,7 @@ int rac_match_spans(const int32_t *hist_tok, int64_t n_hist, const int32_t *quer
     if ((n_hist > 0 && !hist_tok) || (n_query > 0 && (!query_tok || !ref_row))) return RAC_EINVAL;
     if (!workspace) return RAC_EINVAL;
     if (reinterpret_cast<uintptr_t>(workspace) & 15u) return RAC_EALIGN;
-    MatchLayout L = match_layout(n_hist, n_query, max_hits);
+    MatchLayout L = match_layout(n_hist, n_query, max_hits, per);
     if (workspace_bytes < L.total) return RAC_ESIZE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
@@ -921,6 +923,13 @@ int rac_match_spans(const int32_t *hist_tok, int64_t n_hist, const int32_t *quer
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
 }
 
+int rac_match_spans(const int32_t *hist_tok, int64_t n_hist, const int32_t *query_tok, int64_t n_query,
+                    int32_t min_ngram, int32_t max_hits, int32_t *ref_row, rac_span *spans, int32_t *n_spans,
+                    void *workspace, size_t workspace_bytes, void *stream) {
+    return match_spans(hist_tok, n_hist, query_tok, n_query, min_ngram, max_hits, ref_row, spans, n_spans, workspace,
+                       workspace_bytes, kSlotsPerWindow, stream);
+}
+
 int rac_spans_to_rows(const rac_span *spans, const int32_t *n_spans, int64_t n_query, int32_t *ref_row, void *stream) {
     if (n_query < 0 || !n_spans) return RAC_EINVAL;
     if (n_query == 0) return RAC_OK;
@@ -940,14 +949,16 @@ int rac_match_spans_static(const int32_t *hist_tok, int64_t n_hist, const int32_
     // size check first, with the same layout function the caller-workspace entry point uses
     const size_t need = rac_match_workspace_bytes(n_hist, n_query, max_hits);
     if (need == 0) return (n_hist < 0 || n_query < 0) ? RAC_EINVAL : RAC_EUNSUPPORTED;
-    if (need > kStaticMatchBytes) return RAC_ESIZE;  // problem too large for the built-in scratch
+    // where few hits per window leave most of the memory to the table (65536 tokens, four hits), half the table still fits
+    const int per = need <= kStaticMatchBytes ? kSlotsPerWindow : kSlotsPerWindow / 2;
+    if (match_layout(n_hist, n_query, max_hits, per).total > kStaticMatchBytes) return RAC_ESIZE;  // too large for the scratch
     void *scratch = nullptr;
     int rc = static_match_scratch(&scratch);
     if (rc != RAC_OK) return rc;
     // every launch of the matcher re-initialises the table, the rows and the span count, so whatever the
     // previous call left in the scratch is harmless
-    return rac_match_spans(hist_tok, n_hist, query_tok, n_query, min_ngram, max_hits, ref_row, spans, n_spans, scratch,
-                           kStaticMatchBytes, stream);
+    return match_spans(hist_tok, n_hist, query_tok, n_query, min_ngram, max_hits, ref_row, spans, n_spans, scratch,
+                       kStaticMatchBytes, per, stream);
 }
 
 }  // extern "C"

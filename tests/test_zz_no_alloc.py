@@ -63,3 +63,19 @@ def test_static_scratch_matcher_equals_workspace_matcher_twice_in_a_row():
     assert ei.value.code == -3 and "too small" in str(ei.value)
     torch.cuda.synchronize()
     assert int(n.item()) == -1 and torch.all(rows == 4242)
+
+
+@pytest.mark.parametrize("n_hist,n_query,K", [(65536, 2048, 4), (131072, 2048, 1), (65537, 1500, 0), (70000, 5000, 1)])
+def test_static_scratch_with_the_smaller_table(n_hist, n_query, K):
+    """Problems that fit the scratch with two table slots per window only, some with more than half of the slots taken."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_04991_b200 import binding as rac
+    from paper_2608_04991_b200 import synth
+    import oracle
+    rac.load()
+    assert rac.rac_match_workspace_bytes(n_hist, n_query, K) > rac.MATCH_STATIC_BYTES
+    wl = synth.span_workload(n_hist, n_query, seed=n_hist + K)
+    o_rows, o_spans = oracle.match_spans(wl.hist, wl.query, 4, K)
+    for rows, spans, n in _both(rac, torch.device("cuda:0"), wl.hist, wl.query, 4, K):
+        assert n > 0 and np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
