@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
 // above tau are candidates, collected in channel order, one per lane.  (c) While there are more than k, the
 // smallest goes (smallest magnitude; among equals the highest channel): the survivors are the k largest with
 // ties to the lower channel, still in channel order.  More than 32 candidates (many equal magnitudes, e.g. an
-// all-zero residual): k rounds of a maximum over the whole token instead.  (d) The winners go into the record's
+// all-zero residual): a pass over the whole token instead.  (d) The winners go into the record's
 // outlier fields in channel order, their dense codes are cleared (E^d = E - O), and with the sender-side
 // reconstruction those channels of x_hat are replaced.
 constexpr int kOutCap = 32;        // candidates per token: one per lane
@@ -451,43 +451,74 @@ __device__ __forceinline__ float pick8(const float (&v)[8], int i) {
     return (i & 4) ? b1 : b0;
 }
 
-// whole-token path: k rounds of a maximum over all d channels (rare).  Lane r returns the r-th winner:
-// channel, residual, aligned reference.
+// Whole-token path (rare): the k largest |e| of all d channels, ties to the lower channel, by one warp.  One pass over the rows
+// in channel order, 256 channels at a time, eight per lane; lanes 0..k-1 hold the k best so far, lane r returns its channel,
+// residual and aligned reference (in no order).  What comes later has the higher channel, so it replaces the smallest held one
+// only with a larger magnitude, and of equal ones held the highest channel goes: at most k replacements per 256 channels.
+// Bound by the trips for the rows, the next of which is under way while one is looked at.  k rounds of a maximum over the whole
+// token, one channel per lane and trip, took 150 us per token at d = 4096, k = 8; this takes 5.  (16384 such tokens, all residuals
+// zero: 1.61 ms when the warps of a second launch did it, 4.40 ms when the selectors of encode_top_kernel did, 0.17 ms so.)
 __device__ __noinline__ void select_whole_token(int d, int k, int coef_shift, const uint16_t *xrow, const uint16_t *rrow,
                                                 const uint16_t *gain, const uint16_t *bias, const uint32_t *coef,
                                                 int lane, int *c_out, float *e_out, float *rt_out) {
-    unsigned long long prev = ~0ull, mine = 0ull;
-    float minee = 0.f, minert = 0.f;
-    for (int r = 0; r < k; r++) {
-        unsigned long long best = 0ull;
-        float beste = 0.f, bestrt = 0.f;
-        for (int c = lane; c < d; c += 32) {
-            const float h = __uint_as_float((uint32_t)xrow[c] << 16);
-            float rr = 0.f;
-            if (rrow) {
-                rr = __uint_as_float((uint32_t)rrow[c] << 16);
-                if (gain) rr = bf16_round(__fmaf_rn(half_bits_to_float(gain[c]), rr, half_bits_to_float(bias[c])));
+    int held = lane < k ? -1 : 0x7fffffff;     // magnitude (bits) this lane holds, -1: none yet
+    int hc = 0x10000 + lane;                   // its channel
+    float he = 0.f, hrt = 0.f;
+    uint4 xn = make_uint4(0u, 0u, 0u, 0u), rn = xn;
+    auto load = [&](int c) {
+        if (c < d) {
+            xn = __ldcg(reinterpret_cast<const uint4 *>(xrow + c));
+            if (rrow) rn = __ldcg(reinterpret_cast<const uint4 *>(rrow + c));
+        }
+    };
+    load(8 * lane);
+    for (int base = 0; base < d; base += 256) {
+        const int c0 = base + 8 * lane;
+        const bool act = c0 < d;
+        const uint32_t xw[4] = {xn.x, xn.y, xn.z, xn.w};
+        uint32_t rw[4] = {rn.x, rn.y, rn.z, rn.w};      // zero without a reference
+        load(c0 + 256);
+        const uint32_t cf = act ? coef[c0 >> coef_shift] : 0u;
+        if (rrow && gain && act) {
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const int c = c0 + 2 * i;
+                rw[i] = f2_to_bf16x2(__fmaf_rn(half_bits_to_float(gain[c]), __uint_as_float(rw[i] << 16), half_bits_to_float(bias[c])),
+                                     __fmaf_rn(half_bits_to_float(gain[c + 1]), __uint_as_float(rw[i] & 0xffff0000u),
+                                               half_bits_to_float(bias[c + 1])));
             }
-            const uint32_t cf = coef[c >> coef_shift];
-            const float rtc = __fmaf_rn(half_bits_to_float(cf & 0xffff), rr, half_bits_to_float(cf >> 16));
-            const float e = __fsub_rn(h, rtc);
-            const unsigned long long comp =
-                ((unsigned long long)(__float_as_uint(e) & 0x7fffffffu) << 16) | (unsigned long long)(0xffff - c);
-            // a composite is 0 only for |e| == 0 at channel 65535, which d <= 8192 excludes
-            if (comp < prev && comp > best) { best = comp; beste = e; bestrt = rtc; }
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
-            const float othere = __shfl_xor_sync(0xffffffffu, beste, o);
-            const float otherrt = __shfl_xor_sync(0xffffffffu, bestrt, o);
-            if (other > best) { best = other; beste = othere; bestrt = otherrt; }
+        const float ca = half_bits_to_float(cf & 0xffff), cb = half_bits_to_float(cf >> 16);
+        const u64 a2 = pack2(ca, ca), b2 = pack2(cb, cb);
+        float e[8], rt[8];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const u64 rt2 = pfma(a2, bf16x2_to_p(rw[i]), b2);
+            unpack2(rt2, rt[2 * i], rt[2 * i + 1]);
+            unpack2(psub(bf16x2_to_p(xw[i]), rt2), e[2 * i], e[2 * i + 1]);
         }
-        if (lane == r) { mine = best; minee = beste; minert = bestrt; }
-        prev = best;
+        uint32_t left = act ? 0xffu : 0u;      // elements not taken yet
+        while (true) {
+            int best = -1, at = 0;
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                const int mag = (int)(__float_as_uint(e[i]) & 0x7fffffffu);
+                if (((left >> i) & 1u) && mag > best) { best = mag; at = i; }
+            }
+            const int top = __reduce_max_sync(0xffffffffu, best);
+            const int low = __reduce_min_sync(0xffffffffu, held);
+            if (top <= low) break;
+            const int from = __ffs(__ballot_sync(0xffffffffu, best == top)) - 1;      // the lowest channel of them
+            const int worst = __reduce_max_sync(0xffffffffu, held == low ? hc : -1);  // the highest channel of the smallest held
+            const int tc = __shfl_sync(0xffffffffu, c0 + at, from);
+            const float te = __shfl_sync(0xffffffffu, pick8(e, at), from), trt = __shfl_sync(0xffffffffu, pick8(rt, at), from);
+            if (lane == from) left &= ~(1u << at);
+            if (held == low && hc == worst) { held = top; hc = tc; he = te; hrt = trt; }
+        }
     }
-    *c_out = 0xffff - (int)(mine & 0xffffull);
-    *e_out = minee;
-    *rt_out = minert;
+    *c_out = hc;
+    *e_out = he;
+    *rt_out = hrt;
 }
 
 // NV: slab maxima per lane (d <= 32*32*NV).  KT: the number of outliers when it is 8 (unrolled), else 0 = p.topk.
@@ -723,7 +754,7 @@ __global__ void __launch_bounds__(W * 32, W == 7 ? 4 : 3) outlier_kernel(const C
             }
             // ---- (d) outlier fields in channel order, dense codes at those channels cleared
             int pos = __popc(__ballot_sync(0xffffffffu, won) & lt_mask);
-            if (n[u] > kOutCap) {   // the whole-token path returns its winners by rank, not by channel
+            if (n[u] > kOutCap) {   // the whole-token path returns its winners in no order
                 pos = 0;
                 for (int y = 0; y < k; y++) {
                     const int cy = __shfl_sync(0xffffffffu, wc, y);
@@ -1056,7 +1087,7 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
             } else {
                 select_whole_token(d, k, coef_shift, xrow, rrow, p.gain, p.bias, coefp, lane, &wc, &we, &wrt);
                 won = lane < k;
-                pos = 0;                         // the whole-token path returns its winners by rank, not by channel
+                pos = 0;                         // the whole-token path returns its winners in no order
                 for (int y = 0; y < k; y++) {
                     const int cy = __shfl_sync(0xffffffffu, wc, y);
                     pos += cy < wc ? 1 : 0;

@@ -278,6 +278,61 @@ def test_one_launch_outliers_at_shape_edges(env, d, g, bits, k, T):
     assert np.array_equal(o_x.reshape(-1), s.bf16_bits(xs).reshape(-1))
 
 
+@pytest.mark.parametrize("d,g,bits,k,T,predictor", [
+    (32, 32, 4, 1, 40, False), (32, 32, 2, 16, 40, False), (256, 32, 3, 8, 40, True), (288, 32, 4, 16, 40, False),
+    (4096, 128, 4, 8, 700, False), (5120, 128, 2, 5, 300, True), (8160, 32, 3, 8, 50, False), (8192, 64, 4, 16, 1200, False)])
+def test_many_equal_residuals(env, d, g, bits, k, T, predictor):
+    """Tokens whose outliers are looked for in the whole token: all-zero residuals, one magnitude everywhere, magnitudes that rise
+    or fall from one piece of channels to the next (the 256 channels of a step, fewer and more), and a few levels at random.  The
+    whole call with and without x_hat, and the same tokens through two token lists."""
+    s, rac, dev, P = env.synth, env.rac, env.dev, env.P
+    gen = s.generator(d + k, dev)
+    R = s.activations(T, d, s.channel_scale(d, 5, dev), gen)
+    rng = np.random.default_rng(d + k)
+    gain, bias = s.predictor_gain_bias(d, 5, dev) if predictor else (None, None)
+    X = R.clone() if gain is None else torch.addcmul(bias.float(), gain.float(), R.float()).to(torch.bfloat16)
+    rows = np.arange(T, dtype=np.int32)
+    sign = torch.tensor([1.0, -1.0], device=dev).repeat(d // 2)         # pairs cancel: the mean of a group is exactly zero
+    for t in range(T):
+        kind = t % 7                                                    # 0: the (transformed) reference itself
+        if kind == 0:
+            continue
+        piece = int(rng.choice([2, 32, 64, 256, 512]))
+        level = torch.arange(d, device=dev) // piece
+        if kind == 1:
+            level = torch.zeros_like(level)
+        elif kind == 3:
+            level = level.flip(0) // 2 * 2
+        elif kind == 4:
+            level = torch.from_numpy(rng.integers(0, 4, d // 2)).to(dev).repeat_interleave(2)
+        elif kind == 5:                                                 # zeros, and fewer non-zero channels than outliers
+            level = torch.full((d,), -1, device=dev)
+            level[-max(1, (k - 1) // 2) * 2:] = 5
+            level = level if k > 2 else level.clamp(max=-1)
+        elif kind == 6:
+            level = torch.ones_like(level)
+            level[int(rng.integers(0, d // 2)) * 2] = 9
+        X[t] = ((level + 1).float() * 0.25 * sign).to(torch.bfloat16)
+        rows[t] = -1
+    step = np.full((2, d), 0.125, np.float32)
+    rows_d = torch.from_numpy(rows).to(dev)
+    cfg = rac.CodecCfg(d, g, bits, k)
+    _, pay, _ = P.round_trip_case(cfg, X, R, rows_d, gain, bias, step, 1.0 / step)
+    order = rng.permutation(T).astype(np.int32)
+    st = torch.zeros(1, dtype=torch.int32, device=dev)
+    nws = rac.rac_encode_workspace_bytes(cfg, T)
+    ws = torch.empty(nws, dtype=torch.uint8, device=dev)
+    step_d, inv_d = P.to_dev(step, dev), P.to_dev(1.0 / step, dev)
+    listed = torch.full((pay.size,), 0xA5, dtype=torch.uint8, device=dev)
+    xs = torch.full((T, d), -7.0, dtype=torch.bfloat16, device=dev)
+    for part in (order[:T // 3], order[T // 3:]):
+        rac.rac_encode_reconstruct_list(cfg, X, T, torch.from_numpy(part).to(dev),
+                                        torch.tensor([part.size], dtype=torch.int32, device=dev), R, T, rows_d, None, 0, gain, bias,
+                                        step_d, inv_d, listed, pay.size, xs, ws, nws, st)
+    assert int(st.item()) == 0 and np.array_equal(listed.cpu().numpy(), pay)
+    assert torch.equal(xs.view(torch.int16), P.gpu_encode_reconstruct(cfg, X, R, rows_d, gain, bias, step_d, inv_d)[1].view(torch.int16))
+
+
 @pytest.mark.parametrize("T", [0, 1, 31, 128, 4095, 4096, 4097, 12289, 131072, 128 * 4096 + 1])
 def test_split_waves_at_range_edges(env, T):
     """One token up to more ranges than CTAs; mixed rows, all of one wave, and a first row that only the last token reaches."""
