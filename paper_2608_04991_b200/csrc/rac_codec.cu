@@ -458,9 +458,12 @@ __device__ __forceinline__ float pick8(const float (&v)[8], int i) {
 // Bound by the trips for the rows, the next of which is under way while one is looked at.  k rounds of a maximum over the whole
 // token, one channel per lane and trip, took 150 us per token at d = 4096, k = 8; this takes 5.  (16384 such tokens, all residuals
 // zero: 1.61 ms when the warps of a second launch did it, 4.40 ms when the selectors of encode_top_kernel did, 0.17 ms so.)
-__device__ __noinline__ void select_whole_token(int d, int k, int coef_shift, const uint16_t *xrow, const uint16_t *rrow,
-                                                const uint16_t *gain, const uint16_t *bias, const uint32_t *coef,
-                                                int lane, int *c_out, float *e_out, float *rt_out) {
+struct Winner {
+    int c;
+    float e, rt;
+};
+__device__ __noinline__ Winner select_whole_token(int d, int k, int coef_shift, const uint16_t *xrow, const uint16_t *rrow,
+                                                  const uint16_t *gain, const uint16_t *bias, const uint32_t *coef, int lane) {
     int held = lane < k ? -1 : 0x7fffffff;     // magnitude (bits) this lane holds, -1: none yet
     int hc = 0x10000 + lane;                   // its channel
     float he = 0.f, hrt = 0.f;
@@ -516,9 +519,7 @@ __device__ __noinline__ void select_whole_token(int d, int k, int coef_shift, co
             if (held == low && hc == worst) { held = top; hc = tc; he = te; hrt = trt; }
         }
     }
-    *c_out = hc;
-    *e_out = he;
-    *rt_out = hrt;
+    return Winner{hc, he, hrt};
 }
 
 // NV: slab maxima per lane (d <= 32*32*NV).  KT: the number of outliers when it is 8 (unrolled), else 0 = p.topk.
@@ -749,7 +750,10 @@ __global__ void __launch_bounds__(W * 32, W == 7 ? 4 : 3) outlier_kernel(const C
                     if (lane == 31 - __clz(bal)) { mag = 0xffffffffu; won = false; }   // among equals the highest channel
                 }
             } else {
-                select_whole_token(d, k, coef_shift, xrow[u], rrow[u], p.gain, p.bias, coefp[u], lane, &wc, &we, &wrt);
+                const Winner w = select_whole_token(d, k, coef_shift, xrow[u], rrow[u], p.gain, p.bias, coefp[u], lane);
+                wc = w.c;
+                we = w.e;
+                wrt = w.rt;
                 won = lane < k;
             }
             // ---- (d) outlier fields in channel order, dense codes at those channels cleared
@@ -1085,7 +1089,10 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
                 }
                 pos = __popc(__ballot_sync(0xffffffffu, won) & lt_mask);
             } else {
-                select_whole_token(d, k, coef_shift, xrow, rrow, p.gain, p.bias, coefp, lane, &wc, &we, &wrt);
+                const Winner w = select_whole_token(d, k, coef_shift, xrow, rrow, p.gain, p.bias, coefp, lane);
+                wc = w.c;
+                we = w.e;
+                wrt = w.rt;
                 won = lane < k;
                 pos = 0;                         // the whole-token path returns its winners in no order
                 for (int y = 0; y < k; y++) {
