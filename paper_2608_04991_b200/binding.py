@@ -4,8 +4,8 @@ Every function has the name and the argument order of its C entry point in
 ``include/rac.h``.  Arguments are either raw addresses (int) or torch tensors
 living where the C function expects them (device pointers for the ``rac_*``
 calls); the binding checks dtype, contiguity and device, takes the tensor's
-address and the current CUDA stream, calls the library and raises on a non-zero
-return code.  The launching calls are marshalled by the extension module
+address and the current CUDA stream (or ``stream``: a ``torch.cuda.Stream`` or
+an address), calls the library and raises on a non-zero return code.  The launching calls are marshalled by the extension module
 ``_native`` (``csrc/rac_py.cpp``), the others and the plain library by ctypes.
 No arithmetic of the method happens here and there is no fallback: if the
 library cannot be loaded, importing callers get an error.
@@ -197,7 +197,7 @@ def load():
     l.rac_calibrate_steps_shared.restype = C.c_int
     l.rac_calibrate_steps_shared.argtypes = [cfgp, vp, i64, vp, i64, vp, vp, vp, vp, vp, C.c_float, vp, vp, vp, sz, vp, vp]
     from . import _native as native
-    native.set_check(_check)
+    native.setup(_check, _stream_address)
     _native = native
     _lib = l
     return l
@@ -213,6 +213,12 @@ def _calls():
 def _check(fn: str, rc: int) -> None:
     if rc != RAC_OK:
         raise RacError(fn, rc, load().rac_strerror(rc).decode())
+
+
+def _stream_address(stream) -> int:
+    """Address of a stream that is neither None nor an integer: a ``torch.cuda.Stream``, a ``c_void_p``, whatever else
+    ctypes passes as a pointer."""
+    return C.cast(stream, C.c_void_p).value or 0
 
 
 # ----------------------------------------------------------------------------- plain queries

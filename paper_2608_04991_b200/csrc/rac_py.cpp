@@ -48,7 +48,7 @@ constexpr int length(const char *s) {
 
 constexpr int kMaxArgs = 24;
 // kinds: c rac_codec_cfg, x rac_index_cfg; tensors or addresses: b bf16, h binary16, f float32, i int32, u bytes, a any type;
-// numbers: l integer, B truth value, d float; s stream (None = the current one)
+// numbers: l integer, B truth value, d float; s stream (None = the current one, an address, or what ctypes takes for one)
 struct Entry {
     const char *name, *kinds, *args;   // args: names, comma separated (for messages)
     int count;
@@ -104,6 +104,7 @@ const Entry kEntries[] = {
 };
 
 PyObject *g_check = nullptr;   // binding._check(name, return code): raises for a non-zero code
+PyObject *g_stream = nullptr;  // binding._stream_address(object) -> int, for streams that are neither None nor an address
 
 const char *arg_name(const Entry &e, int k, char *buf, size_t cap) {
     const char *s = e.args;
@@ -164,6 +165,12 @@ bool marshal(const Entry &e, int k, PyObject *o, Slot *s) {
             if (o == Py_None) {
                 s->p = c10::cuda::getCurrentCUDAStream().stream();
                 return true;
+            }
+            if (!PyLong_Check(o)) {      // a torch stream, a c_void_p
+                PyObject *n = PyObject_CallOneArg(g_stream, o);
+                const bool ok = n && as_integer(n, &s->i);
+                Py_XDECREF(n);
+                return ok;
             }
             return as_integer(o, &s->i);
         case 'c':
@@ -277,13 +284,16 @@ PyObject *py_prepare(PyObject *, PyObject *const *args, Py_ssize_t n) {
     }
     return reinterpret_cast<PyObject *>(p);
 }
-PyObject *py_set_check(PyObject *, PyObject *f) {
-    Py_XSETREF(g_check, Py_NewRef(f));
+// setup(check, stream_address): the callbacks into binding
+PyObject *py_setup(PyObject *, PyObject *const *args, Py_ssize_t n) {
+    if (n != 2) return PyErr_Format(PyExc_TypeError, "setup(check, stream_address)");
+    Py_XSETREF(g_check, Py_NewRef(args[0]));
+    Py_XSETREF(g_stream, Py_NewRef(args[1]));
     Py_RETURN_NONE;
 }
 PyMethodDef methods[] = {
     {"prepare", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(py_prepare)), METH_FASTCALL, nullptr},
-    {"set_check", py_set_check, METH_O, nullptr},
+    {"setup", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(py_setup)), METH_FASTCALL, nullptr},
     {}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods};
 

@@ -1,4 +1,6 @@
 """What the binding accepts and refuses, without a GPU: nothing here gets as far as a launch."""
+import ctypes as C
+
 import pytest
 import torch
 
@@ -13,8 +15,8 @@ def rac():
     return binding
 
 
-def decode(rac, cfg, payload=A, T=16, ref_base=A, step=A, X_hat=A):
-    rac.rac_decode_reconstruct(cfg, payload, T, ref_base, 16, None, None, None, step, X_hat, A, stream=0)
+def decode(rac, cfg, payload=A, T=16, ref_base=A, step=A, X_hat=A, stream=0):
+    rac.rac_decode_reconstruct(cfg, payload, T, ref_base, 16, None, None, None, step, X_hat, A, stream=stream)
 
 
 @pytest.mark.parametrize("kw,exc,text", [
@@ -61,3 +63,20 @@ def test_prepared_call_checks_like_the_plain_one(rac):
         call(1)
     none = rac.prepare(rac.rac_decode_reconstruct, cfg, A, 0, A, 16, None, None, None, A, A, A, stream=0)
     assert none() is None
+
+
+class _Stream:
+    """What torch.cuda.Stream is to ctypes."""
+    _as_parameter_ = C.c_void_p(0x7000)
+
+
+def test_streams_are_addresses_or_what_ctypes_takes_for_one(rac):
+    cfg = rac.CodecCfg(4096, 128, 4, 0)
+    assert hasattr(torch.cuda.Stream, "_as_parameter_")
+    for stream in (0, 0x7000, True, _Stream(), C.c_void_p(0x7000), C.c_void_p(None), C.pointer(C.c_int(3))):
+        decode(rac, cfg, T=0, stream=stream)
+        rac.prepare(rac.rac_decode_reconstruct, cfg, A, 0, A, 16, None, None, None, A, A, A, stream=stream)()
+    assert rac._stream_address(_Stream()) == 0x7000 and rac._stream_address(C.c_void_p(None)) == 0
+    for stream in (3.7, torch.tensor(5), C.c_int64(5), object()):
+        with pytest.raises((TypeError, C.ArgumentError)):
+            decode(rac, cfg, T=0, stream=stream)
