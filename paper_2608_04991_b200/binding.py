@@ -197,7 +197,7 @@ def load():
     l.rac_calibrate_steps_shared.restype = C.c_int
     l.rac_calibrate_steps_shared.argtypes = [cfgp, vp, i64, vp, i64, vp, vp, vp, vp, vp, C.c_float, vp, vp, vp, sz, vp, vp]
     from . import _native as native
-    native.setup(_check, _stream_address)
+    native.setup(_check, _stream_address, CodecCfg, IndexCfg)
     _native = native
     _lib = l
     return l

@@ -104,6 +104,7 @@ const Entry kEntries[] = {
 };
 
 PyObject *g_check = nullptr;   // binding._check(name, return code): raises for a non-zero code
+PyObject *g_codec_cfg = nullptr, *g_index_cfg = nullptr;   // binding.CodecCfg, binding.IndexCfg: the structs of rac.h
 PyObject *g_stream = nullptr;  // binding._stream_address(object) -> int, for streams that are neither None nor an address
 
 const char *arg_name(const Entry &e, int k, char *buf, size_t cap) {
@@ -175,14 +176,16 @@ bool marshal(const Entry &e, int k, PyObject *o, Slot *s) {
             return as_integer(o, &s->i);
         case 'c':
         case 'x': {
+            // the struct type itself (or a subclass): any other buffer of its size is none
+            if (!PyObject_TypeCheck(o, reinterpret_cast<PyTypeObject *>(kind == 'c' ? g_codec_cfg : g_index_cfg))) {
+                PyErr_Format(PyExc_TypeError, "%s: expected %s", arg_name(e, k, name, sizeof name), kind == 'c' ? "a CodecCfg" : "an IndexCfg");
+                return false;
+            }
             Py_buffer v;
-            const Py_ssize_t want = kind == 'c' ? sizeof(rac_codec_cfg) : sizeof(rac_index_cfg);
             if (PyObject_GetBuffer(o, &v, PyBUF_SIMPLE) != 0) return false;
             s->p = v.buf;      // the caller holds the object for as long as the address is used
-            const bool ok = v.len == want;
             PyBuffer_Release(&v);
-            if (!ok) PyErr_Format(PyExc_TypeError, "%s: expected %s", arg_name(e, k, name, sizeof name), kind == 'c' ? "a CodecCfg" : "an IndexCfg");
-            return ok;
+            return true;
         }
     }
     if (o == Py_None) {
@@ -284,11 +287,14 @@ PyObject *py_prepare(PyObject *, PyObject *const *args, Py_ssize_t n) {
     }
     return reinterpret_cast<PyObject *>(p);
 }
-// setup(check, stream_address): the callbacks into binding
+// setup(check, stream_address, CodecCfg, IndexCfg): the callbacks into binding and its struct types
 PyObject *py_setup(PyObject *, PyObject *const *args, Py_ssize_t n) {
-    if (n != 2) return PyErr_Format(PyExc_TypeError, "setup(check, stream_address)");
+    if (n != 4 || !PyType_Check(args[2]) || !PyType_Check(args[3]))
+        return PyErr_Format(PyExc_TypeError, "setup(check, stream_address, CodecCfg, IndexCfg)");
     Py_XSETREF(g_check, Py_NewRef(args[0]));
     Py_XSETREF(g_stream, Py_NewRef(args[1]));
+    Py_XSETREF(g_codec_cfg, Py_NewRef(args[2]));
+    Py_XSETREF(g_index_cfg, Py_NewRef(args[3]));
     Py_RETURN_NONE;
 }
 PyMethodDef methods[] = {

@@ -80,3 +80,17 @@ def test_streams_are_addresses_or_what_ctypes_takes_for_one(rac):
     for stream in (3.7, torch.tensor(5), C.c_int64(5), object()):
         with pytest.raises((TypeError, C.ArgumentError)):
             decode(rac, cfg, T=0, stream=stream)
+
+
+@pytest.mark.parametrize("cfg", [b"\0" * 36, bytearray(36), (C.c_int32 * 9)(4096, 128, 4), torch.zeros(9, dtype=torch.int32).numpy()])
+def test_other_buffers_of_the_size_of_a_configuration_are_refused(rac, cfg):
+    with pytest.raises(TypeError):
+        decode(rac, cfg, T=0)
+    with pytest.raises(TypeError):
+        rac.rac_index_reset(memoryview(cfg)[:16] if isinstance(cfg, (bytes, bytearray)) else cfg, A, 1 << 30, stream=0)
+    with pytest.raises(TypeError):
+        rac.prepare(rac.rac_decode_reconstruct, cfg, A, 0, A, 16, None, None, None, A, A, A, stream=0)
+
+    class Named(rac.CodecCfg):
+        pass
+    decode(rac, Named(4096, 128, 4, 0), T=0)
