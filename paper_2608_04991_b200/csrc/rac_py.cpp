@@ -246,7 +246,7 @@ struct EntryObject {
 struct PreparedObject {
     PyObject_HEAD
     const Entry *entry;
-    PyObject *keepalive;
+    PyObject *args, *keepalive;   // the marshalled arguments themselves, and what the caller gave
     vectorcallfunc vectorcall;
     Slot slots[kMaxArgs];
 };
@@ -264,11 +264,12 @@ PyObject *prepared_call(PyObject *self, PyObject *const *, size_t nargsf, PyObje
     return finish(*p->entry, p->slots);
 }
 void prepared_dealloc(PyObject *self) {
+    Py_XDECREF(reinterpret_cast<PreparedObject *>(self)->args);
     Py_XDECREF(reinterpret_cast<PreparedObject *>(self)->keepalive);
     Py_TYPE(self)->tp_free(self);
 }
 PyObject *prepared_keepalive(PyObject *self, void *) { return Py_NewRef(reinterpret_cast<PreparedObject *>(self)->keepalive); }
-PyGetSetDef prepared_getset[] = {{"keepalive", prepared_keepalive, nullptr, "what the marshalled addresses refer to", nullptr}, {}};
+PyGetSetDef prepared_getset[] = {{"keepalive", prepared_keepalive, nullptr, "the (args, kwargs) of the call", nullptr}, {}};
 PyTypeObject EntryType = {PyVarObject_HEAD_INIT(nullptr, 0)};
 PyTypeObject PreparedType = {PyVarObject_HEAD_INIT(nullptr, 0)};
 
@@ -280,8 +281,9 @@ PyObject *py_prepare(PyObject *, PyObject *const *args, Py_ssize_t n) {
     if (!p) return nullptr;
     p->entry = reinterpret_cast<EntryObject *>(args[0])->entry;
     p->vectorcall = prepared_call;
-    p->keepalive = PyTuple_Pack(2, args[1], args[2]);   // the marshalled arguments themselves, and the caller's
-    if (!p->keepalive || !marshal_all(*p->entry, &PyTuple_GET_ITEM(args[1], 0), PyTuple_GET_SIZE(args[1]), p->slots)) {
+    p->args = Py_NewRef(args[1]);
+    p->keepalive = Py_NewRef(args[2]);
+    if (!marshal_all(*p->entry, &PyTuple_GET_ITEM(args[1], 0), PyTuple_GET_SIZE(args[1]), p->slots)) {
         Py_DECREF(p);
         return nullptr;
     }

@@ -94,3 +94,9 @@ def test_other_buffers_of_the_size_of_a_configuration_are_refused(rac, cfg):
     class Named(rac.CodecCfg):
         pass
     decode(rac, Named(4096, 128, 4, 0), T=0)
+
+
+def test_prepared_call_shows_what_it_was_given(rac):
+    args = (rac.CodecCfg(4096, 128, 4, 0), A, 0, A, 16, None, None, None, A, A, A)
+    call = rac.prepare(rac.rac_decode_reconstruct, *args, stream=0)
+    assert call.keepalive == (args, {"stream": 0}) and call.keepalive[0][0] is args[0]
