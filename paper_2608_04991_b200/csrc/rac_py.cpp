@@ -159,9 +159,13 @@ bool marshal(const Entry &e, int k, PyObject *o, Slot *s) {
             s->i = v;
             return v >= 0;
         }
-        case 'd':
-            s->d = PyFloat_AsDouble(o);
-            return !(s->d == -1.0 && PyErr_Occurred());
+        case 'd': {
+            PyObject *n = PyNumber_Float(o);
+            if (!n) return false;
+            s->d = PyFloat_AS_DOUBLE(n);
+            Py_DECREF(n);
+            return true;
+        }
         case 's':
             if (o == Py_None) {
                 s->p = c10::cuda::getCurrentCUDAStream().stream();

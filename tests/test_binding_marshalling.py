@@ -100,3 +100,15 @@ def test_prepared_call_shows_what_it_was_given(rac):
     args = (rac.CodecCfg(4096, 128, 4, 0), A, 0, A, 16, None, None, None, A, A, A)
     call = rac.prepare(rac.rac_decode_reconstruct, *args, stream=0)
     assert call.keepalive == (args, {"stream": 0}) and call.keepalive[0][0] is args[0]
+
+
+def test_numbers_are_whatever_float_and_int_take(rac):
+    def steps(clip, T=0):
+        rac.rac_calibrate_steps(rac.CodecCfg(4096, 128, 4, 0), None, T, None, 0, None, None, None, clip, None, None, None, 0, None, stream=0)
+    for clip, T in ((3, 0), (3.0, "0"), ("3.0", 0.9), (torch.tensor(3.0), torch.tensor(0))):
+        with pytest.raises(rac.RacError) as e:      # marshalled; the library then misses the tables
+            steps(clip, T)
+        assert e.value.code == -1
+    for clip in (None, "three", object()):
+        with pytest.raises((TypeError, ValueError)):
+            steps(clip)
