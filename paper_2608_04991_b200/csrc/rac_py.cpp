@@ -218,6 +218,10 @@ bool marshal(const Entry &e, int k, PyObject *o, Slot *s) {
     return true;
 }
 bool marshal_all(const Entry &e, PyObject *const *args, Py_ssize_t n, Slot *s) {
+    if (!g_check) {
+        PyErr_SetString(PyExc_RuntimeError, "the module is set up by binding.load()");
+        return false;
+    }
     if (n != e.count) {
         PyErr_Format(PyExc_TypeError, "%s: expected %d arguments, got %zd", e.name, e.count, n);
         return false;
@@ -237,7 +241,6 @@ PyObject *finish(const Entry &e, const Slot *s) {
     rc = e.call(s);
     Py_END_ALLOW_THREADS
     if (rc == RAC_OK) Py_RETURN_NONE;
-    if (!g_check) return PyErr_Format(PyExc_RuntimeError, "%s failed: %d", e.name, rc);
     return PyObject_CallFunction(g_check, "si", e.name, rc);
 }
 

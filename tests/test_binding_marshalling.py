@@ -112,3 +112,13 @@ def test_numbers_are_whatever_float_and_int_take(rac):
     for clip in (None, "three", object()):
         with pytest.raises((TypeError, ValueError)):
             steps(clip)
+
+
+def test_extension_module_by_itself_raises(rac):
+    """Imported without binding.load(): an error, not a crash."""
+    import subprocess
+    import sys
+    code = ("import torch\nfrom paper_2608_04991_b200 import _native as n\n"
+            "try:\n    n.rac_index_reset(b'', 0, 0, 0)\nexcept RuntimeError as e:\n    print(e)")
+    out = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=rac.LIB_PATH.rsplit("/", 2)[0])
+    assert out.returncode == 0 and "binding.load()" in out.stdout
