@@ -191,7 +191,9 @@ int rac_match_spans_static(const int32_t *hist_tok, int64_t n_hist, const int32_
  *                      Appending requests one by one gives the same index as any other split into calls with the
  *                      same request boundaries: contents do not depend on thread timing.
  *   rac_index_query    the selection of Eq. 3 for one prompt against the indexed history: like rac_match_spans,
- *                      except that a match ends at the end of its request.  With intra != 0, every position that no
+ *                      except that a match ends at the end of its request.  n_hist is where the rows of intra-sequence
+ *                      references begin: the number of tokens in the index, or, say, of rows in the state buffer (<=
+ *                      capacity); the candidates are those of the index either way.  With intra != 0, every position that no
  *                      span covers and whose token occurred EARLIER in the prompt gets
  *                      ref_row = n_hist + (position of the first occurrence of that token in the prompt): a
  *                      reference to the reconstruction of that earlier token of the same prompt.  First occurrences

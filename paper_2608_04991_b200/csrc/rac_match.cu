@@ -51,6 +51,7 @@ struct MatchParams {
     int n_hist, n_query, nwin, w, K;
     unsigned int bmask;    // buckets - 1
     const int32_t *end_of; // [n_hist] end of the request that holds each history position; null = one request
+    const int32_t *indexed;// [1]      tokens the index holds (a query may name more or fewer); null = n_hist
     int first_live;        // only windows that start at or after this history position are candidates (0 = all)
     // intra-sequence references: a table of the prompt's tokens (TokenTable).  One cluster keeps it in shared memory.
     unsigned int *tok;     // [tmask + 1] else null
@@ -373,12 +374,19 @@ __global__ void __launch_bounds__(kChunk, ONE ? 1 : 2) match_query_kernel(const 
             cg::this_cluster().barrier_arrive();
         }
     }
-    if (!p.ahead) grid_dependency_wait();
+    int held_tokens = p.n_hist;           // no history token behind them is read
+    if (!p.ahead) {
+        grid_dependency_wait();
+        if (p.indexed) held_tokens = __ldcg(p.indexed);
+    }
     stage_tokens(s_tok, p.query, base, kChunk + p.w + 8, N);
     __syncthreads();
     const int32_t *win = s_tok + threadIdx.x;
     const u64 h = window_hash(win, p.w);
-    if (p.ahead) grid_dependency_wait();
+    if (p.ahead) {
+        grid_dependency_wait();
+        if (p.indexed) held_tokens = __ldcg(p.indexed);
+    }
     if (p.intra) {
         if constexpr (ONE) cg::this_cluster().barrier_wait();
         if (i < N) tt.insert(win[0], i);
@@ -425,8 +433,8 @@ __global__ void __launch_bounds__(kChunk, ONE ? 1 : 2) match_query_kernel(const 
         const int jj = max(j, 0), at = has_to_match(j);
         int32_t hh[8];
 #pragma unroll
-        for (int u = 0; u < 8; u++) hh[u] = p.hist[min(jj + p.w + u, p.n_hist - 1)];
-        const int32_t h_at = p.hist[min(jj + at, p.n_hist - 1)], q_at = p.query[min(i + at, N - 1)];
+        for (int u = 0; u < 8; u++) hh[u] = p.hist[min(jj + p.w + u, held_tokens - 1)];
+        const int32_t h_at = p.hist[min(jj + at, held_tokens - 1)], q_at = p.query[min(i + at, N - 1)];
         const int end_j = p.end_of ? p.end_of[jj] : p.n_hist;
         Candidate c;
         c.j = j;
@@ -548,7 +556,7 @@ __global__ void __launch_bounds__(kChunk, ONE ? 1 : 2) match_query_kernel(const 
                         int32_t tok[8];
 #pragma unroll
                         for (int r = 0; r < 8; r++)
-                            tok[r] = p.hist[min(max(v[r0 + r], 0) + has_to_match(v[r0 + r]), p.n_hist - 1)];
+                            tok[r] = p.hist[min(max(v[r0 + r], 0) + has_to_match(v[r0 + r]), held_tokens - 1)];
 #pragma unroll
                         for (int r = 0; r < 8; r++)
                             if (tok[r] != (v[r0 + r] > bestj ? q_last : q_beyond)) v[r0 + r] = -1;
@@ -757,6 +765,7 @@ struct IndexParams {
     int32_t *top;       // [capacity*K]
     int32_t *end_of;    // [capacity]
     int32_t *next;      // [capacity]  no cap on the hits: another start of the same window (chain link), else null
+    int32_t *indexed;   // [1]         tokens the index holds
     int a, b;           // the request: tokens [a, b)
     int w, K;
     unsigned int bmask;
@@ -771,6 +780,7 @@ __global__ void __launch_bounds__(64) index_append_kernel(const IndexParams p) {
     const int j = p.b - 1 - (int)(blockIdx.x * blockDim.x + threadIdx.x);   // the latest starts first
     if (j < p.a) return;
     p.end_of[j] = p.b;
+    if (j == p.b - 1) *p.indexed = p.b;
     if (j + p.w <= p.b)      // else the window would leave the request
         index_start(p.slots, p.top, p.next, p.bmask, p.hist, j, p.hist + j, p.w, p.K, window_hash(p.hist + j, p.w));
 }
@@ -966,7 +976,7 @@ int rac_match_spans_static(const int32_t *hist_tok, int64_t n_hist, const int32_
 // ---- persistent index ------------------------------------------------------------------------
 namespace {
 struct IndexLayout {
-    size_t slots, top, filled, end_of, next, total;
+    size_t slots, top, filled, end_of, next, indexed, total;
     unsigned int M;
 };
 bool index_cfg_ok(const rac_index_cfg *c) {
@@ -982,6 +992,7 @@ IndexLayout index_layout(const rac_index_cfg *c) {
     L.filled = o;
     L.end_of = o;   o = align16(o + (size_t)c->capacity * 4);
     L.next = o;     o = align16(o + (size_t)c->capacity * 4);
+    L.indexed = o;  o = align16(o + 4);
     L.total = o;
     return L;
 }
@@ -1014,8 +1025,9 @@ int rac_index_reset(const rac_index_cfg *cfg, void *index, size_t index_bytes, v
     const IndexLayout L = index_layout(cfg);
     if (index_bytes < L.total) return RAC_ESIZE;
     const long long n16 = (long long)(L.filled / 16);
+    unsigned char *ix = static_cast<unsigned char *>(index);
     launch_after(fill_ones_kernel, fill_blocks(n16), 256, 0, static_cast<cudaStream_t>(stream),
-                 reinterpret_cast<uint4 *>(static_cast<unsigned char *>(index) + L.slots), n16, (int32_t *)nullptr);
+                 reinterpret_cast<uint4 *>(ix + L.slots), n16, reinterpret_cast<int32_t *>(ix + L.indexed));
     return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;
 }
 
@@ -1036,6 +1048,7 @@ int rac_index_append(const rac_index_cfg *cfg, void *index, size_t index_bytes, 
     p.top = reinterpret_cast<int32_t *>(ix + L.top);
     p.end_of = reinterpret_cast<int32_t *>(ix + L.end_of);
     p.next = cfg->max_hits == 0 ? reinterpret_cast<int32_t *>(ix + L.next) : nullptr;
+    p.indexed = reinterpret_cast<int32_t *>(ix + L.indexed);
     p.a = (int)n_before;
     p.b = (int)n_after;
     p.w = cfg->min_ngram;
@@ -1095,6 +1108,7 @@ int rac_index_query_live(const rac_index_cfg *cfg, const void *index, size_t ind
     p.next = cfg->max_hits == 0 ? const_cast<int32_t *>(reinterpret_cast<const int32_t *>(ix + L.next)) : nullptr;
     p.first_live = (int)first_live;
     p.end_of = reinterpret_cast<const int32_t *>(ix + L.end_of);
+    p.indexed = reinterpret_cast<const int32_t *>(ix + L.indexed);
     if (n_query == 0) {
         launch_after(fill_ones_kernel, 1, 32, 0, st, (uint4 *)nullptr, 0ll, n_spans);
         return cudaGetLastError() == cudaSuccess ? RAC_OK : RAC_ECUDA;

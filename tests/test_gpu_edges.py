@@ -226,6 +226,37 @@ def test_copy_that_resumes_after_a_changed_token(env):
         assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
 
 
+@pytest.mark.parametrize("N,K", [(600, 8), (4500, 8), (600, 0)])
+@pytest.mark.parametrize("named", [2000, 2990, 2999, 3000, 3500])
+def test_query_that_names_other_than_the_indexed_tokens(env, N, K, named):
+    """n_hist is where the rows of intra-sequence references begin: a caller may give the rows of its state buffer, more or fewer
+    than the tokens in the index.  The candidates are those of the index."""
+    rac, dev = env.rac, env.dev
+    rng = np.random.default_rng(named + N)
+    hist = rng.integers(0, 200, 3000).astype(np.int32)
+    cuts = [0, 900, 1970, 2985, 3000]
+    query = rng.integers(0, 3000, N).astype(np.int32)
+    for i in range(3, N - 40, 43):
+        L = int(rng.integers(4, 41))
+        j = int(rng.integers(1900, 3000 - L + 1))
+        query[i:i + L] = hist[j:j + L]
+    query[N - 15:] = hist[2985:]
+    cfg = rac.IndexCfg(3500, 3, K)
+    nb, nws = rac.rac_index_bytes(cfg), rac.rac_index_query_workspace_bytes(N)
+    mem, ws = (torch.full((n,), 0x5A, dtype=torch.uint8, device=dev) for n in (nb, nws))
+    h, q = torch.from_numpy(hist).to(dev), torch.from_numpy(query).to(dev)
+    rows = torch.full((N,), 12345, dtype=torch.int32, device=dev)
+    spans = torch.full((N // 3 + 1, 3), 777, dtype=torch.int32, device=dev)
+    n = torch.full((1,), -5, dtype=torch.int32, device=dev)
+    rac.rac_index_reset(cfg, mem, nb)
+    for a, b in zip(cuts, cuts[1:]):
+        rac.rac_index_append(cfg, mem, nb, h, a, b)
+    rac.rac_index_query(cfg, mem, nb, h, named, q, N, True, rows, spans, n, ws, nws)
+    o_rows, o_spans = env.orc.match_spans_req(hist, cuts, query, w=3, max_hits=K, intra=True)
+    o_rows[o_rows >= 3000] += named - 3000
+    assert np.array_equal(spans[:int(n.item())].cpu().numpy(), o_spans) and np.array_equal(rows.cpu().numpy(), o_rows)
+
+
 @pytest.mark.parametrize("N", [64, 512, 2048, 4096, 4097])
 @pytest.mark.parametrize("w,K", [(1, 8), (3, 2), (4, 3), (4, 8), (4, 16), (8, 8)])
 def test_edited_copies(env, N, w, K):
