@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(64) index_append_kernel(const IndexParams p) {
     const int j = p.b - 1 - (int)(blockIdx.x * blockDim.x + threadIdx.x);   // the latest starts first
     if (j < p.a) return;
     p.end_of[j] = p.b;
-    if (j == p.b - 1) *p.indexed = p.b;
+    if (j == p.b - 1) atomicMax(p.indexed, p.b);
     if (j + p.w <= p.b)      // else the window would leave the request
         index_start(p.slots, p.top, p.next, p.bmask, p.hist, j, p.hist + j, p.w, p.K, window_hash(p.hist + j, p.w));
 }

@@ -170,7 +170,7 @@ def test_index_and_token_table_at_cluster_edges(env, N, w, K, live):
     assert torch.all(rows[N:] == 12345) and torch.all(ws[nws:] == 0x5A)
 
 
-def _index_query(env, hist, cuts, query, w, K, intra):
+def _index_query(env, hist, requests, query, w, K, intra):
     rac, dev = env.rac, env.dev
     N, H = query.size, hist.size
     cfg = rac.IndexCfg(H, w, K)
@@ -181,8 +181,8 @@ def _index_query(env, hist, cuts, query, w, K, intra):
     spans = torch.full((N // w + 1, 3), 777, dtype=torch.int32, device=dev)
     n = torch.full((1,), -5, dtype=torch.int32, device=dev)
     rac.rac_index_reset(cfg, mem, nb)
-    for a, b in zip(cuts, cuts[1:]):
-        rac.rac_index_append(cfg, mem, nb, h, int(a), int(b))
+    for a, b in requests:
+        rac.rac_index_append(cfg, mem, nb, h, a, b)
     rac.rac_index_query(cfg, mem, nb, h, H, q, N, intra, rows, spans, n, ws, nws)
     return rows.cpu().numpy(), spans[:int(n.item())].cpu().numpy()
 
@@ -222,7 +222,7 @@ def test_copy_that_resumes_after_a_changed_token(env):
         assert o_spans[0, 2] == 12
         rows, spans = _match(env, hist, query, 4, 8)
         assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
-        rows, spans = _index_query(env, hist, [0, hist.size], query, 4, 8, False)
+        rows, spans = _index_query(env, hist, [(0, hist.size)], query, 4, 8, False)
         assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
 
 
@@ -257,6 +257,16 @@ def test_query_that_names_other_than_the_indexed_tokens(env, N, K, named):
     assert np.array_equal(spans[:int(n.item())].cpu().numpy(), o_spans) and np.array_equal(rows.cpu().numpy(), o_rows)
 
 
+def test_requests_in_any_order(env):
+    """The end of the index is that of its last token, not of the request that came last."""
+    rng = np.random.default_rng(12)
+    hist = rng.integers(0, 200, 2000).astype(np.int32)
+    query = np.concatenate([hist[1700:1760], rng.integers(0, 200, 30), hist[1960:], hist[300:350]]).astype(np.int32)
+    o_rows, o_spans = env.orc.match_spans_req(hist, [0, 800, 2000], query, w=3, max_hits=8)
+    rows, spans = _index_query(env, hist, [(800, 2000), (0, 800)], query, 3, 8, False)
+    assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
+
+
 @pytest.mark.parametrize("N", [64, 512, 2048, 4096, 4097])
 @pytest.mark.parametrize("w,K", [(1, 8), (3, 2), (4, 3), (4, 8), (4, 16), (8, 8)])
 def test_edited_copies(env, N, w, K):
@@ -269,7 +279,7 @@ def test_edited_copies(env, N, w, K):
         assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
         cuts = [0, 700, 2500, 2600, hist.size]
         for intra in (False, True):
-            rows, spans = _index_query(env, hist, cuts, query, w, K, intra)
+            rows, spans = _index_query(env, hist, list(zip(cuts, cuts[1:])), query, w, K, intra)
             o_rows, o_spans = env.orc.match_spans_req(hist, cuts, query, w=w, max_hits=K, intra=intra)
             assert np.array_equal(rows, o_rows) and np.array_equal(spans, o_spans)
 
