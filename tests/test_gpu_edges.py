@@ -445,3 +445,27 @@ def test_group_scales_in_calls_of_many_tokens(env, d, bits, kg, T, predictor):
     rows[::7] = -1
     gain, bias = s.predictor_gain_bias(d, 4, env.dev) if predictor else (None, None)
     P.round_trip_case(rac.CodecCfg(d, 128, bits, 0, scale_mode=1, topk_group=kg), X, R, rows, gain, bias)
+
+
+@pytest.mark.parametrize("d", [2048, 4096])
+def test_encode_with_x_hat_on_both_sides_of_the_step_registers(env, d):
+    """Identity rows without outliers, one token below and above the size from which rows of 4 and 8 KB leave the steps in memory:
+    the same records, and x_hat equal to the receiver's."""
+    s, rac, P = env.synth, env.rac, env.P
+    T = 80_000_000 // d + 1
+    gen = s.generator(d, env.dev)
+    X = s.activations(T, d, s.channel_scale(d, 4, env.dev), gen)
+    R = s.affine_noisy_reference(X, 128, gen)
+    step = (X[:2000].float().std(0, unbiased=False) / 7).half().float().clamp(min=2.0 ** -10).repeat(2, 1).contiguous()
+    inv = 1.0 / step
+    cfg = rac.CodecCfg(d, 128, 4, 0)
+    rec = rac.rac_record_bytes(cfg)
+    out = []
+    for n in (T, T - 1):
+        pay, xs, st = P.gpu_encode_reconstruct(cfg, X[:n], R[:n], None, None, None, step, inv)
+        xr, st2 = P.gpu_decode(cfg, pay, n, R[:n], None, None, None, step, env.dev)
+        assert st == 0 and st2 == 0 and torch.equal(xs.view(torch.int16), xr.view(torch.int16))
+        out.append(pay)
+    assert np.array_equal(out[0][:(T - 1) * rec], out[1])
+    P.compare_encode(cfg, out[0][-64 * rec:], s.bf16_bits(X[-64:]), s.bf16_bits(R[-64:]), None, None, None, step.cpu().numpy(),
+                     inv.cpu().numpy())
