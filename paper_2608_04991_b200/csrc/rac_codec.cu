@@ -1650,7 +1650,9 @@ int fill_common(const Geometry &g, CodecParams *p, long long T, const void *ref_
 
 // Encode with outliers, all tokens: the one-launch form.  The shape follows from the number of streaming warps; without x_hat
 // the widths 4096 and 5120 with groups of 128 or 64 channels have variants with these compiled in, and of those one for calls
-// in which every token has its reference row; with x_hat the width is compiled in for groups of 128.
+// in which every token has its reference row; with x_hat the width is compiled in for groups of 128.  Everything else has groups
+// of 128 and of 64 compiled in (groups of 64 read from the parameters / compiled in, 3-bit, four outliers: 195312 x 1536 527 / 501
+// us, 146484 x 2048 398 / 378, 585937 x 512 with x_hat 1187 / 1089; 4-bit, eight: 58593 x 5120 with x_hat 419 / 393).
 template <int BITS, int KT, bool XHAT, int NV, int NSEL, int MAXT, int MINB, int D>
 static int launch_top_shape(const Geometry &g, CodecParams &p, bool allref, cudaStream_t stream) {
     const int nt = g.nthreads + 32 * NSEL, smem = top_smem_layout(g.d, g.rec, (int)sizeof(TopSel<NSEL, XHAT>)).total;
@@ -1661,6 +1663,7 @@ static int launch_top_shape(const Geometry &g, CodecParams &p, bool allref, cuda
     } else if constexpr (D != 0) {
         return RAC_TOP(4, false);
     } else {
+        if (g.lpg == 2) return RAC_TOP(2, false);
         return g.lpg == 4 ? RAC_TOP(4, false) : RAC_TOP(0, false);
     }
 #undef RAC_TOP

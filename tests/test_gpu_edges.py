@@ -321,7 +321,8 @@ def test_one_launch_outliers_at_shape_edges(env, d, g, bits, k, T):
 
 @pytest.mark.parametrize("d,g,bits,k,T,predictor", [
     (32, 32, 4, 1, 40, False), (32, 32, 2, 16, 40, False), (256, 32, 3, 8, 40, True), (288, 32, 4, 16, 40, False),
-    (4096, 128, 4, 8, 700, False), (5120, 128, 2, 5, 300, True), (8160, 32, 3, 8, 50, False), (8192, 64, 4, 16, 1200, False)])
+    (1536, 64, 3, 4, 60, False), (4096, 128, 4, 8, 700, False),
+    (5120, 128, 2, 5, 300, True), (8160, 32, 3, 8, 50, False), (8192, 64, 4, 16, 1200, False)])
 def test_many_equal_residuals(env, d, g, bits, k, T, predictor):
     """Tokens whose outliers are looked for in the whole token: all-zero residuals, one magnitude everywhere, magnitudes that rise
     or fall from one piece of channels to the next (the 256 channels of a step, fewer and more), and a few levels at random.  The
