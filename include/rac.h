@@ -255,9 +255,10 @@ int rac_spans_to_rows(const rac_span *spans, const int32_t *n_spans, int64_t n_q
  *                                result can differ in its last bf16 bit from (alpha*r + beta) + round(code*step).
  *   payload   >= T*record bytes, 16-byte aligned; payload_cap is its capacity
  *   workspace >= rac_encode_workspace_bytes(cfg, T) bytes of scratch, 16-byte aligned (0 bytes, and NULL
- *             allowed, when cfg->topk == 0).  With outliers, the calls that also write x_hat and those over a token
- *             list are two launches: the streaming pass leaves the largest |e| of every 32-channel slab here (4*d/32
- *             bytes per token, rows padded to 16 bytes) and the outlier pass reads it.  Any call with outliers wants it.
+ *             allowed, when cfg->topk == 0).  Some calls with outliers are two launches (those over a token list, and
+ *             with x_hat some of more than 4096 channels): the streaming pass leaves the largest |e| of every
+ *             32-channel slab here (4*d/32 bytes per token, rows padded to 16 bytes) and the outlier pass reads it.
+ *             The others are one launch and do not touch it.  Which is which may change: any call with outliers wants it.
  * The encoder reads only inv_step on the device: keep inv_step[c] == 0 wherever step[c] == 0 ("code 0").
  * The per-group fit is taken in binary32 on the device; its result, rounded to binary16, is what both
  * ends use, so any rounding difference against a binary64 fit shows up only in `coef`. */

@@ -126,6 +126,7 @@ def load():
         raise RuntimeError(f"{LIB_PATH} is missing: build it with `python -m paper_2608_04991_b200.build` "
                            "(there is no CPU fallback)")
     l = C.CDLL(LIB_PATH)
+    # (the launching calls below go through `_native`; their signatures are for callers who use the library returned here)
     vp, i64, i32, sz = C.c_void_p, C.c_int64, C.c_int32, C.c_size_t
     cfgp = C.POINTER(CodecCfg)
     l.rac_version.restype = C.c_char_p

@@ -12,8 +12,9 @@
 // pieces (piece (j + lane/2) mod 4 in step j), which makes the 128-bit accesses bank-conflict free
 // on a plain linear row.
 //
-// Kernels: encode_ws_kernel (streaming pass of encode, optionally also the sender-side x_hat),
-// outlier_kernel (second launch of encode: the k largest |e| per token), decode_kernel and decode_ws_kernel
+// Kernels: encode_ws_kernel (encode without outliers, or the streaming pass of one with them; optionally also the sender-side
+// x_hat), outlier_kernel (second launch of some encodes with outliers: the k largest |e| per token), encode_top_kernel (both in
+// one launch, where that is the better form), decode_kernel and decode_ws_kernel
 // (receiver and sender reconstruction, with and without per-token outliers), split_waves_kernel (tokens that
 // reference the same prompt go second).  The kernels of the per-group-scale quantiser (Eq. 8 as printed) live in
 // rac_codec_dyn.cu; this file holds the C ABI of both.  Step tables, segment fit and reconstruction error: rac_calib.cu.
@@ -261,9 +262,10 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
 // LPG: lanes per alignment group as a compile-time constant (4 = groups of 128 channels, 2 = groups of 64), or 0 to
 // read it from the parameters; the constant removes the uniform branches of the shuffle reductions.
 // D: the hidden width as a compile-time constant (4096 and 5120 are compiled in), or 0 to read it from the parameters;
-// the constant folds the address arithmetic of the rows and stages (downlink call at 131072 x 5120: 0.671 -> 0.658 ms).
+// the constant folds the address arithmetic of the rows and stages (without outliers, 131072 x 5120 485 -> 458 us, x 4096 394 ->
+// 383 us; with x_hat and gathered rows 697 -> 685 us, there with eight outliers 861 -> 849 us in both launches).
 // REF: every token has a reference row (identity rows: no row list, a reference buffer): the per-token test and the
-// second row of the tables go away (downlink call 0.649 -> 0.634 ms).
+// second row of the tables go away (without outliers, 131072 x 5120 474 -> 458 us; with x_hat see launch_stream_lpg).
 template <int BITS, bool TOPK, bool XHAT, int MINB, bool SUB, int LPG = 0, int D = 0, bool REF = false>
 __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(const CodecParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -528,8 +530,8 @@ __device__ __noinline__ Winner select_whole_token(int d, int k, int coef_shift, 
 // bound this pass) overlap.
 constexpr int kOutPair = 2;
 
-// W: warps per CTA.  7 = four CTAs of 72 registers per SM (56 tokens in flight), the faster shape without x_hat;
-// 8 = three CTAs of 80 registers (48 tokens), which the variant that also patches x_hat prefers.
+// W: warps per CTA.  7 = four CTAs of 72 registers per SM (56 tokens in flight), 8 = three CTAs of 80 registers (48 tokens); see
+// launch_encode.
 template <int NV, int KT, bool SUB, int W>
 __global__ void __launch_bounds__(W * 32, W == 7 ? 4 : 3) outlier_kernel(const CodecParams p, const int bits) {
     constexpr int U = kOutPair;
@@ -1716,14 +1718,14 @@ static int launch_top(const Geometry &g, CodecParams &p, cudaStream_t stream) {
 
 // The streaming kernel of one call.  REF (every token has a reference row: identity rows) drops the test per token; with x_hat it
 // also keeps the thread's steps in registers, which is faster at every width (3 to 7 %, 8192 channels 40 %) but in one case: rows of
-// 4 or 8 KB in tensors that L2 does not hold, where all CTAs ask for the same few DRAM banks and a slower kernel asks less evenly
-// (131072 x 4096 583 us with REF, 528 without, 131072 x 2048 308 and 272; both forms are equal at 80 M channels).  Register variants: 64 Ki registers hold two CTAs of 160 threads at 128 registers a
+// 4 or 8 KB in tensors that L2 does not hold (131072 x 4096 583 us with REF, 528 without, 131072 x 2048 308 and 272; both forms are
+// equal at 80 M channels; 3840 and 4352 channels 3 and 6 % faster with it, as everywhere else).  Register variants: 64 Ki registers hold two CTAs of 160 threads at 128 registers a
 // thread beside a third, or four at 96.  Without x_hat four CTAs are the better ones; with x_hat the kernel reads both step
 // tables every token, and at four CTAs per SM the shared-memory carve-out leaves too little L1 for them.
 template <int BITS, bool TOPK, bool XHAT, int LPG, int D>
 static int launch_stream_lpg(const Geometry &g, CodecParams &p, size_t smem, long long max_ctas, cudaStream_t stream) {
-    const bool camped = XHAT && (g.d == 2048 || g.d == 4096) && p.T * g.d > 80'000'000;
-    const bool allref = p.ref_row == nullptr && p.ref_base != nullptr && !camped;
+    const bool long_pow2 = XHAT && (g.d == 2048 || g.d == 4096) && p.T * g.d > 80'000'000;
+    const bool allref = p.ref_row == nullptr && p.ref_base != nullptr && !long_pow2;
 #define RAC_STREAM(M, R) \
     launch_persistent(encode_ws_kernel<BITS, TOPK, XHAT, M, false, LPG, D, R>, p, g.nthreads, smem, max_ctas, stream)
     if constexpr (XHAT) {
@@ -1791,7 +1793,8 @@ static int launch_encode(const Geometry &g, CodecParams &p, long long max_ctas, 
     // A warp per pair of tokens.  Many rounds of them, or a token list: three CTAs of eight warps (80 registers, 48 tokens per
     // SM); few rounds: four CTAs of seven warps (72 registers, 56 tokens).  With more work than one round, every warp gets the
     // same number of rounds (a grid of whole rounds, not a full grid with a ragged last round).
-    // (measured at 131072 x 5120: 0.901 against 0.910 ms; with few rounds the smaller CTAs win: 16384 x 4096 0.105 -> 0.102 ms)
+    // (x_hat, gathered rows, eight against seven warps, both launches: 131072 x 5120 846 / 850 us, 8000 x 8192 115 / 112 and 30000 x
+    // 8192 392 / 391, 14000 x 5120 99 / 100)
     const bool wide = sub || p.T > (long long)di.sms * 3 * 8 * kOutPair * 6;
     const int wpc = wide ? 8 : 7;
     const long long per_cta = wpc * kOutPair;
