@@ -1719,9 +1719,10 @@ static int launch_top(const Geometry &g, CodecParams &p, cudaStream_t stream) {
 // The streaming kernel of one call.  REF (every token has a reference row: identity rows) drops the test per token; with x_hat it
 // also keeps the thread's steps in registers, which is faster at every width (3 to 7 %, 8192 channels 40 %) but in one case: rows of
 // 4 or 8 KB in tensors that L2 does not hold (131072 x 4096 583 us with REF, 528 without, 131072 x 2048 308 and 272; both forms are
-// equal at 80 M channels; 3840 and 4352 channels 3 and 6 % faster with it, as everywhere else).  Register variants: 64 Ki registers hold two CTAs of 160 threads at 128 registers a
-// thread beside a third, or four at 96.  Without x_hat four CTAs are the better ones; with x_hat the kernel reads both step
-// tables every token, and at four CTAs per SM the shared-memory carve-out leaves too little L1 for them.
+// equal at 80 M channels; 3840 and 4352 channels 3 and 6 % faster with it, as everywhere else).  Register variants: 64 Ki registers
+// hold two CTAs of 160 threads at 128 registers a thread beside a third, or four at 96.  Without x_hat four CTAs are the better
+// ones; with x_hat the kernel reads both step tables every token, and at four CTAs per SM the shared-memory carve-out leaves too
+// little L1 for them.
 template <int BITS, bool TOPK, bool XHAT, int LPG, int D>
 static int launch_stream_lpg(const Geometry &g, CodecParams &p, size_t smem, long long max_ctas, cudaStream_t stream) {
     const bool long_pow2 = XHAT && (g.d == 2048 || g.d == 4096) && p.T * g.d > 80'000'000;
