@@ -94,14 +94,13 @@ __global__ void __launch_bounds__(kCalWarps * 32, MOMENTS ? 3 : 2) calib_kernel(
     for (int i = 0; i < 32; i++) acc0[i] = 0.f;
     int cnt_ref = 0, cnt_dir = 0;
     bool timed_out = false;
-    const unsigned int group_mask = 0xffffffffu;   // lanes beyond the row hold zeros and form groups of their own
 
     // one token in stage s; returns false when its data did not arrive
     auto token = [&](int k, int s, uint32_t parity) -> bool {
         const uint32_t xs = stage0 + s * kCalStageBytes;
         if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar0 + 8 * s, parity))) return false;
         const bool has_ref = ref_of[s];
-        uint32_t xw[16], rw[16];
+        uint32_t xw[16], rw[16];     // lanes beyond the row hold zeros and form groups of their own
 #pragma unroll
         for (int i = 0; i < 16; i++) { xw[i] = 0u; rw[i] = 0u; }
         if (valid) {
@@ -131,7 +130,7 @@ __global__ void __launch_bounds__(kCalWarps * 32, MOMENTS ? 3 : 2) calib_kernel(
             a2 = pack2(a, a);
             b2 = pack2(b, b);
         } else {
-            fit_group(xw, rw, has_ref, p.lpg, p.inv_group, group_mask, p.status, a2, b2, nullptr, &st);
+            fit_group_centred(xw, rw, has_ref, p.lpg, p.inv_group, p.status, a2, b2, st);
         }
         if (MOMENTS) {
             if (valid && (lane & (p.lpg - 1)) == 0) p.moments[tok * p.J + (slab >> p.lpg_shift)] = st;

@@ -239,6 +239,36 @@ __device__ __forceinline__ uint4 load_ref_words(uint32_t addr, const uint16_t *g
     return w;
 }
 
+// the thread's whole slab, slot order (off: byte offsets of its four slots in the row).  One test of the transform and all of its
+// loads before any is used: with a test per slot each slot was a trip of its own (300 x 8192 with x_hat 9.0 us, 8.0 so).
+__device__ __forceinline__ void load_ref_slab(uint32_t (&rw)[16], uint32_t rs, const uint32_t (&off)[4], const uint16_t *gain,
+                                              const uint16_t *bias) {
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const uint4 w = lds128(rs + off[j]);
+        rw[4 * j + 0] = w.x; rw[4 * j + 1] = w.y; rw[4 * j + 2] = w.z; rw[4 * j + 3] = w.w;
+    }
+    if (gain) {
+        uint4 gw[4], bw[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            gw[j] = __ldg(reinterpret_cast<const uint4 *>(gain + (off[j] >> 1)));
+            bw[j] = __ldg(reinterpret_cast<const uint4 *>(bias + (off[j] >> 1)));
+        }
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const uint32_t gws[4] = {gw[j].x, gw[j].y, gw[j].z, gw[j].w}, bws[4] = {bw[j].x, bw[j].y, bw[j].z, bw[j].w};
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const uint32_t w = rw[4 * j + i];
+                rw[4 * j + i] = f2_to_bf16x2(
+                    __fmaf_rn(half_bits_to_float(gws[i] & 0xffff), __uint_as_float(w << 16), half_bits_to_float(bws[i] & 0xffff)),
+                    __fmaf_rn(half_bits_to_float(gws[i] >> 16), __uint_as_float(w & 0xffff0000u), half_bits_to_float(bws[i] >> 16)));
+            }
+        }
+    }
+}
+
 // the same for one pair of channels (c even), operation for operation
 __device__ __forceinline__ u64 load_ref_pair(uint32_t addr, const uint16_t *gain, const uint16_t *bias, int c) {
     const uint32_t w = lds32(addr);
@@ -307,33 +337,50 @@ __device__ __forceinline__ void issue_token_loads(const CodecParams &p, Ctrl *ct
     if (row >= 0) bulk_load(stage_addr + r_off, ref_row_ptr<SUB>(p, row), row_bytes, bar);
 }
 
-// Eq. 6 for the group this thread belongs to: centred two-pass sums over the thread's 32 channels (rows as packed bf16
-// words; two accumulators per sum and channel parity), butterflies over the group's lanes, the zero-variance rule, and
-// wire rounding of (alpha, beta) to binary16.  Returns the wire coefficients splatted for packed arithmetic; a16/b16
-// are their bit patterns.  The rows stay packed and enter the sums through the mixed adds above: half the registers of
-// unpacked rows and no unpacking (streaming pass at 131072 x 5120, group 128, 4-bit: with outliers 528 -> 485 us, without
-// 516 -> 467 us, with x_hat 726 -> 700 us).
-__device__ __forceinline__ void fit_group(const uint32_t (&xw)[16], const uint32_t (&rw)[16], bool has_ref, int lpg,
-                                          float inv_group, unsigned int group_mask, uint32_t *status, u64 &a2, u64 &b2,
-                                          uint32_t *coef_word = nullptr, float4 *stats = nullptr) {
-    float ra0 = 0.f, ra1 = 0.f, rb0 = 0.f, rb1 = 0.f, xa0 = 0.f, xa1 = 0.f, xb0 = 0.f, xb1 = 0.f;
+// c + the product of two bf16 halves of packed words: the product is exact, so the one rounding is that of the sum.
+__device__ __forceinline__ float fma_lo(uint32_t v, uint32_t w, float c) {
+    float r;
+    asm("{.reg .b16 l, h, m, n; mov.b32 {l, h}, %1; mov.b32 {m, n}, %2; fma.rn.f32.bf16 %0, l, m, %3;}" : "=f"(r) : "r"(v), "r"(w), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float fma_hi(uint32_t v, uint32_t w, float c) {
+    float r;
+    asm("{.reg .b16 l, h, m, n; mov.b32 {l, h}, %1; mov.b32 {m, n}, %2; fma.rn.f32.bf16 %0, h, n, %3;}" : "=f"(r) : "r"(v), "r"(w), "f"(c));
+    return r;
+}
+// Sums of v, and of v*w, over the thread's 32 channels (even channels, odd channels), two accumulators each.
+__device__ __forceinline__ float sum_slab(const uint32_t (&v)[16]) {
+    float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
-        ra0 = add_lo(rw[i], ra0); ra1 = add_hi(rw[i], ra1); rb0 = add_lo(rw[i + 1], rb0); rb1 = add_hi(rw[i + 1], rb1);
-        xa0 = add_lo(xw[i], xa0); xa1 = add_hi(xw[i], xa1); xb0 = add_lo(xw[i + 1], xb0); xb1 = add_hi(xw[i + 1], xb1);
+        p0 = add_lo(v[i], p0); p1 = add_hi(v[i], p1);
+        p2 = add_lo(v[i + 1], p2); p3 = add_hi(v[i + 1], p3);
     }
-    float sr = (ra0 + rb0) + (ra1 + rb1), sh = (xa0 + xb0) + (xa1 + xb1);
+    return (p0 + p2) + (p1 + p3);
+}
+__device__ __forceinline__ float2 dot_slab(const uint32_t (&v)[16], const uint32_t (&w)[16]) {
+    float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) {
+        p0 = fma_lo(v[i], w[i], p0); p1 = fma_hi(v[i], w[i], p1);
+        p2 = fma_lo(v[i + 1], w[i + 1], p2); p3 = fma_hi(v[i + 1], w[i + 1], p3);
+    }
+    return make_float2(p0 + p2, p1 + p3);
+}
+// butterflies over the lanes of a group, two values at a time
+__device__ __forceinline__ void group_sum2(float &a, float &b, int lpg, unsigned int group_mask) {
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         if (lpg > o) {
-            sr += __shfl_xor_sync(group_mask, sr, o);
-            sh += __shfl_xor_sync(group_mask, sh, o);
+            a += __shfl_xor_sync(group_mask, a, o);
+            b += __shfl_xor_sync(group_mask, b, o);
         }
     }
-    if (!(fabsf(sr) <= 3.0e38f) || !(fabsf(sh) <= 3.0e38f)) {
-        if (status) atomicOr(status, RAC_STATUS_NONFINITE);
-    }
-    const float rbar = sr * inv_group, hbar = sh * inv_group;
+}
+
+// sums of the centred values' products over the group
+__device__ __forceinline__ void centred_sums(const uint32_t (&xw)[16], const uint32_t (&rw)[16], float rbar, float hbar, int lpg,
+                                             unsigned int group_mask, float &sxx, float &sxy) {
     u64 sxxa = 0ull, sxxb = 0ull, sxya = 0ull, sxyb = 0ull;
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
@@ -343,20 +390,15 @@ __device__ __forceinline__ void fit_group(const uint32_t (&xw)[16], const uint32
         sxxa = pfma(dr0, dr0, sxxa); sxya = pfma(dr0, dh0, sxya);
         sxxb = pfma(dr1, dr1, sxxb); sxyb = pfma(dr1, dh1, sxyb);
     }
-    float sxx, sxx_hi, sxy, sxy_hi;
+    float sxx_hi, sxy_hi;
     unpack2(padd(sxxa, sxxb), sxx, sxx_hi);
     unpack2(padd(sxya, sxyb), sxy, sxy_hi);
     sxx += sxx_hi;
     sxy += sxy_hi;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        if (lpg > o) {
-            sxx += __shfl_xor_sync(group_mask, sxx, o);
-            sxy += __shfl_xor_sync(group_mask, sxy, o);
-        }
-    }
-    if (stats) *stats = make_float4(rbar, hbar, sxx, sxy);
-    // zero-variance rule, then wire rounding to binary16
+    group_sum2(sxx, sxy, lpg, group_mask);
+}
+// the zero-variance rule, then wire rounding to binary16: the coefficients splatted for packed arithmetic, and their bit patterns
+__device__ __forceinline__ uint32_t wire_coefficients(bool has_ref, float rbar, float hbar, float sxx, float sxy, u64 &a2, u64 &b2) {
     float a_star = 0.f, b_star = hbar;
     if (has_ref && sxx > 1e-12f && fabsf(sxy) < 65504.0f * sxx) {
         a_star = __fdiv_rn(sxy, sxx);
@@ -366,7 +408,71 @@ __device__ __forceinline__ void fit_group(const uint32_t (&xw)[16], const uint32
     const float a = half_bits_to_float(a16), b = half_bits_to_float(b16);
     a2 = pack2(a, a);
     b2 = pack2(b, b);
-    if (coef_word) *coef_word = a16 | (b16 << 16);
+    return a16 | (b16 << 16);
+}
+__device__ __forceinline__ void flag_nonfinite(float sr, float sh, uint32_t *status) {
+    if (!(fabsf(sr) <= 3.0e38f) || !(fabsf(sh) <= 3.0e38f)) {
+        if (status) atomicOr(status, RAC_STATUS_NONFINITE);
+    }
+}
+
+// Eq. 6 for the group this thread belongs to (rows as packed bf16 words), as the encoders take it.  Returns the bit patterns of the
+// wire coefficients, and the coefficients.
+//
+// The centred sums come out of one pass over the rows: Sxx = sum (r*r) - n*rbar^2 and Sxy = sum (r*h) - n*rbar*hbar, products of
+// bf16 being exact.  Every thread takes the means' part of its 32 channels out of its own sums before they are added up over the
+// group, which costs no rounding more than the sums have anyway.  With means small beside the spread -- activations -- this is
+// closer to 64 bits than sums of centred values, which are rounded one by one (error of alpha, rms, groups of 128: activations
+// 6.8e-8 so, 6.9e-8 centred; a walk's next state 6.6e-8 and 6.7e-8; channels of very different scales 8.1e-8 and 8.4e-8; a mean of a
+// quarter of the spread 6.7e-8 and 6.8e-8, of half of it 6.9e-8 and 6.8e-8).  Hence the line, kMeanRatio: a warp in which some
+// group has n*rbar^2 or n*hbar^2 above a quarter of the centred sum of squares takes the second, centred pass.  That of h is not
+// known, but it is at least Sxy^2 / Sxx; only where this does not suffice (references that have little to do with the token)
+// sum h*h is formed as well.
+// The encoders are bound by issue slots and, in long runs, by the board's power beside DRAM: per pair of channels this is 8
+// operations, and the products do not wait for the means, where two passes took 8 and 2 packed ones.  (131072 x 5120, eight
+// outliers 616 -> 590 us, uplink with x_hat and retrieval 943 -> 917; 20001 x 5120 by Eq. 8, both ends, 209.7 -> 208.0; the sums on the matrix
+// unit by mma.sync, sixteen of them per warp and token, were slower everywhere and truncate.)
+constexpr float kMeanRatio = 0.25f;
+__device__ __forceinline__ uint32_t fit_group(const uint32_t (&xw)[16], const uint32_t (&rw)[16], bool has_ref, int lpg,
+                                              float inv_group, unsigned int group_mask, uint32_t *status, u64 &a2, u64 &b2) {
+    float sr = has_ref ? sum_slab(rw) : 0.f, sh = sum_slab(xw), sxx = 0.f, sxy = 0.f;
+    group_sum2(sr, sh, lpg, group_mask);
+    const float rbar = sr * inv_group, hbar = sh * inv_group;
+    if (has_ref) {
+        const float2 rr = dot_slab(rw, rw), rh = dot_slab(rw, xw);
+        const float r32 = -32.0f * rbar;
+        sxx = rr.x + __fmaf_rn(r32, rbar, rr.y);
+        sxy = rh.x + __fmaf_rn(r32, hbar, rh.y);
+        group_sum2(sxx, sxy, lpg, group_mask);
+        // strict comparisons: whatever is infinite or no number ends in the second pass
+        const bool small_r = sr * rbar < kMeanRatio * sxx;
+        if (__builtin_expect(!__all_sync(group_mask, small_r && (sh * hbar) * sxx < (kMeanRatio * sxy) * sxy), 0)) {
+            const float2 hh = dot_slab(xw, xw);
+            float shh = hh.x + __fmaf_rn(-32.0f * hbar, hbar, hh.y);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1)
+                if (lpg > o) shh += __shfl_xor_sync(group_mask, shh, o);
+            if (!__all_sync(group_mask, small_r && sh * hbar < kMeanRatio * shh && shh < 1e30f && sxx < 1e30f)) {
+                flag_nonfinite(sr, sh, status);
+                centred_sums(xw, rw, rbar, hbar, lpg, group_mask, sxx, sxy);
+            }
+        }
+    } else {
+        flag_nonfinite(sr, sh, status);
+    }
+    return wire_coefficients(has_ref, rbar, hbar, sxx, sxy, a2, b2);
+}
+// The same by centred sums in any case, as the calibration takes it, and the statistics.  (There the rows are waited for, and the
+// one-pass form was slower: 4096 x 2880 with encode and error 50.2 us, 47.8 so.)
+__device__ __forceinline__ void fit_group_centred(const uint32_t (&xw)[16], const uint32_t (&rw)[16], bool has_ref, int lpg,
+                                                  float inv_group, uint32_t *status, u64 &a2, u64 &b2, float4 &stats) {
+    float sr = sum_slab(rw), sh = sum_slab(xw), sxx, sxy;
+    group_sum2(sr, sh, lpg, 0xffffffffu);
+    flag_nonfinite(sr, sh, status);
+    const float rbar = sr * inv_group, hbar = sh * inv_group;
+    centred_sums(xw, rw, rbar, hbar, lpg, 0xffffffffu, sxx, sxy);
+    stats = make_float4(rbar, hbar, sxx, sxy);
+    wire_coefficients(has_ref, rbar, hbar, sxx, sxy, a2, b2);
 }
 
 // ------------------------------------------------------------------------------------------------

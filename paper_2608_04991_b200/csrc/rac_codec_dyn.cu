@@ -184,11 +184,7 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_dyn_kernel
                 xw[4 * j + 0] = w.x; xw[4 * j + 1] = w.y; xw[4 * j + 2] = w.z; xw[4 * j + 3] = w.w;
             }
             if (has_ref) {
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    const uint4 w = load_ref_words(rs + off[j], p.gain, p.bias, (int)(off[j] >> 1));
-                    rw[4 * j + 0] = w.x; rw[4 * j + 1] = w.y; rw[4 * j + 2] = w.z; rw[4 * j + 3] = w.w;
-                }
+                load_ref_slab(rw, rs, off, p.gain, p.bias);
             } else {
 #pragma unroll
                 for (int i = 0; i < 16; i++) rw[i] = 0u;
@@ -202,8 +198,7 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_dyn_kernel
                 a2 = pack2(a, a);
                 b2 = pack2(b, b);
             } else {
-                uint32_t coef_word;
-                fit_group(xw, rw, has_ref, lpg, p.inv_group, group_mask, p.status, a2, b2, &coef_word);
+                const uint32_t coef_word = fit_group(xw, rw, has_ref, lpg, p.inv_group, group_mask, p.status, a2, b2);
                 if ((lane & (lpg - 1)) == 0) reinterpret_cast<uint32_t *>(rec)[tid >> lpg_shift] = coef_word;
             }
             // residual, and the largest magnitude of each slot of 8 channels

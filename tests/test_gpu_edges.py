@@ -470,3 +470,57 @@ def test_encode_with_x_hat_on_both_sides_of_the_step_registers(env, d):
     assert np.array_equal(out[0][:(T - 1) * rec], out[1])
     P.compare_encode(cfg, out[0][-64 * rec:], s.bf16_bits(X[-64:]), s.bf16_bits(R[-64:]), None, None, None, step.cpu().numpy(),
                      inv.cpu().numpy())
+
+
+# --------------------------------------------------------------------------------------------- the three ways of the fit
+@pytest.mark.parametrize("d,g", [(4096, 128), (3584, 64), (2880, 32), (8192, 1024), (5120, 256)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_fit_with_means_small_and_large_beside_the_spread(env, d, g, mode):
+    """Means that stay inside the one-pass form, means around its line (n*mean^2 a quarter of the centred sum of squares, of the
+    reference and of the token), references that say nothing about the token, constant and zero groups, all among the groups of
+    one warp and as whole tokens.  Coefficients against the oracle's binary64 fit by the protocol's windows; the rest bit for
+    bit."""
+    s, rac, P = env.synth, env.rac, env.P
+    T, J = 24, d // g
+    rng = np.random.default_rng(d + g)
+    r = rng.standard_normal((T, J, g))
+    h = 0.9 * r + 0.05 * rng.standard_normal((T, J, g))
+    kind = rng.integers(0, 8, (T, J))
+    kind[:8] = np.arange(8)[:, None]                      # tokens of one kind; the others mixed
+    pick = lambda k: (kind == k)[:, :, None]
+    r = r + 0.45 * pick(1) + 0.55 * pick(2) + 40.0 * pick(3)
+    h = h + 0.40 * pick(1) + 0.50 * pick(2) + 36.0 * pick(3) + 0.5 * pick(4)
+    h = np.where(pick(5), rng.standard_normal((T, J, g)) + 0.45, h)      # unrelated
+    r = np.where(pick(6), 1.25, np.where(pick(7), 0.0, r))
+    X = torch.from_numpy(h.reshape(T, d)).float().to(torch.bfloat16).to(env.dev)
+    R = torch.from_numpy(r.reshape(T, d)).float().to(torch.bfloat16).to(env.dev)
+    if mode == 0:
+        cfg = rac.CodecCfg(d, g, 4, 8)
+        step = np.full((2, d), 0.03125, np.float32)
+        P.round_trip_case(cfg, X, ref_base=R, step=step, inv_step=(np.float32(1) / step).astype(np.float32))
+    else:
+        P.round_trip_case(rac.CodecCfg(d, g, 4, 0, scale_mode=1, topk_group=1), X, ref_base=R)
+
+
+def test_fit_flags_values_that_are_not_finite(env):
+    """An infinity or a NaN in the token or in the reference, in one group of one token: the status bit, and the records of all
+    other tokens as without it."""
+    s, rac, P = env.synth, env.rac, env.P
+    d, T = 4096, 6
+    gen = s.generator(5, env.dev)
+    X = s.activations(T, d, s.channel_scale(d, 5, env.dev), gen)
+    R = s.affine_noisy_reference(X, 128, gen)
+    step = np.full((2, d), 0.03125, np.float32)
+    inv = (np.float32(1) / step).astype(np.float32)
+    cfg = rac.CodecCfg(d, 128, 4, 0)
+    rec = rac.rac_record_bytes(cfg)
+    clean, _, st = P.gpu_encode_reconstruct(cfg, X, R, None, None, None, torch.from_numpy(step).to(env.dev), torch.from_numpy(inv).to(env.dev))
+    assert st == 0
+    for bad in (float("inf"), float("nan"), -float("inf")):
+        for which in (0, 1):
+            x, r = X.clone(), R.clone()
+            (x, r)[which][3, 777] = bad
+            pay, _, st = P.gpu_encode_reconstruct(cfg, x, r, None, None, None, torch.from_numpy(step).to(env.dev), torch.from_numpy(inv).to(env.dev))
+            assert st & rac.STATUS_NONFINITE
+            keep = [t for t in range(T) if t != 3]
+            assert np.array_equal(pay.reshape(T, rec)[keep], clean.reshape(T, rec)[keep])
