@@ -180,7 +180,8 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
         float ev[8];
         uint32_t xh[4];
         uint32_t w = 0;
-        if (BITS == 3) {
+        if (BITS == 3 || XHAT) {
+            // clamped on both sides: 3-bit codes have no saturating pack, and with x_hat the float is used again
             uint32_t bits8[8];
 #pragma unroll
             for (int i = 0; i < 4; i++) {
@@ -203,9 +204,9 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
                     xh[i] = f2_to_bf16x2(x0, x1);
                 }
             }
-            w = pack8<BITS>(bits8);
+            w = pack8_sum<BITS>(bits8);
         } else {
-            // 4- and 2-bit codes: clamp from below in binary32, round by the magic add, take the integer
+            // 4- and 2-bit codes without x_hat: clamp from below in binary32, round by the magic add, take the integer
             // out of the mantissa and let the saturating pack clamp from above (its range is
             // [-2^(BITS-1), 2^(BITS-1)-1], whose upper end is Qmax)
 #pragma unroll
@@ -216,16 +217,10 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
                 unpack2(pmul(e, inv2[i]), v0, v1);
                 v0 = fmaxf(v0, -qmax);
                 v1 = fmaxf(v1, -qmax);
-                if (XHAT) { v0 = fminf(v0, qmax); v1 = fminf(v1, qmax); }  // the float is used again below
                 const u64 tt = padd(pack2(v0, v1), magic2);
                 unpack2(tt, t0, t1);
                 w = sat_pack2<BITS>((int)__float_as_uint(t1) - 0x4b400000, (int)__float_as_uint(t0) - 0x4b400000, w);
                 unpack2(e, ev[2 * i], ev[2 * i + 1]);
-                if (XHAT) {
-                    float x0, x1;
-                    unpack2(pfma(psub(tt, magic2), st2[i], rt), x0, x1);
-                    xh[i] = f2_to_bf16x2(x0, x1);
-                }
             }
         }
         words[j] = w;

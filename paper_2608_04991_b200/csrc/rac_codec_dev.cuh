@@ -184,6 +184,20 @@ __device__ __forceinline__ uint32_t pack8(const uint32_t (&b)[8]) {
     }
 }
 
+// The same for codes that lie in [-(2^(BITS-1) - 1), 2^(BITS-1) - 1], given as the bits of code + kMagic: one sum of the shifted
+// bits (a shift-and-add per code), whose constant part is taken out again; codes + 2^(BITS-1) fill their fields without carries.
+// 9 operations for eight codes, where selecting the bits field by field takes 15 (11 for 4 bits) and the saturating pack, which
+// wants the integers themselves, 12.  (3-bit encode of 16384 x 4096, eight outliers, 65.8 -> 62.3 us.)
+template <int BITS>
+__device__ __forceinline__ uint32_t pack8_sum(const uint32_t (&b)[8]) {
+    constexpr uint32_t ones = BITS == 4 ? 0x11111111u : BITS == 3 ? 0x00249249u : 0x00005555u;   // 1 in every field
+    constexpr uint32_t offset = ones << (BITS - 1);
+    uint32_t w = b[7];
+#pragma unroll
+    for (int i = 6; i >= 0; i--) w = (w << BITS) + b[i];
+    return (w + (offset - 0x4b400000u * ones)) ^ offset;
+}
+
 // Two signed integers saturated to BITS-bit two's complement and packed below the bits of c
 // (d = c << 2*BITS | sat(hi) << BITS | sat(lo)); BITS is 4 or 2.
 template <int BITS>
