@@ -119,13 +119,28 @@ __host__ __device__ inline WsSmem ws_smem_layout(int d, int rec, int stages, boo
     return s;
 }
 
+// Both step tables in shared memory, laid out by thread: the 16-byte pieces that a thread reads in one step of its work (for half h
+// of slot j piece 2j + h of the inverse steps; a slot's binary16 steps are one piece) stand side by side for all threads of a
+// token, so that a warp's access is 512 consecutive bytes.  Read in place a warp's access touches 32 cache lines (9 wavefronts of
+// the L1 data pipe against 4), and with x_hat the four rows of a width of 5120 are more than the L1 beside the stages.
+struct SlabTables {
+    uint32_t inv = 0, step = 0;            // this thread's first pieces
+    uint32_t pitch = 0;                    // bytes from one piece of a thread to its next
+    bool half_steps = false;               // the steps as binary16 (as binary32 where that does not hold them exactly)
+};
+__device__ __forceinline__ float4 lds128f(uint32_t addr) {
+    const uint4 w = lds128(addr);
+    return make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
+}
+
 // One thread's 32 channels of one token, rows and record in shared memory: Eq. 6, Eq. 7, Eq. 8 with the static table, packing,
 // the sender-side reconstruction (over the X row), and the largest |e| of the slab.
 // STEPREG: every token has a reference, and the thread holds its steps (row 0 of the table, slot order) in st0.
-template <int BITS, bool TOPK, bool XHAT, int LPG, bool STEPREG>
+template <int BITS, bool TOPK, bool XHAT, int LPG, bool STEPREG, bool TABLES = false>
 __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int lane, int rot, int d, int Jc, bool shared, int coff,
                                             const uint32_t (&off)[4], unsigned int group_mask, uint32_t xs, uint32_t rs,
-                                            bool has_ref, int seg, unsigned char *rec, float *tm, const u64 (&st0)[STEPREG ? 16 : 1]) {
+                                            bool has_ref, int seg, unsigned char *rec, float *tm, const u64 (&st0)[STEPREG ? 16 : 1],
+                                            const SlabTables tab = SlabTables()) {
     constexpr float qmax = (float)((1 << (BITS - 1)) - 1);
     const u64 magic2 = pack2(kMagic, kMagic);
     // ---- (1) the slab: 4 slots of 8 channels, slot j holds piece (j + rot) & 3
@@ -163,17 +178,39 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
 #pragma unroll
     for (int j = 0; j < 4; j++) {
         const int c = (int)(off[j] >> 1);
-        const float4 iv0 = __ldg(reinterpret_cast<const float4 *>(inv_tab + c));
-        const float4 iv1 = __ldg(reinterpret_cast<const float4 *>(inv_tab + c + 4));
+        float4 iv0, iv1;
+        if (TABLES) {
+            const uint32_t a = tab.inv + (has_ref ? 0u : 8u * tab.pitch) + 2 * j * tab.pitch;
+            iv0 = lds128f(a);
+            iv1 = lds128f(a + tab.pitch);
+        } else {
+            iv0 = __ldg(reinterpret_cast<const float4 *>(inv_tab + c));
+            iv1 = __ldg(reinterpret_cast<const float4 *>(inv_tab + c + 4));
+        }
         const u64 inv2[4] = {pack2(iv0.x, iv0.y), pack2(iv0.z, iv0.w), pack2(iv1.x, iv1.y), pack2(iv1.z, iv1.w)};
         u64 st2[4] = {0ull, 0ull, 0ull, 0ull};
         if (XHAT) {
             if (STEPREG) {
 #pragma unroll
                 for (int i = 0; i < 4; i++) st2[i] = st0[STEPREG ? 4 * j + i : 0];
+            } else if (TABLES && tab.half_steps) {
+                const uint4 w = lds128(tab.step + (has_ref ? 0u : 4u * tab.pitch) + j * tab.pitch);
+                const uint32_t hw[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&hw[i]));
+                    st2[i] = pack2(f.x, f.y);
+                }
             } else {
-                const float4 s0 = __ldg(reinterpret_cast<const float4 *>(step_tab + c));
-                const float4 s1 = __ldg(reinterpret_cast<const float4 *>(step_tab + c + 4));
+                float4 s0, s1;
+                if (TABLES) {
+                    const uint32_t a = tab.step + (has_ref ? 0u : 8u * tab.pitch) + 2 * j * tab.pitch;
+                    s0 = lds128f(a);
+                    s1 = lds128f(a + tab.pitch);
+                } else {
+                    s0 = __ldg(reinterpret_cast<const float4 *>(step_tab + c));
+                    s1 = __ldg(reinterpret_cast<const float4 *>(step_tab + c + 4));
+                }
                 st2[0] = pack2(s0.x, s0.y); st2[1] = pack2(s0.z, s0.w); st2[2] = pack2(s1.x, s1.y); st2[3] = pack2(s1.z, s1.w);
             }
         }
@@ -253,7 +290,7 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
 // read it from the parameters; the constant removes the uniform branches of the shuffle reductions.
 // D: the hidden width as a compile-time constant (4096 and 5120 are compiled in), or 0 to read it from the parameters;
 // the constant folds the address arithmetic of the rows and stages (without outliers, 131072 x 5120 485 -> 458 us, x 4096 394 ->
-// 383 us; with x_hat and gathered rows 697 -> 685 us, there with eight outliers 861 -> 849 us in both launches).
+// 383 us; with x_hat and gathered rows 697 -> 685 us).
 // REF: every token has a reference row (identity rows: no row list, a reference buffer): the per-token test and the
 // second row of the tables go away (without outliers, 131072 x 5120 474 -> 458 us; with x_hat see launch_stream_lpg).
 template <int BITS, bool TOPK, bool XHAT, int MINB, bool SUB, int LPG = 0, int D = 0, bool REF = false>
@@ -265,12 +302,12 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
     const int d = D ? D : p.d;
     const bool valid = tid * 32 < d;
     constexpr int S = 2;   // stages of the ring (the host sets p.stages to the same)
-    // with the width and the group compiled in, the record geometry is a constant too (those variants are launched for
-    // no outliers or eight per token only)
+    // with the width and the group compiled in, the record geometry is a constant too (those variants are without outliers)
+    static_assert(!(TOPK && D != 0), "the geometry below has no outliers");
     constexpr bool kGeo = D != 0 && LPG != 0;
     const int Jc = kGeo ? D / (32 * (LPG ? LPG : 1)) : p.J;
     const int codeb = kGeo ? D * BITS / 8 : p.code_bytes;
-    const int recb = kGeo ? (4 * (D / (32 * (LPG ? LPG : 1))) + D * BITS / 8 + (TOPK ? 32 : 0) + 15) / 16 * 16 : p.rec;
+    const int recb = kGeo ? (4 * (D / (32 * (LPG ? LPG : 1))) + D * BITS / 8 + 15) / 16 * 16 : p.rec;
     const WsSmem L = ws_smem_layout(d, recb, S, TOPK);
     WsCtrl *ctrl = reinterpret_cast<WsCtrl *>(smem);
     const uint32_t sbase = smem_u32(smem);
@@ -790,6 +827,14 @@ __global__ void __launch_bounds__(W * 32, W == 7 ? 4 : 3) outlier_kernel(const C
 // 0.601); at 16384 x 4096 4 CTAs of 4 + 2 66 us, 4 of 4 + 3 68, 5 of 4 + 2 72 (two launches 81).  Reading the slabs from the
 // stage and refilling it afterwards was slower in every shape.  With x_hat the CTAs keep two selectors and the registers that
 // three of them per SM leave; see one_launch for where that form is the better one.
+//
+// Teams: with x_hat a token needs the inverse steps and the steps, in calls with direct tokens two rows of each, and several CTAs
+// per SM each with their stages leave them too little L1.  So in calls of many tokens an SM runs ONE CTA of several teams, each
+// of which is what is a CTA otherwise (its streaming and selector warps, stages and barriers), and all of them read one copy of the tables in
+// shared memory (SlabTables).  131072 x 5120, 28 % direct tokens, in long runs: 759 us against 915 with a CTA per token and 717
+// and about 130 in two launches; 100000 x 4096 487 -> 439, x 3072 382 -> 348, x 6144 708 against 704 and about 100; long uplink with
+// retrieval 926 -> 812.  (More teams with fewer registers, four at 4096 channels, 437 and spills.)
+// Teams without x_hat (one row in L1 is no trouble there) 574 against 568.
 struct TopCtrl {
     unsigned long long full[2];     // data of the stage has landed
     unsigned long long done[4];     // every streaming warp has finished token (mod 4)
@@ -822,11 +867,13 @@ __host__ __device__ inline TopSmem top_smem_layout(int d, int rec, int sel_bytes
 }
 
 // NV: slab maxima per lane (d <= 1024 * NV).  KT: the number of outliers when it is 8, else 0 = p.topk.  LPG, D, REF: as for
-// encode_ws_kernel.
-template <int BITS, int KT, bool XHAT, int NV, int NSEL, int MAXT, int MINB, int LPG, int D = 0, bool REF = false>
+// encode_ws_kernel.  TEAMS > 1: tables in shared memory; no gain and bias (they would be read past an L1 that is not there).
+template <int BITS, int KT, bool XHAT, int NV, int NSEL, int MAXT, int MINB, int LPG, int D = 0, bool REF = false, int TEAMS = 1>
 __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParams p) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    const int tid = threadIdx.x, nt = blockDim.x;
+    extern __shared__ __align__(128) unsigned char smem_all[];
+    // everything below is about this thread's team
+    const int nt = TEAMS == 1 ? blockDim.x : blockDim.x / TEAMS, team = TEAMS == 1 ? 0 : threadIdx.x / nt;
+    const int tid = TEAMS == 1 ? threadIdx.x : threadIdx.x - team * nt;
     const int lane = tid & 31, warp = tid >> 5, nstream = D ? (D / 32 + 31) / 32 : (nt >> 5) - NSEL;
     const int rot = (lane >> 1) & 3;
     const int d = D ? D : p.d;
@@ -836,11 +883,12 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
     const int recb = kGeo ? (4 * (D / (32 * (LPG ? LPG : 1))) + D * BITS / 8 + 32 + 15) / 16 * 16 : p.rec;
     const int coff = 4 * Jc;
     const TopSmem L = top_smem_layout(d, recb, (int)sizeof(TopSel<NSEL, XHAT>));
+    unsigned char *smem = smem_all + (TEAMS == 1 ? 0 : team * align_up(L.total, 128));
     TopCtrl *ctrl = reinterpret_cast<TopCtrl *>(smem);
     const uint32_t sbase = smem_u32(smem);
     const uint32_t row_bytes = 2u * (uint32_t)d;
 
-    if (p.T <= gridDim.x) grid_launch_dependents();
+    if (TEAMS == 1 && p.T <= gridDim.x) grid_launch_dependents();
     if (tid == 0) {
         for (int s = 0; s < 2; s++) mbar_init(smem_u32(&ctrl->full[s]), 1);
         for (int s = 0; s < 4; s++) {
@@ -859,8 +907,49 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
     }
     __syncthreads();
     grid_dependency_wait();
-    const int first = blockIdx.x, stride = gridDim.x;
-    const int n_my = (p.T > first) ? (int)((p.T - first + stride - 1) / stride) : 0;
+    int teams = TEAMS;       // at work
+    SlabTables tab;
+    if constexpr (TEAMS > 1) {
+        const bool mine = warp < nstream && tid * 32 < d;
+        const uint32_t t0 = smem_u32(smem_all) + TEAMS * align_up(L.total, 128);
+        tab.pitch = (uint32_t)nstream * 512u;
+        tab.inv = t0 + tid * 16u;
+        tab.step = tab.inv + 16u * tab.pitch;
+        tab.half_steps = true;
+        // row r, slot j of both tables by team (4r + j) mod TEAMS
+        for (int q = team; mine && q < 8; q += TEAMS) {
+            const int r = q >> 2, j = q & 3, c = r * d + tid * 32 + ((j + rot) & 3) * 8;
+            const uint4 i0 = __ldg(reinterpret_cast<const uint4 *>(p.inv_step + c)), i1 = __ldg(reinterpret_cast<const uint4 *>(p.inv_step + c + 4));
+            sts128(tab.inv + (8 * r + 2 * j) * tab.pitch, i0);
+            sts128(tab.inv + (8 * r + 2 * j + 1) * tab.pitch, i1);
+            const float4 s0 = __ldg(reinterpret_cast<const float4 *>(p.step + c)), s1 = __ldg(reinterpret_cast<const float4 *>(p.step + c + 4));
+            const float v[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+            uint32_t hw[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const __half2 h = __floats2half2_rn(v[2 * i], v[2 * i + 1]);
+                const float2 back = __half22float2(h);
+                tab.half_steps = tab.half_steps && back.x == v[2 * i] && back.y == v[2 * i + 1];
+                hw[i] = *reinterpret_cast<const uint32_t *>(&h);
+            }
+            sts128(tab.step + (4 * r + j) * tab.pitch, make_uint4(hw[0], hw[1], hw[2], hw[3]));
+        }
+        tab.half_steps = __syncthreads_and(tab.half_steps) != 0;
+        if (!tab.half_steps) {
+            // Steps that binary16 does not hold (calibrated tables are binary16 values): the last team stands back and its stages
+            // hold them as they are (the host sees to it that they fit).
+            teams = TEAMS - 1;
+            tab.step = smem_u32(smem_all) + (TEAMS - 1) * align_up(L.total, 128) + L.stage0 + tid * 16u;
+            for (int q = team; mine && q < 8; q += TEAMS) {
+                const int r = q >> 2, j = q & 3, c = r * d + tid * 32 + ((j + rot) & 3) * 8;
+                sts128(tab.step + (8 * r + 2 * j) * tab.pitch, __ldg(reinterpret_cast<const uint4 *>(p.step + c)));
+                sts128(tab.step + (8 * r + 2 * j + 1) * tab.pitch, __ldg(reinterpret_cast<const uint4 *>(p.step + c + 4)));
+            }
+            __syncthreads();
+        }
+    }
+    const int first = blockIdx.x + gridDim.x * team, stride = gridDim.x * teams;
+    const int n_my = (team < teams && p.T > first) ? (int)((p.T - first + stride - 1) / stride) : 0;
     auto token = [&](int k) -> long long { return first + (long long)k * stride; };   // this CTA's k-th token
     auto raw_row_of = [&](int k) -> int { return p.ref_row ? p.ref_row[token(k)] : (int)token(k); };
     // one lane: start the copies of this CTA's k-th token
@@ -892,9 +981,9 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
             if (!__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&ctrl->full[stage]), parity))) { timed_out = true; break; }
             const bool has_ref = REF ? true : ctrl->row[stage] >= 0;
             if (valid)
-                encode_slab<BITS, true, XHAT, LPG, false>(p, tid, lane, rot, d, Jc, false, coff, off, group_mask, xs, xs + row_bytes,
+                encode_slab<BITS, true, XHAT, LPG, false, (TEAMS > 1)>(p, tid, lane, rot, d, Jc, false, coff, off, group_mask, xs, xs + row_bytes,
                                                     has_ref, 0, stg + L.rec_off + parity * recb,
-                                                    reinterpret_cast<float *>(stg + L.tm_off), no_steps);
+                                                    reinterpret_cast<float *>(stg + L.tm_off), no_steps, tab);
             fence_async_smem();     // the record bytes written above will be read by the copy engine
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&ctrl->done[it & 3])) : "memory");
@@ -1695,6 +1784,44 @@ static bool one_launch(const Geometry &g, const CodecParams &p) {
     if (g.nthreads <= 160) return p.ref_row == nullptr || p.T <= 8192;
     return p.T <= 1024;
 }
+// The one-launch form in teams: with x_hat, from 2080 to 7168 channels, where one CTA's shared memory holds the teams and the tables,
+// in calls of so many tokens that the tables' way there and the CTA's longer start are made up for.  NS: most streaming warps of
+// a team.  Tokens (CTA per token, or two launches in parentheses / teams, us): gathered rows 3000 x 5120 28.9 / 27.1, 6000 x 5120 51.2 /
+// 44.7, identity rows 6000 x 5120 44.2 / 46.4, 12000 x 5120 82.9 / 80.6; 2048 x 4096 16.5 / 16.6, 12000 x 4096 61.7 / 58.3; 2048 x 3072
+// 13.9 / 14.7, 12000 x 3072 50.9 / 49.0; 2048 x 6144 (about 25) / 24.4, 12000 x 6144 (about 103) / 94.4.
+template <int BITS, int KT, int NV, int NS, int NSEL, int TEAMS, int D>
+static int launch_teams_shape(const Geometry &g, CodecParams &p, const DeviceInfo &di, cudaStream_t stream) {
+    const TopSmem L = top_smem_layout(g.d, g.rec, (int)sizeof(TopSel<NSEL, true>));
+    const int table = g.nthreads * 16;                  // bytes of a piece for all threads of a token
+    const int smem = TEAMS * align_up(L.total, 128) + 24 * table, nt = TEAMS * (g.nthreads + 32 * NSEL);
+    if (smem > di.max_smem_optin || 16 * table > 2 * L.stage_bytes) return RAC_EUNSUPPORTED;
+    constexpr int kMaxT = TEAMS * 32 * (NS + NSEL);
+#define RAC_TEAMS(G, W) launch_persistent(encode_top_kernel<BITS, KT, true, NV, NSEL, kMaxT, 1, G, W, false, TEAMS>, p, nt, smem, p.T, stream)
+    if (D != 0 && g.d == D && g.lpg == 4) return RAC_TEAMS(4, D);
+    if (g.lpg == 2) return RAC_TEAMS(2, 0);
+    return g.lpg == 4 ? RAC_TEAMS(4, 0) : RAC_TEAMS(0, 0);
+#undef RAC_TEAMS
+}
+// RAC_EUNSUPPORTED: not a call for them
+static int launch_teams(const Geometry &g, CodecParams &p, cudaStream_t stream) {
+    if (!p.X_hat || p.gain || g.nthreads <= 64 || g.nthreads > 224) return RAC_EUNSUPPORTED;
+    DeviceInfo di;
+    if (int rc = device_info(&di)) return rc;
+    const long long per_sm = g.nthreads > 160 || (g.nthreads > 128 && p.ref_row) ? 20 : 54;
+    if (p.T < per_sm * di.sms) return RAC_EUNSUPPORTED;
+#define RAC_TEAMS(B, K)                                                                             \
+    (g.nthreads <= 96    ? launch_teams_shape<B, K, 3, 3, 2, 4, 0>(g, p, di, stream)                 \
+     : g.nthreads <= 128 ? launch_teams_shape<B, K, 4, 4, 2, 3, K == 8 ? 4096 : 0>(g, p, di, stream) \
+     : g.nthreads <= 160 ? launch_teams_shape<B, K, 5, 5, 3, 3, K == 8 ? 5120 : 0>(g, p, di, stream) \
+                         : launch_teams_shape<B, K, 7, 7, 2, 2, 0>(g, p, di, stream))
+    switch (g.bits) {
+        case 4: return g.topk == 8 ? RAC_TEAMS(4, 8) : RAC_TEAMS(4, 0);
+        case 3: return g.topk == 8 ? RAC_TEAMS(3, 8) : RAC_TEAMS(3, 0);
+        case 2: return g.topk == 8 ? RAC_TEAMS(2, 8) : RAC_TEAMS(2, 0);
+    }
+#undef RAC_TEAMS
+    return RAC_EUNSUPPORTED;
+}
 static int launch_top(const Geometry &g, CodecParams &p, cudaStream_t stream) {
 #define RAC_TOPB(B) (g.topk == 8 ? launch_top_bits<B, 8>(g, p, stream) : launch_top_bits<B, 0>(g, p, stream))
     switch (g.bits) {
@@ -1720,10 +1847,7 @@ static int launch_stream_lpg(const Geometry &g, CodecParams &p, size_t smem, lon
 #define RAC_STREAM(M, R) \
     launch_persistent(encode_ws_kernel<BITS, TOPK, XHAT, M, false, LPG, D, R>, p, g.nthreads, smem, max_ctas, stream)
     if constexpr (XHAT) {
-        if constexpr (!(TOPK && D != 0)) {   // (at that width, identity rows with outliers are always one launch)
-            if (allref) return RAC_STREAM(2, true);
-        }
-        return RAC_STREAM(2, false);
+        return allref ? RAC_STREAM(2, true) : RAC_STREAM(2, false);
     } else if constexpr (D != 0) {
         return allref ? RAC_STREAM(4, true) : RAC_STREAM(4, false);
     } else {
@@ -1732,18 +1856,17 @@ static int launch_stream_lpg(const Geometry &g, CodecParams &p, size_t smem, lon
 #undef RAC_STREAM
 }
 
-// Widths 4096 and 5120 have variants with the record geometry compiled in; 4096 with outliers is always one launch (one_launch),
-// and so is every call with outliers and without x_hat: what those would need is not instantiated.
+// Widths 4096 and 5120 without outliers have variants with the record geometry compiled in.  With outliers 4096 is always one
+// launch and 5120 comes here with a predictor in front only; every call with outliers and without x_hat is one launch (launch_teams,
+// one_launch): what those would need is not instantiated.
 template <int BITS, bool TOPK, bool XHAT>
 static int launch_stream(const Geometry &g, CodecParams &p, size_t smem, long long max_ctas, cudaStream_t stream) {
     if (p.tok_list || p.intra_base || p.coef_ext)   // the subset form has one variant: it is not the hot path
         return launch_persistent(encode_ws_kernel<BITS, TOPK, XHAT, 2, true, 0>, p, g.nthreads, smem, max_ctas, stream);
     if constexpr (!TOPK || XHAT) {
-        if (g.d == 5120 && (!TOPK || g.topk == 8)) {
-            if (g.lpg == 4) return launch_stream_lpg<BITS, TOPK, XHAT, 4, 5120>(g, p, smem, max_ctas, stream);
-            if (g.lpg == 2) return launch_stream_lpg<BITS, TOPK, XHAT, 2, 5120>(g, p, smem, max_ctas, stream);
-        }
         if constexpr (!TOPK) {
+            if (g.d == 5120 && g.lpg == 4) return launch_stream_lpg<BITS, TOPK, XHAT, 4, 5120>(g, p, smem, max_ctas, stream);
+            if (g.d == 5120 && g.lpg == 2) return launch_stream_lpg<BITS, TOPK, XHAT, 2, 5120>(g, p, smem, max_ctas, stream);
             if (g.d == 4096 && g.lpg == 4) return launch_stream_lpg<BITS, TOPK, XHAT, 4, 4096>(g, p, smem, max_ctas, stream);
             if (g.d == 4096 && g.lpg == 2) return launch_stream_lpg<BITS, TOPK, XHAT, 2, 4096>(g, p, smem, max_ctas, stream);
         }
@@ -1768,7 +1891,11 @@ static int launch_encode(const Geometry &g, CodecParams &p, long long max_ctas, 
     if (g.scale_mode == 1) return launch_encode_dyn(g, p, max_ctas, stream);
     const bool topk = g.topk > 0;
     const bool sub = p.tok_list || p.intra_base || p.coef_ext;
-    if (topk && !sub && one_launch(g, p)) return launch_top(g, p, stream);
+    if (topk && !sub) {
+        const int rc = launch_teams(g, p, stream);
+        if (rc != RAC_EUNSUPPORTED) return rc;
+        if (one_launch(g, p)) return launch_top(g, p, stream);
+    }
     p.stages = 2;
     const size_t smem = ws_smem_layout(g.d, g.rec, p.stages, topk).total;
     int rc = RAC_EUNSUPPORTED;

@@ -524,3 +524,52 @@ def test_fit_flags_values_that_are_not_finite(env):
             assert st & rac.STATUS_NONFINITE
             keep = [t for t in range(T) if t != 3]
             assert np.array_equal(pay.reshape(T, rec)[keep], clean.reshape(T, rec)[keep])
+
+
+# ------------------------------------------------------------------- one launch with x_hat: teams of one CTA per SM, from a size on
+@pytest.mark.parametrize("d,g,bits,k,per_sm,gathered", [
+    (5120, 128, 4, 8, 20, True),      # three teams, width compiled in
+    (5120, 64, 3, 5, 54, False),
+    (4128, 32, 2, 16, 20, True),      # five warps, the last with one lane
+    (5120, 32, 4, 16, 20, True),      # three teams and the tables do not fit: the other forms
+    (4096, 128, 4, 8, 54, True),      # three teams, width compiled in
+    (4096, 256, 3, 8, 54, True),
+    (2080, 32, 4, 8, 54, True),       # four teams of three warps, the last with one lane
+    (7168, 256, 2, 8, 20, True),      # two teams, the widest
+    (5376, 128, 4, 1, 20, False),
+    (7168, 128, 4, 8, 20, True),      # two teams do not fit
+])
+@pytest.mark.parametrize("table", ["binary16", "binary32"])
+def test_encode_in_teams_at_its_first_sizes(env, d, g, bits, k, per_sm, gathered, table):
+    """The last token count of the other forms and the first of this one, where a team gets one token more than another: records
+    as without x_hat (another kernel) and against the oracle, x_hat equal to the receiver's; steps that binary16 holds, and steps
+    that it does not (there one team stands back)."""
+    s, rac, P = env.synth, env.rac, env.P
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    T = per_sm * sms
+    gen = s.generator(d + bits, env.dev)
+    X = s.activations(T, d, s.channel_scale(d, 4, env.dev), gen)
+    R = s.affine_noisy_reference(X, g, gen)
+    rows = None
+    if gathered:
+        rows = torch.arange(T, dtype=torch.int32, device=env.dev)
+        rows[::5] = -1
+    step = torch.stack([torch.full((d,), 0.05, device=env.dev), X[:2000].float().std(0, unbiased=False) * (3.0 / 7)]).clamp(min=2.0 ** -10)
+    step = step.half().float() if table == "binary16" else step + step * 2.0 ** -14
+    inv = 1.0 / step
+    cfg = rac.CodecCfg(d, g, bits, k)
+    rec = rac.rac_record_bytes(cfg)
+    out = []
+    for n in (T, T - 1):
+        r = None if rows is None else rows[:n]
+        pay, xs, st = P.gpu_encode_reconstruct(cfg, X[:n], R[:n], r, None, None, step, inv)
+        plain, st2 = P.gpu_encode(cfg, X[:n], R[:n], r, None, None, step, inv)
+        xr, st3 = P.gpu_decode(cfg, pay, n, R[:n], r, None, None, step, env.dev)
+        assert st == 0 and st2 == 0 and st3 == 0
+        assert np.array_equal(pay, plain) and torch.equal(xs.view(torch.int16), xr.view(torch.int16))
+        out.append(pay)
+    assert np.array_equal(out[0][:(T - 1) * rec], out[1])
+    at = slice(T - 700, T)
+    P.compare_encode(cfg, out[0][(T - 700) * rec:], s.bf16_bits(X[at]), s.bf16_bits(R),
+                     np.arange(T - 700, T, dtype=np.int32) if rows is None else rows[at].cpu().numpy(), None, None,
+                     step.cpu().numpy(), inv.cpu().numpy())
