@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kCalWarps * 32, MOMENTS ? 3 : 2) calib_kernel(
 
 // Step tables from the per-partition sums: 32 channels per CTA, eight threads per channel, each adding every eighth
 // partition in binary64, then the eight in order (a fixed summation order -> deterministic).  One thread per channel and
-// all partitions in a row took 21 us at d = 2880 (a chain of 128 loads), this takes 5.6 us.
+// all partitions in a row took 21 us at d = 2880 (a chain of 128 loads), eight with four loads at a time 5.4; all sixteen are loaded at once now (one trip).
 constexpr int kFinSlices = 8;
 __global__ void __launch_bounds__(32 * kFinSlices) calib_finalize_kernel(const float *partial, int parts, int d, int bits,
                                                                          float clip_sigmas, float *step, float *inv_step) {
@@ -224,9 +224,13 @@ __global__ void __launch_bounds__(32 * kFinSlices) calib_finalize_kernel(const f
     grid_dependency_wait();
     const int *cnt = reinterpret_cast<const int *>(partial + (long long)parts * 2 * d);
     double sum = 0.0;
-#pragma unroll 4
-    for (int b = slice; b < parts; b += kFinSlices) sum += (double)partial[(long long)b * 2 * d + c];
+    float v[kCalParts / kFinSlices];     // one trip
+#pragma unroll
+    for (int u = 0; u < kCalParts / kFinSlices; u++)
+        v[u] = slice + u * kFinSlices < parts ? partial[(long long)(slice + u * kFinSlices) * 2 * d + c] : 0.f;
     if (threadIdx.x < parts) atomicAdd(&s_n, cnt[2 * threadIdx.x + row]);
+#pragma unroll
+    for (int u = 0; u < kCalParts / kFinSlices; u++) sum += (double)v[u];
     s_sum[slice][lane] = sum;
     __syncthreads();
     if (slice != 0) return;
@@ -347,20 +351,31 @@ __device__ __forceinline__ void err_add(ErrSum &s, const uint4 &a, const uint4 &
         s.mx = fmaxf(s.mx, fmaxf(fabsf(d0), fabsf(d1)));
     }
 }
-// sums of a CTA by a fixed tree (the same order on every run); thread 0 holds them afterwards
+// Sums of a CTA by a fixed tree (the same order on every run): halves of the threads down to one; thread 0 holds them afterwards.
+// The three levels above a warp's width are taken by the first warp behind one barrier, the rest by shuffles.
 __device__ __forceinline__ void err_reduce(double &se, double &sx, double &mx) {
     __shared__ double s_se[kErrThreads], s_sx[kErrThreads], s_mx[kErrThreads];
-    s_se[threadIdx.x] = se; s_sx[threadIdx.x] = sx; s_mx[threadIdx.x] = mx;
+    const int t = threadIdx.x;
+    s_se[t] = se; s_sx[t] = sx; s_mx[t] = mx;
     __syncthreads();
-    for (int o = kErrThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            s_se[threadIdx.x] += s_se[threadIdx.x + o];
-            s_sx[threadIdx.x] += s_sx[threadIdx.x + o];
-            s_mx[threadIdx.x] = fmax(s_mx[threadIdx.x], s_mx[threadIdx.x + o]);
-        }
-        __syncthreads();
+    static_assert(kErrThreads == 256, "the tree below");
+    if (t >= 32) return;
+    auto top = [&](const double *v, auto join) {
+        const double a = join(v[t], v[t + 128]), b = join(v[t + 64], v[t + 192]);
+        const double c = join(v[t + 32], v[t + 160]), e = join(v[t + 96], v[t + 224]);
+        return join(join(a, b), join(c, e));
+    };
+    auto add = [](double a, double b) { return a + b; };
+    auto most = [](double a, double b) { return fmax(a, b); };
+    se = top(s_se, add);
+    sx = top(s_sx, add);
+    mx = top(s_mx, most);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        se += __shfl_down_sync(0xffffffffu, se, o);
+        sx += __shfl_down_sync(0xffffffffu, sx, o);
+        mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, o));
     }
-    se = s_se[0]; sx = s_sx[0]; mx = s_mx[0];
 }
 // partial[b] = (sum (x - x_hat)^2, sum x^2, max |x - x_hat|) over the 8-element chunks b, b + grid, ...; four chunks of a
 // thread are loaded before the first is used
@@ -369,15 +384,18 @@ __global__ void __launch_bounds__(kErrThreads) recon_error_kernel(const uint4 *X
     grid_dependency_wait();
     constexpr long long stride = (long long)kErrGrid * kErrThreads;
     ErrSum s = {0.0, 0.0, 0.f};
-    long long i = blockIdx.x * (long long)kErrThreads + threadIdx.x;
-    for (; i + 3 * stride < n8; i += 4 * stride) {
+    for (long long i = blockIdx.x * (long long)kErrThreads + threadIdx.x; i < n8; i += 4 * stride) {
         uint4 a[4], b[4];
 #pragma unroll
-        for (int u = 0; u < 4; u++) { a[u] = X[i + u * stride]; b[u] = Xh[i + u * stride]; }
+        for (int u = 0; u < 4; u++) {
+            const long long at = i + u * stride < n8 ? i + u * stride : i;      // loads without a branch
+            a[u] = X[at];
+            b[u] = Xh[at];
+        }
 #pragma unroll
-        for (int u = 0; u < 4; u++) err_add(s, a[u], b[u]);
+        for (int u = 0; u < 4; u++)
+            if (i + u * stride < n8) err_add(s, a[u], b[u]);
     }
-    for (; i < n8; i += stride) err_add(s, X[i], Xh[i]);
     double mx = (double)s.mx;
     err_reduce(s.se, s.sx, mx);
     if (threadIdx.x == 0) {
