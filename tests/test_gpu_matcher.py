@@ -168,6 +168,30 @@ def test_spans_to_rows(env):
     assert np.all(o[:4090] == -1) and o[4090:].tolist() == list(range(10, 16))
 
 
+@pytest.mark.parametrize("n_query,n_spans", [(1, 1), (1023, 40), (1024, 0), (1025, 60), (30000, 3001), (262144, 2048), (262145, 900)])
+def test_spans_to_rows_at_chunk_edges(env, n_query, n_spans):
+    """Spans in no order, of lengths 0 and up, some outside [0, n_query) in part or as a whole, one of them as long as lengths go;
+    more of them than a CTA looks at in one go; the last size of the one-launch form and the first of the other."""
+    rac, dev = env.rac, env.dev
+    rng = np.random.default_rng(n_query)
+    cuts = np.sort(rng.integers(-50, n_query + 50, 2 * n_spans))
+    q0, q1 = cuts[0::2], cuts[1::2]                        # disjoint, so that their order has no meaning
+    sp = np.stack([q0, rng.integers(0, 10 ** 6, n_spans), q1 - q0], 1).astype(np.int32)
+    if n_spans > 1 and (sp[-1, 0] >= q1[:-1].max()):
+        sp[-1, 2] = 2 ** 31 - 1
+    sp = sp[rng.permutation(n_spans)]
+    want = np.full(n_query, -1, np.int64)
+    for a, h, n in sp.astype(np.int64):
+        lo, hi = max(a, 0), min(a + n, n_query)
+        if hi > lo:
+            want[lo:hi] = h + np.arange(lo - a, hi - a)
+    spans = torch.from_numpy(np.concatenate([sp, np.full((1, 3), 7, np.int32)])).to(dev)
+    out = torch.full((n_query + 2,), 99, dtype=torch.int32, device=dev)
+    rac.rac_spans_to_rows(spans, torch.tensor([n_spans], dtype=torch.int32, device=dev), n_query, out[1:n_query + 1])
+    o = out.cpu().numpy()
+    assert o[0] == 99 and o[-1] == 99 and np.array_equal(o[1:-1], want)
+
+
 # --------------------------------------------------------------------------- persistent index over earlier requests
 class GpuIndex:
     """Drives rac_index_* the way a serving loop would: one append per finished request, one query per prompt."""
