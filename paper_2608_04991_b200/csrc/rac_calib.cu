@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kCalWarps * 32, MOMENTS ? 3 : 2) calib_kernel(
             a2 = pack2(a, a);
             b2 = pack2(b, b);
         } else {
-            fit_group_centred(xw, rw, has_ref, p.lpg, p.inv_group, p.status, a2, b2, st);
+            fit_group(xw, rw, has_ref, p.lpg, p.inv_group, 0xffffffffu, p.status, a2, b2, &st);
         }
         if (MOMENTS) {
             if (valid && (lane & (p.lpg - 1)) == 0) p.moments[tok * p.J + (slab >> p.lpg_shift)] = st;

@@ -351,36 +351,6 @@ __device__ __forceinline__ void issue_token_loads(const CodecParams &p, Ctrl *ct
     if (row >= 0) bulk_load(stage_addr + r_off, ref_row_ptr<SUB>(p, row), row_bytes, bar);
 }
 
-// c + the product of two bf16 halves of packed words: the product is exact, so the one rounding is that of the sum.
-__device__ __forceinline__ float fma_lo(uint32_t v, uint32_t w, float c) {
-    float r;
-    asm("{.reg .b16 l, h, m, n; mov.b32 {l, h}, %1; mov.b32 {m, n}, %2; fma.rn.f32.bf16 %0, l, m, %3;}" : "=f"(r) : "r"(v), "r"(w), "f"(c));
-    return r;
-}
-__device__ __forceinline__ float fma_hi(uint32_t v, uint32_t w, float c) {
-    float r;
-    asm("{.reg .b16 l, h, m, n; mov.b32 {l, h}, %1; mov.b32 {m, n}, %2; fma.rn.f32.bf16 %0, h, n, %3;}" : "=f"(r) : "r"(v), "r"(w), "f"(c));
-    return r;
-}
-// Sums of v, and of v*w, over the thread's 32 channels (even channels, odd channels), two accumulators each.
-__device__ __forceinline__ float sum_slab(const uint32_t (&v)[16]) {
-    float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
-#pragma unroll
-    for (int i = 0; i < 16; i += 2) {
-        p0 = add_lo(v[i], p0); p1 = add_hi(v[i], p1);
-        p2 = add_lo(v[i + 1], p2); p3 = add_hi(v[i + 1], p3);
-    }
-    return (p0 + p2) + (p1 + p3);
-}
-__device__ __forceinline__ float2 dot_slab(const uint32_t (&v)[16], const uint32_t (&w)[16]) {
-    float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
-#pragma unroll
-    for (int i = 0; i < 16; i += 2) {
-        p0 = fma_lo(v[i], w[i], p0); p1 = fma_hi(v[i], w[i], p1);
-        p2 = fma_lo(v[i + 1], w[i + 1], p2); p3 = fma_hi(v[i + 1], w[i + 1], p3);
-    }
-    return make_float2(p0 + p2, p1 + p3);
-}
 // butterflies over the lanes of a group, two values at a time
 __device__ __forceinline__ void group_sum2(float &a, float &b, int lpg, unsigned int group_mask) {
 #pragma unroll
@@ -392,27 +362,51 @@ __device__ __forceinline__ void group_sum2(float &a, float &b, int lpg, unsigned
     }
 }
 
-// sums of the centred values' products over the group
-__device__ __forceinline__ void centred_sums(const uint32_t (&xw)[16], const uint32_t (&rw)[16], float rbar, float hbar, int lpg,
-                                             unsigned int group_mask, float &sxx, float &sxy) {
-    u64 sxxa = 0ull, sxxb = 0ull, sxya = 0ull, sxyb = 0ull;
+// Eq. 6 for the group this thread belongs to: centred two-pass sums over the thread's 32 channels (rows as packed bf16
+// words; two accumulators per sum and channel parity), butterflies over the group's lanes, the zero-variance rule, and
+// wire rounding of (alpha, beta) to binary16.  Returns their bit patterns and, in a2 and b2, the coefficients splatted for
+// packed arithmetic; a token without a reference has no second pass.  The rows stay packed and enter the sums through the
+// mixed adds above: half the registers of unpacked rows and no unpacking (streaming pass at 131072 x 5120, group 128,
+// 4-bit: with outliers 528 -> 485 us, without 516 -> 467 us, with x_hat 726 -> 700 us).
+// Sums of products in one pass, the means' part taken out afterwards, are less work only where means are small beside the
+// spread, and need the centred pass behind them where they are not: 131072 x 5120, 4-bit, eight outliers, groups of 128 616 us so,
+// 583 to 588 in one pass with means of zero, but 695 to 709 with means of 0.6 of the spread and more (16384 x 4096, 3-bit 65.1, 62.7 and
+// 72.7; groups of 1024 72.3, 70.7 and 86); and from groups of 256 on the error of alpha against 64 bits is up to 6 % larger.
+__device__ __forceinline__ uint32_t fit_group(const uint32_t (&xw)[16], const uint32_t (&rw)[16], bool has_ref, int lpg,
+                                              float inv_group, unsigned int group_mask, uint32_t *status, u64 &a2, u64 &b2,
+                                              float4 *stats = nullptr) {
+    float ra0 = 0.f, ra1 = 0.f, rb0 = 0.f, rb1 = 0.f, xa0 = 0.f, xa1 = 0.f, xb0 = 0.f, xb1 = 0.f;
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
-        const u64 dr0 = pack2(sub_lo(rw[i], rbar), sub_hi(rw[i], rbar)), dh0 = pack2(sub_lo(xw[i], hbar), sub_hi(xw[i], hbar));
-        const u64 dr1 = pack2(sub_lo(rw[i + 1], rbar), sub_hi(rw[i + 1], rbar));
-        const u64 dh1 = pack2(sub_lo(xw[i + 1], hbar), sub_hi(xw[i + 1], hbar));
-        sxxa = pfma(dr0, dr0, sxxa); sxya = pfma(dr0, dh0, sxya);
-        sxxb = pfma(dr1, dr1, sxxb); sxyb = pfma(dr1, dh1, sxyb);
+        ra0 = add_lo(rw[i], ra0); ra1 = add_hi(rw[i], ra1); rb0 = add_lo(rw[i + 1], rb0); rb1 = add_hi(rw[i + 1], rb1);
+        xa0 = add_lo(xw[i], xa0); xa1 = add_hi(xw[i], xa1); xb0 = add_lo(xw[i + 1], xb0); xb1 = add_hi(xw[i + 1], xb1);
     }
-    float sxx_hi, sxy_hi;
-    unpack2(padd(sxxa, sxxb), sxx, sxx_hi);
-    unpack2(padd(sxya, sxyb), sxy, sxy_hi);
-    sxx += sxx_hi;
-    sxy += sxy_hi;
-    group_sum2(sxx, sxy, lpg, group_mask);
-}
-// the zero-variance rule, then wire rounding to binary16: the coefficients splatted for packed arithmetic, and their bit patterns
-__device__ __forceinline__ uint32_t wire_coefficients(bool has_ref, float rbar, float hbar, float sxx, float sxy, u64 &a2, u64 &b2) {
+    float sr = (ra0 + rb0) + (ra1 + rb1), sh = (xa0 + xb0) + (xa1 + xb1);
+    group_sum2(sr, sh, lpg, group_mask);
+    if (!(fabsf(sr) <= 3.0e38f) || !(fabsf(sh) <= 3.0e38f)) {
+        if (status) atomicOr(status, RAC_STATUS_NONFINITE);
+    }
+    const float rbar = sr * inv_group, hbar = sh * inv_group;
+    float sxx = 0.f, sxy = 0.f;
+    if (has_ref || stats) {
+        u64 sxxa = 0ull, sxxb = 0ull, sxya = 0ull, sxyb = 0ull;
+#pragma unroll
+        for (int i = 0; i < 16; i += 2) {
+            const u64 dr0 = pack2(sub_lo(rw[i], rbar), sub_hi(rw[i], rbar)), dh0 = pack2(sub_lo(xw[i], hbar), sub_hi(xw[i], hbar));
+            const u64 dr1 = pack2(sub_lo(rw[i + 1], rbar), sub_hi(rw[i + 1], rbar));
+            const u64 dh1 = pack2(sub_lo(xw[i + 1], hbar), sub_hi(xw[i + 1], hbar));
+            sxxa = pfma(dr0, dr0, sxxa); sxya = pfma(dr0, dh0, sxya);
+            sxxb = pfma(dr1, dr1, sxxb); sxyb = pfma(dr1, dh1, sxyb);
+        }
+        float sxx_hi, sxy_hi;
+        unpack2(padd(sxxa, sxxb), sxx, sxx_hi);
+        unpack2(padd(sxya, sxyb), sxy, sxy_hi);
+        sxx += sxx_hi;
+        sxy += sxy_hi;
+        group_sum2(sxx, sxy, lpg, group_mask);
+    }
+    if (stats) *stats = make_float4(rbar, hbar, sxx, sxy);
+    // zero-variance rule, then wire rounding to binary16
     float a_star = 0.f, b_star = hbar;
     if (has_ref && sxx > 1e-12f && fabsf(sxy) < 65504.0f * sxx) {
         a_star = __fdiv_rn(sxy, sxx);
@@ -423,70 +417,6 @@ __device__ __forceinline__ uint32_t wire_coefficients(bool has_ref, float rbar, 
     a2 = pack2(a, a);
     b2 = pack2(b, b);
     return a16 | (b16 << 16);
-}
-__device__ __forceinline__ void flag_nonfinite(float sr, float sh, uint32_t *status) {
-    if (!(fabsf(sr) <= 3.0e38f) || !(fabsf(sh) <= 3.0e38f)) {
-        if (status) atomicOr(status, RAC_STATUS_NONFINITE);
-    }
-}
-
-// Eq. 6 for the group this thread belongs to (rows as packed bf16 words), as the encoders take it.  Returns the bit patterns of the
-// wire coefficients, and the coefficients.
-//
-// The centred sums come out of one pass over the rows: Sxx = sum (r*r) - n*rbar^2 and Sxy = sum (r*h) - n*rbar*hbar, products of
-// bf16 being exact.  Every thread takes the means' part of its 32 channels out of its own sums before they are added up over the
-// group, which costs no rounding more than the sums have anyway.  With means small beside the spread -- activations -- this is
-// closer to 64 bits than sums of centred values, which are rounded one by one (error of alpha, rms, groups of 128: activations
-// 6.8e-8 so, 6.9e-8 centred; a walk's next state 6.6e-8 and 6.7e-8; channels of very different scales 8.1e-8 and 8.4e-8; a mean of a
-// quarter of the spread 6.7e-8 and 6.8e-8, of half of it 6.9e-8 and 6.8e-8).  Hence the line, kMeanRatio: a warp in which some
-// group has n*rbar^2 or n*hbar^2 above a quarter of the centred sum of squares takes the second, centred pass.  That of h is not
-// known, but it is at least Sxy^2 / Sxx; only where this does not suffice (references that have little to do with the token)
-// sum h*h is formed as well.
-// The encoders are bound by issue slots and, in long runs, by the board's power beside DRAM: per pair of channels this is 8
-// operations, and the products do not wait for the means, where two passes took 8 and 2 packed ones.  (131072 x 5120, eight
-// outliers 616 -> 590 us, uplink with x_hat and retrieval 943 -> 917; 20001 x 5120 by Eq. 8, both ends, 209.7 -> 208.0; the sums on the matrix
-// unit by mma.sync, sixteen of them per warp and token, were slower everywhere and truncate.)
-constexpr float kMeanRatio = 0.25f;
-__device__ __forceinline__ uint32_t fit_group(const uint32_t (&xw)[16], const uint32_t (&rw)[16], bool has_ref, int lpg,
-                                              float inv_group, unsigned int group_mask, uint32_t *status, u64 &a2, u64 &b2) {
-    float sr = has_ref ? sum_slab(rw) : 0.f, sh = sum_slab(xw), sxx = 0.f, sxy = 0.f;
-    group_sum2(sr, sh, lpg, group_mask);
-    const float rbar = sr * inv_group, hbar = sh * inv_group;
-    if (has_ref) {
-        const float2 rr = dot_slab(rw, rw), rh = dot_slab(rw, xw);
-        const float r32 = -32.0f * rbar;
-        sxx = rr.x + __fmaf_rn(r32, rbar, rr.y);
-        sxy = rh.x + __fmaf_rn(r32, hbar, rh.y);
-        group_sum2(sxx, sxy, lpg, group_mask);
-        // strict comparisons: whatever is infinite or no number ends in the second pass
-        const bool small_r = sr * rbar < kMeanRatio * sxx;
-        if (__builtin_expect(!__all_sync(group_mask, small_r && (sh * hbar) * sxx < (kMeanRatio * sxy) * sxy), 0)) {
-            const float2 hh = dot_slab(xw, xw);
-            float shh = hh.x + __fmaf_rn(-32.0f * hbar, hbar, hh.y);
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1)
-                if (lpg > o) shh += __shfl_xor_sync(group_mask, shh, o);
-            if (!__all_sync(group_mask, small_r && sh * hbar < kMeanRatio * shh && shh < 1e30f && sxx < 1e30f)) {
-                flag_nonfinite(sr, sh, status);
-                centred_sums(xw, rw, rbar, hbar, lpg, group_mask, sxx, sxy);
-            }
-        }
-    } else {
-        flag_nonfinite(sr, sh, status);
-    }
-    return wire_coefficients(has_ref, rbar, hbar, sxx, sxy, a2, b2);
-}
-// The same by centred sums in any case, as the calibration takes it, and the statistics.  (There the rows are waited for, and the
-// one-pass form was slower: 4096 x 2880 with encode and error 50.2 us, 47.8 so.)
-__device__ __forceinline__ void fit_group_centred(const uint32_t (&xw)[16], const uint32_t (&rw)[16], bool has_ref, int lpg,
-                                                  float inv_group, uint32_t *status, u64 &a2, u64 &b2, float4 &stats) {
-    float sr = sum_slab(rw), sh = sum_slab(xw), sxx, sxy;
-    group_sum2(sr, sh, lpg, 0xffffffffu);
-    flag_nonfinite(sr, sh, status);
-    const float rbar = sr * inv_group, hbar = sh * inv_group;
-    centred_sums(xw, rw, rbar, hbar, lpg, 0xffffffffu, sxx, sxy);
-    stats = make_float4(rbar, hbar, sxx, sxy);
-    wire_coefficients(has_ref, rbar, hbar, sxx, sxy, a2, b2);
 }
 
 // ------------------------------------------------------------------------------------------------

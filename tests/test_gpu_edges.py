@@ -472,14 +472,13 @@ def test_encode_with_x_hat_on_both_sides_of_the_step_registers(env, d):
                      inv.cpu().numpy())
 
 
-# --------------------------------------------------------------------------------------------- the three ways of the fit
+# ------------------------------------------------------------------------------------------------------------- the fit
 @pytest.mark.parametrize("d,g", [(4096, 128), (3584, 64), (2880, 32), (8192, 1024), (5120, 256)])
 @pytest.mark.parametrize("mode", [0, 1])
 def test_fit_with_means_small_and_large_beside_the_spread(env, d, g, mode):
-    """Means that stay inside the one-pass form, means around its line (n*mean^2 a quarter of the centred sum of squares, of the
-    reference and of the token), references that say nothing about the token, constant and zero groups, all among the groups of
-    one warp and as whole tokens.  Coefficients against the oracle's binary64 fit by the protocol's windows; the rest bit for
-    bit."""
+    """Means of zero, about half of the spread and large beside it (of the reference and of the token), references that say
+    nothing about the token, constant and zero groups, all among the groups of one warp and as whole tokens.  Coefficients
+    against the oracle's binary64 fit by the protocol's windows; the rest bit for bit."""
     s, rac, P = env.synth, env.rac, env.P
     T, J = 24, d // g
     rng = np.random.default_rng(d + g)
@@ -500,6 +499,44 @@ def test_fit_with_means_small_and_large_beside_the_spread(env, d, g, mode):
         P.round_trip_case(cfg, X, ref_base=R, step=step, inv_step=(np.float32(1) / step).astype(np.float32))
     else:
         P.round_trip_case(rac.CodecCfg(d, g, 4, 0, scale_mode=1, topk_group=1), X, ref_base=R)
+
+
+@pytest.mark.parametrize("d,g", [(2880, 32), (3584, 64), (4096, 128), (5120, 256), (8192, 1024)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_encoders_fit_by_the_calibrations_centred_sums(env, d, g, mode):
+    """The segment fit leaves its centred statistics per token and group (mean r, mean h, Sxx, Sxy) in its workspace.  The
+    encoders' coefficient words are those statistics' division and multiply-add, correctly rounded, bit for bit: a fit whose
+    sums round in another way flips a word in some ten thousand (its relative difference over the 2^-11 of a binary16 step).
+    Means from zero to half of the spread; some tokens without a reference."""
+    s, rac, dev = env.synth, env.rac, env.dev
+    T, J = 4096, d // g
+    rng = np.random.default_rng(d + mode)
+    gen = s.generator(g, dev)
+    R = torch.randn((T, J, g), device=dev, generator=gen) + torch.rand((T, J, 1), device=dev, generator=gen) * 0.5
+    X = 0.9 * R + 0.05 * torch.randn((T, J, g), device=dev, generator=gen)
+    X, R = X.to(torch.bfloat16).view(T, d), R.to(torch.bfloat16).view(T, d)
+    rows = rng.permutation(T).astype(np.int32)
+    rows[::9] = -1
+    X = X[torch.from_numpy(np.where(rows >= 0, rows, np.arange(T))).to(dev).long()]      # next to its reference row
+    rows_d = torch.from_numpy(rows).to(dev)
+    scfg = rac.CodecCfg(d, g, 4, 0, coef_fmt=1)
+    nb = rac.rac_fit_segments_workspace_bytes(scfg, T)
+    ws = torch.zeros(nb, dtype=torch.uint8, device=dev)
+    st = torch.zeros(1, dtype=torch.int32, device=dev)
+    rac.rac_fit_segments(scfg, X, T, R, T, rows_d, None, None, torch.tensor([0, T], dtype=torch.int32, device=dev), 1,
+                         torch.zeros((1, J), dtype=torch.int32, device=dev), torch.zeros(T, dtype=torch.int32, device=dev), ws, nb, st)
+    rbar, hbar, sxx, sxy = np.moveaxis(ws[:16 * T * J].cpu().numpy().view(np.float32).reshape(T, J, 4), 2, 0)
+    assert int(st.item()) == 0 and np.all(sxx[rows >= 0] > 1.0)
+    ref = (rows >= 0)[:, None]
+    a = np.where(ref, sxy / np.where(ref, sxx, np.float32(1)), np.float32(0))
+    b = np.where(ref, (hbar - a.astype(np.longdouble) * rbar).astype(np.float32), hbar)
+    want = a.astype(np.float16).view(np.uint16) | (b.astype(np.float16).view(np.uint16).astype(np.uint32) << 16)
+    step = torch.full((2, d), 0.03125, device=dev)
+    cfg = rac.CodecCfg(d, g, 4, 8) if mode == 0 else rac.CodecCfg(d, g, 4, 0, scale_mode=1, topk_group=1)
+    rec = rac.rac_record_bytes(cfg)
+    pay, st = env.P.gpu_encode(cfg, X, R, rows_d, None, None, *((step, 1 / step) if mode == 0 else (None, None)))
+    got = np.ascontiguousarray(pay.reshape(T, rec)[:, :4 * J]).view(np.uint32)
+    assert st == 0 and np.array_equal(got, want)
 
 
 def test_fit_flags_values_that_are_not_finite(env):
