@@ -253,8 +253,10 @@ __device__ __forceinline__ uint4 load_ref_words(uint32_t addr, const uint16_t *g
     return w;
 }
 
-// the thread's whole slab, slot order (off: byte offsets of its four slots in the row).  One test of the transform and all of its
-// loads before any is used: with a test per slot each slot was a trip of its own (300 x 8192 with x_hat 9.0 us, 8.0 so).
+// the thread's whole slab, slot order (off: byte offsets of its four slots in the row).  One test of the transform, and the loads
+// of two slots before either is used: with a test per slot each slot was a trip of its own (a token's chain with x_hat and a
+// predictor, 300 x 8192, 8.8 us, 8.2 to 8.3 so; all four slots at once 8.0, but the registers for that made calls WITHOUT a predictor
+// 1 % slower: 131072 x 5120 with eight outliers 612 us slot by slot, 620 at once, 605 to 608 so).
 __device__ __forceinline__ void load_ref_slab(uint32_t (&rw)[16], uint32_t rs, const uint32_t (&off)[4], const uint16_t *gain,
                                               const uint16_t *bias) {
 #pragma unroll
@@ -263,21 +265,24 @@ __device__ __forceinline__ void load_ref_slab(uint32_t (&rw)[16], uint32_t rs, c
         rw[4 * j + 0] = w.x; rw[4 * j + 1] = w.y; rw[4 * j + 2] = w.z; rw[4 * j + 3] = w.w;
     }
     if (gain) {
-        uint4 gw[4], bw[4];
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            gw[j] = __ldg(reinterpret_cast<const uint4 *>(gain + (off[j] >> 1)));
-            bw[j] = __ldg(reinterpret_cast<const uint4 *>(bias + (off[j] >> 1)));
-        }
+        for (int j0 = 0; j0 < 4; j0 += 2) {
+            uint4 gw[2], bw[2];
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            const uint32_t gws[4] = {gw[j].x, gw[j].y, gw[j].z, gw[j].w}, bws[4] = {bw[j].x, bw[j].y, bw[j].z, bw[j].w};
+            for (int h = 0; h < 2; h++) {
+                gw[h] = __ldg(reinterpret_cast<const uint4 *>(gain + (off[j0 + h] >> 1)));
+                bw[h] = __ldg(reinterpret_cast<const uint4 *>(bias + (off[j0 + h] >> 1)));
+            }
 #pragma unroll
-            for (int i = 0; i < 4; i++) {
-                const uint32_t w = rw[4 * j + i];
-                rw[4 * j + i] = f2_to_bf16x2(
-                    __fmaf_rn(half_bits_to_float(gws[i] & 0xffff), __uint_as_float(w << 16), half_bits_to_float(bws[i] & 0xffff)),
-                    __fmaf_rn(half_bits_to_float(gws[i] >> 16), __uint_as_float(w & 0xffff0000u), half_bits_to_float(bws[i] >> 16)));
+            for (int h = 0; h < 2; h++) {
+                const uint32_t gws[4] = {gw[h].x, gw[h].y, gw[h].z, gw[h].w}, bws[4] = {bw[h].x, bw[h].y, bw[h].z, bw[h].w};
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    uint32_t &w = rw[4 * (j0 + h) + i];
+                    w = f2_to_bf16x2(
+                        __fmaf_rn(half_bits_to_float(gws[i] & 0xffff), __uint_as_float(w << 16), half_bits_to_float(bws[i] & 0xffff)),
+                        __fmaf_rn(half_bits_to_float(gws[i] >> 16), __uint_as_float(w & 0xffff0000u), half_bits_to_float(bws[i] >> 16)));
+                }
             }
         }
     }
