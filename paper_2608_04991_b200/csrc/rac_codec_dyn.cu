@@ -64,15 +64,16 @@ __device__ __forceinline__ void rot_right4f(float (&w)[4], int rot) {
 }
 
 // codes of the 8 channels of one slot -> BITS bytes (one word, or two for 8-bit codes)
-// RANGE: the codes lie in [-Qmax, Qmax] (no outliers among them)
-template <int BITS, bool RANGE>
+// (by fields, not by a sum: an outlier's code leaves its range, a residual that is no number has none, and neither may touch the
+// channels beside it)
+template <int BITS>
 __device__ __forceinline__ void pack_slot(const uint32_t (&t)[8], uint32_t &w0, uint32_t &w1) {
     // t[i]: binary32 bit pattern of (code + 1.5*2^23): the low mantissa bits hold the code in two's complement
     if constexpr (BITS == 8) {
         w0 = __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
         w1 = __byte_perm(__byte_perm(t[4], t[5], 0x0040), __byte_perm(t[6], t[7], 0x0040), 0x5410);
     } else {
-        w0 = RANGE ? pack8_sum<BITS>(t) : pack8<BITS>(t);
+        w0 = pack8<BITS>(t);
         w1 = 0;
     }
 }
@@ -438,7 +439,7 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_dyn_kernel
                             xh[i] = f2_to_bf16x2(x0, x1);
                         }
                     }
-                    pack_slot<BITS, KG == 0>(t8, words[j][0], words[j][1]);
+                    pack_slot<BITS>(t8, words[j][0], words[j][1]);
                     if (XHAT) sts128(xs + off[j], make_uint4(xh[0], xh[1], xh[2], xh[3]));
                 }
             };

@@ -563,6 +563,38 @@ def test_fit_flags_values_that_are_not_finite(env):
             assert np.array_equal(pay.reshape(T, rec)[keep], clean.reshape(T, rec)[keep])
 
 
+@pytest.mark.parametrize("bits", [2, 3, 4, 8])
+@pytest.mark.parametrize("kg", [0, 1])
+def test_group_scales_keep_a_value_that_is_no_number_in_its_channel(env, bits, kg):
+    """A reference value that is not finite (slope 0, the mean alone: one residual without a number), and a NaN of the token
+    beside given coefficients: the codes of the channels around it are those that the sender's x_hat was formed with, so the
+    receiver's x_hat has the same bits everywhere else.  The fit reports the value; with given coefficients nobody looks."""
+    s, rac, dev = env.synth, env.rac, env.dev
+    d, g, T, at = 4096, 128, 6, 777
+    gen = s.generator(bits, dev)
+    X = s.activations(T, d, s.channel_scale(d, 5, dev), gen)
+    R = s.affine_noisy_reference(X, g, gen)
+    words = torch.full((1, d // g), 0x3C00, dtype=torch.int32, device=dev)          # alpha 1, beta 0
+    for bad in (float("nan"), float("inf"), -float("inf"), None):
+        x, r = X.clone(), R.clone()
+        if bad is None:
+            x[3, at] = float("nan")
+        else:
+            r[3, at] = bad
+        cfg = rac.CodecCfg(d, g, bits, 0, scale_mode=1, topk_group=kg, coef_fmt=1 if bad is None else 0)
+        seg = dict(coef_seg=words, seg_of=torch.zeros(T, dtype=torch.int32, device=dev)) if bad is None else {}
+        pay = torch.zeros(T * rac.rac_record_bytes(cfg), dtype=torch.uint8, device=dev)
+        xs, xr = torch.zeros_like(X), torch.zeros_like(X)
+        st = torch.zeros(1, dtype=torch.int32, device=dev)
+        rac.rac_encode_reconstruct_list(cfg, x, T, None, None, r, T, None, None, 0, None, None, None, None, pay, pay.numel(), xs, None, 0,
+                                        st, **seg)
+        rac.rac_decode_reconstruct_list(cfg, pay, T, None, None, r, T, None, None, 0, None, None, None, xr, st, **seg)
+        assert bool(int(st.item()) & rac.STATUS_NONFINITE) == (bad is not None)
+        same = xs.view(torch.int16) == xr.view(torch.int16)
+        same[3, at] = True
+        assert bool(same.all()), (bad, (~same).nonzero()[:8].tolist())
+
+
 # ------------------------------------------------------------------- one launch with x_hat: teams of one CTA per SM, from a size on
 @pytest.mark.parametrize("d,g,bits,k,per_sm,gathered", [
     (5120, 128, 4, 8, 20, True),      # three teams, width compiled in
