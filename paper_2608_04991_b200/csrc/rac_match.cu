@@ -699,39 +699,54 @@ __global__ void spans_to_rows_kernel(const rac_span *spans, const int32_t *n_spa
     }
 }
 
-// The same in one launch: a CTA owns 1024 positions, looks at all spans, 1024 at a time, and hands out those that reach into its
-// own.  Bound by launches and two trips to L2: behind a fill of its own the kernel above ended a prompt of 2048 tokens later (its whole pass 49.7 us, 48.3 so).
-// Every CTA reads every span, so it serves up to kSpanRowsQuery positions; beyond, the work of the form above grows more slowly.
-constexpr int kSpanRows = 1024;
+// The same in one launch: a CTA owns kSpanRows positions, looks at all spans and keeps what reaches into its own.  A piece of up to
+// kSpanShort positions is written by the thread that sees it, longer ones wait in a list and are written by whole warps (a list of
+// more than kSpanList -- only overlapping spans make one -- goes the short way).  Bound by launches and two trips to L2 where spans
+// have the usual length (132 tokens, gaps of 56: 2.2 us up to 98304 positions, 2.8 at 262144; 4.1 in the two launches of a fill and
+// the kernel above), by reading the list where they are as short as they get: 4 tokens, no gaps, 2.2 us at 4096 positions (3.7), 6.3 at
+// 65536 (11.3), 19.9 at 262144 (20.4).  Every CTA reads every span, so that beyond kSpanRowsQuery the two launches are the better
+// ones.
+constexpr int kSpanRows = 1024, kSpanShort = 8, kSpanList = 128;
 constexpr long long kSpanRowsQuery = 262144;
+static_assert(kSpanList > kSpanRows / (kSpanShort + 1), "spans that do not overlap fit the list");
 __global__ void __launch_bounds__(kSpanRows) span_rows_kernel(const rac_span *spans, const int32_t *n_spans, int n_query, int32_t *ref_row) {
-    __shared__ int s_row[kSpanRows], s_n[2];
-    __shared__ rac_span s_span[kSpanRows];
+    __shared__ int s_row[kSpanRows], s_n;
+    __shared__ rac_span s_span[kSpanList];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int lo = blockIdx.x * kSpanRows, hi = min(lo + kSpanRows, n_query);
     grid_launch_dependents();
     s_row[tid] = -1;
-    if (tid < 2) s_n[tid] = 0;
+    if (tid == 0) s_n = 0;
     __syncthreads();
     grid_dependency_wait();
     const int ns = *n_spans;
-    for (int base = 0, b = 0; base < ns; base += kSpanRows, b ^= 1) {
-        if (tid < ns - base) {
-            const rac_span sp = spans[base + tid];
-            const long long q0 = sp.q_start, q1 = q0 + sp.len;
-            if (q0 < hi && q1 > lo && q1 > q0) s_span[atomicAdd(&s_n[b], 1)] = sp;
+    for (long long base = tid; base < ns; base += 4 * kSpanRows) {
+        rac_span sp[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) sp[u] = spans[base + u * kSpanRows < ns ? base + u * kSpanRows : base];   // loads without a branch
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            if (base + u * kSpanRows >= ns) continue;
+            const long long q0 = sp[u].q_start, q1 = q0 + sp[u].len;
+            if (q0 >= hi || q1 <= lo || q1 <= q0) continue;
+            const int a = (int)(q0 > lo ? q0 : lo), b = (int)(q1 < hi ? q1 : hi);
+            const int at = b - a > kSpanShort ? atomicAdd(&s_n, 1) : kSpanList;
+            if (at < kSpanList) {
+                s_span[at] = sp[u];
+            } else {
+                for (int q = a; q < b; q++) s_row[q - lo] = sp[u].h_start + (int)(q - q0);
+            }
         }
-        __syncthreads();
-        const int n = s_n[b];
-        if (tid == 0) s_n[b ^ 1] = 0;
-        for (int k = warp; k < n; k += kSpanRows / 32) {
-            const rac_span sp = s_span[k];
-            const long long q0 = sp.q_start, q1 = q0 + sp.len;
-            const int last = (int)(q1 < hi ? q1 : hi);
-            for (int q = (int)(q0 > lo ? q0 : lo) + lane; q < last; q += 32) s_row[q - lo] = sp.h_start + (int)(q - q0);
-        }
-        __syncthreads();
     }
+    __syncthreads();
+    const int n = min(s_n, kSpanList);
+    for (int k = warp; k < n; k += kSpanRows / 32) {
+        const rac_span sp = s_span[k];
+        const long long q0 = sp.q_start, q1 = q0 + sp.len;
+        const int b = (int)(q1 < hi ? q1 : hi);
+        for (int q = (int)(q0 > lo ? q0 : lo) + lane; q < b; q += 32) s_row[q - lo] = sp.h_start + (int)(q - q0);
+    }
+    __syncthreads();
     if (lo + tid < hi) ref_row[lo + tid] = s_row[tid];
 }
 

@@ -168,7 +168,8 @@ def test_spans_to_rows(env):
     assert np.all(o[:4090] == -1) and o[4090:].tolist() == list(range(10, 16))
 
 
-@pytest.mark.parametrize("n_query,n_spans", [(1, 1), (1023, 40), (1024, 0), (1025, 60), (30000, 3001), (262144, 2048), (262145, 900)])
+@pytest.mark.parametrize("n_query,n_spans", [(1, 1), (1023, 40), (1024, 0), (1025, 60), (30000, 3001), (262144, 2048), (262145, 900),
+                                              (4096, 1024), (65536, 16384), (65537, 4000), (140000, 5000), (262144, 65536)])
 def test_spans_to_rows_at_chunk_edges(env, n_query, n_spans):
     """Spans in no order, of lengths 0 and up, some outside [0, n_query) in part or as a whole, one of them as long as lengths go;
     more of them than a CTA looks at in one go; the last size of the one-launch form and the first of the other."""
