@@ -290,7 +290,7 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
 // read it from the parameters; the constant removes the uniform branches of the shuffle reductions.
 // D: the hidden width as a compile-time constant (4096 and 5120 are compiled in), or 0 to read it from the parameters;
 // the constant folds the address arithmetic of the rows and stages (without outliers, 131072 x 5120 485 -> 458 us, x 4096 394 ->
-// 383 us; with x_hat and gathered rows 697 -> 685 us).
+// 383 us; with x_hat, gathered rows and a predictor, with eight outliers, 100000 x 5120 815 -> 786 us in both launches).
 // REF: every token has a reference row (identity rows: no row list, a reference buffer): the per-token test and the
 // second row of the tables go away (without outliers, 131072 x 5120 474 -> 458 us; with x_hat see launch_stream_lpg).
 template <int BITS, bool TOPK, bool XHAT, int MINB, bool SUB, int LPG = 0, int D = 0, bool REF = false>
@@ -302,12 +302,12 @@ __global__ void __launch_bounds__(MINB == 4 ? 160 : 256, MINB) encode_ws_kernel(
     const int d = D ? D : p.d;
     const bool valid = tid * 32 < d;
     constexpr int S = 2;   // stages of the ring (the host sets p.stages to the same)
-    // with the width and the group compiled in, the record geometry is a constant too (those variants are without outliers)
-    static_assert(!(TOPK && D != 0), "the geometry below has no outliers");
+    // with the width and the group compiled in, the record geometry is a constant too (those variants are launched for
+    // no outliers or eight per token only)
     constexpr bool kGeo = D != 0 && LPG != 0;
     const int Jc = kGeo ? D / (32 * (LPG ? LPG : 1)) : p.J;
     const int codeb = kGeo ? D * BITS / 8 : p.code_bytes;
-    const int recb = kGeo ? (4 * (D / (32 * (LPG ? LPG : 1))) + D * BITS / 8 + 15) / 16 * 16 : p.rec;
+    const int recb = kGeo ? (4 * (D / (32 * (LPG ? LPG : 1))) + D * BITS / 8 + (TOPK ? 32 : 0) + 15) / 16 * 16 : p.rec;
     const WsSmem L = ws_smem_layout(d, recb, S, TOPK);
     WsCtrl *ctrl = reinterpret_cast<WsCtrl *>(smem);
     const uint32_t sbase = smem_u32(smem);
@@ -1847,7 +1847,10 @@ static int launch_stream_lpg(const Geometry &g, CodecParams &p, size_t smem, lon
 #define RAC_STREAM(M, R) \
     launch_persistent(encode_ws_kernel<BITS, TOPK, XHAT, M, false, LPG, D, R>, p, g.nthreads, smem, max_ctas, stream)
     if constexpr (XHAT) {
-        return allref ? RAC_STREAM(2, true) : RAC_STREAM(2, false);
+        if constexpr (!(TOPK && D != 0)) {   // (at that width, identity rows with outliers are always one launch)
+            if (allref) return RAC_STREAM(2, true);
+        }
+        return RAC_STREAM(2, false);
     } else if constexpr (D != 0) {
         return allref ? RAC_STREAM(4, true) : RAC_STREAM(4, false);
     } else {
@@ -1856,17 +1859,20 @@ static int launch_stream_lpg(const Geometry &g, CodecParams &p, size_t smem, lon
 #undef RAC_STREAM
 }
 
-// Widths 4096 and 5120 without outliers have variants with the record geometry compiled in.  With outliers 4096 is always one
-// launch and 5120 comes here with a predictor in front only; every call with outliers and without x_hat is one launch (launch_teams,
-// one_launch): what those would need is not instantiated.
+// Widths 4096 and 5120 have variants with the record geometry compiled in; 4096 with outliers is always one launch (one_launch),
+// and so is every call with outliers and without x_hat: what those would need is not instantiated.  With eight outliers 5120 comes
+// here with gathered rows and a predictor (16384 tokens, groups of 128 137.4 us without the constants, 135.0 with; of 64 149.0 and 145.0),
+// or in groups of 32, which have no constants and whose teams do not fit (launch_teams).
 template <int BITS, bool TOPK, bool XHAT>
 static int launch_stream(const Geometry &g, CodecParams &p, size_t smem, long long max_ctas, cudaStream_t stream) {
     if (p.tok_list || p.intra_base || p.coef_ext)   // the subset form has one variant: it is not the hot path
         return launch_persistent(encode_ws_kernel<BITS, TOPK, XHAT, 2, true, 0>, p, g.nthreads, smem, max_ctas, stream);
     if constexpr (!TOPK || XHAT) {
+        if (g.d == 5120 && (!TOPK || g.topk == 8)) {
+            if (g.lpg == 4) return launch_stream_lpg<BITS, TOPK, XHAT, 4, 5120>(g, p, smem, max_ctas, stream);
+            if (g.lpg == 2) return launch_stream_lpg<BITS, TOPK, XHAT, 2, 5120>(g, p, smem, max_ctas, stream);
+        }
         if constexpr (!TOPK) {
-            if (g.d == 5120 && g.lpg == 4) return launch_stream_lpg<BITS, TOPK, XHAT, 4, 5120>(g, p, smem, max_ctas, stream);
-            if (g.d == 5120 && g.lpg == 2) return launch_stream_lpg<BITS, TOPK, XHAT, 2, 5120>(g, p, smem, max_ctas, stream);
             if (g.d == 4096 && g.lpg == 4) return launch_stream_lpg<BITS, TOPK, XHAT, 4, 4096>(g, p, smem, max_ctas, stream);
             if (g.d == 4096 && g.lpg == 2) return launch_stream_lpg<BITS, TOPK, XHAT, 2, 4096>(g, p, smem, max_ctas, stream);
         }

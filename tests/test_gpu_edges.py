@@ -642,3 +642,32 @@ def test_encode_in_teams_at_its_first_sizes(env, d, g, bits, k, per_sm, gathered
     P.compare_encode(cfg, out[0][(T - 700) * rec:], s.bf16_bits(X[at]), s.bf16_bits(R),
                      np.arange(T - 700, T, dtype=np.int32) if rows is None else rows[at].cpu().numpy(), None, None,
                      step.cpu().numpy(), inv.cpu().numpy())
+
+
+@pytest.mark.parametrize("d,g,k,predictor", [(5120, 128, 8, True), (5120, 64, 8, True), (5120, 128, 5, True), (5120, 32, 8, False), (5376, 128, 8, True)])
+def test_encode_with_x_hat_in_two_launches(env, d, g, k, predictor):
+    """Gathered rows with direct tokens, one token more than the one-launch form takes at these widths, where a predictor or the
+    size of the groups keeps the call from the form in teams: records as without x_hat (another kernel) and against the oracle,
+    x_hat equal to the receiver's."""
+    s, rac, P = env.synth, env.rac, env.P
+    T = 8193
+    gen = s.generator(d + g + k, env.dev)
+    X = s.activations(T, d, s.channel_scale(d, 4, env.dev), gen)
+    R = s.affine_noisy_reference(X, g, gen)
+    rows = torch.arange(T, dtype=torch.int32, device=env.dev)
+    rows[::5] = -1
+    gain, bias = s.predictor_gain_bias(d, 7, env.dev) if predictor else (None, None)
+    step = torch.stack([torch.full((d,), 0.0625, device=env.dev), X[:2000].float().std(0, unbiased=False) * (3.0 / 7)]).clamp(min=2.0 ** -10)
+    step = step.half().float()
+    inv = 1.0 / step
+    cfg = rac.CodecCfg(d, g, 4, k)
+    rec = rac.rac_record_bytes(cfg)
+    pay, xs, st = P.gpu_encode_reconstruct(cfg, X, R, rows, gain, bias, step, inv)
+    plain, st2 = P.gpu_encode(cfg, X, R, rows, gain, bias, step, inv)
+    xr, st3 = P.gpu_decode(cfg, pay, T, R, rows, gain, bias, step, env.dev)
+    assert st == 0 and st2 == 0 and st3 == 0
+    assert np.array_equal(pay, plain) and torch.equal(xs.view(torch.int16), xr.view(torch.int16))
+    at = slice(T - 300, T)
+    gb, bb = (None, None) if gain is None else (s.f16_bits(gain), s.f16_bits(bias))
+    P.compare_encode(cfg, pay[(T - 300) * rec:], s.bf16_bits(X[at]), s.bf16_bits(R), rows[at].cpu().numpy(), gb, bb,
+                     step.cpu().numpy(), inv.cpu().numpy())
