@@ -120,13 +120,17 @@ __host__ __device__ inline WsSmem ws_smem_layout(int d, int rec, int stages, boo
 }
 
 // Both step tables in shared memory, laid out by thread: the 16-byte pieces that a thread reads in one step of its work (for half h
-// of slot j piece 2j + h of the inverse steps; a slot's binary16 steps are one piece) stand side by side for all threads of a
+// of slot j piece 2j + h of a row of inverse steps; a slot's binary16 steps are one piece) stand side by side for all threads of a
 // token, so that a warp's access is 512 consecutive bytes.  Read in place a warp's access touches 32 cache lines (9 wavefronts of
 // the L1 data pipe against 4), and with x_hat the four rows of a width of 5120 are more than the L1 beside the stages.
+// There is room for 24 pieces per thread.  TABLES = 1: both rows of inverse steps and both rows of steps as binary16, which holds
+// calibrated tables.  TABLES = 2, for a caller's own steps that it does not hold: both rows of steps as binary32 and the first row of
+// inverse steps; directly coded tokens read the second in place.  (Gathered rows, 28 % of them direct, binary16 / binary32 / without
+// these tables, us: 12000 x 3072 48.4 / 49.0 / 51.5, x 4096 61.1 / 63.2 / 65.4, x 5120 80.9 / 87.5 / 88.0, 16000 x 6144 123.0 / 132.3 / 139.0;
+// groups of 256 at 24000 x 5120 165 / 184 / 173.  One body for both, with a test per slot, took 2 to 5 % longer than two.)
 struct SlabTables {
     uint32_t inv = 0, step = 0;            // this thread's first pieces
     uint32_t pitch = 0;                    // bytes from one piece of a thread to its next
-    bool half_steps = false;               // the steps as binary16 (as binary32 where that does not hold them exactly)
 };
 __device__ __forceinline__ float4 lds128f(uint32_t addr) {
     const uint4 w = lds128(addr);
@@ -136,7 +140,7 @@ __device__ __forceinline__ float4 lds128f(uint32_t addr) {
 // One thread's 32 channels of one token, rows and record in shared memory: Eq. 6, Eq. 7, Eq. 8 with the static table, packing,
 // the sender-side reconstruction (over the X row), and the largest |e| of the slab.
 // STEPREG: every token has a reference, and the thread holds its steps (row 0 of the table, slot order) in st0.
-template <int BITS, bool TOPK, bool XHAT, int LPG, bool STEPREG, bool TABLES = false>
+template <int BITS, bool TOPK, bool XHAT, int LPG, bool STEPREG, int TABLES = 0>
 __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int lane, int rot, int d, int Jc, bool shared, int coff,
                                             const uint32_t (&off)[4], unsigned int group_mask, uint32_t xs, uint32_t rs,
                                             bool has_ref, int seg, unsigned char *rec, float *tm, const u64 (&st0)[STEPREG ? 16 : 1],
@@ -179,7 +183,7 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
     for (int j = 0; j < 4; j++) {
         const int c = (int)(off[j] >> 1);
         float4 iv0, iv1;
-        if (TABLES) {
+        if (TABLES == 1 || (TABLES == 2 && has_ref)) {
             const uint32_t a = tab.inv + (has_ref ? 0u : 8u * tab.pitch) + 2 * j * tab.pitch;
             iv0 = lds128f(a);
             iv1 = lds128f(a + tab.pitch);
@@ -193,7 +197,7 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
             if (STEPREG) {
 #pragma unroll
                 for (int i = 0; i < 4; i++) st2[i] = st0[STEPREG ? 4 * j + i : 0];
-            } else if (TABLES && tab.half_steps) {
+            } else if (TABLES == 1) {
                 const uint4 w = lds128(tab.step + (has_ref ? 0u : 4u * tab.pitch) + j * tab.pitch);
                 const uint32_t hw[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
@@ -203,7 +207,7 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
                 }
             } else {
                 float4 s0, s1;
-                if (TABLES) {
+                if (TABLES == 2) {
                     const uint32_t a = tab.step + (has_ref ? 0u : 8u * tab.pitch) + 2 * j * tab.pitch;
                     s0 = lds128f(a);
                     s1 = lds128f(a + tab.pitch);
@@ -907,15 +911,14 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
     }
     __syncthreads();
     grid_dependency_wait();
-    int teams = TEAMS;       // at work
     SlabTables tab;
+    bool half_steps = true;
     if constexpr (TEAMS > 1) {
         const bool mine = warp < nstream && tid * 32 < d;
         const uint32_t t0 = smem_u32(smem_all) + TEAMS * align_up(L.total, 128);
         tab.pitch = (uint32_t)nstream * 512u;
         tab.inv = t0 + tid * 16u;
         tab.step = tab.inv + 16u * tab.pitch;
-        tab.half_steps = true;
         // row r, slot j of both tables by team (4r + j) mod TEAMS
         for (int q = team; mine && q < 8; q += TEAMS) {
             const int r = q >> 2, j = q & 3, c = r * d + tid * 32 + ((j + rot) & 3) * 8;
@@ -929,17 +932,14 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
             for (int i = 0; i < 4; i++) {
                 const __half2 h = __floats2half2_rn(v[2 * i], v[2 * i + 1]);
                 const float2 back = __half22float2(h);
-                tab.half_steps = tab.half_steps && back.x == v[2 * i] && back.y == v[2 * i + 1];
+                half_steps = half_steps && back.x == v[2 * i] && back.y == v[2 * i + 1];
                 hw[i] = *reinterpret_cast<const uint32_t *>(&h);
             }
             sts128(tab.step + (4 * r + j) * tab.pitch, make_uint4(hw[0], hw[1], hw[2], hw[3]));
         }
-        tab.half_steps = __syncthreads_and(tab.half_steps) != 0;
-        if (!tab.half_steps) {
-            // Steps that binary16 does not hold (calibrated tables are binary16 values): the last team stands back and its stages
-            // hold them as they are (the host sees to it that they fit).
-            teams = TEAMS - 1;
-            tab.step = smem_u32(smem_all) + (TEAMS - 1) * align_up(L.total, 128) + L.stage0 + tid * 16u;
+        half_steps = __syncthreads_and(half_steps) != 0;
+        if (!half_steps) {      // calibrated tables are binary16 values, a caller's own need not be
+            tab.step = tab.inv + 8u * tab.pitch;
             for (int q = team; mine && q < 8; q += TEAMS) {
                 const int r = q >> 2, j = q & 3, c = r * d + tid * 32 + ((j + rot) & 3) * 8;
                 sts128(tab.step + (8 * r + 2 * j) * tab.pitch, __ldg(reinterpret_cast<const uint4 *>(p.step + c)));
@@ -948,8 +948,8 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
             __syncthreads();
         }
     }
-    const int first = blockIdx.x + gridDim.x * team, stride = gridDim.x * teams;
-    const int n_my = (team < teams && p.T > first) ? (int)((p.T - first + stride - 1) / stride) : 0;
+    const int first = blockIdx.x + gridDim.x * team, stride = gridDim.x * TEAMS;
+    const int n_my = p.T > first ? (int)((p.T - first + stride - 1) / stride) : 0;
     auto token = [&](int k) -> long long { return first + (long long)k * stride; };   // this CTA's k-th token
     auto raw_row_of = [&](int k) -> int { return p.ref_row ? p.ref_row[token(k)] : (int)token(k); };
     // one lane: start the copies of this CTA's k-th token
@@ -980,10 +980,15 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
             const uint32_t xs = sbase + L.stage0 + stage * L.stage_bytes;
             if (!__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&ctrl->full[stage]), parity))) { timed_out = true; break; }
             const bool has_ref = REF ? true : ctrl->row[stage] >= 0;
-            if (valid)
-                encode_slab<BITS, true, XHAT, LPG, false, (TEAMS > 1)>(p, tid, lane, rot, d, Jc, false, coff, off, group_mask, xs, xs + row_bytes,
-                                                    has_ref, 0, stg + L.rec_off + parity * recb,
+            auto slab = [&](auto tables) {
+                encode_slab<BITS, true, XHAT, LPG, false, decltype(tables)::value>(p, tid, lane, rot, d, Jc, false, coff, off, group_mask, xs,
+                                                    xs + row_bytes, has_ref, 0, stg + L.rec_off + parity * recb,
                                                     reinterpret_cast<float *>(stg + L.tm_off), no_steps, tab);
+            };
+            if (valid) {
+                if (TEAMS > 1 && !half_steps) slab(std::integral_constant<int, TEAMS == 1 ? 0 : 2>{});
+                else slab(std::integral_constant<int, TEAMS == 1 ? 0 : 1>{});
+            }
             fence_async_smem();     // the record bytes written above will be read by the copy engine
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&ctrl->done[it & 3])) : "memory");
@@ -1794,7 +1799,7 @@ static int launch_teams_shape(const Geometry &g, CodecParams &p, const DeviceInf
     const TopSmem L = top_smem_layout(g.d, g.rec, (int)sizeof(TopSel<NSEL, true>));
     const int table = g.nthreads * 16;                  // bytes of a piece for all threads of a token
     const int smem = TEAMS * align_up(L.total, 128) + 24 * table, nt = TEAMS * (g.nthreads + 32 * NSEL);
-    if (smem > di.max_smem_optin || 16 * table > 2 * L.stage_bytes) return RAC_EUNSUPPORTED;
+    if (smem > di.max_smem_optin) return RAC_EUNSUPPORTED;
     constexpr int kMaxT = TEAMS * 32 * (NS + NSEL);
 #define RAC_TEAMS(G, W) launch_persistent(encode_top_kernel<BITS, KT, true, NV, NSEL, kMaxT, 1, G, W, false, TEAMS>, p, nt, smem, p.T, stream)
     if (D != 0 && g.d == D && g.lpg == 4) return RAC_TEAMS(4, D);

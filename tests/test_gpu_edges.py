@@ -612,7 +612,7 @@ def test_group_scales_keep_a_value_that_is_no_number_in_its_channel(env, bits, k
 def test_encode_in_teams_at_its_first_sizes(env, d, g, bits, k, per_sm, gathered, table):
     """The last token count of the other forms and the first of this one, where a team gets one token more than another: records
     as without x_hat (another kernel) and against the oracle, x_hat equal to the receiver's; steps that binary16 holds, and steps
-    that it does not (there one team stands back)."""
+    that it does not (these stand as binary32 over the second row of inverse steps)."""
     s, rac, P = env.synth, env.rac, env.P
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     T = per_sm * sms
