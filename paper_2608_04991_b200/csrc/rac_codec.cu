@@ -1791,9 +1791,15 @@ static bool one_launch(const Geometry &g, const CodecParams &p) {
 }
 // The one-launch form in teams: with x_hat, from 2080 to 7168 channels, where one CTA's shared memory holds the teams and the tables,
 // in calls of so many tokens that the tables' way there and the CTA's longer start are made up for.  NS: most streaming warps of
-// a team.  Tokens (CTA per token, or two launches in parentheses / teams, us): gathered rows 3000 x 5120 28.9 / 27.1, 6000 x 5120 51.2 /
-// 44.7, identity rows 6000 x 5120 44.2 / 46.4, 12000 x 5120 82.9 / 80.6; 2048 x 4096 16.5 / 16.6, 12000 x 4096 61.7 / 58.3; 2048 x 3072
-// 13.9 / 14.7, 12000 x 3072 50.9 / 49.0; 2048 x 6144 (about 25) / 24.4, 12000 x 6144 (about 103) / 94.4.
+// a team.  The line by the threads of a token (one_launch's choice / teams, us; rows g: gathered, 28 % direct):
+// up to 96, 64 tokens per SM: 8000 x 3072 35.3 / 35.6, 10000 44.6 / 43.0, 10000 x 2112 40.7 / 38.4;
+// up to 128, 54: 6000 x 4096 33.9 / 34.1, 8000 46.3 / 44.6, 8000 x 3584 49.1 / 42.1;
+// up to 160, identity rows, 160: 8000 x 5120 59.0 / 59.7, 12000 x 4608 83.7 / 84.4, 24000 x 4608 164.8 / 160.5, x 5120 169.6 / 165.3;
+// up to 160, rows g, 56, where one_launch goes over to two launches: 8000 x 4608 55.9 / 57.3, 8300 61.3 / 58.6, 12000 83.7 / 80.4; from
+// 4896 channels on 40, since the rows of the tables are more than L1 there: 6000 x 4864 43.7 / 45.8, x 5120 46.8 / 45.4, 8000 x 5120
+// 62.8 / 57.0;
+// beyond, where it is two launches from 1025 tokens on, 20: 2960 x 6144 32.5 / 30.6, g 33.5 / 28.8, 16000 136.6 / 126.9, g 139.0 / 123.0.
+// The width as a constant: 131072 x 5120 rows g 840 -> 828, 12000 82.3 -> 80.9, 12000 x 4096 61.7 -> 61.1.
 template <int BITS, int KT, int NV, int NS, int NSEL, int TEAMS, int D>
 static int launch_teams_shape(const Geometry &g, CodecParams &p, const DeviceInfo &di, cudaStream_t stream) {
     const TopSmem L = top_smem_layout(g.d, g.rec, (int)sizeof(TopSel<NSEL, true>));
@@ -1812,7 +1818,12 @@ static int launch_teams(const Geometry &g, CodecParams &p, cudaStream_t stream) 
     if (!p.X_hat || p.gain || g.nthreads <= 64 || g.nthreads > 224) return RAC_EUNSUPPORTED;
     DeviceInfo di;
     if (int rc = device_info(&di)) return rc;
-    const long long per_sm = g.nthreads > 160 || (g.nthreads > 128 && p.ref_row) ? 20 : 54;
+    const long long per_sm = g.nthreads <= 96    ? 64
+                             : g.nthreads <= 128 ? 54
+                             : g.nthreads > 160  ? 20
+                             : !p.ref_row        ? 160
+                             : g.d > 4864        ? 40
+                                                 : 56;
     if (p.T < per_sm * di.sms) return RAC_EUNSUPPORTED;
 #define RAC_TEAMS(B, K)                                                                             \
     (g.nthreads <= 96    ? launch_teams_shape<B, K, 3, 3, 2, 4, 0>(g, p, di, stream)                 \

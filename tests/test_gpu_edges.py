@@ -607,6 +607,11 @@ def test_group_scales_keep_a_value_that_is_no_number_in_its_channel(env, bits, k
     (7168, 256, 2, 8, 20, True),      # two teams, the widest
     (5376, 128, 4, 1, 20, False),
     (7168, 128, 4, 8, 20, True),      # two teams do not fit
+    (2112, 64, 3, 8, 64, False),      # the lines of up to 96 threads,
+    (5120, 128, 4, 8, 160, False),    # of up to 160 with identity rows,
+    (4608, 256, 4, 8, 56, True),      # with gathered rows,
+    (4896, 32, 2, 4, 40, True),       # and from 4896 channels on
+    (5120, 128, 4, 8, 40, True),
 ])
 @pytest.mark.parametrize("table", ["binary16", "binary32"])
 def test_encode_in_teams_at_its_first_sizes(env, d, g, bits, k, per_sm, gathered, table):
