@@ -390,7 +390,7 @@ def rac_sender_reconstruct(cfg, payload, T, ref_base, ref_rows, ref_row, ref_gai
 
 def rac_selftest_bounded_wait(cfg, which, inp, T, ref_base, ref_rows, step, inv_step, out, out_cap, workspace,
                               workspace_bytes, dev_status, stream=None) -> None:
-    """Runs the encode (which=0) or reconstruction (which=1) kernels with waits that cannot complete; see rac.h."""
+    """Runs the encode (which=0), reconstruction (1) or encode-and-reconstruct (2) kernels with waits that cannot complete; see rac.h."""
     _calls().rac_selftest_bounded_wait(cfg, which, inp, T, ref_base, ref_rows, step, inv_step, out, out_cap, workspace,
                                        workspace_bytes, dev_status, stream)
 

@@ -2277,8 +2277,15 @@ int rac_encode_reconstruct(const rac_codec_cfg *cfg, const void *X, int64_t T, c
 int rac_selftest_bounded_wait(const rac_codec_cfg *cfg, int32_t which, const void *in, int64_t T, const void *ref_base,
                               int64_t ref_rows, const float *step, const float *inv_step, void *out, size_t out_cap,
                               void *workspace, size_t workspace_bytes, uint32_t *dev_status, void *stream) {
-    if (T < 1 || T > 1024 || !dev_status) return RAC_EINVAL;
+    if (T < 1 || T > (which == 2 ? 16384 : 1024) || !dev_status) return RAC_EINVAL;
     const WaitTest wt = {16u};   // every stage announces 16 bytes that never come
+    if (which == 2) {
+        const size_t rec = rac_record_bytes(cfg), pay = (size_t)T * rec;
+        if (rec == 0 || !out) return RAC_EINVAL;
+        if (out_cap < pay + (size_t)T * (size_t)cfg->d * 2) return RAC_ESIZE;
+        return encode_impl(cfg, in, T, ref_base, ref_rows, nullptr, nullptr, nullptr, step, inv_step, out, pay,
+                           static_cast<uint8_t *>(out) + pay, workspace, workspace_bytes, dev_status, stream, Subset(), &wt);
+    }
     if (which == 0)
         return encode_impl(cfg, in, T, ref_base, ref_rows, nullptr, nullptr, nullptr, step, inv_step, out, out_cap, nullptr,
                            workspace, workspace_bytes, dev_status, stream, Subset(), &wt);

@@ -676,3 +676,33 @@ def test_encode_with_x_hat_in_two_launches(env, d, g, k, predictor):
     gb, bb = (None, None) if gain is None else (s.f16_bits(gain), s.f16_bits(bias))
     P.compare_encode(cfg, pay[(T - 300) * rec:], s.bf16_bits(X[at]), s.bf16_bits(R), rows[at].cpu().numpy(), gb, bb,
                      step.cpu().numpy(), inv.cpu().numpy())
+
+
+@pytest.mark.parametrize("d,bits,k,per_sm", [(4096, 4, 8, 54), (6144, 3, 5, 20)])
+@pytest.mark.parametrize("table", ["binary16", "binary32"])
+def test_teams_whose_waits_cannot_complete_give_up(env, d, bits, k, per_sm, table):
+    """The give-up path of the form in teams, in its safe shape: every stage announces more bytes than its copies deliver and each
+    wait gives up after its polls.  Every team of a CTA sets the status and returns, none waits for another without a bound, and
+    the next ordinary call on the stream gives the bits it always gives."""
+    s, rac, P, dev = env.synth, env.rac, env.P, env.dev
+    T = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + 1
+    gen = s.generator(d + bits, dev)
+    X = s.activations(T, d, s.channel_scale(d, 4, dev), gen)
+    R = s.affine_noisy_reference(X, 128, gen)
+    step = torch.full((2, d), 0.0625, device=dev) * (1.0 if table == "binary16" else 1.0 + 2.0 ** -14)
+    inv = 1.0 / step
+    cfg = rac.CodecCfg(d, 128, bits, k)
+    good = P.gpu_encode_reconstruct(cfg, X, R, None, None, None, step, inv)
+    assert good[2] == 0
+    n = T * rac.rac_record_bytes(cfg)
+    out = torch.zeros(n + 2 * T * d, dtype=torch.uint8, device=dev)
+    nws = rac.rac_encode_workspace_bytes(cfg, T)
+    ws = torch.zeros(max(nws, 16), dtype=torch.uint8, device=dev)
+    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    rac.rac_selftest_bounded_wait(cfg, 2, X, T, R, T, step, inv, out, out.numel(), ws if nws else None, nws, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) & rac.STATUS_TIMEOUT
+    with pytest.raises(rac.RacError):      # no room for x_hat behind the records
+        rac.rac_selftest_bounded_wait(cfg, 2, X, T, R, T, step, inv, out, out.numel() - 1, ws if nws else None, nws, status)
+    pay, xs, st = P.gpu_encode_reconstruct(cfg, X, R, None, None, None, step, inv)
+    assert st == 0 and np.array_equal(pay, good[0]) and torch.equal(xs, good[1])
