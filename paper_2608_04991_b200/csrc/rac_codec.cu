@@ -140,7 +140,11 @@ __device__ __forceinline__ float4 lds128f(uint32_t addr) {
 // One thread's 32 channels of one token, rows and record in shared memory: Eq. 6, Eq. 7, Eq. 8 with the static table, packing,
 // the sender-side reconstruction (over the X row), and the largest |e| of the slab.
 // STEPREG: every token has a reference, and the thread holds its steps (row 0 of the table, slot order) in st0.
-template <int BITS, bool TOPK, bool XHAT, int LPG, bool STEPREG, int TABLES = 0>
+// SATPACK: 4- and 2-bit codes beside x_hat through the saturating pack, as without x_hat, instead of the sum of shifted bits: that
+// is more operations in a shorter chain.  One CTA per token of up to 160 threads: gathered 2960 x 5120 24.7 us by the sum, 23.4 so,
+// x 4608 22.4 and 21.9, 64 x 4096 6.28 and 6.22; of more threads 300 x 6144 7.5 and 7.8; teams 16384 x 3072 63.7 and 64.8; the streaming pass
+// the same by either.
+template <int BITS, bool TOPK, bool XHAT, int LPG, bool STEPREG, int TABLES = 0, bool SATPACK = false>
 __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int lane, int rot, int d, int Jc, bool shared, int coff,
                                             const uint32_t (&off)[4], unsigned int group_mask, uint32_t xs, uint32_t rs,
                                             bool has_ref, int seg, unsigned char *rec, float *tm, const u64 (&st0)[STEPREG ? 16 : 1],
@@ -221,7 +225,7 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
         float ev[8];
         uint32_t xh[4];
         uint32_t w = 0;
-        if (BITS == 3 || XHAT) {
+        if (BITS == 3 || (XHAT && !SATPACK)) {
             // clamped on both sides: 3-bit codes have no saturating pack, and with x_hat the float is used again
             uint32_t bits8[8];
 #pragma unroll
@@ -247,7 +251,7 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
             }
             w = pack8_sum<BITS>(bits8);
         } else {
-            // 4- and 2-bit codes without x_hat: clamp from below in binary32, round by the magic add, take the integer
+            // 4- and 2-bit codes: clamp from below in binary32, round by the magic add, take the integer
             // out of the mantissa and let the saturating pack clamp from above (its range is
             // [-2^(BITS-1), 2^(BITS-1)-1], whose upper end is Qmax)
 #pragma unroll
@@ -258,10 +262,16 @@ __device__ __forceinline__ void encode_slab(const CodecParams &p, int tid, int l
                 unpack2(pmul(e, inv2[i]), v0, v1);
                 v0 = fmaxf(v0, -qmax);
                 v1 = fmaxf(v1, -qmax);
+                if (XHAT) { v0 = fminf(v0, qmax); v1 = fminf(v1, qmax); }  // the float is used again below
                 const u64 tt = padd(pack2(v0, v1), magic2);
                 unpack2(tt, t0, t1);
                 w = sat_pack2<BITS>((int)__float_as_uint(t1) - 0x4b400000, (int)__float_as_uint(t0) - 0x4b400000, w);
                 unpack2(e, ev[2 * i], ev[2 * i + 1]);
+                if (XHAT) {
+                    float x0, x1;
+                    unpack2(pfma(psub(tt, magic2), st2[i], rt), x0, x1);
+                    xh[i] = f2_to_bf16x2(x0, x1);
+                }
             }
         }
         words[j] = w;
@@ -981,9 +991,9 @@ __global__ void __launch_bounds__(MAXT, MINB) encode_top_kernel(const CodecParam
             if (!__all_sync(0xffffffffu, mbar_wait_bounded(smem_u32(&ctrl->full[stage]), parity))) { timed_out = true; break; }
             const bool has_ref = REF ? true : ctrl->row[stage] >= 0;
             auto slab = [&](auto tables) {
-                encode_slab<BITS, true, XHAT, LPG, false, decltype(tables)::value>(p, tid, lane, rot, d, Jc, false, coff, off, group_mask, xs,
-                                                    xs + row_bytes, has_ref, 0, stg + L.rec_off + parity * recb,
-                                                    reinterpret_cast<float *>(stg + L.tm_off), no_steps, tab);
+                encode_slab<BITS, true, XHAT, LPG, false, decltype(tables)::value, TEAMS == 1 && NV <= 5>(
+                    p, tid, lane, rot, d, Jc, false, coff, off, group_mask, xs, xs + row_bytes, has_ref, 0, stg + L.rec_off + parity * recb,
+                    reinterpret_cast<float *>(stg + L.tm_off), no_steps, tab);
             };
             if (valid) {
                 if (TEAMS > 1 && !half_steps) slab(std::integral_constant<int, TEAMS == 1 ? 0 : 2>{});
