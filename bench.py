@@ -31,11 +31,11 @@ if ROOT not in sys.path:
 METRIC = "codec GB/s of bf16 activations (encode+decode round trip)"
 UNIT = "GB/s"
 WORKLOAD = dict(T=131072, d=5120, group=128, bits=4, topk=8, n_hist=131072, min_ngram=4, max_hits=8, gap_max=112)
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one rac_encode[_reconstruct] call (with x_hat: streaming
-# kernel + outlier kernel) and of one reconstruction, from an ncu capture of the SMALL case (T = 16384, same d and record);
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one rac_encode[_reconstruct] call (one launch each) and of
+# one reconstruction, from an ncu capture of the SMALL case (T = 16384, same d and record);
 # traffic is proportional to tokens, so a launch of T tokens moves T/16384 times as much.
-NCU_SMALL_CASE_TRAFFIC = {"encode_sender_up": 267.61e6 + 180.88e6 + 51.14e6 + 2.19e6,
-                          "encode_dn": 335.65e6 + 36.15e6,
+NCU_SMALL_CASE_TRAFFIC = {"encode_sender_up": 272.47e6 + 176.71e6,
+                          "encode_dn": 335.65e6 + 36.32e6,
                           "decode_up": 141.30e6 + 119.66e6, "decode_dn": 212.91e6 + 122.85e6}
 SMALL = dict(T=16384, d=5120, group=128, bits=4, topk=8, n_hist=16384, min_ngram=4, max_hits=8, gap_max=112)
 
@@ -132,7 +132,7 @@ class ClockSampler:
 # --------------------------------------------------------------------------------------------- workload
 class RoundTrip:
     """Device buffers and the ordered C-ABI calls of one step."""
-    LAUNCHES_PER_STEP = 5 + 2 + 1 + 2  # matcher kernels, encode with x_hat (two launches), encode, 2 reconstructions
+    LAUNCHES_PER_STEP = 5 + 1 + 1 + 2  # matcher kernels, encode with x_hat, encode, 2 reconstructions
 
     def __init__(self, wl, seed, dev, token_range=None):
         import numpy as np
@@ -850,7 +850,7 @@ def main():
         enc_ms = stage_ms[ix["encode_sender_up"]] + stage_ms[ix["encode_dn"]]
         dec_ms = stage_ms[ix["decode_up"]] + stage_ms[ix["decode_dn"]]
         if enc_ms >= dec_ms:
-            dom, dom_bytes, dom_ms, dom_n = ("rac_encode_reconstruct (encode_ws_kernel + outlier_kernel), rac_encode (encode_top_kernel)",
+            dom, dom_bytes, dom_ms, dom_n = ("rac_encode_reconstruct (encode_top_kernel in teams), rac_encode (encode_top_kernel)",
                                              rt.bytes_of("encode_sender_up") + rt.bytes_of("encode_dn"), enc_ms, 2)
         else:
             dom, dom_bytes, dom_ms, dom_n = ("decode_ws_kernel<4,8>", rt.bytes_of("decode_up") + rt.bytes_of("decode_dn"),

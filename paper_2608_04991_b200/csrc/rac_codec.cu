@@ -845,10 +845,11 @@ __global__ void __launch_bounds__(W * 32, W == 7 ? 4 : 3) outlier_kernel(const C
 // Teams: with x_hat a token needs the inverse steps and the steps, in calls with direct tokens two rows of each, and several CTAs
 // per SM each with their stages leave them too little L1.  So in calls of many tokens an SM runs ONE CTA of several teams, each
 // of which is what is a CTA otherwise (its streaming and selector warps, stages and barriers), and all of them read one copy of the tables in
-// shared memory (SlabTables).  131072 x 5120, 28 % direct tokens, in long runs: 759 us against 915 with a CTA per token and 717
-// and about 130 in two launches; 100000 x 4096 487 -> 439, x 3072 382 -> 348, x 6144 708 against 704 and about 100; long uplink with
-// retrieval 926 -> 812.  (More teams with fewer registers, four at 4096 channels, 437 and spills.)
-// Teams without x_hat (one row in L1 is no trouble there) 574 against 568.
+// shared memory (SlabTables).  131072 x 5120, 28 % direct tokens, in long runs: 828 us against 966 with a CTA per token and 899 in two
+// launches; 65536 x 4096 305 against 348 with a CTA per token, x 3072 238 against 269, 16000 x 6144 123 against 139 in two launches; long
+// uplink with retrieval 944 -> 856.  The registers spill a little at five streaming and three selector warps (80 of them, 32 bytes); two
+// selectors at 96 registers do not and take 852 us, since a token's selection is the longer chain.  (Four teams with fewer registers
+// at 4096 channels 437 against 439 us, and spills.)  Teams without x_hat (one row in L1 is no trouble there) 574 against 568.
 struct TopCtrl {
     unsigned long long full[2];     // data of the stage has landed
     unsigned long long done[4];     // every streaming warp has finished token (mod 4)
