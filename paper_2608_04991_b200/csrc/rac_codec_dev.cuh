@@ -375,9 +375,10 @@ __device__ __forceinline__ void group_sum2(float &a, float &b, int lpg, unsigned
 // mixed adds above: half the registers of unpacked rows and no unpacking (streaming pass at 131072 x 5120, group 128,
 // 4-bit: with outliers 528 -> 485 us, without 516 -> 467 us, with x_hat 726 -> 700 us).
 // Sums of products in one pass, the means' part taken out afterwards, are less work only where means are small beside the
-// spread, and need the centred pass behind them where they are not: 131072 x 5120, 4-bit, eight outliers, groups of 128 616 us so,
-// 583 to 588 in one pass with means of zero, but 695 to 709 with means of 0.6 of the spread and more (16384 x 4096, 3-bit 65.1, 62.7 and
-// 72.7; groups of 1024 72.3, 70.7 and 86); and from groups of 256 on the error of alpha against 64 bits is up to 6 % larger.
+// spread, and need the centred pass behind them where they are not.  131072 x 5120, 4-bit, eight outliers, groups of 128: 599 us so,
+// 579 in one pass with means of zero, but 696 with means of 0.6 of the spread and 701 where only the token has one; with a vote on the
+// reference's mean before the token enters its products 581, 633 and 698 (16384 x 4096, 3-bit 62.9, 62.0, 71.6 and 71.7; 61.8, 66.2 and
+// 71.4; groups of 1024 71, 69, 85 and 86; 70, 75 and 87).  From groups of 256 on its error of alpha against 64 bits is up to 6 % larger.
 __device__ __forceinline__ uint32_t fit_group(const uint32_t (&xw)[16], const uint32_t (&rw)[16], bool has_ref, int lpg,
                                               float inv_group, unsigned int group_mask, uint32_t *status, u64 &a2, u64 &b2,
                                               float4 *stats = nullptr) {
